@@ -66,8 +66,8 @@ typedef enum {
                           correlations over the scan grid (Methods, Efficient
                           reconstruction based on scanning symmetries), restated
                           exactly by the correlation theorem on a zero-padded
-                          P x P grid (P a power of two >= max(py, px) + R, at most
-                          2048), with the slab's real lateral spectrum stored once
+                          P x P grid (P >= max(py, px) + R, an even size with factors
+                          2, 3 and 5 up to 512, else 1024 or 2048), with the slab's real lateral spectrum stored once
                           per frequency orbit */
 } oam_precision;
 

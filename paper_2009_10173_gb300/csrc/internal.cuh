@@ -182,6 +182,18 @@ double fft_flops(const oam_model *m);
 double fft_bytes(const oam_model *m);
 oam_status fft_plan_bytes(const oam_model *m, size_t *bytes);
 
+// mix_rows.cu, mix_cols.cu: transforms of the lateral-FFT form at the
+// mixed-radix sizes.  mix_size_for: the smallest such size >= need, 0 beyond
+// the largest; tw: the size's roots (mix_roots) in device memory.
+int mix_size_for(int need);
+std::vector<float2> mix_roots(int P);
+oam_status mix_rows_r2c(int P, cudaStream_t st, const float *X, int py, int px, int Ctot, int c0, int C,
+                        const float2 *tw, float2 *Y);
+oam_status mix_cols(int P, bool inverse, cudaStream_t st, const float2 *Z, int nin, int nout, int C, const float2 *tw,
+                    float2 *W);
+oam_status mix_rows_c2r(int P, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0, int C,
+                        const float2 *tw, float scale, float *X);
+
 // op_filter.cu: y = F x over the model's py*px A-lines (x and y may alias)
 oam_status fir_apply(const oam_model *m, const float *x, float *y, cudaStream_t st);
 float *fir_stage(const oam_model *m);

@@ -3,8 +3,8 @@
 // A and A^T are 2-D correlations of the single-position slab with the volume
 // over the scan grid (Methods, Efficient reconstruction based on scanning
 // symmetries: the model is the same for every scanning position).  With the
-// volume and the signals zero-padded to P x P, P a power of two with
-// P >= max(py, px) + R, no circular wrap reaches the output window, and the
+// volume and the signals zero-padded to P x P, P >= max(py, px) + R one of the
+// mixed-radix transform sizes up to 512 or a power of two, no circular wrap reaches the output window, and the
 // correlation theorem restates both operators exactly per lateral frequency
 // (v, u):
 //   A:    s^(v,u,n) = sum_k S^(v,u,k,n) H^(v,u,k)
@@ -21,9 +21,10 @@
 // u in [0, P/2]), FFT along y, the per-orbit banded real matrix times up to
 // four complex frequency vectors, inverse FFT along y, inverse FFT along x
 // back to real rows (Hermitian extension) with zero fill outside the band.
-// FFTs are radix-2 in shared memory with twiddles from sincospi; every sum
-// runs in a fixed order, so results are deterministic.
+// The transforms keep their points in registers between trips through shared
+// memory; every sum runs in a fixed order, so results are deterministic.
 #include <algorithm>
+#include <cmath>
 #include <set>
 #include <vector>
 
@@ -35,8 +36,10 @@ using namespace oam;
 namespace oam {
 
 struct FftLayout {
-  int P = 0, lgP = 0, Q = 0;  // transform size, its log2, half-spectrum columns P/2 + 1
-  int KC = 0;                 // channels per FFT block
+  int P = 0, lgP = 0, Q = 0;  // transform size, its log2 (powers of two above 512), half-spectrum columns P/2 + 1
+  int KC = 0;                 // channels per FFT block (power-of-two kernels)
+  float2 *d_tw = nullptr;     // [P] roots W_P^j of the mixed-radix kernels; none for P > 512
+  bool mixed = false;         // a mixed-radix size
   bool d4 = false;            // S^(v,u) = S^(u,v)
   int n_rep = 0;              // frequency orbits
   int NS = 0;                 // support length n_hi - n_lo
@@ -72,113 +75,9 @@ constexpr int kAdjChunk = 160;  // adjoint products: depths per block (0: all de
 constexpr int kBuildThreads = 128;
 
 
-// Real rows -> half spectrum along x.  X[py][px][Ctot] (channels c0 .. c0+C-1
-// used), Y[Q][py][C] complex.  Block (y, channel block of KC).  Channels l and
-// l + KC/2 ride as the real and imaginary parts of one complex line; with
-// Z = FFT(x + i y), X(u) = (Z(u) + conj Z(-u)) / 2 and Y(u) = (Z(u) - conj Z(-u)) / 2i.
-template <int KC>
-__global__ void __launch_bounds__(kFftThreads) k_fft_rows_r2c(const float *__restrict__ X, int py, int px, int Ctot,
-                                                              int c0, int C, int P, int lgP, int Q,
-                                                              float2 *__restrict__ Y) {
-  constexpr int KH = KC / 2;  // complex lines
-  extern __shared__ float2 sm[];
-  float2 *tw = sm, *a = sm + (P >> 1);
-  const int y = blockIdx.x, cb = blockIdx.y * KC;
-  load_twiddles(tw, P);
-  for (int i = threadIdx.x; i < P * KH; i += blockDim.x) {
-    const int x = i / KH, l = i % KH;
-    float re = 0.0f, im = 0.0f;
-    if (x < px) {
-      const float *row = X + ((size_t)y * px + x) * Ctot + c0 + cb;
-      if (cb + l < C) re = row[l];
-      if (cb + l + KH < C) im = row[l + KH];
-    }
-    a[bitrev(x, lgP) * KH + l] = make_float2(re, im);
-  }
-  fft_lines<KH>(a, tw, P, lgP, false);
-  for (int i = threadIdx.x; i < Q * KC; i += blockDim.x) {
-    const int u = i / KC, c = i % KC, l = c % KH;
-    if (cb + c >= C) continue;
-    const float2 z = a[u * KH + l], w = a[((P - u) & (P - 1)) * KH + l];
-    Y[((size_t)u * py + y) * C + cb + c] = c < KH ? make_float2(0.5f * (z.x + w.x), 0.5f * (z.y - w.y))
-                                                  : make_float2(0.5f * (z.y + w.y), 0.5f * (w.x - z.x));
-  }
-}
-
-// Complex transform along the row index of Z[Q][nin][C] -> W[Q][nout][C]
-// (rows >= nin read as zero, rows >= nout dropped).  Block (u, channel block).
-template <int KC>
-__global__ void __launch_bounds__(kFftThreads) k_fft_cols(const float2 *__restrict__ Z, int nin, int nout, int C, int P,
-                                                          int lgP, int inverse, float2 *__restrict__ W) {
-  extern __shared__ float2 sm[];
-  float2 *tw = sm, *a = sm + (P >> 1);
-  const int u = blockIdx.x, cb = blockIdx.y * KC;
-  load_twiddles(tw, P);
-  for (int i = threadIdx.x; i < P * KC; i += blockDim.x) {
-    const int r = i / KC, c = i % KC;
-    float2 v = make_float2(0.0f, 0.0f);
-    if (r < nin && cb + c < C) v = Z[((size_t)u * nin + r) * C + cb + c];
-    a[bitrev(r, lgP) * KC + c] = v;
-  }
-  fft_lines<KC>(a, tw, P, lgP, inverse != 0);
-  for (int i = threadIdx.x; i < nout * KC; i += blockDim.x) {
-    const int r = i / KC, c = i % KC;
-    if (cb + c < C) W[((size_t)u * nout + r) * C + cb + c] = a[r * KC + c];
-  }
-}
-
-// Half spectrum along x -> real rows, scaled by 1/P^2.  Z[Q][py][C] holds
-// channels c0 .. c0+C-1 of the output X[py][px][Ctot]; every other output
-// channel is written as zero.  Block (y, output channel block of KC).
-// Channels l and l + KC/2 share one complex line W = X + i Y (each extended
-// Hermitian, the imaginary parts of its u = 0 and u = P/2 terms dropped): the
-// inverse transform's real and imaginary parts are the two real rows.
-template <int KC>
-__global__ void __launch_bounds__(kFftThreads) k_fft_rows_c2r(const float2 *__restrict__ Z, int py, int px, int Ctot,
-                                                              int c0, int C, int P, int lgP, int Q,
-                                                              float scale, float *__restrict__ X) {
-  constexpr int KH = KC / 2;
-  extern __shared__ float2 sm[];
-  float2 *tw = sm, *a = sm + (P >> 1);
-  const int y = blockIdx.x, ob = blockIdx.y * KC;
-  if (ob >= c0 + C || ob + KC <= c0) {  // block entirely outside the band: zeros
-    for (int i = threadIdx.x; i < px * KC; i += blockDim.x) {
-      const int x = i / KC, c = i % KC;
-      if (ob + c < Ctot) X[((size_t)y * px + x) * Ctot + ob + c] = 0.0f;
-    }
-    return;
-  }
-  load_twiddles(tw, P);
-  for (int i = threadIdx.x; i < P * KH; i += blockDim.x) {
-    const int f = i / KH, l = i % KH;
-    const int fh = f < Q ? f : P - f;  // Hermitian source column
-    float2 xs = make_float2(0.0f, 0.0f), ys = make_float2(0.0f, 0.0f);
-    const int zx = ob + l - c0, zy = ob + l + KH - c0;
-    if (zx >= 0 && zx < C) xs = Z[((size_t)fh * py + y) * C + zx];
-    if (zy >= 0 && zy < C) ys = Z[((size_t)fh * py + y) * C + zy];
-    if (f == 0 || f == (P >> 1)) {
-      xs.y = 0.0f;
-      ys.y = 0.0f;
-    } else if (f >= Q) {
-      xs.y = -xs.y;
-      ys.y = -ys.y;
-    }
-    a[bitrev(f, lgP) * KH + l] = make_float2(xs.x - ys.y, xs.y + ys.x);
-  }
-  fft_lines<KH>(a, tw, P, lgP, true);
-  for (int i = threadIdx.x; i < px * KC; i += blockDim.x) {
-    const int x = i / KC, c = i % KC, l = c % KH;
-    const int oc = ob + c, zc = oc - c0;
-    if (oc >= Ctot) continue;
-    const float2 v = a[x * KH + l];
-    X[((size_t)y * px + x) * Ctot + oc] = (zc >= 0 && zc < C) ? (c < KH ? v.x : v.y) * scale : 0.0f;
-  }
-}
-
-// ---- transforms in register passes (P >= 16) ------------------------------
-// The kernels above move every point through shared memory once per two
-// radix-2 stages and scatter it to its bit-reversed slot first.  The kernels
-// below run up to four stages per pass in registers: a forward transform is
+// ---- power-of-two transforms in register passes (P = 1024, 2048) -----------
+// Sizes up to 512 run in the mixed-radix kernels (mix_rows.cu, mix_cols.cu).
+// The kernels below run up to four stages per pass in registers: a forward transform is
 // decimation in frequency (natural order in, bit-reversed out: the point at
 // position i ends as frequency bitrev(i), which goes to global row bitrev(i)),
 // an inverse transform decimation in time (position i loads frequency
@@ -317,7 +216,7 @@ __device__ __forceinline__ void xtransform(float2 *a, int P, int lgP, First firs
   }
 }
 
-// k_fft_rows_r2c in register passes (P >= 16): same arguments and results.
+// Real rows -> half spectrum along x (arguments and results as k_mix_rows_r2c).
 template <int KC>
 __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_r2c(const float *__restrict__ X, int py, int px, int Ctot,
                                                                int c0, int C, int P, int lgP, int Q,
@@ -347,7 +246,7 @@ __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_r2c(const float *__re
   }
 }
 
-// k_fft_cols in register passes (P >= 16): same arguments and results.
+// Complex transform along the row index (as k_mix_cols).
 template <int KC, bool kInverse>
 __global__ void __launch_bounds__(kFftThreads) k_xfft_cols(const float2 *__restrict__ Z, int nin, int nout, int C,
                                                            int P, int lgP, float2 *__restrict__ W) {
@@ -366,7 +265,7 @@ __global__ void __launch_bounds__(kFftThreads) k_xfft_cols(const float2 *__restr
   xtransform<KC, !kInverse, false>(sm, P, lgP, load, store);
 }
 
-// k_fft_rows_c2r in register passes (P >= 16): same arguments and results.
+// Half spectrum along x -> real rows (as k_mix_rows_c2r).
 template <int KC>
 __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_c2r(const float2 *__restrict__ Z, int py, int px, int Ctot,
                                                                int c0, int C, int P, int lgP, int Q, float scale,
@@ -618,7 +517,11 @@ __global__ void __launch_bounds__(kBuildThreads) k_shat_pass1(const float *__res
   }
   for (int u = 0; u < Q; ++u) {
     float acc = 0.0f;
-    for (int ap = 0; ap <= R; ++ap) acc = fmaf(cosT[(u * ap) & (P - 1)], sv[ap * ts + tid], acc);
+    for (int ap = 0, j = 0; ap <= R; ++ap) {  // j = u ap mod P
+      acc = fmaf(cosT[j], sv[ap * ts + tid], acc);
+      j += u;
+      if (j >= P) j -= P;
+    }
     T[((size_t)bp * Q + u) * row_len + e] = acc;
   }
 }
@@ -652,13 +555,15 @@ __global__ void __launch_bounds__(kBuildThreads) k_shat_pass2(const float *__res
     const int r = rep_of[v0 * Q + u0];
     if (r < 0) continue;
     float acc = 0.0f;
-    for (int bp = 0; bp <= R; ++bp) acc = fmaf(cosT[(v0 * bp) & (P - 1)], tv[bp * ts + tid], acc);
+    for (int bp = 0, j = 0; bp <= R; ++bp) {  // j = v0 bp mod P
+      acc = fmaf(cosT[j], tv[bp * ts + tid], acc);
+      j += v0;
+      if (j >= P) j -= P;
+    }
     shat[(size_t)r * stride + e] = acc;
     shat_t[(size_t)r * stride_t + et] = acc;
   }
 }
-
-size_t fft_smem(int P, int KC) { return sizeof(float2) * ((size_t)(P >> 1) + (size_t)P * KC); }
 
 // Host tables of the lateral-FFT layout, planned from the model's bands.
 struct FftPlan {
@@ -672,17 +577,25 @@ struct FftPlan {
 // Fill L's sizes and the host tables (no device call).
 oam_status fft_plan(const oam_model *m, FftLayout *L, FftPlan &pl) {
   const int R = m->R, W = m->W, nz = m->grid.nz;
+  // The transform size is the smallest mixed-radix one that the scan and its
+  // halo fit (S^ grows with its square: 96 for 64 positions and R = 30, 160
+  // for 128, 288 for 256); beyond 512 the next power of two.
   const int need = std::max(m->grid.py, m->grid.px) + R;
-  int P = 2, lgP = 1;
-  while (P < need) {
-    P <<= 1;
-    ++lgP;
+  int P = mix_size_for(need), lgP = 0;
+  L->mixed = P > 0;
+  if (!P) {
+    P = 1024;
+    lgP = 10;
+    while (P < need) {
+      P <<= 1;
+      ++lgP;
+    }
   }
   if (P > 2048) return OAM_ERR_UNSUPPORTED;
   L->P = P;
   L->lgP = lgP;
   L->Q = P / 2 + 1;
-  L->KC = std::max(2, std::min(16, 4096 / P));
+  L->KC = 4096 / P;  // power-of-two kernels: 4 or 2
   const int Q = L->Q;
   // D4 when the tap -> orbit map is symmetric under b <-> a
   L->d4 = true;
@@ -770,7 +683,7 @@ oam_status fft_plan(const oam_model *m, FftLayout *L, FftPlan &pl) {
 
 // Device bytes fft_build allocates and keeps (host only).
 oam_status fft_layout_bytes(const FftLayout &L, const FftPlan &pl, int nz, size_t *bytes) {
-  *bytes = alloc_bytes<int>(nz) * 2 + alloc_bytes<long long>(nz) + alloc_bytes<int4>(pl.members.size()) +
+  *bytes = (L.mixed ? alloc_bytes<float2>(L.P) : 0) + alloc_bytes<int>(nz) * 2 + alloc_bytes<long long>(nz) + alloc_bytes<int4>(pl.members.size()) +
            alloc_bytes<int2>(L.NS) + alloc_bytes<long long>(L.NS) +
            alloc_bytes<float>((size_t)L.n_rep * L.row_stride_t) + alloc_bytes<float>((size_t)L.n_rep * L.row_stride) +
            2 * alloc_bytes<float2>((size_t)L.Q * L.P * L.C);
@@ -797,7 +710,7 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
     oam_status rc0 = fft_plan(m, L, pl);
     if (rc0) return rc0;
   }
-  const int P = L->P, Q = L->Q, lgP = L->lgP;
+  const int P = L->P, Q = L->Q;
   std::vector<int> &klo = pl.klo, &klen = pl.klen, &rep_of = pl.rep_of;
   std::vector<long long> &koff = pl.koff, &noff = pl.noff;
   std::vector<int2> &krange = pl.krange, &entry_kn = pl.entry_kn;
@@ -810,6 +723,12 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
       (rc = dev_alloc(m, &L->d_shat, (size_t)L->n_rep * L->row_stride)) ||
       (rc = dev_alloc(m, &L->d_w1, (size_t)Q * P * L->C)) || (rc = dev_alloc(m, &L->d_w2, (size_t)Q * P * L->C)))
     return rc;
+  std::vector<float2> roots;
+  if (L->mixed) {
+    if ((rc = dev_alloc(m, &L->d_tw, (size_t)P))) return rc;
+    roots = mix_roots(P);
+    OAM_CUDA_TRY(cudaMemcpyAsync(L->d_tw, roots.data(), sizeof(float2) * P, cudaMemcpyHostToDevice, st));
+  }
   OAM_CUDA_TRY(cudaMemcpyAsync(L->d_klo, klo.data(), sizeof(int) * nz, cudaMemcpyHostToDevice, st));
   OAM_CUDA_TRY(cudaMemcpyAsync(L->d_klen, klen.data(), sizeof(int) * nz, cudaMemcpyHostToDevice, st));
   OAM_CUDA_TRY(cudaMemcpyAsync(L->d_koff, koff.data(), sizeof(long long) * nz, cudaMemcpyHostToDevice, st));
@@ -861,7 +780,7 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
   const double half = (double)Q * P;
   const double fft_lines = (double)m->grid.py * m->grid.nz + half / P * m->grid.nz + half / P * L->NS +
                            (double)m->grid.py * L->NS;
-  L->flops = 4.0 * half * (double)L->row_len + 5.0 * P * lgP * fft_lines;
+  L->flops = 4.0 * half * (double)L->row_len + 5.0 * P * std::log2((double)P) * fft_lines;
   const double c8 = sizeof(float2);
   L->bytes = 4.0 * (double)L->n_rep * L->row_len +                              // S^
              4.0 * vol_elems(m) + 4.0 * (double)m->grid.py * m->grid.px * m->grid.nt +  // input, output
@@ -873,7 +792,7 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
 void oam::fft_free(oam_model *m, cudaStream_t st) {
   FftLayout *L = m->fft;
   if (!L) return;
-  for (void *p : {(void *)L->d_klo, (void *)L->d_klen, (void *)L->d_koff, (void *)L->d_members, (void *)L->d_krange,
+  for (void *p : {(void *)L->d_tw, (void *)L->d_klo, (void *)L->d_klen, (void *)L->d_koff, (void *)L->d_members, (void *)L->d_krange,
                   (void *)L->d_noff, (void *)L->d_shat_t, (void *)L->d_shat,
                   (void *)L->d_w1, (void *)L->d_w2})
     if (p) cudaFreeAsync(p, st);
@@ -900,74 +819,66 @@ namespace {
 // four-stage passes (KL lines x P/16 groups), 64 to 256.
 int xthreads(int P, int KL) { return std::max(64, std::min(kFftThreads, (((P >> 4) * KL + 31) / 32) * 32)); }
 
-// The transforms of one application in register passes (P >= 16); the
-// spectral products are launched by run_fft between them.
+// The transforms of one application, KC channels per block; the spectral
+// products are launched by run_fft between them.  Register passes (P = 1024, 2048).
 template <int KC>
 struct XKernels {
-  static oam_status prepare(int P) {
-    oam_status rc;
-    const size_t sr = sizeof(float2) * xslots<KC / 2>(P), sc = sizeof(float2) * xslots<KC>(P);
-    if ((rc = set_smem((const void *)k_xfft_rows_r2c<KC>, sr)) || (rc = set_smem((const void *)k_xfft_rows_c2r<KC>, sr)) ||
-        (rc = set_smem((const void *)k_xfft_cols<KC, false>, sc)) || (rc = set_smem((const void *)k_xfft_cols<KC, true>, sc)))
-      return rc;
+  static oam_status rows_r2c(const FftLayout *L, cudaStream_t st, const float *X, int py, int px, int Ctot, int c0,
+                             int C, float2 *Y) {
+    const size_t sm = sizeof(float2) * xslots<KC / 2>(L->P);
+    oam_status rc = set_smem((const void *)k_xfft_rows_r2c<KC>, sm);
+    if (rc) return rc;
+    k_xfft_rows_r2c<KC><<<dim3(py, (C + KC - 1) / KC), xthreads(L->P, KC / 2), sm, st>>>(X, py, px, Ctot, c0, C, L->P,
+                                                                                        L->lgP, L->Q, Y);
+    OAM_LAUNCHED();
     return OAM_OK;
   }
-  static void rows_r2c(dim3 g, cudaStream_t st, const float *X, int py, int px, int Ctot, int c0, int C, int P, int lgP,
-                       int Q, float2 *Y) {
-    k_xfft_rows_r2c<KC><<<g, xthreads(P, KC / 2), sizeof(float2) * xslots<KC / 2>(P), st>>>(X, py, px, Ctot, c0, C, P,
-                                                                                           lgP, Q, Y);
+  template <bool kInverse>
+  static oam_status cols(const FftLayout *L, cudaStream_t st, const float2 *Z, int nin, int nout, int C, float2 *W) {
+    const size_t sm = sizeof(float2) * xslots<KC>(L->P);
+    oam_status rc = set_smem((const void *)k_xfft_cols<KC, kInverse>, sm);
+    if (rc) return rc;
+    k_xfft_cols<KC, kInverse><<<dim3(L->Q, (C + KC - 1) / KC), xthreads(L->P, KC), sm, st>>>(Z, nin, nout, C, L->P,
+                                                                                            L->lgP, W);
+    OAM_LAUNCHED();
+    return OAM_OK;
   }
-  static void cols(dim3 g, cudaStream_t st, const float2 *Z, int nin, int nout, int C, int P, int lgP, int inverse,
-                   float2 *W) {
-    if (inverse)
-      k_xfft_cols<KC, true><<<g, xthreads(P, KC), sizeof(float2) * xslots<KC>(P), st>>>(Z, nin, nout, C, P, lgP, W);
-    else
-      k_xfft_cols<KC, false><<<g, xthreads(P, KC), sizeof(float2) * xslots<KC>(P), st>>>(Z, nin, nout, C, P, lgP, W);
-  }
-  static void rows_c2r(dim3 g, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0, int C, int P,
-                       int lgP, int Q, float scale, float *X) {
-    k_xfft_rows_c2r<KC><<<g, xthreads(P, KC / 2), sizeof(float2) * xslots<KC / 2>(P), st>>>(Z, py, px, Ctot, c0, C,
-                                                                                           P, lgP, Q, scale, X);
+  static oam_status rows_c2r(const FftLayout *L, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0,
+                             int C, float scale, float *X) {
+    const size_t sm = sizeof(float2) * xslots<KC / 2>(L->P);
+    oam_status rc = set_smem((const void *)k_xfft_rows_c2r<KC>, sm);
+    if (rc) return rc;
+    k_xfft_rows_c2r<KC><<<dim3(py, (Ctot + KC - 1) / KC), xthreads(L->P, KC / 2), sm, st>>>(
+        Z, py, px, Ctot, c0, C, L->P, L->lgP, L->Q, scale, X);
+    OAM_LAUNCHED();
+    return OAM_OK;
   }
 };
 
-// The same in the radix-2 kernels (any P).
-template <int KC>
-struct RKernels {
-  static oam_status prepare(int P) {
-    oam_status rc;
-    const size_t sm = fft_smem(P, KC), smr = fft_smem(P, KC / 2);  // row kernels: two channels per line
-    if ((rc = set_smem((const void *)k_fft_rows_r2c<KC>, smr)) || (rc = set_smem((const void *)k_fft_cols<KC>, sm)) ||
-        (rc = set_smem((const void *)k_fft_rows_c2r<KC>, smr)))
-      return rc;
-    return OAM_OK;
+// The same in the mixed-radix kernels (P <= 512).
+struct MKernels {
+  static oam_status rows_r2c(const FftLayout *L, cudaStream_t st, const float *X, int py, int px, int Ctot, int c0,
+                             int C, float2 *Y) {
+    return mix_rows_r2c(L->P, st, X, py, px, Ctot, c0, C, L->d_tw, Y);
   }
-  static void rows_r2c(dim3 g, cudaStream_t st, const float *X, int py, int px, int Ctot, int c0, int C, int P, int lgP,
-                       int Q, float2 *Y) {
-    k_fft_rows_r2c<KC><<<g, kFftThreads, fft_smem(P, KC / 2), st>>>(X, py, px, Ctot, c0, C, P, lgP, Q, Y);
+  template <bool kInverse>
+  static oam_status cols(const FftLayout *L, cudaStream_t st, const float2 *Z, int nin, int nout, int C, float2 *W) {
+    return mix_cols(L->P, kInverse, st, Z, nin, nout, C, L->d_tw, W);
   }
-  static void cols(dim3 g, cudaStream_t st, const float2 *Z, int nin, int nout, int C, int P, int lgP, int inverse,
-                   float2 *W) {
-    k_fft_cols<KC><<<g, kFftThreads, fft_smem(P, KC), st>>>(Z, nin, nout, C, P, lgP, inverse, W);
-  }
-  static void rows_c2r(dim3 g, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0, int C, int P,
-                       int lgP, int Q, float scale, float *X) {
-    k_fft_rows_c2r<KC><<<g, kFftThreads, fft_smem(P, KC / 2), st>>>(Z, py, px, Ctot, c0, C, P, lgP, Q, scale, X);
+  static oam_status rows_c2r(const FftLayout *L, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0,
+                             int C, float scale, float *X) {
+    return mix_rows_c2r(L->P, st, Z, py, px, Ctot, c0, C, L->d_tw, scale, X);
   }
 };
 
-template <int KC, class K>
+template <class K>
 oam_status run_fft(const oam_model *m, const FftLayout *L, bool fwd, const float *in, float *out, cudaStream_t st) {
-  const int P = L->P, Q = L->Q, lgP = L->lgP, nz = m->grid.nz, py = m->grid.py, px = m->grid.px, NS = L->NS;
-  oam_status rc = K::prepare(P);
-  if (rc) return rc;
-  const unsigned cbz = (unsigned)((nz + KC - 1) / KC), cbs = (unsigned)((NS + KC - 1) / KC);
+  const int P = L->P, nz = m->grid.nz, py = m->grid.py, px = m->grid.px, NS = L->NS;
+  oam_status rc;
   const float scale = 1.0f / ((float)P * (float)P);
   if (fwd) {
-    K::rows_r2c(dim3(py, cbz), st, in, py, px, nz, 0, nz, P, lgP, Q, L->d_w2);
-    OAM_LAUNCHED();
-    K::cols(dim3(Q, cbz), st, L->d_w2, py, P, nz, P, lgP, 0, L->d_w1);
-    OAM_LAUNCHED();
+    if ((rc = K::rows_r2c(L, st, in, py, px, nz, 0, nz, L->d_w2))) return rc;
+    if ((rc = K::template cols<false>(L, st, L->d_w2, py, P, nz, L->d_w1))) return rc;
     const size_t sa = sizeof(float4) * 2 * nz + sizeof(int) * (2 * nz + 2) + sizeof(long long) * nz;
     if ((rc = set_smem((const void *)k_fft_apply_fwd, sa))) return rc;
     const int fchunk = kFwdChunk > 0 ? kFwdChunk : NS;
@@ -976,16 +887,11 @@ oam_status run_fft(const oam_model *m, const FftLayout *L, bool fwd, const float
     k_fft_apply_fwd<<<fblocks, fwd_threads, sa, st>>>(L->d_shat, L->row_stride, L->d_members, L->d_klo, L->d_klen,
                                                       L->d_koff, L->d_krange, nz, m->n_lo, NS, L->d_w1, L->d_w2);
     OAM_LAUNCHED();
-    K::cols(dim3(Q, cbs), st, L->d_w2, P, py, NS, P, lgP, 1, L->d_w1);
-    OAM_LAUNCHED();
-    const unsigned cbt = (unsigned)((m->grid.nt + KC - 1) / KC);
-    K::rows_c2r(dim3(py, cbt), st, L->d_w1, py, px, m->grid.nt, m->n_lo, NS, P, lgP, Q, scale, out);
-    OAM_LAUNCHED();
+    if ((rc = K::template cols<true>(L, st, L->d_w2, P, py, NS, L->d_w1))) return rc;
+    if ((rc = K::rows_c2r(L, st, L->d_w1, py, px, m->grid.nt, m->n_lo, NS, scale, out))) return rc;
   } else {
-    K::rows_r2c(dim3(py, cbs), st, in, py, px, m->grid.nt, m->n_lo, NS, P, lgP, Q, L->d_w2);
-    OAM_LAUNCHED();
-    K::cols(dim3(Q, cbs), st, L->d_w2, py, P, NS, P, lgP, 0, L->d_w1);
-    OAM_LAUNCHED();
+    if ((rc = K::rows_r2c(L, st, in, py, px, m->grid.nt, m->n_lo, NS, L->d_w2))) return rc;
+    if ((rc = K::template cols<false>(L, st, L->d_w2, py, P, NS, L->d_w1))) return rc;
     const size_t sa = (sizeof(float4) * 2 + sizeof(int2) + sizeof(long long)) * NS;
     if ((rc = set_smem((const void *)k_fft_apply_adj, sa))) return rc;
     const int achunk = kAdjChunk > 0 ? kAdjChunk : nz;
@@ -994,10 +900,8 @@ oam_status run_fft(const oam_model *m, const FftLayout *L, bool fwd, const float
     k_fft_apply_adj<<<ablocks, adj_threads, sa, st>>>(L->d_shat_t, L->row_stride_t, L->d_members, L->d_klo, L->d_klen,
                                                       L->d_krange, L->d_noff, nz, m->n_lo, NS, L->d_w1, L->d_w2);
     OAM_LAUNCHED();
-    K::cols(dim3(Q, cbz), st, L->d_w2, P, py, nz, P, lgP, 1, L->d_w1);
-    OAM_LAUNCHED();
-    K::rows_c2r(dim3(py, cbz), st, L->d_w1, py, px, nz, 0, nz, P, lgP, Q, scale, out);
-    OAM_LAUNCHED();
+    if ((rc = K::template cols<true>(L, st, L->d_w2, P, py, nz, L->d_w1))) return rc;
+    if ((rc = K::rows_c2r(L, st, L->d_w1, py, px, nz, 0, nz, scale, out))) return rc;
   }
   return OAM_OK;
 }
@@ -1006,13 +910,8 @@ oam_status run_fft_any(const oam_model *m, bool fwd, const float *in, float *out
   const FftLayout *L = m->fft;
   if (!L) return OAM_ERR_UNSUPPORTED;
   ProfScope prof(m, st, fwd);
-  const bool x = L->P >= 16;  // register-pass transforms need a four-stage pass
-  switch (L->KC) {
-    case 16: return x ? run_fft<16, XKernels<16>>(m, L, fwd, in, out, st) : run_fft<16, RKernels<16>>(m, L, fwd, in, out, st);
-    case 8: return x ? run_fft<8, XKernels<8>>(m, L, fwd, in, out, st) : run_fft<8, RKernels<8>>(m, L, fwd, in, out, st);
-    case 4: return x ? run_fft<4, XKernels<4>>(m, L, fwd, in, out, st) : run_fft<4, RKernels<4>>(m, L, fwd, in, out, st);
-    default: return x ? run_fft<2, XKernels<2>>(m, L, fwd, in, out, st) : run_fft<2, RKernels<2>>(m, L, fwd, in, out, st);
-  }
+  if (L->d_tw) return run_fft<MKernels>(m, L, fwd, in, out, st);
+  return L->KC == 4 ? run_fft<XKernels<4>>(m, L, fwd, in, out, st) : run_fft<XKernels<2>>(m, L, fwd, in, out, st);
 }
 
 }  // namespace
