@@ -60,8 +60,14 @@ typedef enum {
 
 typedef enum {
   OAM_PREC_FP32 = 0,  /* plain FP32 slab and FP32 CUDA-core operators */
-  OAM_PREC_BF16X3 = 1, /* split-BF16 (hi+lo) slab and iterate on tcgen05 tensor cores,
-                          FP32 accumulation in tensor memory: hi*hi + hi*lo + lo*hi */
+  OAM_PREC_BF16X3 = 1, /* two-term 16-bit splits (hi+lo) of the slab and the iterate on
+                          tcgen05 tensor cores, FP32 accumulation in tensor memory:
+                          hi*hi + hi*lo + lo*hi, at least as accurate as BF16 terms
+                          (the terms are FP16 of operands scaled by powers of two).
+                          The scan's y axis is taken to the lateral frequency domain
+                          by FP32 line transforms, so each frequency is a correlation
+                          along x; positions whose window holds only zeros get exact
+                          zeros, those whose window holds a non-finite value NaN */
   OAM_PREC_FFT = 2     /* FP32 lateral-FFT form of the same operators: both are 2-D
                           correlations over the scan grid (Methods, Efficient
                           reconstruction based on scanning symmetries), restated
@@ -152,7 +158,8 @@ oam_status oam_build_model(const oam_sensor *sensor, const oam_grid *grid, const
  * compressed model is a single scanning position's, so its size depends on
  * the window, depths, samples and sensor, not on the number of scan
  * positions (Results; Methods, Efficient reconstruction based on scanning
- * symmetries) -- only the tensor-core staging buffers grow with the scan.
+ * symmetries) -- only the tensor-core form's transformed slab and staging
+ * buffers grow with the scan.
  * The bands are planned from host-side distances with two samples of margin
  * per band edge, so the result bounds the built model's device_bytes from
  * above (by a few per cent).  Same argument errors as oam_build_model
@@ -338,7 +345,8 @@ oam_status oam_model_get_tiles(const oam_model *model, int32_t direction, int32_
  * not depend on the shape (fixed summation order per accumulator). */
 oam_status oam_model_set_tiles(oam_model *model, int32_t direction, int32_t fold_warps, int32_t ring);
 /* Position tiling of the split-BF16 kernels, direction 0 or 1: the grid whose
- * 128 consecutive positions a block takes.  1 = the padded scan grid (rows of
+ * 128 consecutive positions a block takes (rows: the real and the imaginary part
+ * of a transformed scan row each).  1 = the padded grid (rows of
  * px + R positions, the R padding positions per row computed and dropped;
  * strips of 128 + 2R staged rows), 2 = the scan grid itself (every position an
  * output; a tile that wraps w scan rows stages 128 + (w + 2) R rows, so it

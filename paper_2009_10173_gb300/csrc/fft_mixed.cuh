@@ -143,26 +143,31 @@ __host__ __device__ constexpr int mix_threads() {
   return n > 256 ? 256 : (n + 31) / 32 * 32;
 }
 
-// One transform of KL lines.  src(i, l) yields point i, dst(f, l, v) takes
-// frequency f (inverse: src takes the frequency, dst the point).  tw holds
-// W_P^j, j < P (global memory, read through L1).
-template <int R1, int R2, int KL, bool kInverse, class Src, class Dst>
-__device__ __forceinline__ void mix_transform(float2 *a, const float2 *__restrict__ tw, Src src, Dst dst) {
+// One transform of KL lines, in two passes with a barrier between.  src(i2, l, v)
+// fills v[m] with points m R2 + i2 (all of a thread's loads together, so that
+// they are in flight at once), dst(f, l, v) takes frequency f (inverse: src fills
+// frequencies, dst takes a point).  tw holds W_P^j, j < P (global memory, read
+// through L1).
+template <int R1, int R2, int KL, bool kInverse, class Src>
+__device__ __forceinline__ void mix_pass1(float2 *a, const float2 *__restrict__ tw, Src src) {
   constexpr int RS = mix_stride<R2, KL>();
   for (int id = threadIdx.x; id < R2 * KL; id += blockDim.x) {
     const int l = id % KL, i2 = id / KL;
     float2 v[R1];
+    src(i2, l, v);
+    if (kInverse) {
 #pragma unroll
-    for (int m = 0; m < R1; ++m) {
-      const float2 u = src(m * R2 + i2, l);
-      v[m] = kInverse ? make_float2(u.y, u.x) : u;
+      for (int m = 0; m < R1; ++m) v[m] = make_float2(v[m].y, v[m].x);
     }
     dft<R1>(v);
     a[i2 * KL + l] = v[0];
 #pragma unroll
     for (int m = 1; m < R1; ++m) a[m * RS + i2 * KL + l] = cmulc(v[m], __ldg(tw + m * i2));
   }
-  __syncthreads();
+}
+template <int R1, int R2, int KL, bool kInverse, class Dst>
+__device__ __forceinline__ void mix_pass2(float2 *a, Dst dst) {
+  constexpr int RS = mix_stride<R2, KL>();
   for (int id = threadIdx.x; id < R1 * KL; id += blockDim.x) {
     const int l = id % KL, k1 = id / KL;
     float2 v[R2];
@@ -173,6 +178,12 @@ __device__ __forceinline__ void mix_transform(float2 *a, const float2 *__restric
     for (int m = 0; m < R2; ++m) dst(k1 + R1 * m, l, kInverse ? make_float2(v[m].y, v[m].x) : v[m]);
   }
 }
+template <int R1, int R2, int KL, bool kInverse, class Src, class Dst>
+__device__ __forceinline__ void mix_transform(float2 *a, const float2 *__restrict__ tw, Src src, Dst dst) {
+  mix_pass1<R1, R2, KL, kInverse>(a, tw, src);
+  __syncthreads();
+  mix_pass2<R1, R2, KL, kInverse>(a, dst);
+}
 
 // The transform sizes, smallest first: even, at most 512, steps of at most a third
 // from 12 on and a quarter or less over most of 64 .. 320 (the batched scans with a
@@ -180,7 +191,7 @@ __device__ __forceinline__ void mix_transform(float2 *a, const float2 *__restric
 #define OAM_MIX_SIZES(X)                                                                                     \
   X(4, 2, 2) X(8, 2, 4) X(12, 3, 4) X(16, 4, 4) X(20, 4, 5) X(24, 4, 6) X(32, 4, 8) X(40, 5, 8) X(48, 6, 8) \
   X(64, 8, 8) X(80, 8, 10) X(96, 8, 12) X(128, 8, 16) X(160, 10, 16) X(192, 12, 16) X(240, 15, 16)         \
-  X(256, 16, 16) X(288, 18, 16) X(320, 20, 16) X(384, 24, 16) X(512, 32, 16)
+  X(256, 16, 16) X(288, 16, 18) X(320, 16, 20) X(384, 16, 24) X(512, 16, 32)
 constexpr int kMixMax = 512;
 
 // Smallest size >= need (need <= kMixMax).

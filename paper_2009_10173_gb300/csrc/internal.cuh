@@ -33,6 +33,7 @@ struct __align__(32) Patch {
 
 // Tensor-core operator layout of one direction (forward or adjoint); defined in op_tc.cu.
 struct TcLayout;
+struct TcLine;
 // Lateral-FFT form of the operators (OAM_PREC_FFT); defined in op_fft.cu.
 struct FftLayout;
 // Band-pass filter along time of a filtered model; defined in op_filter.cu.
@@ -77,14 +78,11 @@ struct oam_model {
   long long *d_adj_off = nullptr;
   float *d_adj = nullptr;
 
-  // tensor-core layouts (OAM_PREC_BF16X3) and the staging buffer for the
-  // split-BF16 copy of the operator input ([chunks][qtot][8] hi, then lo)
+  // tensor-core layouts (OAM_PREC_BF16X3) per direction, and the plan and buffers
+  // of the line transforms around them
   oam::TcLayout *tc_fwd = nullptr;
   oam::TcLayout *tc_adj = nullptr;
-  uint8_t *d_tc_pack = nullptr;
-  size_t tc_pack_bytes = 0;
-  long long tc_qtot = 0;
-  float *d_tc_part = nullptr;  // per-part partial sums of the tensor-core operators
+  oam::TcLine *tc_line = nullptr;
 
   oam::FftLayout *fft = nullptr;  // lateral-FFT form (OAM_PREC_FFT)
   oam::FirLayout *fir = nullptr;  // band-pass filter: forward is F A, adjoint A^T F (none: nullptr)
@@ -193,6 +191,28 @@ oam_status mix_cols(int P, bool inverse, cudaStream_t st, const float2 *Z, int n
                     float2 *W);
 oam_status mix_rows_c2r(int P, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0, int C,
                         const float2 *tw, float scale, float *X);
+
+// mix_lines.cu: transforms along the scan's y axis around the tensor-core
+// correlation along x.  Lines longer than the largest transform are cut into
+// `segs` overlapping segments of P input rows and `valid` output rows.
+struct LineShape {
+  int px, py, R;           // scan grid, half window
+  int halo;                // rows coupled along y: min(R, py - 1)
+  int segs, valid;         // segments, output rows of each
+  int len, in_lo, elems;   // input row length, first channel packed, packed channels per position
+  int wp, rows;            // positions per packed row (px + R), packed positions per frequency
+  int nr;                  // packed rows per frequency: 2 segs (re and im)
+  int out_len, out_lo, acc, parts;  // output row length, output channel of accumulator column 0, columns, partial sums
+  int words;               // 32-row mark words per column
+  unsigned *marks;         // [2][px][words]: positions with a non-zero, with a non-finite input
+  unsigned *vmax;          // [frequencies] largest magnitude of the transformed lines, as float bits
+  int *any_bad;            // some position has a non-finite input
+  const unsigned *grown;   // [2][px][words]: positions whose window holds one
+  __host__ __device__ int out_row(int seg) const { return seg * valid; }  // first output row of a segment
+  __host__ __device__ int first_row(int seg) const { return segs > 1 ? seg * valid - halo : 0; }  // point 0's row
+};
+oam_status line_r2c(int P, cudaStream_t st, const LineShape &s, const float *in, const float2 *tw, float *packed);
+oam_status line_c2r(int P, cudaStream_t st, const LineShape &s, const float *part, const float2 *tw, float *out);
 
 // op_filter.cu: y = F x over the model's py*px A-lines (x and y may alias)
 oam_status fir_apply(const oam_model *m, const float *x, float *y, cudaStream_t st);

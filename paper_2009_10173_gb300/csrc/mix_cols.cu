@@ -14,17 +14,21 @@ namespace {
 constexpr int kColCh = 16;  // complex channels per block
 
 // Complex transform along the row index of Z[Q][nin][C] -> W[Q][nout][C]
-// (rows >= nin read as zero, rows >= nout dropped).  Block (u, channel block).
+// (rows >= nin read as zero, rows >= nout dropped).  Block (channel block, u).
 template <int R1, int R2, int KC, bool kInverse>
 __global__ void __launch_bounds__(mix_threads<R1, R2, KC>())
     k_mix_cols(const float2 *__restrict__ Z, int nin, int nout, int C, const float2 *__restrict__ tw,
                float2 *__restrict__ W) {
   extern __shared__ float2 sm[];
-  const int u = blockIdx.x, cb = blockIdx.y * KC;
+  const int u = blockIdx.y, cb = blockIdx.x * KC;
   const float2 *zin = Z + (size_t)u * nin * C + cb;
   float2 *wout = W + (size_t)u * nout * C + cb;
-  auto load = [&](int i, int l) {
-    return (i < nin && cb + l < C) ? zin[(size_t)i * C + l] : make_float2(0.0f, 0.0f);
+  auto load = [&](int i2, int l, float2 (&v)[R1]) {
+#pragma unroll
+    for (int m = 0; m < R1; ++m) {
+      const int i = m * R2 + i2;
+      v[m] = (i < nin && cb + l < C) ? zin[(size_t)i * C + l] : make_float2(0.0f, 0.0f);
+    }
   };
   auto store = [&](int i, int l, float2 v) {
     if (i < nout && cb + l < C) wout[(size_t)i * C + l] = v;
@@ -38,7 +42,7 @@ oam_status cols(cudaStream_t st, const float2 *Z, int Q, int nin, int nout, int 
   if (sm > 48 * 1024)
     OAM_CUDA_TRY(cudaFuncSetAttribute(k_mix_cols<R1, R2, kColCh, kInverse>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k_mix_cols<R1, R2, kColCh, kInverse><<<dim3(Q, (C + kColCh - 1) / kColCh), mix_threads<R1, R2, kColCh>(), sm, st>>>(
+  k_mix_cols<R1, R2, kColCh, kInverse><<<dim3((C + kColCh - 1) / kColCh, Q), mix_threads<R1, R2, kColCh>(), sm, st>>>(
       Z, nin, nout, C, tw, W);
   OAM_LAUNCHED();
   return OAM_OK;

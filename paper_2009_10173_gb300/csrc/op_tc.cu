@@ -1,46 +1,56 @@
 // Split-BF16 forward and adjoint operators on the 5th-generation tensor cores
 // (tcgen05 MMA, accumulators in tensor memory, operands staged by the TMA
 // engine).  Both are the lateral correlations of Eq. 4 ("two coordinate
-// systems", Methods, Efficient reconstruction based on scanning symmetries)
-// written as one implicit GEMM per block of 128 scan positions:
+// systems", Methods, Efficient reconstruction based on scanning symmetries).
 //
-//   forward  D[pos][n] += sum_{tap, k}  X[pos + tap][k] * S_tap[k][n]
-//   adjoint  D[pos][k] += sum_{tap, n}  X[pos - tap][n] * S_tap[k][n]
+// Along the scan's y axis the correlation is diagonal in the lateral frequency:
+// with the lines of the input zero-padded to P points (mix_lines.cu), and the
+// slab's transform over its row offset real because the slab is even in it
+// (Results, axial symmetry),
+//   S_v[a][k][n] = sum_b S[b][a][k][n] cos(2 pi v b / P),
+// each of the P/2 + 1 frequencies v is a correlation along x alone, the same for
+// the real and the imaginary part of the transformed lines:
 //
-// M = 128 positions (one tensor-memory lane each), N = the slab band of one
-// 16-deep K chunk (time samples for A, depths for A^T), K = (tap, 16-chunk).
+//   forward  D_v[row][n] += sum_{a, k}  X_v[row + a][k] * S_v[a][k][n]
+//   adjoint  D_v[row][k] += sum_{a, n}  X_v[row + a][n] * S_v[a][k][n]
 //
-// Mirror folding.  The sensor is axially symmetric and its patch set is
-// mirror-symmetric (Results, axial symmetry), so S[b][a] = S[+-b][+-a] exactly
-// (one stored orbit).  The four mirrored taps therefore share one slab tile,
+// One implicit GEMM per block of 128 rows (positions x of a frequency's real and
+// imaginary part): M = 128 rows (one tensor-memory lane each), N = the slab band
+// of one 16-deep K chunk (time samples for A, depths for A^T), K = (tap a,
+// 16-chunk).  The P/2 + 1 frequencies of two rows each stand for py + R padded
+// scan rows, and a row meets R + 1 folded taps instead of (R + 1)^2: 24x fewer
+// products than the correlation over both axes at a 61x61 window, for a slab
+// (P/2 + 1) / (R + 1) = 4 times the size at 200 lines and two line transforms.
+// Measured on a GB300 against that form (one application): 200x200x300 forward
+// 5.78 -> 0.49 ms, adjoint 5.71 -> 0.47 ms, 96x96x192 forward 0.86 -> 0.10 ms.
+//
+// Mirror folding.  S_v[a] = S_v[-a], so the two mirrored taps share one slab tile
 // and their operand rows are summed before the product:
-//   F[pos][k] = X[pos + (b, a)] + X[pos + (b, -a)] + X[pos + (-b, a)] + X[pos + (-b, -a)]
-// (duplicates dropped when a or b is 0).  One block handles one 128-position
-// tile and a group of kBPerBlock consecutive |b|, one after the other into the
-// same accumulator; for each it stages the FP32 rows y+b and y-b (TMA, 128-byte
-// swizzle) and adds them once per stage, sixteen warps build F from two shifted
-// rows of that sum (8 of the stage's 32 K elements each), split it into BF16
-// hi/lo in tensor memory, and one warp walks the items while an elected lane
-// issues the MMAs with A read from tensor memory.  This cuts the MMA count by
-// ~4 for a 61x61 window.
+//   F[row][k] = X_v[row + a][k] + X_v[row - a][k]
+// (one row for a = 0).  A block stages the rows of 32 K elements at a time (TMA,
+// 128-byte swizzle); the fold warps build F from two shifted rows, split it into
+// FP16 hi/lo in tensor memory, and one warp walks the items while an elected
+// lane issues the MMAs with A read from tensor memory.
 //
-// The iterate is packed with a padded flat index q = y*Wp + x, Wp = px + R
-// (zero columns px .. Wp-1 and R+1 zero rows above and below), so a lateral
-// offset a is a shift by a rows of a staged strip.  A block's 128 positions
-// are consecutive in one of two grids (the position tiling, a tile parameter):
-// the padded grid (o = y*Wp + x; padding positions compute and are dropped;
-// strips of 128 + 2R rows) or the scan grid (o = y*px + x, every lane an
-// output; lane m reads strip row m + R*(rows wrapped before m) + R + a, and a
-// strip holds 128 + (w + 2) R rows for tiles that wrap w scan rows).
+// The packed input holds, per frequency, R zero positions, then each row of px
+// positions followed by R zeros (stride Wp = px + R), so a lateral offset a is a
+// shift by a positions of a staged strip.  A block's 128 positions are
+// consecutive in one of two grids (the position tiling, a tile parameter): the
+// padded grid (o = row*Wp + x; padding positions compute and are dropped; strips
+// of 128 + 2R positions) or the scan grid (o = row*px + x, every lane an output;
+// lane m reads strip position m + R*(rows wrapped before m) + R + a, and a strip
+// holds 128 + (w + 2) R positions for tiles that wrap w rows).
 //
-// Each product uses hi = bf16(v), lo = bf16(v - hi) splits of the slab and of
-// the folded iterate: D += F_hi S_hi + F_hi S_lo + F_lo S_hi, accumulated in
-// FP32 in tensor memory.  Each block's tensor-memory sums are written as one
-// partial per |b| group; k_sum_parts adds them in index order (this bounds how many
-// MMA results any one accumulator takes, which keeps the tensor cores' FP32
-// accumulation within 1e-4 of the FP64 oracle).
+// Each product uses two-term 16-bit splits v = hi + lo of the slab and of the
+// folded iterate: D += F_hi S_hi + F_hi S_lo + F_lo S_hi, accumulated in FP32 in
+// tensor memory.  The terms are FP16 (22 significant bits together, BF16 terms
+// hold 16) of operands scaled by powers of two: the slab by one for the model,
+// the iterate by one for each frequency, from the magnitudes that the line
+// transform finds.  Few blocks (small scans, or a nearly empty last wave)
+// split the taps over `parts` blocks, whose partial sums the inverse line
+// transform adds in index order.
 #include <cuda.h>
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <cstring>
@@ -57,14 +67,14 @@ constexpr int kTileM = 128;        // positions per block
 constexpr int kFoldWarpChoices[] = {4, 8, 16};  // warps that build the folded operand (then run the epilogue)
 constexpr int kDefaultFoldWarps = 8;
 constexpr int kMaxItems = 8;       // item ring depth (slab tile + folded operand)
-constexpr int kBPerBlock = 4;      // consecutive |b| per block (one partial sum per group)
 constexpr int kFoldCols = 32;      // tensor-memory columns per folded operand: 2 chunks x (hi, lo) x 8
 constexpr int kSmemLimit = 227 * 1024;
 
-// One ring item: the slab tiles of one (orbit, stage), hi then lo of each of
-// its two 16-deep chunks; 8 bytes, so a block's item tables stay small.
+// One ring item: the slab tiles of one (|a|, stage), hi then lo of each of
+// its two 16-deep chunks; 8 bytes, so a block's item tables stay small.  The
+// same for every frequency, whose tiles lie v_stride bytes apart.
 struct __align__(8) TcItem {
-  uint32_t off16;  // byte offset of the item's tiles in data, in 16-byte units
+  uint32_t off16;  // byte offset of the item's tiles in a frequency's data, in 16-byte units
   uint8_t c16[2];  // accumulator column / 16 of each tile
   uint8_t n16[2];  // MMA N / 16 of each tile (0 = no tile)
   __host__ __device__ uint32_t col(int c) const { return 16u * c16[c]; }
@@ -73,28 +83,43 @@ struct __align__(8) TcItem {
 };
 
 struct TcTile {
-  int orbit, chunk, col, n;
-  long long off;  // byte offset of the hi part; lo follows after n*32 bytes
+  int a, chunk, col, n;
+  long long off;  // byte offset of the hi part in a frequency's data; lo follows after n*32 bytes
 };
 
 struct TcLayout {
   int dir = 0;            // 0 forward, 1 adjoint
   int stages = 0;         // K stages of kStageK
   int acc_cols = 0;       // accumulator width (multiple of 16)
-  int tmem_cols = 0;      // allocated tensor-memory columns (power of two >= 32)
   int out_lo = 0;         // output index of accumulator column 0
   int in_lo = 0;          // input index of packed element 0
   int in_elems = 0;       // packed elements per position (32 * stages)
   int slot_bytes = 0;     // shared-memory slot per item
   int ring_pref = 0;      // item-ring depth chosen by oam_model_autotune (0 = deepest that fits)
   int tiling = 0;         // position tiling: 0 auto, 1 padded grid, 2 scan grid
-  std::vector<double> row_cols;  // per |b|: MMA columns x 16 summed over a = 0 .. R and the stages
+  int parts = 1;          // blocks that share a tile's taps
+  bool wide = false;      // some tile is wider than one MMA
+  double cols = 0;        // MMA columns x 16 summed over a = 0 .. R and the stages
   int fold_warps = kDefaultFoldWarps;  // fold-warp count chosen by oam_model_autotune (4, 8 or 16)
-  TcItem *d_items = nullptr;
-  uint8_t *d_data = nullptr;
-  size_t data_bytes = 0;
+  TcItem *d_items = nullptr;  // [R + 1][stages]
+  uint8_t *d_data = nullptr;  // [P/2 + 1][v_stride]
+  size_t v_stride = 0;        // bytes of one frequency's tiles
+  float *d_pack = nullptr;    // packed input [(P/2 + 1) rows][in_elems]
   CUtensorMap tmap;       // FP32 packed input [qtot][in_elems], box 32 x (128 + 2R), 128-byte swizzle
-  CUtensorMap tmap_scan;  // the same with the scan-grid strip rows (when they fit one box)
+  CUtensorMap tmap_scan;  // the same with the scan-grid strip positions (when they fit one box)
+};
+
+// The line transforms' plan, common to both directions.
+struct TcLine {
+  int P = 0, Q = 0;           // transform size, frequencies P/2 + 1
+  int halo = 0;               // rows coupled along y: min(R, py - 1)
+  int segs = 1, valid = 0;    // segments of a line, output rows of each
+  int nr = 0, rows = 0;       // packed rows and positions per frequency
+  int words = 0;              // mark words per column
+  float2 *d_tw = nullptr;     // [P] roots
+  unsigned *d_marks = nullptr;  // [2][px][words], [Q] magnitudes, the non-finite flag, [2][px][words] grown
+  unsigned *d_smax = nullptr;   // bound of the transformed slab's magnitude, as float bits
+  float *d_part = nullptr;    // partial sums [parts][Q][nr][px][acc_cols]
 };
 
 }  // namespace oam
@@ -102,16 +127,21 @@ struct TcLayout {
 namespace {
 
 struct CorrParams {
-  long long qtot;
-  int wp, px, py, R, W, stages;
-  int sp;  // row stride of the grid the position tiles follow: Wp (padded) or px (scan)
-  const int *tap_orbit;
-  const TcItem *items;  // [n_orb][stages]
+  int wp, px, R, stages;
+  int sp;          // row stride of the grid the position tiles follow: Wp (padded) or px (scan)
+  int nr, rows;    // packed rows and positions per frequency
+  const TcItem *items;  // [R + 1][stages]
   const uint8_t *data;
+  size_t v_stride;
   int slot_bytes, n_items, strip_rows, strip_bytes, items_bytes;
   int acc_cols, tmem_cols, fold_col0;
-  float *part;         // partial sums [groups][py*px][acc_cols], one slice per group of kBPerBlock |b|
-  size_t part_stride;  // py*px
+  const unsigned *marks;  // [2][px][words]: positions with a non-zero, with a non-finite input
+  unsigned *grown;        // [2][px][words]: positions whose window holds one
+  const int *any_bad;     // some position has a non-finite input
+  int words;
+  const unsigned *vmax;  // [frequencies] largest magnitude of the transformed lines, as float bits
+  const unsigned *smax;  // the slab's, over its transform (an upper bound)
+  float *part;         // partial sums [parts][frequencies][nr][px][acc_cols]
   int *status;
   long long budget;
 };
@@ -124,28 +154,11 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
       : "memory");
 }
 
-// Does row offset `off` put any of the tile's rows inside the grid?
-__device__ __forceinline__ bool row_live(const CorrParams &p, int tile, int off) {
-  const int o0 = tile * kTileM, o1 = min(o0 + kTileM, p.py * p.sp) - 1;
-  const int y_first = o0 / p.sp, y_last = o1 / p.sp;
-  return !(y_last + off < 0 || y_first + off >= p.py);
-}
-
 // Lateral offset |a| of the j-th item of a stage.  Items alternate between
 // the small and the large offsets (0, R, 1, R - 1, ...): the band, and with it
 // the MMA width N, grows with the offset, so each pair of items costs about
 // the same MMA time while its fold work is the same for every pair.
 __device__ __forceinline__ int a_of(int j, int R) { return (j & 1) ? R - (j >> 1) : (j >> 1); }
-
-// Index of the n-th set bit of mask (n counted from 0).
-__device__ __forceinline__ int nth_set(unsigned mask, int n) {
-  for (int i = 0; i < kBPerBlock; ++i)
-    if ((mask >> i) & 1u) {
-      if (n == 0) return i;
-      --n;
-    }
-  return 0;
-}
 
 // Packed FP32 pairs (two lanes of one 64-bit register) and their arithmetic.
 __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
@@ -191,31 +204,47 @@ __device__ __forceinline__ void add_row(const float *strip, int row, int q, uint
   }
 }
 
-// Split four FP32 pairs into BF16 pairs hi = bf16(v) and lo = bf16(v - hi),
-// both rounded to nearest even; element 2e in the low half of word e.
-__device__ __forceinline__ void split_bf16(const uint64_t (&v)[4], uint32_t (&hv)[4], uint32_t (&lv)[4]) {
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// 2^e, -126 <= e <= 127.
+__device__ __forceinline__ float pow2(int e) { return __int_as_float((e + 127) << 23); }
+
+// Exponent e of the power of two that brings a magnitude of at most `top` into
+// [2^14, 2^15), below FP16's largest 65504 (0 for an all-zero operand).
+__device__ __forceinline__ int scale_exp(float top) {
+  return top > 0.0f ? min(126, max(-126, 14 - ilogbf(top))) : 0;
+}
+
+// Split four FP32 pairs (scaled into FP16's range) into FP16 pairs: hi = v with
+// its low 13 fraction bits cleared (an FP16 value), lo = v - hi rounded to
+// nearest even; element 2e in the low half of word e.
+__device__ __forceinline__ void split_f16(const uint64_t (&v)[4], uint32_t (&hv)[4], uint32_t (&lv)[4]) {
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     float x, y;
     unpack_f32x2(v[e], x, y);
-    const __nv_bfloat162 h2 = __floats2bfloat162_rn(x, y);
-    const uint32_t hb = *reinterpret_cast<const uint32_t *>(&h2);
-    const uint64_t lo = sub_f32x2(v[e], pack_f32x2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xffff0000u)));
+    x = __uint_as_float(__float_as_uint(x) & 0xffffe000u);
+    y = __uint_as_float(__float_as_uint(y) & 0xffffe000u);
+    const __half2 h2 = __floats2half2_rn(x, y);
     float lx, ly;
-    unpack_f32x2(lo, lx, ly);
-    const __nv_bfloat162 l2 = __floats2bfloat162_rn(lx, ly);
-    hv[e] = hb;
+    unpack_f32x2(sub_f32x2(v[e], pack_f32x2(x, y)), lx, ly);
+    const __half2 l2 = __floats2half2_rn(lx, ly);
+    hv[e] = *reinterpret_cast<const uint32_t *>(&h2);
     lv[e] = *reinterpret_cast<const uint32_t *>(&l2);
   }
 }
 
-// Fold one item: F = P[m + R + a] + P[m + R - a] (P[m + R] alone for a = 0)
+// Fold one item: F = X[m + R + a] + X[m + R - a] (X[m + R] alone for a = 0)
 // for this thread's row m and its E of the stage's 32 K elements (8-element
-// quarters q0 .. q0 + E/8 - 1), split into BF16 hi/lo words in the order the
-// tensor-memory store takes them: E = 8: hi[4], lo[4]; E >= 16: per 16-deep
-// chunk, hi[8] then lo[8].
+// quarters q0 .. q0 + E/8 - 1), times the power of two `sc`, split into FP16
+// hi/lo words in the order the tensor-memory store takes them: E = 8: hi[4],
+// lo[4]; E >= 16: per 16-deep chunk, hi[8] then lo[8].
 template <int E>
-__device__ __forceinline__ void fold_item(const float *X1, int m, int R, int a, int q0, uint32_t (&w)[E]) {
+__device__ __forceinline__ void fold_item(const float *X1, int m, int R, int a, int q0, uint64_t sc, uint32_t (&w)[E]) {
   constexpr int NQ = E / 8;
   uint64_t f[NQ][4];
 #pragma unroll
@@ -226,8 +255,10 @@ __device__ __forceinline__ void fold_item(const float *X1, int m, int R, int a, 
   }
 #pragma unroll
   for (int i = 0; i < NQ; ++i) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) f[i][e] = mul_f32x2(f[i][e], sc);
     uint32_t hv[4], lv[4];
-    split_bf16(f[i], hv, lv);
+    split_f16(f[i], hv, lv);
     const int hb = E == 8 ? 0 : 16 * (i >> 1) + 4 * (i & 1);  // word of the quarter's first hi pair
     const int lb = E == 8 ? 4 : hb + 8;
 #pragma unroll
@@ -240,7 +271,7 @@ __device__ __forceinline__ void fold_item(const float *X1, int m, int R, int a, 
 
 // Store one folded item into its tensor-memory slot (slot column 0 = chunk 0
 // hi, 8 = chunk 0 lo, 16 = chunk 1 hi, 24 = chunk 1 lo; a column holds two
-// BF16 K elements).
+// FP16 K elements).
 template <int E>
 __device__ __forceinline__ void store_item(uint32_t slot_addr, int q0, const uint32_t (&w)[E]) {
   if constexpr (E == 8) {
@@ -255,11 +286,54 @@ __device__ __forceinline__ void store_item(uint32_t slot_addr, int q0, const uin
   }
 }
 
-template <int FW>
-__global__ void __launch_bounds__(64 + 32 * FW, 1)
-    k_corr_fold(const __grid_constant__ CUtensorMap tmap, const CorrParams p) {
+// D (col d) += A (tensor memory, 16 deep) x B (n columns); kWide: n above one MMA's 256.
+template <bool kWide>
+__device__ __forceinline__ void mma_cols(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t n) {
+  if (!kWide || n <= 256u) {
+    ptx::mma_f16_ta(d, a, b, idesc | ((n >> 3) << 17), 1);
+  } else {  // 256 columns, then the rest: 256 rows of 16 bytes further in the tile
+    ptx::mma_f16_ta(d, a, b, idesc | (32u << 17), 1);
+    ptx::mma_f16_ta(d + 256u, a, b + 256u, idesc | (((n - 256u) >> 3) << 17), 1);
+  }
+}
+
+// The marks of column x (mix_lines.cu), or-ed over the columns within R and grown by
+// R rows: one warp, lanes over columns, then over the rows of a word.
+__device__ __forceinline__ void grow_marks(const CorrParams &p, int x, int lane) {
+  const int xa = max(0, x - p.R), xb = min(p.px - 1, x + p.R);
+  const bool bad = *p.any_bad != 0;
+  for (int which = 0; which < 2; ++which) {
+    const unsigned *src = p.marks + (size_t)(which * p.px) * p.words;
+    unsigned *dst = p.grown + (size_t)(which * p.px + x) * p.words;
+    unsigned win[5] = {0, 0, 0, 0, 0};  // words w - 2 .. w + 2 (R <= 64)
+    for (int j = -2; j < p.words; ++j) {  // word j + 2 joins; word j is complete
+      unsigned m = 0;
+      if (j + 2 < p.words && (which == 0 || bad))
+        for (int xx = xa + lane; xx <= xb; xx += 32) m |= __ldcg(src + (size_t)xx * p.words + j + 2);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) win[i] = win[i + 1];
+      win[4] = __reduce_or_sync(0xffffffffu, m);
+      if (j < 0) continue;
+      bool any = false;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {  // rows lane - R .. lane + R of word j
+        const int lo = max(lane - p.R - 32 * (i - 2), 0), hi = min(lane + p.R - 32 * (i - 2), 31);
+        if (lo <= hi) any = any || (win[i] & (0xffffffffu << lo) & (0xffffffffu >> (31 - hi))) != 0;
+      }
+      const unsigned out = __ballot_sync(0xffffffffu, any);
+      if (lane == 0) dst[j] = out;
+    }
+  }
+}
+
+// Block (position tile, tap part, frequency).  What bounds it: the fold warps and
+// the MMA issue take about the same time per pair of items (~0.45 us at 320
+// accumulator columns), each waiting on the other through the item ring.
+template <int FW, bool kWide>
+__global__ void __launch_bounds__(96 + 32 * FW, 1)
+    k_corr_line(const __grid_constant__ CUtensorMap tmap, const CorrParams p) {
   constexpr int kFoldWarps = FW;
-  constexpr int kThreads = 64 + 32 * FW;
+  constexpr int kThreads = 96 + 32 * FW;
   constexpr int G = FW / 4;   // K groups per tensor-memory lane quarter
   constexpr int E = 32 / G;   // stage K elements folded per thread and item
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -275,27 +349,17 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + 512);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + 516);
   volatile int *never = reinterpret_cast<volatile int *>(smem + 520);  // stays 0: waits that ignore abort
-  TcItem *sitems = reinterpret_cast<TcItem *>(smem + 1024);           // [kBPerBlock][stages][R+1]: the group's items
-  // Three strip buffers in rotation: stage gs stages its row y+b in buffer
-  // gs % 3 (which then holds P = X(y+b) + X(y-b)) and its row y-b in buffer
-  // (gs + 1) % 3, free again once P is formed, so stage gs + 1 reuses it and
-  // the buffer stage gs - 1 held P.
-  uint8_t *strips = smem + 1024 + p.items_bytes;                       // [3][strip_bytes]
+  TcItem *sitems = reinterpret_cast<TcItem *>(smem + 1024);           // [stages][nj]: this part's items
+  uint8_t *strips = smem + 1024 + p.items_bytes;                       // [3][strip_bytes]: stage st in buffer st % 3
   uint8_t *slots = strips + 3 * p.strip_bytes;                         // [K][slot_bytes]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tile = blockIdx.x;
-  const int grp = (int)blockIdx.y;  // |b| = kBPerBlock * grp + i: rows y + b and y - b
-  const int R = p.R, NA = R + 1;    // a = 0 .. R
-  unsigned live = 0;                // group members i whose rows meet the grid
-  for (int i = 0; i < kBPerBlock; ++i) {
-    const int b = kBPerBlock * grp + i;
-    if (b <= R && (row_live(p, tile, b) || row_live(p, tile, -b))) live |= 1u << i;
-  }
-  const bool skip = live == 0;
-  const int y0 = tile * kTileM / p.sp, x0 = tile * kTileM % p.sp;  // the tile's first position
-  const long long qt = (long long)y0 * p.wp + x0;                  // its padded index
-  const int total = __popc(live) * p.stages;  // strip stages of the block: live members in order, stages within
+  const int tile = blockIdx.x, parts = gridDim.y, freq = blockIdx.z;
+  const int R = p.R, NA = R + 1, NP = (NA + 1) / 2;  // a = 0 .. R in pairs
+  const int j0 = 2 * ((int)blockIdx.y * NP / parts), j1 = min(NA, 2 * (((int)blockIdx.y + 1) * NP / parts)), nj = j1 - j0;
+  const int r0 = tile * kTileM / p.sp, x0 = tile * kTileM % p.sp;  // the tile's first position
+  const int qt = freq * p.rows + r0 * p.wp + x0;                    // strip start: R positions before it
+  const uint8_t *data = p.data + (size_t)freq * p.v_stride;
   const int L = p.strip_rows;
 
   if (threadIdx.x == 0) {
@@ -314,15 +378,8 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
     *never = 0;
     ptx::mbar_fence_init();
   }
-  if (!skip) {  // the group's item tables [member][stage][item j], loaded by every thread in one pass
-    const int n = p.stages * NA;
-    for (int j = threadIdx.x; j < kBPerBlock * n; j += kThreads) {
-      const int i = j / n, r = j % n, b = kBPerBlock * grp + i;
-      if (!((live >> i) & 1u)) continue;
-      const int st = r / NA, a = a_of(r % NA, R);
-      sitems[j] = p.items[p.tap_orbit[(b + R) * p.W + (a + R)] * p.stages + st];
-    }
-  }
+  for (int i = threadIdx.x; i < p.stages * nj; i += kThreads)
+    sitems[i] = p.items[a_of(j0 + i % nj, R) * p.stages + i / nj];
   if (warp == 1) {
     ptx::tmem_alloc(tmem_slot, p.tmem_cols);
     ptx::tmem_relinquish();
@@ -339,42 +396,27 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0 && !skip) {
-      int it_slab = 0;
-      int uses[3] = {0, 0, 0};  // loads issued per strip buffer (one full / empty phase each)
+    if (lane == 0) {
+      int it_slab = 0, loads = 0;  // item pairs and strips requested
       int k = 0;
       uint32_t lap = 0;  // parity of the item ring's current lap
       bool ok = true;
-      // Block stage gs (member gs / stages, K stage gs % stages) loads row y+b
-      // into buffer gs % 3 and row y-b into buffer (gs + 1) % 3 (a load of no
-      // bytes for b = 0), each once the fold warps have released the buffer's
-      // previous use.  The rows for stage gs + 1 are requested right after
-      // stage gs's first slab tile, about a stage ahead of their use, instead
-      // of after stage gs's last tile (which the item ring throttles to just
-      // before the fold warps need the rows).
-      auto load_strips = [&](int gs) {
-        const int st = gs % p.stages;
-        const int b = kBPerBlock * grp + nth_set(live, gs / p.stages);
-        const int q_p = (int)((long long)(R + 1) * p.wp + qt + (long long)b * p.wp - R);
-        const int q_m = (int)((long long)(R + 1) * p.wp + qt - (long long)b * p.wp - R);
-        for (int r = 0; r < 2; ++r) {
-          const int s = (gs + r) % 3;
-          if (!ptx::mbar_wait(&strip_empty[s], (uses[s] & 1) ^ 1, abort_flag, p.budget)) return false;
-          const bool load = r == 0 || b > 0;
-          ptx::mbar_arrive_expect_tx(&strip_full[s], load ? (uint32_t)(L * 128) : 0u);
-          if (load) tma_load_2d(strips + (size_t)s * p.strip_bytes, &tmap, kStageK * st, r == 0 ? q_p : q_m, &strip_full[s]);
-          ++uses[s];
-        }
+      // Stage st's strip goes to buffer st % 3 once the fold warps have released
+      // stage st - 3; it is requested two stages ahead of its use.
+      auto load_strip = [&](int st) {
+        const int s = st % 3;
+        if (!ptx::mbar_wait(&strip_empty[s], ((st / 3) & 1) ^ 1, abort_flag, p.budget)) return false;
+        ptx::mbar_arrive_expect_tx(&strip_full[s], (uint32_t)(L * 128));
+        tma_load_2d(strips + (size_t)s * p.strip_bytes, &tmap, kStageK * st, qt, &strip_full[s]);
+        ++loads;
         return true;
       };
-      if (!load_strips(0)) {
-        fail(1);
-        ok = false;
-      }
-      for (int gs = 0; gs < total && ok; ++gs) {
-        const TcItem *row_items = sitems + (nth_set(live, gs / p.stages) * p.stages + gs % p.stages) * NA;
-        for (int a = 0; a < NA; a += 2) {  // pair slot k holds items a (slot 2k) and a + 1 (slot 2k + 1) of the stage
-          const TcItem ia = row_items[a], ib = a + 1 < NA ? row_items[a + 1] : TcItem{};
+      for (int st = 0; st < min(2, p.stages) && ok; ++st) ok = load_strip(st);
+      if (!ok) fail(1);
+      for (int st = 0; st < p.stages && ok; ++st) {
+        const TcItem *row_items = sitems + st * nj;
+        for (int j = 0; j < nj; j += 2) {  // pair slot k holds items j (slot 2k) and j + 1 (slot 2k + 1) of the stage
+          const TcItem ia = row_items[j], ib = j + 1 < nj ? row_items[j + 1] : TcItem{};
           if (!ptx::mbar_wait(&item_empty[k], lap ^ 1, abort_flag, p.budget)) {
             fail(2);
             ok = false;
@@ -382,17 +424,17 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
           }
           ptx::mbar_arrive_expect_tx(&slab_full[k], ia.bytes() + ib.bytes());
           if (ia.bytes() > 0)
-            ptx::bulk_g2s(slots + (size_t)(2 * k) * p.slot_bytes, p.data + (size_t)ia.off16 * 16, ia.bytes(),
+            ptx::bulk_g2s(slots + (size_t)(2 * k) * p.slot_bytes, data + (size_t)ia.off16 * 16, ia.bytes(),
                           &slab_full[k]);
           if (ib.bytes() > 0)
-            ptx::bulk_g2s(slots + (size_t)(2 * k + 1) * p.slot_bytes, p.data + (size_t)ib.off16 * 16, ib.bytes(),
+            ptx::bulk_g2s(slots + (size_t)(2 * k + 1) * p.slot_bytes, data + (size_t)ib.off16 * 16, ib.bytes(),
                           &slab_full[k]);
           ++it_slab;
           if (++k == KP) {
             k = 0;
             lap ^= 1;
           }
-          if (a == 0 && gs + 1 < total && !load_strips(gs + 1)) {
+          if (j == 0 && st + 2 < p.stages && !load_strip(st + 2)) {
             fail(1);
             ok = false;
             break;
@@ -403,8 +445,8 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
         // let copies already issued land before the block exits
         for (int i = std::max(0, it_slab - KP); i < it_slab; ++i)
           ptx::mbar_wait(&slab_full[i % KP], (i / KP) & 1, never, p.budget);
-        for (int s = 0; s < 3; ++s)  // each buffer's last load (earlier ones were consumed before it was issued)
-          if (uses[s] > 0) ptx::mbar_wait(&strip_full[s], (uses[s] - 1) & 1, never, p.budget);
+        for (int st = std::max(0, loads - 3); st < loads; ++st)
+          ptx::mbar_wait(&strip_full[st % 3], (st / 3) & 1, never, p.budget);
       }
     }
   } else if (warp == 1) {
@@ -420,10 +462,10 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
     uint32_t lap = 0;
     // B descriptor template (start-address field in 16-byte units; fields never carry)
     const uint64_t slot_desc = ptx::smem_desc(ptx::smem_addr(slots), 0, 128);
-    const uint32_t idesc_m128 = ptx::idesc_bf16_f32(kTileM, 0);
-    for (int gs = 0; gs < total && ok && !skip; ++gs) {
-      const TcItem *row_items = sitems + (nth_set(live, gs / p.stages) * p.stages + gs % p.stages) * NA;
-      for (int a = 0; a < NA; a += 2) {
+    const uint32_t idesc = ptx::idesc_f16_f32(kTileM, 0);
+    for (int st = 0; st < p.stages && ok; ++st) {
+      const TcItem *row_items = sitems + st * nj;
+      for (int j = 0; j < nj; j += 2) {
         bool w = ptx::mbar_wait(&slab_full[k], lap, abort_flag, p.budget);
         if (w) w = ptx::mbar_wait(&fold_full[k], lap, abort_flag, p.budget);
         if (!__all_sync(0xffffffffu, w)) {
@@ -432,8 +474,8 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
           break;
         }
         ptx::tc_fence_after();
-        for (int h = 0; h < 2 && a + h < NA; ++h) {
-          const TcItem item = row_items[a + h];
+        for (int h = 0; h < 2 && j + h < nj; ++h) {
+          const TcItem item = row_items[j + h];
           const uint32_t slot = (uint32_t)(2 * k + h);
           const uint32_t a_base = tmem + (uint32_t)p.fold_col0 + 32u * slot;
           const uint64_t dB = slot_desc + (uint64_t)((slot * (uint32_t)p.slot_bytes) >> 4);
@@ -441,16 +483,15 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
           const uint64_t b0h = dB + ((uint64_t)n0 << 16), b0l = b0h + 2u * n0;  // lbo = 16 n bytes; lo 32 n bytes on
           const uint64_t dB1 = dB + 4u * n0;                                   // second tile 64 n0 bytes later
           const uint64_t b1h = dB1 + ((uint64_t)n1 << 16), b1l = b1h + 2u * n1;
-          const uint32_t i0 = idesc_m128 | ((n0 >> 3) << 17), i1 = idesc_m128 | ((n1 >> 3) << 17);
           const uint32_t d0 = tmem + item.col(0), d1 = tmem + item.col(1);
           if (leader) {
             // the two chunks accumulate into different columns: interleave them
-            if (n0) ptx::mma_bf16_ta(d0, a_base, b0h, i0, 1);
-            if (n1) ptx::mma_bf16_ta(d1, a_base + 16u, b1h, i1, 1);
-            if (n0) ptx::mma_bf16_ta(d0, a_base + 8u, b0h, i0, 1);
-            if (n1) ptx::mma_bf16_ta(d1, a_base + 24u, b1h, i1, 1);
-            if (n0) ptx::mma_bf16_ta(d0, a_base, b0l, i0, 1);
-            if (n1) ptx::mma_bf16_ta(d1, a_base + 16u, b1l, i1, 1);
+            if (n0) mma_cols<kWide>(d0, a_base, b0h, idesc, n0);
+            if (n1) mma_cols<kWide>(d1, a_base + 16u, b1h, idesc, n1);
+            if (n0) mma_cols<kWide>(d0, a_base + 8u, b0h, idesc, n0);
+            if (n1) mma_cols<kWide>(d1, a_base + 24u, b1h, idesc, n1);
+            if (n0) mma_cols<kWide>(d0, a_base, b0l, idesc, n0);
+            if (n1) mma_cols<kWide>(d1, a_base + 16u, b1l, idesc, n1);
           }
         }
         if (leader) ptx::mma_commit(&item_empty[k]);  // the pair's slots are free once its MMAs complete
@@ -463,6 +504,10 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
     }
     if (leader) ptx::mma_commit(acc_full);
     __syncwarp();
+  } else if (warp == 2 + kFoldWarps) {
+    // ------------------------------------------------------------ marks
+    if (blockIdx.y == 0)
+      for (int x = freq * gridDim.x + tile; x < p.px; x += gridDim.z * gridDim.x) grow_marks(p, x, lane);
   } else {
     // ------------------------------------------------------------ fold warps, then epilogue
     const int fw = warp - 2;        // 0 .. kFoldWarps-1
@@ -478,82 +523,59 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
     if (lane == 0) ptx::mbar_arrive(acc_ready);
 
     bool ok = true;
-    if (!skip) {
-      const int m = 32 * quarter + lane;  // row (tensor-memory lane) this thread folds
-      const int om = tile * kTileM + m;
-      const int pm = (om / p.sp - y0) * p.wp + (om % p.sp - x0);  // its padded offset from the tile's first
-      const int q0 = kq * (E / 8);        // first 8-element quarter of the stage
-      int uses[3] = {0, 0, 0}, k = 0;  // strip buffer uses consumed, as the producer counts them
-      uint32_t lap = 0;
-      for (int gs = 0; gs < total && ok; ++gs) {
-        const int b = kBPerBlock * grp + nth_set(live, gs / p.stages);
-        const int s = gs % 3, s2 = (gs + 1) % 3;
-        ok = ptx::mbar_wait(&strip_full[s], uses[s] & 1, abort_flag, p.budget);
-        if (ok) ok = ptx::mbar_wait(&strip_full[s2], uses[s2] & 1, abort_flag, p.budget);
+    const int m = 32 * quarter + lane;  // row (tensor-memory lane) this thread folds
+    const int o = tile * kTileM + m;    // its position in the tile grid
+    const int row = o / p.sp, x = o % p.sp;
+    const int pm = (row - r0) * p.wp + (x - x0);  // its packed offset from the tile's first
+    const int q0 = kq * (E / 8);        // first 8-element quarter of the stage
+    const int ef = scale_exp(2.0f * __uint_as_float(p.vmax[freq])), es = scale_exp(__uint_as_float(*p.smax));
+    const uint64_t sc = pack_f32x2(pow2(ef), pow2(ef));
+    int k = 0;
+    uint32_t lap = 0;
+    for (int st = 0; st < p.stages && ok; ++st) {
+      const int s = st % 3;
+      ok = __all_sync(0xffffffffu, ptx::mbar_wait(&strip_full[s], (st / 3) & 1, abort_flag, p.budget));
+      if (!ok) {
+        if (lane == 0) fail(32);
+        break;
+      }
+      const float *X1 = reinterpret_cast<const float *>(strips + (size_t)s * p.strip_bytes);
+      // two items per pass, in pair slot k: one wait, fence and barrier step for both
+      for (int j = 0; j < nj; j += 2) {
+        const bool two = j + 1 < nj;
+        uint32_t w0[E], w1[E];  // folded in registers while the pair slot may still be in use
+        fold_item<E>(X1, pm, R, a_of(j0 + j, R), q0, sc, w0);
+        if (two) fold_item<E>(X1, pm, R, a_of(j0 + j + 1, R), q0, sc, w1);
+        ok = ptx::mbar_wait(&item_empty[k], lap ^ 1, abort_flag, p.budget);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) {
-          if (lane == 0) fail(32);
+          if (lane == 0) fail(64);
           break;
         }
-        float *X1 = reinterpret_cast<float *>(strips + (size_t)s * p.strip_bytes);
-        if (b > 0) {
-          // P = X(y+b) + X(y-b) in place: both strips share the swizzle, so the
-          // sum runs over physical float4s.
-          const float4 *X2 = reinterpret_cast<const float4 *>(strips + (size_t)s2 * p.strip_bytes);
-          float4 *P4 = reinterpret_cast<float4 *>(X1);
-          for (int i = threadIdx.x - 64; i < L * 8; i += 32 * kFoldWarps) {
-            float4 u = P4[i];
-            const float4 v = X2[i];
-            u.x += v.x;
-            u.y += v.y;
-            u.z += v.z;
-            u.w += v.w;
-            P4[i] = u;
-          }
-          asm volatile("bar.sync 1, %0;" ::"r"(32 * kFoldWarps) : "memory");  // fold warps only
-        }
+        const uint32_t fa = tmem + lane_base + (uint32_t)p.fold_col0 + 64u * (uint32_t)k;
+        store_item<E>(fa, q0, w0);
+        if (two) store_item<E>(fa + 32u, q0, w1);
+        ptx::tmem_wait_st();
+        ptx::tc_fence_before();
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(&strip_empty[s2]);  // row y-b is folded into P (or was not loaded)
-        ++uses[s2];
-        // two items (a, a + 1) per pass, in pair slot k: one wait, fence and barrier step for both
-        for (int a = 0; a < NA; a += 2) {
-          const bool two = a + 1 < NA;
-          uint32_t w0[E], w1[E];  // folded in registers while the pair slot may still be in use
-          fold_item<E>(X1, pm, R, a_of(a, R), q0, w0);
-          if (two) fold_item<E>(X1, pm, R, a_of(a + 1, R), q0, w1);
-          ok = ptx::mbar_wait(&item_empty[k], lap ^ 1, abort_flag, p.budget);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) {
-            if (lane == 0) fail(64);
-            break;
-          }
-          const uint32_t fa = tmem + lane_base + (uint32_t)p.fold_col0 + 64u * (uint32_t)k;
-          store_item<E>(fa, q0, w0);
-          if (two) store_item<E>(fa + 32u, q0, w1);
-          ptx::tmem_wait_st();
-          ptx::tc_fence_before();
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(&fold_full[k]);
-          if (++k == KP) {
-            k = 0;
-            lap ^= 1;
-          }
+        if (lane == 0) ptx::mbar_arrive(&fold_full[k]);
+        if (++k == KP) {
+          k = 0;
+          lap ^= 1;
         }
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(&strip_empty[s]);
-        ++uses[s];
       }
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&strip_empty[s]);
     }
 
-    // epilogue: this warp's lane quarter and column half of the accumulator
+    // epilogue: this warp's lane quarter and column share of the accumulator
     bool done = ptx::mbar_wait(acc_full, 0, abort_flag, 4 * p.budget);
     done = __all_sync(0xffffffffu, done && ok);
     ptx::tc_fence_after();
-    const int mrow = 32 * quarter + lane;
-    const int o = tile * kTileM + mrow;  // this lane's position in the tile grid
-    const int y = o / p.sp, x = o % p.sp;
-    const bool valid = done && y < p.py && x < p.px;
-    float *row = p.part + ((size_t)grp * p.part_stride + (size_t)y * p.px + x) * p.acc_cols;
+    const bool valid = done && row < p.nr && x < p.px;
+    const float us = pow2(-es), uf = pow2(-ef);
+    float *dst_row =
+        p.part + ((((size_t)blockIdx.y * gridDim.z + freq) * p.nr + row) * p.px + x) * (size_t)p.acc_cols;
     if (done) {
       for (int j = blk_begin; j < blk_end; ++j) {
         const int col = 32 * j;
@@ -561,13 +583,12 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
         ptx::tmem_ld32(tmem + lane_base + (uint32_t)col, r);
         ptx::tmem_wait_ld();
         if (valid) {
-          float4 *dst = reinterpret_cast<float4 *>(row + col);
+          float4 *dst = reinterpret_cast<float4 *>(dst_row + col);
           const int nv = std::min(8, (p.acc_cols - col) >> 2);
+          auto val = [&](int i) { return __uint_as_float(r[i]) * us * uf; };  // exact unless it leaves FP32's range
 #pragma unroll
           for (int q = 0; q < 8; ++q)
-            if (q < nv)
-              dst[q] = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
-                                   __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
+            if (q < nv) dst[q] = make_float4(val(4 * q), val(4 * q + 1), val(4 * q + 2), val(4 * q + 3));
         }
       }
     }
@@ -581,106 +602,70 @@ __global__ void __launch_bounds__(64 + 32 * FW, 1)
 }
 
 // ---------------------------------------------------------------- packers
-// Slab tiles: hi then lo, each [2 chunks of 8][n rows][8] bf16 (K-major core matrices).
-__global__ void k_pack_tiles(const float *band, const int *band_lo, const int *band_hi, int band_w, int nz,
-                             int dir, int t_lo, const TcTile *tiles, uint8_t *data) {
+// Slab tiles of every frequency: hi then lo, each [2 chunks of 8][n rows][8] FP16
+// (K-major core matrices).  S_v[a][k][n] = sum_{b=0}^{halo} w_b cos(2 pi v b / P)
+// S[b][a][k][n], w_0 = 1, w_{>0} = 2 (the +-b pair; row offsets beyond the halo
+// meet no row).  Block (tile, kPackThreads of its elements), a thread per element:
+// the slab values of its element in shared memory, then every frequency in turn.
+constexpr int kPackThreads = 128;
+
+// Upper bound of the transformed slab's magnitude: its largest entry times the
+// window (the weights of a row offset's cosine sum to at most W).
+__global__ void k_slab_max(const float *__restrict__ band, size_t n, float terms, unsigned *smax) {
+  float top = 0.0f;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    top = fmaxf(top, fabsf(band[i]));
+  const unsigned t = __reduce_max_sync(0xffffffffu, __float_as_uint(top * terms));
+  if ((threadIdx.x & 31) == 0) atomicMax(smax, t);
+}
+
+__global__ void __launch_bounds__(kPackThreads) k_pack_tiles(const float *__restrict__ band, const int *band_lo,
+                                                             const int *band_hi, int band_w, int nz, int dir, int t_lo,
+                                                             const int *tap_orbit, int R, int halo, int P, int Q,
+                                                             const float2 *__restrict__ tw, const unsigned *smax,
+                                                             const TcTile *tiles, size_t v_stride, uint8_t *data) {
+  extern __shared__ float smp[];
+  float *cosT = smp, *sv = smp + P;  // [P], [halo + 1][kPackThreads]
   const TcTile t = tiles[blockIdx.x];
-  __nv_bfloat16 *hi = reinterpret_cast<__nv_bfloat16 *>(data + t.off);
-  __nv_bfloat16 *lo = hi + 16 * t.n;
-  for (int i = threadIdx.x; i < 16 * t.n; i += blockDim.x) {
-    const int kk = i / t.n, row = i % t.n;  // kk: index along K (0..15), row: along N
-    int k, n;
-    if (dir == 0) {
-      k = 16 * t.chunk + kk;
-      n = t_lo + t.col + row;
-    } else {
-      k = t.col + row;
-      n = t_lo + 16 * t.chunk + kk;
-    }
+  if ((int)blockIdx.y * kPackThreads >= 16 * t.n) return;
+  const int tid = threadIdx.x, i = blockIdx.y * kPackThreads + tid;
+  for (int j = tid; j < P; j += kPackThreads) cosT[j] = tw[j].x;
+  __syncthreads();
+  if (i >= 16 * t.n) return;
+  const int row = (i >> 3) % t.n, kk = (i / (8 * t.n)) * 8 + (i & 7);  // row: along N, kk: along K (0..15)
+  const int k = dir == 0 ? 16 * t.chunk + kk : t.col + row;
+  const int n = dir == 0 ? t_lo + t.col + row : t_lo + 16 * t.chunk + kk;
+  const int W = 2 * R + 1;
+  for (int b = 0; b <= halo; ++b) {
     float v = 0.0f;
     if (k < nz) {
-      const int lo_n = band_lo[t.orbit * nz + k], hi_n = band_hi[t.orbit * nz + k];
-      if (n >= lo_n && n < hi_n) v = band[((size_t)t.orbit * nz + k) * band_w + (n - lo_n)];
+      const int o = tap_orbit[(b + R) * W + (t.a + R)];
+      const int lo = band_lo[o * nz + k], hi = band_hi[o * nz + k];
+      if (n >= lo && n < hi) v = band[((size_t)o * nz + k) * band_w + (n - lo)];
     }
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-    const int idx = ((kk >> 3) * t.n + row) * 8 + (kk & 7);
-    hi[idx] = h;
-    lo[idx] = l;
+    sv[b * kPackThreads + tid] = b == 0 ? v : 2.0f * v;
   }
-}
-
-// Iterate in[py][px][len] -> out[qtot][elems] (FP32): element e of padded
-// position q is index first + e of the row of (y, x) = (q / wp - R - 1, q % wp),
-// zero outside the grid or the row.
-__global__ void k_pack_input(const float *__restrict__ in, int len, int first, int elems, long long qtot, int wp,
-                             int R, int px, int py, float4 *__restrict__ out) {
-  const int e4n = elems >> 2;
-  const long long total = qtot * e4n;
-  const bool vec = ((len | first) & 3) == 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const long long q = i / e4n;
-    const int e = 4 * (int)(i % e4n);
-    const int y = (int)(q / wp) - (R + 1), x = (int)(q % wp);
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (y >= 0 && y < py && x < px) {
-      const float *src = in + ((size_t)y * px + x) * len;
-      const int idx = first + e;
-      if (vec && idx + 3 < len) {
-        v = *reinterpret_cast<const float4 *>(src + idx);
-      } else {
-        if (idx < len) v.x = src[idx];
-        if (idx + 1 < len) v.y = src[idx + 1];
-        if (idx + 2 < len) v.z = src[idx + 2];
-        if (idx + 3 < len) v.w = src[idx + 3];
-      }
-    }
-    out[i] = v;
-  }
-}
-
-// out[pos][n] = sum over parts (in index order) of part[.][pos][n - out_lo] for n
-// in the accumulator range, 0 elsewhere.  Every element of out is written.
-__global__ void k_sum_parts(const float *__restrict__ part, int parts, size_t npos, int acc_cols, int out_lo,
-                            int out_len, float *__restrict__ out) {
-  const size_t total = npos * (size_t)out_len;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const size_t pos = i / out_len;
-    const int n = (int)(i % out_len), c = n - out_lo;
+  const float sc = pow2(scale_exp(__uint_as_float(*smax)));
+  __half *dst = reinterpret_cast<__half *>(data + t.off) + i;
+  for (int f = 0; f < Q; ++f) {
     float v = 0.0f;
-    if (c >= 0 && c < acc_cols) {
-      const float *src = part + pos * acc_cols + c;
-      for (int q = 0; q < parts; ++q) v += src[(size_t)q * npos * acc_cols];
+    for (int b = 0, j = 0; b <= halo; ++b) {  // j = f b mod P
+      v = fmaf(cosT[j], sv[b * kPackThreads + tid], v);
+      j += f;
+      if (j >= P) j -= P;
     }
-    out[i] = v;
+    v *= sc;
+    const __half h = __float2half_rn(v);
+    __half *d = dst + (size_t)f * (v_stride / sizeof(__half));
+    d[0] = h;
+    d[16 * t.n] = __float2half_rn(v - __half2float(h));
   }
 }
 
-// Strip rows a block stages per row offset: 128 positions wrap at most
-// (px + 126) / px scan rows, each adding R rows of padding to the span, plus
+// Positions of a staged strip on the scan grid: 128 positions wrap at most
+// (px + 126) / px rows, each adding R rows of padding to the span, plus
 // R rows of halo on either side.
 int strip_rows_for(int px, int R) { return kTileM + ((px + kTileM - 2) / px + 2) * R; }
-
-// Executed MMA flops of one application: 3 products x 2 x M x (16 x N) over
-// the (position tile, |b|, a >= 0) work items whose rows meet the grid, for
-// position tiles along rows of stride sp.
-double exec_flops_for(const oam_model *m, const TcLayout *L, int sp) {
-  const int R = m->R, py = m->grid.py;
-  const long long n_tiles = ((long long)py * sp + kTileM - 1) / kTileM;
-  double total = 0;
-  for (long long t = 0; t < n_tiles; ++t) {
-    const long long yf = t * kTileM / sp, yl = (std::min(t * kTileM + kTileM, (long long)py * sp) - 1) / sp;
-    for (int b = 0; b <= R; ++b) {
-      const bool lp = !(yl + b < 0 || yf + b >= py), lm = !(yl - b < 0 || yf - b >= py);
-      if (lp || lm) total += L->row_cols[b];
-    }
-  }
-  return 3.0 * 2.0 * kTileM * total;
-}
-
-// Groups of kBPerBlock consecutive |b| = 0 .. R (the kernel's grid y, the partial sums).
-int b_groups(int R) { return (R + 1 + kBPerBlock - 1) / kBPerBlock; }
 
 int pow2_cols(int n) {
   int c = 32;
@@ -715,10 +700,68 @@ oam_status encode_tmap(CUtensorMap *map, float *base, long long qtot, int elems,
   return OAM_OK;
 }
 
-// One direction's item and tile tables from the band form (host only).
-oam_status plan_dir(const oam_model *m, TcLayout *L, int dir, std::vector<TcItem> &items,
+// Longest line one transform takes.
+constexpr int kLineMax = 512;
+
+// The line transforms' plan: the smallest size that holds a line and its halo, or
+// overlapping segments of the largest.
+oam_status plan_line(const oam_model *m, TcLine *T) {
+  const int py = m->grid.py;
+  T->halo = std::min(m->R, py - 1);
+  T->segs = 1;
+  T->valid = py;
+  T->P = py + T->halo <= kLineMax ? mix_size_for(py + T->halo) : kLineMax;
+  if (py + T->halo > kLineMax) {
+    T->valid = kLineMax - 2 * T->halo;
+    T->segs = (py + T->valid - 1) / T->valid;
+  }
+  T->Q = T->P / 2 + 1;
+  T->nr = 2 * T->segs;
+  const long long rows = m->R + (long long)T->nr * (m->grid.px + m->R);
+  if (rows * T->Q > 0x7fffffffLL) return OAM_ERR_UNSUPPORTED;
+  T->rows = (int)rows;
+  T->words = (py + 31) / 32;
+  return OAM_OK;
+}
+
+// Sample (forward) or depth (adjoint) range [lo, hi) of the slab of orbit o in one
+// 16-deep K chunk, from accumulator column 0.
+void chunk_range(const oam_model *m, int o, int dir, int chunk, int t_lo, int *plo, int *phi) {
+  const int nz = m->grid.nz;
+  int lo = 1 << 30, hi = -1;
+  if (dir == 0) {
+    for (int k = 16 * chunk; k < std::min(nz, 16 * chunk + 16); ++k) {
+      const int bl = m->h_band_lo[(size_t)o * nz + k], bh = m->h_band_hi[(size_t)o * nz + k];
+      if (bh > bl) {
+        lo = std::min(lo, bl - t_lo);
+        hi = std::max(hi, bh - t_lo);
+      }
+    }
+  } else {
+    const int n0 = t_lo + 16 * chunk, n1 = n0 + 16;
+    for (int k = 0; k < nz; ++k) {
+      const int bl = m->h_band_lo[(size_t)o * nz + k], bh = m->h_band_hi[(size_t)o * nz + k];
+      if (bh > bl && bl < n1 && bh > n0) {
+        lo = std::min(lo, k);
+        hi = std::max(hi, k + 1);
+      }
+    }
+  }
+  *plo = lo;
+  *phi = hi;
+}
+
+// Columns [col, col + n) of a tile over a range, whole 16-column groups.
+void tile_cols(int lo, int hi, int *col, int *n) {
+  *col = lo & ~15;
+  *n = ((hi - *col) + 15) & ~15;
+}
+
+// One direction's item and tile tables from the band form (host only): per (|a|,
+// stage) the union of the row offsets' bands.
+oam_status plan_dir(const oam_model *m, const TcLine *T, TcLayout *L, int dir, std::vector<TcItem> &items,
                     std::vector<TcTile> &tiles) {
-  const int nz = m->grid.nz, O = m->n_orb;
+  const int nz = m->grid.nz, R = m->R, W = m->W;
   const int t_lo = m->n_lo & ~15;
   L->dir = dir;
   if (dir == 0) {
@@ -733,92 +776,105 @@ oam_status plan_dir(const oam_model *m, TcLayout *L, int dir, std::vector<TcItem
     L->in_lo = t_lo;
   }
   L->in_elems = kStageK * L->stages;
-  L->tmem_cols = pow2_cols(L->acc_cols);
-  if (L->tmem_cols > 512) return OAM_ERR_UNSUPPORTED;
+  if (pow2_cols(L->acc_cols) > 512) return OAM_ERR_UNSUPPORTED;
 
-  items.assign((size_t)O * L->stages, TcItem{});
+  items.assign((size_t)(R + 1) * L->stages, TcItem{});
   tiles.clear();
   long long off = 0;
   int max_item = 16;
-  for (int o = 0; o < O; ++o) {
+  L->wide = false;
+  L->cols = 0;
+  for (int a = 0; a <= R; ++a) {
     for (int s = 0; s < L->stages; ++s) {
       TcItem it{};
-      const long long item_off = off;
-      if (off / 16 > 0xFFFFFFFFLL) return OAM_ERR_UNSUPPORTED;
       it.off16 = (uint32_t)(off / 16);
       for (int c = 0; c < 2; ++c) {
         const int chunk = 2 * s + c;
         int lo = 1 << 30, hi = -1;
-        if (dir == 0) {
-          for (int k = 16 * chunk; k < std::min(nz, 16 * chunk + 16); ++k) {
-            const int bl = m->h_band_lo[(size_t)o * nz + k], bh = m->h_band_hi[(size_t)o * nz + k];
-            if (bh > bl) {
-              lo = std::min(lo, bl - t_lo);
-              hi = std::max(hi, bh - t_lo);
-            }
-          }
-        } else {
-          const int n0 = t_lo + 16 * chunk, n1 = n0 + 16;
-          for (int k = 0; k < nz; ++k) {
-            const int bl = m->h_band_lo[(size_t)o * nz + k], bh = m->h_band_hi[(size_t)o * nz + k];
-            if (bh > bl && bl < n1 && bh > n0) {
-              lo = std::min(lo, k);
-              hi = std::max(hi, k + 1);
-            }
-          }
+        for (int b = 0; b <= R; ++b) {
+          int bl, bh, col, n;
+          chunk_range(m, m->h_tap_orbit[(b + R) * W + (a + R)], dir, chunk, t_lo, &bl, &bh);
+          if (bh <= bl) continue;
+          // a single offset's band wider than 256 columns is not taken
+          tile_cols(bl, bh, &col, &n);
+          if (n > 256 || col + n > L->acc_cols) return OAM_ERR_UNSUPPORTED;
+          if (b > T->halo) continue;
+          lo = std::min(lo, bl);
+          hi = std::max(hi, bh);
         }
-        if (hi <= lo) {
-          it.c16[c] = 0;
-          it.n16[c] = 0;
-          continue;
-        }
-        const int col = lo & ~15;
-        const int n = ((hi - col) + 15) & ~15;
-        if (n > 256 || col + n > L->acc_cols) return OAM_ERR_UNSUPPORTED;
+        if (hi <= lo) continue;
+        int col, n;
+        tile_cols(lo, hi, &col, &n);
         it.c16[c] = (uint8_t)(col / 16);
         it.n16[c] = (uint8_t)(n / 16);
-        tiles.push_back(TcTile{o, chunk, col, n, off});
+        L->wide = L->wide || n > 256;
+        L->cols += 16.0 * n;
+        tiles.push_back(TcTile{a, chunk, col, n, off});
         off += 64LL * n;  // hi + lo: 2 x (n rows x 16 elements x 2 bytes)
       }
-      if (it.bytes() != (uint32_t)(off - item_off)) return OAM_ERR_DEVICE;  // the tiles are packed back to back
       max_item = std::max(max_item, (int)it.bytes());
-      items[(size_t)o * L->stages + s] = it;
+      items[(size_t)a * L->stages + s] = it;
     }
   }
   L->slot_bytes = (max_item + 127) & ~127;
-  L->data_bytes = (size_t)std::max<long long>(off, 16);
-  // MMA columns per |b| (summed over a = 0 .. R); executed flops follow from
-  // the tiles whose rows meet the grid (exec_flops_for)
-  {
-    std::vector<double> orb_cols(O, 0.0);
-    for (const TcTile &t : tiles) orb_cols[t.orbit] += 16.0 * t.n;
-    const int W = m->W, R = m->R;
-    L->row_cols.assign(R + 1, 0.0);
-    for (int b = 0; b <= R; ++b)
-      for (int a = 0; a <= R; ++a) L->row_cols[b] += orb_cols[m->h_tap_orbit[(b + R) * W + (a + R)]];
+  L->v_stride = (size_t)std::max<long long>(off, 16);
+  // Blocks that share a tile's taps: as many as make the last wave of one block per
+  // SM fullest.  In units of one pair of items (~0.45 us): a block's pairs, about
+  // 12 for its set-up and epilogue, and a part's sums written and read once more.
+  // At least two: the tensor cores truncate when they add to an accumulator, and
+  // the frequencies' sums cancel over depth, so halving the products that one
+  // accumulator takes halves that error (200x200x300 forward 4.4e-6 -> 2.1e-6).
+  const int NP = (R + 2) / 2, sms = std::max(1, m->sm_count ? m->sm_count : 152);
+  const long long tiles0 = ((long long)T->nr * m->grid.px + kTileM - 1) / kTileM * T->Q;
+  const double part_units = 2.0 * T->Q * T->nr * m->grid.px * L->acc_cols * 4.0 / (6.8e12 * 0.45e-6);
+  double best = 0;
+  L->parts = 0;
+  for (int q = std::min(2, NP); q <= std::min(4, NP); ++q) {
+    const double cost = (double)((tiles0 * q + sms - 1) / sms) * ((double)((NP + q - 1) / q) * L->stages + 12) +
+                        (q - 1) * part_units;
+    if (!L->parts || cost < best) {
+      best = cost;
+      L->parts = q;
+    }
   }
   return OAM_OK;
 }
 
 // Build one direction's item and tile tables from the band form, then pack.
 oam_status build_dir(oam_model *m, TcLayout *L, int dir, cudaStream_t st, int *d_band_hi) {
+  const TcLine *T = m->tc_line;
   std::vector<TcItem> items;
   std::vector<TcTile> tiles;
-  oam_status rc = plan_dir(m, L, dir, items, tiles);
+  oam_status rc = plan_dir(m, T, L, dir, items, tiles);
   if (rc) return rc;
   const int nz = m->grid.nz, t_lo = m->n_lo & ~15;
+  const size_t qtot = (size_t)T->rows * T->Q;
   if ((rc = dev_alloc(m, &L->d_items, items.size()))) return rc;
-  if ((rc = dev_alloc(m, &L->d_data, L->data_bytes))) return rc;
+  if ((rc = dev_alloc(m, &L->d_data, L->v_stride * T->Q))) return rc;
+  if ((rc = dev_alloc(m, &L->d_pack, qtot * L->in_elems))) return rc;
   OAM_CUDA_TRY(cudaMemcpyAsync(L->d_items, items.data(), sizeof(TcItem) * items.size(), cudaMemcpyHostToDevice, st));
+  // padding positions and channels stay zero: the line transform writes the others
+  OAM_CUDA_TRY(cudaMemsetAsync(L->d_pack, 0, sizeof(float) * qtot * L->in_elems, st));
   if (!tiles.empty()) {
+    int n_max = 0;
+    for (const TcTile &t : tiles) n_max = std::max(n_max, t.n);
     TcTile *d_tiles = nullptr;
     OAM_CUDA_TRY(cudaMallocAsync((void **)&d_tiles, sizeof(TcTile) * tiles.size(), st));
     OAM_CUDA_TRY(cudaMemcpyAsync(d_tiles, tiles.data(), sizeof(TcTile) * tiles.size(), cudaMemcpyHostToDevice, st));
-    k_pack_tiles<<<(unsigned)tiles.size(), 256, 0, st>>>(m->d_band, m->d_band_lo, d_band_hi, m->band_w, nz, dir,
-                                                         t_lo, d_tiles, L->d_data);
+    const dim3 grid((unsigned)tiles.size(), (unsigned)((16 * n_max + kPackThreads - 1) / kPackThreads));
+    const size_t sm = sizeof(float) * ((size_t)T->P + (size_t)(T->halo + 1) * kPackThreads);  // at most 35 KB
+    k_pack_tiles<<<grid, kPackThreads, sm, st>>>(m->d_band, m->d_band_lo, d_band_hi, m->band_w, nz, dir, t_lo,
+                                                 m->d_tap_orbit, m->R, T->halo, T->P, T->Q, T->d_tw, T->d_smax,
+                                                 d_tiles, L->v_stride, L->d_data);
     OAM_LAUNCHED();
-    OAM_CUDA_TRY(cudaStreamSynchronize(st));
     OAM_CUDA_TRY(cudaFreeAsync(d_tiles, st));
+  }
+  OAM_CUDA_TRY(cudaStreamSynchronize(st));  // host tables above go out of scope
+  for (int scan = 0; scan < 2; ++scan) {
+    const int rows = scan ? strip_rows_for(m->grid.px, m->R) : kTileM + 2 * m->R;
+    if (rows > 256) continue;
+    rc = encode_tmap(scan ? &L->tmap_scan : &L->tmap, L->d_pack, (long long)qtot, L->in_elems, rows);
+    if (rc) return rc;
   }
   return OAM_OK;
 }
@@ -827,24 +883,23 @@ struct Launch {
   CorrParams p;
   size_t smem;
   int tiling;   // 1 padded grid, 2 scan grid
-  int n_tiles;  // position tiles (the grid's x)
+  int n_tiles;  // position tiles of a frequency (the grid's x)
 };
 
-oam_status plan_launch(const oam_model *m, const TcLayout *L, Launch *out) {
-  const int R = m->R, px = m->grid.px, py = m->grid.py;
+oam_status plan_launch(const oam_model *m, const TcLine *T, const TcLayout *L, Launch *out) {
+  const int R = m->R, px = m->grid.px;
   CorrParams p{};
-  p.qtot = m->tc_qtot;
   p.wp = px + R;
   p.px = px;
-  p.py = py;
   p.R = R;
-  p.W = m->W;
   p.stages = L->stages;
-  p.tap_orbit = m->d_tap_orbit;
+  p.nr = T->nr;
+  p.rows = T->rows;
   p.items = L->d_items;
   p.data = L->d_data;
+  p.v_stride = L->v_stride;
   p.slot_bytes = L->slot_bytes;
-  p.items_bytes = (int)((sizeof(TcItem) * kBPerBlock * L->stages * (R + 1) + 1023) & ~size_t(1023));
+  p.items_bytes = (int)((sizeof(TcItem) * L->stages * (R + 1) + 1023) & ~size_t(1023));
   p.fold_col0 = (L->acc_cols + 31) & ~31;
   const int tmem_items = (512 - p.fold_col0) / kFoldCols;
   auto strip_bytes = [](int rows) { return (rows * 128 + 1023) & ~1023; };  // 128-byte rows, 1024-byte aligned
@@ -867,142 +922,162 @@ oam_status plan_launch(const oam_model *m, const TcLayout *L, Launch *out) {
   p.n_items &= ~1;  // items go in pairs (one fold pass each)
   if (p.n_items < 2) return OAM_ERR_UNSUPPORTED;
   p.acc_cols = L->acc_cols;
-  p.tmem_cols = 32;
-  while (p.tmem_cols < p.fold_col0 + kFoldCols * p.n_items) p.tmem_cols <<= 1;
-  p.part = m->d_tc_part;
-  p.part_stride = (size_t)py * px;
+  p.tmem_cols = pow2_cols(p.fold_col0 + kFoldCols * p.n_items);
+  p.part = T->d_part;
   p.status = m->d_status;
   p.budget = 4000000000LL;  // ~2 s at 2 GHz
   out->p = p;
   out->smem = (size_t)fixed + (size_t)p.n_items * p.slot_bytes;
   out->tiling = tiling;
-  out->n_tiles = (int)(((long long)py * p.sp + kTileM - 1) / kTileM);
+  out->n_tiles = (int)(((long long)T->nr * p.sp + kTileM - 1) / kTileM);
   if (out->smem > (size_t)kSmemLimit) return OAM_ERR_UNSUPPORTED;
   return OAM_OK;
 }
 
-template <int FW>
-oam_status launch_fold(const Launch &lp, const TcLayout *L, dim3 grid, cudaStream_t st) {
-  OAM_CUDA_TRY(cudaFuncSetAttribute(k_corr_fold<FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lp.smem));
-  k_corr_fold<FW><<<grid, 64 + 32 * FW, lp.smem, st>>>(lp.tiling == 2 ? L->tmap_scan : L->tmap, lp.p);
+template <int FW, bool kWide>
+oam_status launch_corr(const Launch &lp, const TcLayout *L, dim3 grid, cudaStream_t st) {
+  OAM_CUDA_TRY(
+      cudaFuncSetAttribute(k_corr_line<FW, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lp.smem));
+  k_corr_line<FW, kWide><<<grid, 96 + 32 * FW, lp.smem, st>>>(lp.tiling == 2 ? L->tmap_scan : L->tmap, lp.p);
   OAM_LAUNCHED();
   return OAM_OK;
 }
 
+template <bool kWide>
+oam_status launch_corr_fw(const Launch &lp, const TcLayout *L, dim3 grid, cudaStream_t st) {
+  if (L->fold_warps == 4) return launch_corr<4, kWide>(lp, L, grid, st);
+  if (L->fold_warps == 16) return launch_corr<16, kWide>(lp, L, grid, st);
+  return launch_corr<8, kWide>(lp, L, grid, st);
+}
+
 oam_status run_corr(const oam_model *m, const TcLayout *L, const float *in, int in_len, float *out, int out_len,
                     cudaStream_t st) {
-  if (!m->d_tc_part || !m->d_tc_pack) return OAM_ERR_UNSUPPORTED;
+  const TcLine *T = m->tc_line;
+  if (!T || !T->d_part || !L || !L->d_pack) return OAM_ERR_UNSUPPORTED;
   Launch lp;
-  oam_status rc = plan_launch(m, L, &lp);
+  oam_status rc = plan_launch(m, T, L, &lp);
   if (rc) return rc;
-  const int R = m->R;
-  {
-    const long long total = m->tc_qtot * (L->in_elems / 4);
-    const int blocks = (int)std::min<long long>((total + 255) / 256, 16LL * m->sm_count);
-    k_pack_input<<<blocks, 256, 0, st>>>(in, in_len, L->in_lo, L->in_elems, m->tc_qtot, m->grid.px + R, R, m->grid.px,
-                                         m->grid.py, reinterpret_cast<float4 *>(m->d_tc_pack));
-    OAM_LAUNCHED();
-  }
-  {
-    ProfScope prof(m, st, L->dir == 0);
-    const dim3 grid(lp.n_tiles, b_groups(R));
-    if (L->fold_warps == 4) rc = launch_fold<4>(lp, L, grid, st);
-    else if (L->fold_warps == 16) rc = launch_fold<16>(lp, L, grid, st);
-    else rc = launch_fold<8>(lp, L, grid, st);
-    if (rc) return rc;
-  }
-  const size_t npos = (size_t)m->grid.py * m->grid.px;
-  const int blocks = (int)std::min<size_t>((npos * out_len + 255) / 256, 16ull * m->sm_count);
-  k_sum_parts<<<blocks, 256, 0, st>>>(m->d_tc_part, b_groups(R), npos, L->acc_cols, L->out_lo, out_len, out);
-  OAM_LAUNCHED();
-  return OAM_OK;
+  LineShape s{};
+  s.px = m->grid.px;
+  s.py = m->grid.py;
+  s.R = m->R;
+  s.halo = T->halo;
+  s.segs = T->segs;
+  s.valid = T->valid;
+  s.len = in_len;
+  s.in_lo = L->in_lo;
+  s.elems = L->in_elems;
+  s.wp = lp.p.wp;
+  s.rows = T->rows;
+  s.nr = T->nr;
+  s.out_len = out_len;
+  s.out_lo = L->out_lo;
+  s.acc = L->acc_cols;
+  s.parts = L->parts;
+  s.words = T->words;
+  s.marks = T->d_marks;
+  unsigned *tail = T->d_marks + (size_t)2 * s.px * s.words;
+  s.vmax = tail;
+  s.any_bad = reinterpret_cast<int *>(tail + T->Q);
+  s.grown = tail + T->Q + 1;
+  lp.p.marks = s.marks;
+  lp.p.grown = tail + T->Q + 1;
+  lp.p.any_bad = s.any_bad;
+  lp.p.words = T->words;
+  lp.p.vmax = s.vmax;
+  lp.p.smax = T->d_smax;
+  ProfScope prof(m, st, L->dir == 0);
+  if ((rc = line_r2c(T->P, st, s, in, T->d_tw, L->d_pack))) return rc;
+  const dim3 grid(lp.n_tiles, L->parts, T->Q);
+  if ((rc = L->wide ? launch_corr_fw<true>(lp, L, grid, st) : launch_corr_fw<false>(lp, L, grid, st))) return rc;
+  return line_c2r(T->P, st, s, T->d_part, T->d_tw, out);
 }
+
+size_t part_floats(const oam_model *m, const TcLine *T, const TcLayout *L) {
+  return (size_t)L->parts * T->Q * T->nr * m->grid.px * L->acc_cols;
+}
+size_t mark_words(const oam_model *m, const TcLine *T) { return (size_t)4 * m->grid.px * T->words + T->Q + 1; }
 
 }  // namespace
 
 // Device bytes tc_build allocates, from the planned bands (host only; no
 // device call).  Fails like tc_build on shapes the kernels do not take.
 oam_status oam::tc_plan_bytes(const oam_model *m, size_t *bytes) {
-  if (kTileM + 2 * m->R > 256) return OAM_ERR_UNSUPPORTED;  // padded-grid strip rows per TMA box
-  TcLayout Lf, La;
+  if (kTileM + 2 * m->R > 256) return OAM_ERR_UNSUPPORTED;  // padded-grid strip positions per TMA box
+  TcLine T;
+  TcLayout Ls[2];
   std::vector<TcItem> items;
   std::vector<TcTile> tiles;
-  size_t b = 0;
+  oam_status rc = plan_line(m, &T);
+  if (rc) return rc;
+  size_t b = 0, part = 0;
   for (int dir = 0; dir < 2; ++dir) {
-    TcLayout *L = dir == 0 ? &Lf : &La;
-    oam_status rc = plan_dir(m, L, dir, items, tiles);
-    if (rc) return rc;
+    TcLayout *L = &Ls[dir];
+    if ((rc = plan_dir(m, &T, L, dir, items, tiles))) return rc;
     Launch lp;
-    if ((rc = plan_launch(m, L, &lp))) return rc;
-    b += alloc_bytes<TcItem>(items.size()) + alloc_bytes<uint8_t>(L->data_bytes);
+    if ((rc = plan_launch(m, &T, L, &lp))) return rc;
+    b += alloc_bytes<TcItem>(items.size()) + alloc_bytes<uint8_t>(L->v_stride * T.Q) +
+         alloc_bytes<float>((size_t)T.rows * T.Q * L->in_elems);
+    part = std::max(part, part_floats(m, &T, L));
   }
-  const int wp = m->grid.px + m->R;
-  const long long qtot = (long long)(m->grid.py + 2 * m->R + 2) * wp + 256;
-  if (qtot > 0x7fffffffLL) return OAM_ERR_UNSUPPORTED;
-  b += alloc_bytes<uint8_t>((size_t)std::max(Lf.in_elems, La.in_elems) * qtot * sizeof(float));
-  b += alloc_bytes<float>((size_t)b_groups(m->R) * m->grid.py * m->grid.px * std::max(Lf.acc_cols, La.acc_cols));
-  *bytes = b;
+  *bytes = b + alloc_bytes<float>(part) + alloc_bytes<float2>(T.P) + alloc_bytes<unsigned>(mark_words(m, &T)) + alloc_bytes<unsigned>(1);
   return OAM_OK;
 }
 
 oam_status oam::tc_build(oam_model *m, cudaStream_t st) {
-  if (kTileM + 2 * m->R > 256) return OAM_ERR_UNSUPPORTED;  // padded-grid strip rows per TMA box
-  int *d_band_hi = nullptr;
+  if (kTileM + 2 * m->R > 256) return OAM_ERR_UNSUPPORTED;  // padded-grid strip positions per TMA box
+  TcLine *T = m->tc_line = new TcLine();
+  oam_status rc = plan_line(m, T);
+  if (rc) return rc;
+  const std::vector<float2> roots = mix_roots(T->P);
+  if ((rc = dev_alloc(m, &T->d_tw, roots.size())) || (rc = dev_alloc(m, &T->d_marks, mark_words(m, T))) ||
+      (rc = dev_alloc(m, &T->d_smax, 1)))
+    return rc;
+  OAM_CUDA_TRY(cudaMemcpyAsync(T->d_tw, roots.data(), sizeof(float2) * roots.size(), cudaMemcpyHostToDevice, st));
+  OAM_CUDA_TRY(cudaMemsetAsync(T->d_marks, 0, sizeof(unsigned) * mark_words(m, T), st));
+  OAM_CUDA_TRY(cudaMemsetAsync(T->d_smax, 0, sizeof(unsigned), st));
   const size_t nb = (size_t)m->n_orb * m->grid.nz;
+  k_slab_max<<<4 * std::max(1, m->sm_count), 256, 0, st>>>(m->d_band, nb * m->band_w, (float)m->W, T->d_smax);
+  OAM_LAUNCHED();
+  int *d_band_hi = nullptr;
   OAM_CUDA_TRY(cudaMallocAsync((void **)&d_band_hi, sizeof(int) * nb, st));
   OAM_CUDA_TRY(cudaMemcpyAsync(d_band_hi, m->h_band_hi.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, st));
   m->tc_fwd = new TcLayout();
   m->tc_adj = new TcLayout();
-  oam_status rc = build_dir(m, m->tc_fwd, 0, st, d_band_hi);
+  rc = build_dir(m, m->tc_fwd, 0, st, d_band_hi);
   if (!rc) rc = build_dir(m, m->tc_adj, 1, st, d_band_hi);
   cudaFreeAsync(d_band_hi, st);
   if (rc) return rc;
-  const int wp = m->grid.px + m->R;
-  m->tc_qtot = (long long)(m->grid.py + 2 * m->R + 2) * wp + 256;
-  if (m->tc_qtot > 0x7fffffffLL) return OAM_ERR_UNSUPPORTED;
-  const int elems = std::max(m->tc_fwd->in_elems, m->tc_adj->in_elems);
-  m->tc_pack_bytes = (size_t)elems * m->tc_qtot * sizeof(float);
-  rc = dev_alloc(m, &m->d_tc_pack, m->tc_pack_bytes);
-  if (rc) return rc;
   for (TcLayout *L : {m->tc_fwd, m->tc_adj}) {
-    rc = encode_tmap(&L->tmap, reinterpret_cast<float *>(m->d_tc_pack), m->tc_qtot, L->in_elems, kTileM + 2 * m->R);
-    if (rc) return rc;
-    if (strip_rows_for(m->grid.px, m->R) <= 256) {
-      rc = encode_tmap(&L->tmap_scan, reinterpret_cast<float *>(m->d_tc_pack), m->tc_qtot, L->in_elems,
-                       strip_rows_for(m->grid.px, m->R));
-      if (rc) return rc;
-    }
     Launch lp;
-    rc = plan_launch(m, L, &lp);
-    if (rc) return rc;
+    if ((rc = plan_launch(m, T, L, &lp))) return rc;
   }
-  // One partial per (position, |b| group): bounds the MMA results summed into
-  // one tensor-memory accumulator; the parts are added in FP32 in a fixed order.
-  const int acc = std::max(m->tc_fwd->acc_cols, m->tc_adj->acc_cols);
-  rc = dev_alloc(m, &m->d_tc_part, (size_t)b_groups(m->R) * m->grid.py * m->grid.px * acc);
-  if (rc) return rc;
-  return OAM_OK;
+  return dev_alloc(m, &T->d_part, std::max(part_floats(m, T, m->tc_fwd), part_floats(m, T, m->tc_adj)));
 }
 
 void oam::tc_free(oam_model *m, cudaStream_t st) {
   for (TcLayout *L : {m->tc_fwd, m->tc_adj}) {
     if (!L) continue;
-    if (L->d_items) cudaFreeAsync(L->d_items, st);
-    if (L->d_data) cudaFreeAsync(L->d_data, st);
+    for (void *p : {(void *)L->d_items, (void *)L->d_data, (void *)L->d_pack})
+      if (p) cudaFreeAsync(p, st);
     delete L;
   }
   m->tc_fwd = m->tc_adj = nullptr;
-  if (m->d_tc_pack) cudaFreeAsync(m->d_tc_pack, st);
-  m->d_tc_pack = nullptr;
-  if (m->d_tc_part) cudaFreeAsync(m->d_tc_part, st);
-  m->d_tc_part = nullptr;
+  if (TcLine *T = m->tc_line) {
+    for (void *p : {(void *)T->d_tw, (void *)T->d_marks, (void *)T->d_smax, (void *)T->d_part})
+      if (p) cudaFreeAsync(p, st);
+    delete T;
+  }
+  m->tc_line = nullptr;
 }
 
+// Executed MMA flops of one application: 3 products x 2 x M x (16 x N) over the
+// (frequency, position tile, a >= 0) work items.
 double oam::tc_exec_flops(const oam_model *m, int dir) {
   const TcLayout *L = dir == 0 ? m->tc_fwd : m->tc_adj;
   Launch lp;
-  if (!L || plan_launch(m, L, &lp)) return 0.0;
-  return exec_flops_for(m, L, lp.p.sp);
+  if (!L || plan_launch(m, m->tc_line, L, &lp)) return 0.0;
+  return 3.0 * 2.0 * kTileM * (double)lp.n_tiles * m->tc_line->Q * L->cols;
 }
 
 oam_status oam::forward_tc(const oam_model *m, const float *H, float *s, cudaStream_t st) {
@@ -1038,7 +1113,7 @@ oam_status oam::tc_autotune(oam_model *m, int reps, cudaStream_t st, int *best_f
       L->tiling = tiling;
       L->ring_pref = 0;
       Launch lp;
-      if (plan_launch(m, L, &lp)) continue;  // this tiling does not fit the model
+      if (plan_launch(m, m->tc_line, L, &lp)) continue;  // this tiling does not fit the model
       const int deepest = lp.p.n_items;
       for (int fw : kFoldWarpChoices) {
         L->fold_warps = fw;
@@ -1086,7 +1161,7 @@ oam_status oam::tc_set_tiles(oam_model *m, int dir, int fold_warps, int ring) {
   L->ring_pref = ring;
   L->fold_warps = fold_warps;
   Launch lp;
-  oam_status rc = plan_launch(m, L, &lp);
+  oam_status rc = plan_launch(m, m->tc_line, L, &lp);
   if (rc || (ring >= 2 && lp.p.n_items != ring)) {
     L->ring_pref = keep_ring;
     L->fold_warps = keep_w;
@@ -1102,7 +1177,7 @@ oam_status oam::tc_set_tiling(oam_model *m, int dir, int tiling) {
   const int keep = L->tiling;
   L->tiling = tiling;
   Launch lp;
-  const oam_status rc = plan_launch(m, L, &lp);
+  const oam_status rc = plan_launch(m, m->tc_line, L, &lp);
   if (rc) L->tiling = keep;
   return rc;
 }
@@ -1110,7 +1185,7 @@ oam_status oam::tc_set_tiling(oam_model *m, int dir, int tiling) {
 int oam::tc_get_tiling(const oam_model *m, int dir) {
   const TcLayout *L = dir == 0 ? m->tc_fwd : m->tc_adj;
   Launch lp;
-  return L && plan_launch(m, L, &lp) == OAM_OK ? lp.tiling : 0;
+  return L && plan_launch(m, m->tc_line, L, &lp) == OAM_OK ? lp.tiling : 0;
 }
 
 void oam::tc_get_tiles(const oam_model *m, int dir, int *fold_warps, int *ring) {
@@ -1121,5 +1196,5 @@ void oam::tc_get_tiles(const oam_model *m, int dir, int *fold_warps, int *ring) 
   }
   Launch lp;
   *fold_warps = L->fold_warps;
-  *ring = plan_launch(m, L, &lp) == OAM_OK ? lp.p.n_items : 0;
+  *ring = plan_launch(m, m->tc_line, L, &lp) == OAM_OK ? lp.p.n_items : 0;
 }

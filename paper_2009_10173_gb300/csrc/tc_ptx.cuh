@@ -124,29 +124,16 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
   return d;                // base offset 0, absolute LBO mode, layout type 0 (no swizzle)
 }
 
-// Instruction descriptor, kind::f16: BF16 A and B (both K-major), FP32 D.
-__device__ __forceinline__ uint32_t idesc_bf16_f32(uint32_t M, uint32_t N) {
-  return (1u << 4)            // D format: F32
-         | (1u << 7)          // A format: BF16
-         | (1u << 10)         // B format: BF16
+// Instruction descriptor, kind::f16: FP16 A and B (both K-major), FP32 D.
+__device__ __forceinline__ uint32_t idesc_f16_f32(uint32_t M, uint32_t N) {
+  return (1u << 4)            // D format: F32; A and B formats: F16 (0)
          | ((N >> 3) << 17)   // N / 8
          | ((M >> 4) << 24);  // M / 16
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, one CTA, issued by one thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// Same with the A operand read from tensor memory: M rows in lanes, each row's
-// 16 BF16 K-elements packed two per 32-bit column (8 columns).
-__device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+// D[tmem] (+)= A[tmem] * B[smem]^T, one CTA, issued by one thread.  A: M rows in
+// lanes, each row's 16 FP16 K-elements packed two per 32-bit column (8 columns).
+__device__ __forceinline__ void mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                             uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
