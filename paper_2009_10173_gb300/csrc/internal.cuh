@@ -185,11 +185,12 @@ oam_status fft_plan_bytes(const oam_model *m, size_t *bytes);
 // the largest; tw: the size's roots (mix_roots) in device memory.
 int mix_size_for(int need);
 std::vector<float2> mix_roots(int P);
-oam_status mix_rows_r2c(int P, cudaStream_t st, const float *X, int py, int px, int Ctot, int c0, int C,
+// C channels in rows of CO (a multiple of 4) in the half spectrum.
+oam_status mix_rows_r2c(int P, cudaStream_t st, const float *X, int py, int px, int Ctot, int c0, int C, int CO,
                         const float2 *tw, float2 *Y);
 oam_status mix_cols(int P, bool inverse, cudaStream_t st, const float2 *Z, int nin, int nout, int C, const float2 *tw,
                     float2 *W);
-oam_status mix_rows_c2r(int P, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0, int C,
+oam_status mix_rows_c2r(int P, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0, int C, int CO,
                         const float2 *tw, float scale, float *X);
 
 // mix_lines.cu: transforms along the scan's y axis around the tensor-core

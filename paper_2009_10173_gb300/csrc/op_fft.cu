@@ -35,6 +35,18 @@ using namespace oam;
 
 namespace oam {
 
+// S^ for one direction: per frequency orbit a row of `stride` floats that holds, for
+// each input element e (forward: depth, adjoint: sample), the outputs of the
+// four-output groups [glo, ghi) that its band meets (zeros outside the band).
+struct ApplyRows {
+  int n_in = 0, n_out = 0;    // elements
+  int windows = 0;            // 32-output windows
+  long long stride = 0;       // floats per orbit row (a multiple of 4)
+  int2 *d_elem = nullptr;     // [n_in] (float4 index of group 0 in the row, glo | ghi << 16)
+  int2 *d_window = nullptr;   // [windows] input elements [x, y) whose groups meet the window
+  float *d_s = nullptr;       // [n_rep][stride]
+};
+
 struct FftLayout {
   int P = 0, lgP = 0, Q = 0;  // transform size, its log2 (powers of two above 512), half-spectrum columns P/2 + 1
   int KC = 0;                 // channels per FFT block (power-of-two kernels)
@@ -42,20 +54,11 @@ struct FftLayout {
   bool mixed = false;         // a mixed-radix size
   bool d4 = false;            // S^(v,u) = S^(u,v)
   int n_rep = 0;              // frequency orbits
-  int NS = 0;                 // support length n_hi - n_lo
-  int C = 0;                  // max(nz, NS): channels of the work buffers
-  long long row_len = 0;      // sum_k klen_k: entries of one orbit row of S^
-  long long row_stride = 0;   // row_len rounded up to 4 floats: each row starts on a 16-byte boundary
-  int *d_klo = nullptr, *d_klen = nullptr;  // [nz] union band per depth (absolute samples)
-  long long *d_koff = nullptr;              // [nz] offset of depth k in an orbit row
-  int4 *d_members = nullptr;                // [n_rep] half-spectrum indices u*P + v (-1 unused)
-  int2 *d_krange = nullptr;                 // [NS] depths [x, y) whose band can hold sample n_lo + j
-  long long *d_noff = nullptr;              // [NS] offset of sample n_lo + j in a transposed orbit row
-  long long row_len_t = 0;                  // sum_j (krange_j.y - krange_j.x)
-  long long row_stride_t = 0;               // row_len_t rounded up to 4 floats
-  float *d_shat_t = nullptr;                // [n_rep][row_stride_t]: S^ by sample, depths krange_j (adjoint)
-  float *d_shat = nullptr;                  // [n_rep][row_stride]
-  float2 *d_w1 = nullptr, *d_w2 = nullptr;  // [Q][P][C] work buffers
+  int n0 = 0, NS = 0;         // support: samples n0 .. n0 + NS - 1 (n0: n_lo rounded down to 4)
+  int CZ = 0, CS = 0;         // channel strides of the work buffers: nz and NS rounded up to 4
+  int4 *d_members = nullptr;  // [n_rep] half-spectrum indices u*P + v (-1 unused)
+  ApplyRows rows[2];          // S^ by depth (forward), by sample (adjoint)
+  float2 *d_w1 = nullptr, *d_w2 = nullptr;  // [Q][P][max(CZ, CS)] work buffers
   double flops = 0;                         // flops of one application (matrix part + FFTs)
   double bytes = 0;                         // device bytes read + written per application
 };
@@ -67,11 +70,9 @@ namespace {
 using namespace oam::fftdev;
 
 constexpr int kFftThreads = 256;
-constexpr int kApplyMaxThreads = 1024;
-constexpr int kUnroll = 8;  // spectral products: independent row loads per lane in flight
-constexpr int kFwdPhases = 2;  // forward products: lane groups of a warp that walk interleaved depths
-constexpr int kFwdChunk = 256;  // forward products: samples per block (0: all samples of the orbit)
-constexpr int kAdjChunk = 160;  // adjoint products: depths per block (0: all depths of the orbit)
+constexpr int kApplyWarps = 5;  // spectral products: warps per block
+constexpr int kUnroll = 4;      // 16-byte row loads per lane and step, two steps in flight
+constexpr int kStep = 4 * kUnroll;  // input elements per step
 constexpr int kBuildThreads = 128;
 
 
@@ -219,7 +220,7 @@ __device__ __forceinline__ void xtransform(float2 *a, int P, int lgP, First firs
 // Real rows -> half spectrum along x (arguments and results as k_mix_rows_r2c).
 template <int KC>
 __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_r2c(const float *__restrict__ X, int py, int px, int Ctot,
-                                                               int c0, int C, int P, int lgP, int Q,
+                                                               int c0, int C, int CO, int P, int lgP, int Q,
                                                                float2 *__restrict__ Y) {
   constexpr int KH = KC / 2;
   extern __shared__ float2 sm[];
@@ -241,7 +242,7 @@ __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_r2c(const float *__re
     const int u = i / KC, c = i % KC, l = c % KH;
     if (cb + c >= C) continue;
     const float2 z = a[xslot<KH>(bitrev(u, lgP), l)], w = a[xslot<KH>(bitrev((P - u) & (P - 1), lgP), l)];
-    Y[((size_t)u * py + y) * C + cb + c] = c < KH ? make_float2(0.5f * (z.x + w.x), 0.5f * (z.y - w.y))
+    Y[((size_t)u * py + y) * CO + cb + c] = c < KH ? make_float2(0.5f * (z.x + w.x), 0.5f * (z.y - w.y))
                                                   : make_float2(0.5f * (z.y + w.y), 0.5f * (w.x - z.x));
   }
 }
@@ -268,8 +269,8 @@ __global__ void __launch_bounds__(kFftThreads) k_xfft_cols(const float2 *__restr
 // Half spectrum along x -> real rows (as k_mix_rows_c2r).
 template <int KC>
 __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_c2r(const float2 *__restrict__ Z, int py, int px, int Ctot,
-                                                               int c0, int C, int P, int lgP, int Q, float scale,
-                                                               float *__restrict__ X) {
+                                                               int c0, int C, int CO, int P, int lgP, int Q,
+                                                               float scale, float *__restrict__ X) {
   constexpr int KH = KC / 2;
   extern __shared__ float2 sm[];
   const int y = blockIdx.x, ob = blockIdx.y * KC;
@@ -287,8 +288,8 @@ __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_c2r(const float2 *__r
     const int fh = f < Q ? f : P - f;
     float2 xs = make_float2(0.0f, 0.0f), ys = make_float2(0.0f, 0.0f);
     const int zx = ob + l - c0, zy = ob + l + KH - c0;
-    if (zx >= 0 && zx < C) xs = Z[((size_t)fh * py + y) * C + zx];
-    if (zy >= 0 && zy < C) ys = Z[((size_t)fh * py + y) * C + zy];
+    if (zx >= 0 && zx < C) xs = Z[((size_t)fh * py + y) * CO + zx];
+    if (zy >= 0 && zy < C) ys = Z[((size_t)fh * py + y) * CO + zy];
     if (f == 0 || f == (P >> 1)) {
       xs.y = 0.0f;
       ys.y = 0.0f;
@@ -308,182 +309,116 @@ __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_c2r(const float2 *__r
   xtransform<KH, false, false>(sm, P, lgP, load, store);
 }
 
-// Forward, per frequency orbit r: s^_f[j] = sum_k S^_r[k][n - klo_k] H^_f[k]
-// for the orbit's member frequencies f, n = n_lo + j; thread j visits the
-// depths [kr_j.x, kr_j.y) whose band holds n.  Block per orbit.
-__global__ void __launch_bounds__(kApplyMaxThreads) k_fft_apply_fwd(const float *__restrict__ shat, long long row_len,
-                                                        const int4 *__restrict__ members,
-                                                        const int *__restrict__ klo, const int *__restrict__ klen,
-                                                        const long long *__restrict__ koff,
-                                                        const int2 *__restrict__ krange, int nz, int n_lo, int NS,
-                                                        const float2 *__restrict__ Hh, float2 *__restrict__ sh) {
-  extern __shared__ float4 smf[];
-  float4 *Hs = smf;                                  // [nz][2]: members (0, 1) and (2, 3), (re, im) pairs
-  int *s_lo = reinterpret_cast<int *>(Hs + 2 * nz);   // [nz]
-  int *s_len = s_lo + nz;                             // [nz]
-  long long *s_off = reinterpret_cast<long long *>(s_len + nz);  // [nz]: 40 nz bytes in, 8-byte aligned
-  // linear grid, chunk fastest: an orbit's sample chunks run back to back and share its vectors in L2
-  const int nch = kFwdChunk > 0 ? (NS + kFwdChunk - 1) / kFwdChunk : 1;
-  const int r = (int)(blockIdx.x / nch), chunk = (int)(blockIdx.x % nch);
-  const int4 mem = members[r];
-  for (int k = threadIdx.x; k < nz; k += blockDim.x) {
-    const float2 z = make_float2(0.0f, 0.0f);
-    const float2 h0 = mem.x >= 0 ? Hh[(size_t)mem.x * nz + k] : z, h1 = mem.y >= 0 ? Hh[(size_t)mem.y * nz + k] : z;
-    const float2 h2 = mem.z >= 0 ? Hh[(size_t)mem.z * nz + k] : z, h3 = mem.w >= 0 ? Hh[(size_t)mem.w * nz + k] : z;
-    Hs[2 * k] = make_float4(h0.x, h0.y, h1.x, h1.y);
-    Hs[2 * k + 1] = make_float4(h2.x, h2.y, h3.x, h3.y);
-    s_lo[k] = klo[k];
-    s_len[k] = klen[k];
-    s_off[k] = koff[k];
-  }
-  __syncthreads();
-  const float *row = shat + (size_t)r * row_len;
-  constexpr int kLanes = 32 / kFwdPhases;  // samples per warp
-  const int lane = threadIdx.x & 31, sub = lane % kLanes, ph = lane / kLanes;
-  const int jb = kFwdChunk > 0 ? chunk * kFwdChunk : 0;
-  const int je = kFwdChunk > 0 ? min(NS, jb + kFwdChunk) : NS;
-  // a warp serves kLanes samples; its lane groups walk interleaved depths of
-  // the warp's common depth range (coalesced row reads), then add their sums
-  for (int g0 = jb + (threadIdx.x >> 5) * kLanes; g0 < je; g0 += (blockDim.x >> 5) * kLanes) {
-    const int j = g0 + sub;
-    const bool live = j < je;
-    const int n = n_lo + j;
-    const int2 kr = live ? krange[j] : make_int2(nz, 0);
-    const int k0 = __reduce_min_sync(0xffffffffu, kr.x), k1 = __reduce_max_sync(0xffffffffu, kr.y);
-    float acc[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.0f;
-    int k = k0 + ph;
-    for (; k + kFwdPhases * (kUnroll - 1) < k1; k += kFwdPhases * kUnroll) {  // kUnroll loads in flight per lane
-      float sv[kUnroll];
-#pragma unroll
-      for (int q = 0; q < kUnroll; ++q) {
-        const int kk = k + kFwdPhases * q, d = n - s_lo[kk];
-        sv[q] = (live && (unsigned)d < (unsigned)s_len[kk]) ? __ldg(row + s_off[kk] + d) : 0.0f;
-      }
-#pragma unroll
-      for (int q = 0; q < kUnroll; ++q) {
-        const float4 a = Hs[2 * (k + kFwdPhases * q)], b = Hs[2 * (k + kFwdPhases * q) + 1];
-        acc[0] = fmaf(sv[q], a.x, acc[0]);
-        acc[1] = fmaf(sv[q], a.y, acc[1]);
-        acc[2] = fmaf(sv[q], a.z, acc[2]);
-        acc[3] = fmaf(sv[q], a.w, acc[3]);
-        acc[4] = fmaf(sv[q], b.x, acc[4]);
-        acc[5] = fmaf(sv[q], b.y, acc[5]);
-        acc[6] = fmaf(sv[q], b.z, acc[6]);
-        acc[7] = fmaf(sv[q], b.w, acc[7]);
-      }
-    }
-    for (; k < k1; k += kFwdPhases) {
-      const int d = n - s_lo[k];
-      const float sv = (live && (unsigned)d < (unsigned)s_len[k]) ? __ldg(row + s_off[k] + d) : 0.0f;
-      const float4 a = Hs[2 * k], b = Hs[2 * k + 1];
-      acc[0] = fmaf(sv, a.x, acc[0]);
-      acc[1] = fmaf(sv, a.y, acc[1]);
-      acc[2] = fmaf(sv, a.z, acc[2]);
-      acc[3] = fmaf(sv, a.w, acc[3]);
-      acc[4] = fmaf(sv, b.x, acc[4]);
-      acc[5] = fmaf(sv, b.y, acc[5]);
-      acc[6] = fmaf(sv, b.z, acc[6]);
-      acc[7] = fmaf(sv, b.w, acc[7]);
-    }
-#pragma unroll
-    for (int off = 16; off >= kLanes; off >>= 1)
-#pragma unroll
-      for (int q = 0; q < 8; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], off);
-    if (!live || ph != 0) continue;
-    if (mem.x >= 0) sh[(size_t)mem.x * NS + j] = make_float2(acc[0], acc[1]);
-    if (mem.y >= 0) sh[(size_t)mem.y * NS + j] = make_float2(acc[2], acc[3]);
-    if (mem.z >= 0) sh[(size_t)mem.z * NS + j] = make_float2(acc[4], acc[5]);
-    if (mem.w >= 0) sh[(size_t)mem.w * NS + j] = make_float2(acc[6], acc[7]);
-  }
+// Spectral products of one frequency orbit r and direction: out_f[o] = sum_e S^_r[e][o]
+// in_f[e] for the orbit's up to four member frequencies f.  A warp serves a window of
+// 32 outputs: lanes hold eight groups of four outputs, their four quarters walk
+// interleaved input elements of the window's range; a lane reads its four outputs'
+// S^ with one 16-byte load and multiplies them with the element's four complex values
+// from shared memory as packed (re, im) pairs.
+//
+// What bounds it: reading S^ once from HBM.  Four outputs per load and packed products
+// take 7 issue slots per S^ value instead of 20 (a lane per output, scalar loads), and
+// the next step's loads are issued before this step's products.  200x200x300 (0.77 GB),
+// cold caches: 200 us forward, 191 adjoint (3.9 TB/s), against 270 and 217 for the scalar
+// form with its own kernel per direction.
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t splat2(float v) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+  return r;
 }
 
-// Adjoint, per frequency orbit r: H^_f[k] = sum_n S^_r[k][n] s^_f[n - n_lo], from
-// the orbit's row by sample (entries of sample n_lo + j are depths krange_j).
-// Thread k; every lane of a warp walks the same samples (coalesced reads).
-__global__ void __launch_bounds__(kApplyMaxThreads) k_fft_apply_adj(const float *__restrict__ shat_t,
-                                                                    long long row_len_t,
-                                                                    const int4 *__restrict__ members,
-                                                                    const int *__restrict__ klo,
-                                                                    const int *__restrict__ klen,
-                                                                    const int2 *__restrict__ krange,
-                                                                    const long long *__restrict__ noff, int nz,
-                                                                    int n_lo, int NS, const float2 *__restrict__ sh,
-                                                                    float2 *__restrict__ Hh) {
-  extern __shared__ float4 sma[];
-  float4 *Ss = sma;                                      // [NS][2]: members (0, 1) and (2, 3)
-  int2 *s_kr = reinterpret_cast<int2 *>(Ss + 2 * NS);     // [NS]
-  long long *s_no = reinterpret_cast<long long *>(s_kr + NS);  // [NS]
-  // linear grid, chunk fastest: an orbit's depth chunks run back to back
-  const int nch = kAdjChunk > 0 ? (nz + kAdjChunk - 1) / kAdjChunk : 1;
-  const int r = (int)(blockIdx.x / nch), chunk = (int)(blockIdx.x % nch);
-  const int kb = kAdjChunk > 0 ? chunk * kAdjChunk : 0, ke = kAdjChunk > 0 ? min(nz, kb + kAdjChunk) : nz;
+__global__ void __launch_bounds__(32 * kApplyWarps, 4)
+    k_fft_apply(const float *__restrict__ S, long long stride, const int4 *__restrict__ members,
+                const int2 *__restrict__ elem, const int2 *__restrict__ window, int windows, int n_in, int in_stride,
+                int n_out, int out_stride, const float2 *__restrict__ in, float2 *__restrict__ out) {
+  extern __shared__ ulonglong2 sma[];
+  // members (0, 1) and (2, 3) as (re, im) pairs; kStep elements beyond the last meet no output
+  ulonglong2 *X = sma;                                            // [n_in + kStep][2]
+  int2 *E = reinterpret_cast<int2 *>(X + 2 * (n_in + kStep));     // [n_in + kStep]
+  const int r = blockIdx.x;
   const int4 mem = members[r];
-  for (int j = threadIdx.x; j < NS; j += blockDim.x) {
+  {
+    float2 *X2 = reinterpret_cast<float2 *>(X);
     const float2 z = make_float2(0.0f, 0.0f);
-    const float2 x0 = mem.x >= 0 ? sh[(size_t)mem.x * NS + j] : z, x1 = mem.y >= 0 ? sh[(size_t)mem.y * NS + j] : z;
-    const float2 x2 = mem.z >= 0 ? sh[(size_t)mem.z * NS + j] : z, x3 = mem.w >= 0 ? sh[(size_t)mem.w * NS + j] : z;
-    Ss[2 * j] = make_float4(x0.x, x0.y, x1.x, x1.y);
-    Ss[2 * j + 1] = make_float4(x2.x, x2.y, x3.x, x3.y);
-    s_kr[j] = krange[j];
-    s_no[j] = noff[j];
+    for (int e = threadIdx.x; e < n_in + kStep; e += blockDim.x) {
+      const bool ok = e < n_in;
+      const float2 x0 = ok && mem.x >= 0 ? in[(size_t)mem.x * in_stride + e] : z;
+      const float2 x1 = ok && mem.y >= 0 ? in[(size_t)mem.y * in_stride + e] : z;
+      const float2 x2 = ok && mem.z >= 0 ? in[(size_t)mem.z * in_stride + e] : z;
+      const float2 x3 = ok && mem.w >= 0 ? in[(size_t)mem.w * in_stride + e] : z;
+      X2[4 * e] = x0;
+      X2[4 * e + 1] = x1;
+      X2[4 * e + 2] = x2;
+      X2[4 * e + 3] = x3;
+      E[e] = ok ? elem[e] : make_int2(0, 0);
+    }
   }
   __syncthreads();
-  const float *row = shat_t + (size_t)r * row_len_t;
-  const int lane = threadIdx.x & 31, sub = lane & 15, ph = lane >> 4;
-  // a warp serves 16 depths; its two half-warps walk alternate samples of the
-  // warp's common sample range (coalesced reads), then add their sums
-  for (int g0 = kb + (threadIdx.x >> 5) * 16; g0 < ke; g0 += (blockDim.x >> 5) * 16) {
-    const int k = g0 + sub;
-    const bool live = k < ke && klen[k] > 0;
-    const int lo = live ? klo[k] - n_lo : NS, hi = live ? klo[k] - n_lo + klen[k] : 0;
-    const int j0 = __reduce_min_sync(0xffffffffu, lo), j1 = __reduce_max_sync(0xffffffffu, hi);
-    float acc[8];
+  const float4 *row = reinterpret_cast<const float4 *>(S + (size_t)r * stride);
+  const int lane = threadIdx.x & 31, ph = lane >> 3;
+  for (int w = threadIdx.x >> 5; w < windows; w += blockDim.x >> 5) {
+    const int g = 8 * w + (lane & 7);
+    const int2 win = window[w];
+    uint64_t acc[4][4];  // [output][member]
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.0f;
-    int j = j0 + ph;
-    for (; j + 2 * (kUnroll - 1) < j1; j += 2 * kUnroll) {  // kUnroll loads in flight per lane
-      float sv[kUnroll];
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int q = 0; q < kUnroll; ++q) {
-        const int jj = j + 2 * q;
-        const int2 kr = s_kr[jj];
-        sv[q] = (k >= kr.x && k < kr.y) ? __ldg(row + s_no[jj] + (k - kr.x)) : 0.0f;
-      }
+      for (int j = 0; j < 4; ++j) acc[i][j] = 0;
+    auto load = [&](int e) {
+      const int2 d = E[e];
+      const bool in_band = g >= (d.y & 0xffff) && g < (int)((unsigned)d.y >> 16);
+      return in_band ? __ldg(row + d.x + g) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    auto add = [&](int e, float4 v) {
+      const ulonglong2 h0 = X[2 * e], h1 = X[2 * e + 1];
+      const uint64_t h[4] = {h0.x, h0.y, h1.x, h1.y}, s[4] = {splat2(v.x), splat2(v.y), splat2(v.z), splat2(v.w)};
 #pragma unroll
-      for (int q = 0; q < kUnroll; ++q) {
-        const float4 a = Ss[2 * (j + 2 * q)], b = Ss[2 * (j + 2 * q) + 1];
-        acc[0] = fmaf(sv[q], a.x, acc[0]);
-        acc[1] = fmaf(sv[q], a.y, acc[1]);
-        acc[2] = fmaf(sv[q], a.z, acc[2]);
-        acc[3] = fmaf(sv[q], a.w, acc[3]);
-        acc[4] = fmaf(sv[q], b.x, acc[4]);
-        acc[5] = fmaf(sv[q], b.y, acc[5]);
-        acc[6] = fmaf(sv[q], b.z, acc[6]);
-        acc[7] = fmaf(sv[q], b.w, acc[7]);
-      }
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fma2(s[i], h[j], acc[i][j]);
+    };
+    // the next step's loads are issued before this step's products
+    float4 v[kUnroll], next[kUnroll];
+#pragma unroll
+    for (int q = 0; q < kUnroll; ++q) v[q] = load(win.x + 4 * q + ph);
+    for (int e0 = win.x; e0 < win.y; e0 += kStep) {
+      const bool more = e0 + kStep < win.y;
+#pragma unroll
+      for (int q = 0; q < kUnroll; ++q)
+        next[q] = more ? load(e0 + kStep + 4 * q + ph) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int q = 0; q < kUnroll; ++q) add(e0 + 4 * q + ph, v[q]);
+#pragma unroll
+      for (int q = 0; q < kUnroll; ++q) v[q] = next[q];
     }
-    for (; j < j1; j += 2) {
-      const int2 kr = s_kr[j];
-      const float sv = (k >= kr.x && k < kr.y) ? __ldg(row + s_no[j] + (k - kr.x)) : 0.0f;
-      const float4 a = Ss[2 * j], b = Ss[2 * j + 1];
-      acc[0] = fmaf(sv, a.x, acc[0]);
-      acc[1] = fmaf(sv, a.y, acc[1]);
-      acc[2] = fmaf(sv, a.z, acc[2]);
-      acc[3] = fmaf(sv, a.w, acc[3]);
-      acc[4] = fmaf(sv, b.x, acc[4]);
-      acc[5] = fmaf(sv, b.y, acc[5]);
-      acc[6] = fmaf(sv, b.z, acc[6]);
-      acc[7] = fmaf(sv, b.w, acc[7]);
-    }
+    // sum the quarters, each keeping the member of its number
+    uint64_t b[4][2], c[4];
+    const bool hi = ph & 2, odd = ph & 1;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 16);
-    if (k >= ke || ph != 0) continue;
-    if (mem.x >= 0) Hh[(size_t)mem.x * nz + k] = make_float2(acc[0], acc[1]);
-    if (mem.y >= 0) Hh[(size_t)mem.y * nz + k] = make_float2(acc[2], acc[3]);
-    if (mem.z >= 0) Hh[(size_t)mem.z * nz + k] = make_float2(acc[4], acc[5]);
-    if (mem.w >= 0) Hh[(size_t)mem.w * nz + k] = make_float2(acc[6], acc[7]);
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        b[i][j] = add2(hi ? acc[i][2 + j] : acc[i][j],
+                       __shfl_xor_sync(0xffffffffu, hi ? acc[i][j] : acc[i][2 + j], 16));
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      c[i] = add2(odd ? b[i][1] : b[i][0], __shfl_xor_sync(0xffffffffu, odd ? b[i][0] : b[i][1], 8));
+    const int f = ph == 0 ? mem.x : ph == 1 ? mem.y : ph == 2 ? mem.z : mem.w;
+    if (f >= 0 && 4 * g < n_out) {  // whole groups: out_stride is a multiple of 4
+      ulonglong2 *o = reinterpret_cast<ulonglong2 *>(out + (size_t)f * out_stride + 4 * g);
+      o[0] = make_ulonglong2(c[0], c[1]);
+      o[1] = make_ulonglong2(c[2], c[3]);
+    }
   }
 }
 
@@ -530,9 +465,9 @@ __global__ void __launch_bounds__(kBuildThreads) k_shat_pass1(const float *__res
 // every orbit r = (v0, u0) with this u0.  Block (entry block, u0).
 __global__ void __launch_bounds__(kBuildThreads) k_shat_pass2(const float *__restrict__ T, long long row_len, int R,
                                                               int P, int Q, const int *__restrict__ rep_of,
-                                                              const int2 *__restrict__ entry_kn, int n_lo,
-                                                              const int2 *__restrict__ krange,
-                                                              const long long *__restrict__ noff,
+                                                              const int2 *__restrict__ entry_kn, int n0,
+                                                              const int2 *__restrict__ by_depth,
+                                                              const int2 *__restrict__ by_sample,
                                                               long long stride, long long stride_t,
                                                               float *__restrict__ shat, float *__restrict__ shat_t) {
   extern __shared__ float smb[];
@@ -549,8 +484,8 @@ __global__ void __launch_bounds__(kBuildThreads) k_shat_pass2(const float *__res
     tv[bp * ts + tid] = bp == 0 ? t : 2.0f * t;
   }
   const int2 kn = entry_kn[e];
-  const int jn = kn.y - n_lo;
-  const long long et = noff[jn] + (kn.x - krange[jn].x);  // same entry in the row by sample
+  const int jn = kn.y - n0;
+  const long long ef = 4LL * by_depth[kn.x].x + jn, et = 4LL * by_sample[jn].x + kn.x;  // its place in the two rows
   for (int v0 = 0; v0 < Q; ++v0) {
     const int r = rep_of[v0 * Q + u0];
     if (r < 0) continue;
@@ -560,19 +495,41 @@ __global__ void __launch_bounds__(kBuildThreads) k_shat_pass2(const float *__res
       j += v0;
       if (j >= P) j -= P;
     }
-    shat[(size_t)r * stride + e] = acc;
+    shat[(size_t)r * stride + ef] = acc;
     shat_t[(size_t)r * stride_t + et] = acc;
   }
 }
 
 // Host tables of the lateral-FFT layout, planned from the model's bands.
 struct FftPlan {
-  std::vector<int> klo, klen;
-  std::vector<long long> koff, noff;
-  std::vector<int2> krange, entry_kn;
+  std::vector<int2> elem[2], window[2], entry_kn;  // entry_kn: (depth, sample) of the S^ entries of an orbit
   std::vector<int> rep_of;
   std::vector<int4> members;
 };
+
+// Row layout of one direction: lo[e] .. hi[e] - 1 are the outputs that element e meets.
+void plan_apply(const std::vector<int> &lo, const std::vector<int> &hi, int n_out, ApplyRows *A,
+                std::vector<int2> *elem, std::vector<int2> *window) {
+  A->n_in = (int)lo.size();
+  A->n_out = n_out;
+  A->windows = (n_out + 31) / 32;
+  elem->assign(A->n_in, make_int2(0, 0));
+  window->assign(A->windows, make_int2(A->n_in, 0));
+  int used = 0;  // groups
+  for (int e = 0; e < A->n_in; ++e) {
+    if (hi[e] <= lo[e]) continue;
+    const int glo = lo[e] / 4, ghi = (hi[e] + 3) / 4;
+    (*elem)[e] = make_int2(used - glo, glo | (ghi << 16));
+    used += ghi - glo;
+    for (int w = glo / 8; w <= (ghi - 1) / 8; ++w) {
+      (*window)[w].x = std::min((*window)[w].x, e);
+      (*window)[w].y = e + 1;
+    }
+  }
+  for (int2 &w : *window)
+    if (w.y <= w.x) w = make_int2(0, 0);
+  A->stride = 4LL * std::max(used, 1);
+}
 
 // Fill L's sizes and the host tables (no device call).
 oam_status fft_plan(const oam_model *m, FftLayout *L, FftPlan &pl) {
@@ -605,13 +562,13 @@ oam_status fft_plan(const oam_model *m, FftLayout *L, FftPlan &pl) {
         L->d4 = false;
         break;
       }
-  // union band per depth over all orbits
-  std::vector<int> &klo = pl.klo, &klen = pl.klen;
-  std::vector<long long> &koff = pl.koff;
-  klo.assign(nz, 0);
-  klen.assign(nz, 0);
-  koff.assign(nz, 0);
-  long long row = 0;
+  // union band per depth over all orbits, and the depths per sample
+  L->n0 = m->n_lo & ~3;
+  L->NS = std::max(1, m->n_hi - L->n0);
+  L->CZ = (nz + 3) & ~3;
+  L->CS = (L->NS + 3) & ~3;
+  std::vector<int> klo(nz, 0), khi(nz, 0), slo(L->NS, nz), shi(L->NS, 0);  // samples from n0
+  pl.entry_kn.clear();
   for (int k = 0; k < nz; ++k) {
     int lo = 1 << 30, hi = -1;
     for (int o = 0; o < m->n_orb; ++o) {
@@ -621,41 +578,19 @@ oam_status fft_plan(const oam_model *m, FftLayout *L, FftPlan &pl) {
         hi = std::max(hi, bh);
       }
     }
-    if (hi <= lo) lo = hi = m->n_lo;
-    klo[k] = lo;
-    klen[k] = hi - lo;
-    koff[k] = row;
-    row += hi - lo;
+    if (hi <= lo) continue;
+    klo[k] = lo - L->n0;
+    khi[k] = hi - L->n0;
+    for (int j = klo[k]; j < khi[k]; ++j) {
+      slo[j] = std::min(slo[j], k);
+      shi[j] = k + 1;
+      pl.entry_kn.push_back(make_int2(k, L->n0 + j));
+    }
   }
-  L->row_len = std::max<long long>(row, 1);
-  L->row_stride = (L->row_len + 3) & ~3LL;
-  L->NS = std::max(1, m->n_hi - m->n_lo);
-  std::vector<int2> &krange = pl.krange;
-  krange.assign(L->NS, make_int2(0, 0));
-  for (int j = 0; j < L->NS; ++j) {
-    const int n = m->n_lo + j;
-    int kf = nz, kl = -1;
-    for (int k = 0; k < nz; ++k)
-      if (n >= klo[k] && n < klo[k] + klen[k]) {
-        kf = std::min(kf, k);
-        kl = std::max(kl, k);
-      }
-    krange[j] = kl >= kf ? make_int2(kf, kl + 1) : make_int2(0, 0);
-  }
-  std::vector<long long> &noff = pl.noff;
-  noff.assign(L->NS, 0);
-  long long rowt = 0;
-  for (int j = 0; j < L->NS; ++j) {
-    noff[j] = rowt;
-    rowt += krange[j].y - krange[j].x;
-  }
-  L->row_len_t = std::max<long long>(rowt, 1);
-  L->row_stride_t = (L->row_len_t + 3) & ~3LL;
-  L->C = std::max(nz, L->NS);
-  std::vector<int2> &entry_kn = pl.entry_kn;
-  entry_kn.assign((size_t)L->row_len, make_int2(0, 0));
-  for (int k = 0; k < nz; ++k)
-    for (int j = 0; j < klen[k]; ++j) entry_kn[(size_t)koff[k] + j] = make_int2(k, klo[k] + j);
+  if (pl.entry_kn.empty()) pl.entry_kn.push_back(make_int2(0, L->n0));  // an empty slab: one zero entry
+  if (nz > 4 * 65535 || L->NS > 4 * 65535) return OAM_ERR_UNSUPPORTED;  // 16-bit group indices (beyond the API's sizes)
+  plan_apply(klo, khi, L->NS, &L->rows[0], &pl.elem[0], &pl.window[0]);
+  plan_apply(slo, shi, nz, &L->rows[1], &pl.elem[1], &pl.window[1]);
   // frequency orbits and their members in the half spectrum (index u*P + v)
   std::vector<int> &rep_of = pl.rep_of;
   std::vector<int4> &members = pl.members;
@@ -682,11 +617,12 @@ oam_status fft_plan(const oam_model *m, FftLayout *L, FftPlan &pl) {
 }
 
 // Device bytes fft_build allocates and keeps (host only).
-oam_status fft_layout_bytes(const FftLayout &L, const FftPlan &pl, int nz, size_t *bytes) {
-  *bytes = (L.mixed ? alloc_bytes<float2>(L.P) : 0) + alloc_bytes<int>(nz) * 2 + alloc_bytes<long long>(nz) + alloc_bytes<int4>(pl.members.size()) +
-           alloc_bytes<int2>(L.NS) + alloc_bytes<long long>(L.NS) +
-           alloc_bytes<float>((size_t)L.n_rep * L.row_stride_t) + alloc_bytes<float>((size_t)L.n_rep * L.row_stride) +
-           2 * alloc_bytes<float2>((size_t)L.Q * L.P * L.C);
+oam_status fft_layout_bytes(const FftLayout &L, const FftPlan &pl, size_t *bytes) {
+  size_t b = (L.mixed ? alloc_bytes<float2>(L.P) : 0) + alloc_bytes<int4>(pl.members.size()) +
+             2 * alloc_bytes<float2>((size_t)L.Q * L.P * std::max(L.CZ, L.CS));
+  for (const ApplyRows &A : L.rows)
+    b += alloc_bytes<int2>(A.n_in) + alloc_bytes<int2>(A.windows) + alloc_bytes<float>((size_t)L.n_rep * A.stride);
+  *bytes = b;
   return OAM_OK;
 }
 
@@ -697,7 +633,7 @@ oam_status oam::fft_plan_bytes(const oam_model *m, size_t *bytes) {
   FftPlan pl;
   oam_status rc = fft_plan(m, &L, pl);
   if (rc) return rc;
-  return fft_layout_bytes(L, pl, m->grid.nz, bytes);
+  return fft_layout_bytes(L, pl, bytes);
 }
 
 oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
@@ -711,17 +647,14 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
     if (rc0) return rc0;
   }
   const int P = L->P, Q = L->Q;
-  std::vector<int> &klo = pl.klo, &klen = pl.klen, &rep_of = pl.rep_of;
-  std::vector<long long> &koff = pl.koff, &noff = pl.noff;
-  std::vector<int2> &krange = pl.krange, &entry_kn = pl.entry_kn;
-  std::vector<int4> &members = pl.members;
+  const std::vector<int> &rep_of = pl.rep_of;
+  const std::vector<int2> &entry_kn = pl.entry_kn;
+  const std::vector<int4> &members = pl.members;
+  const long long entries = (long long)entry_kn.size();
   oam_status rc;
-  if ((rc = dev_alloc(m, &L->d_klo, nz)) || (rc = dev_alloc(m, &L->d_klen, nz)) ||
-      (rc = dev_alloc(m, &L->d_koff, nz)) || (rc = dev_alloc(m, &L->d_members, members.size())) ||
-      (rc = dev_alloc(m, &L->d_krange, (size_t)L->NS)) || (rc = dev_alloc(m, &L->d_noff, (size_t)L->NS)) ||
-      (rc = dev_alloc(m, &L->d_shat_t, (size_t)L->n_rep * L->row_stride_t)) ||
-      (rc = dev_alloc(m, &L->d_shat, (size_t)L->n_rep * L->row_stride)) ||
-      (rc = dev_alloc(m, &L->d_w1, (size_t)Q * P * L->C)) || (rc = dev_alloc(m, &L->d_w2, (size_t)Q * P * L->C)))
+  const size_t chan = (size_t)Q * P * std::max(L->CZ, L->CS);
+  if ((rc = dev_alloc(m, &L->d_members, members.size())) || (rc = dev_alloc(m, &L->d_w1, chan)) ||
+      (rc = dev_alloc(m, &L->d_w2, chan)))
     return rc;
   std::vector<float2> roots;
   if (L->mixed) {
@@ -729,15 +662,19 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
     roots = mix_roots(P);
     OAM_CUDA_TRY(cudaMemcpyAsync(L->d_tw, roots.data(), sizeof(float2) * P, cudaMemcpyHostToDevice, st));
   }
-  OAM_CUDA_TRY(cudaMemcpyAsync(L->d_klo, klo.data(), sizeof(int) * nz, cudaMemcpyHostToDevice, st));
-  OAM_CUDA_TRY(cudaMemcpyAsync(L->d_klen, klen.data(), sizeof(int) * nz, cudaMemcpyHostToDevice, st));
-  OAM_CUDA_TRY(cudaMemcpyAsync(L->d_koff, koff.data(), sizeof(long long) * nz, cudaMemcpyHostToDevice, st));
   OAM_CUDA_TRY(cudaMemcpyAsync(L->d_members, members.data(), sizeof(int4) * members.size(), cudaMemcpyHostToDevice,
                                st));
-  OAM_CUDA_TRY(cudaMemcpyAsync(L->d_krange, krange.data(), sizeof(int2) * krange.size(), cudaMemcpyHostToDevice, st));
-  OAM_CUDA_TRY(cudaMemcpyAsync(L->d_noff, noff.data(), sizeof(long long) * noff.size(), cudaMemcpyHostToDevice, st));
-  // entries of the row by sample whose depth band misses the sample stay zero
-  OAM_CUDA_TRY(cudaMemsetAsync(L->d_shat_t, 0, sizeof(float) * (size_t)L->n_rep * L->row_stride_t, st));
+  for (int d = 0; d < 2; ++d) {
+    ApplyRows &A = L->rows[d];
+    if ((rc = dev_alloc(m, &A.d_elem, (size_t)A.n_in)) || (rc = dev_alloc(m, &A.d_window, (size_t)A.windows)) ||
+        (rc = dev_alloc(m, &A.d_s, (size_t)L->n_rep * A.stride)))
+      return rc;
+    OAM_CUDA_TRY(cudaMemcpyAsync(A.d_elem, pl.elem[d].data(), sizeof(int2) * A.n_in, cudaMemcpyHostToDevice, st));
+    OAM_CUDA_TRY(
+        cudaMemcpyAsync(A.d_window, pl.window[d].data(), sizeof(int2) * A.windows, cudaMemcpyHostToDevice, st));
+    // outputs of a group that the element's band does not meet stay zero
+    OAM_CUDA_TRY(cudaMemsetAsync(A.d_s, 0, sizeof(float) * (size_t)L->n_rep * A.stride, st));
+  }
   // build S^ (temporaries: entry table, band_hi, rep table, T)
   int2 *d_entry = nullptr;
   int *d_band_hi = nullptr, *d_rep_of = nullptr;
@@ -746,7 +683,7 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
   if (cudaMallocAsync((void **)&d_entry, sizeof(int2) * entry_kn.size(), st) != cudaSuccess ||
       cudaMallocAsync((void **)&d_band_hi, sizeof(int) * nb, st) != cudaSuccess ||
       cudaMallocAsync((void **)&d_rep_of, sizeof(int) * rep_of.size(), st) != cudaSuccess ||
-      cudaMallocAsync((void **)&d_T, sizeof(float) * (size_t)(R + 1) * Q * L->row_len, st) != cudaSuccess) {
+      cudaMallocAsync((void **)&d_T, sizeof(float) * (size_t)(R + 1) * Q * entries, st) != cudaSuccess) {
     cudaGetLastError();
     if (d_entry) cudaFreeAsync(d_entry, st);
     if (d_band_hi) cudaFreeAsync(d_band_hi, st);
@@ -757,18 +694,18 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
   cudaMemcpyAsync(d_entry, entry_kn.data(), sizeof(int2) * entry_kn.size(), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(d_band_hi, m->h_band_hi.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(d_rep_of, rep_of.data(), sizeof(int) * rep_of.size(), cudaMemcpyHostToDevice, st);
-  const unsigned eblocks = (unsigned)((L->row_len + kBuildThreads - 1) / kBuildThreads);
+  const unsigned eblocks = (unsigned)((entries + kBuildThreads - 1) / kBuildThreads);
   const size_t sb = sizeof(float) * ((size_t)P + (size_t)(R + 1) * kBuildThreads);
   if (sb > 48 * 1024) {
     OAM_CUDA_TRY(cudaFuncSetAttribute(k_shat_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb));
     OAM_CUDA_TRY(cudaFuncSetAttribute(k_shat_pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb));
   }
   k_shat_pass1<<<dim3(eblocks, R + 1), kBuildThreads, sb, st>>>(
-      m->d_band, m->d_band_lo, d_band_hi, m->band_w, m->d_tap_orbit, R, W, nz, d_entry, L->row_len, P, Q, d_T);
+      m->d_band, m->d_band_lo, d_band_hi, m->band_w, m->d_tap_orbit, R, W, nz, d_entry, entries, P, Q, d_T);
   OAM_LAUNCHED();
-  k_shat_pass2<<<dim3(eblocks, Q), kBuildThreads, sb, st>>>(d_T, L->row_len, R, P, Q, d_rep_of, d_entry, m->n_lo,
-                                                            L->d_krange, L->d_noff, L->row_stride, L->row_stride_t, L->d_shat,
-                                                            L->d_shat_t);
+  k_shat_pass2<<<dim3(eblocks, Q), kBuildThreads, sb, st>>>(d_T, entries, R, P, Q, d_rep_of, d_entry, L->n0,
+                                                            L->rows[0].d_elem, L->rows[1].d_elem, L->rows[0].stride,
+                                                            L->rows[1].stride, L->rows[0].d_s, L->rows[1].d_s);
   OAM_LAUNCHED();
   OAM_CUDA_TRY(cudaStreamSynchronize(st));  // host tables above go out of scope
   cudaFreeAsync(d_entry, st);
@@ -780,9 +717,9 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
   const double half = (double)Q * P;
   const double fft_lines = (double)m->grid.py * m->grid.nz + half / P * m->grid.nz + half / P * L->NS +
                            (double)m->grid.py * L->NS;
-  L->flops = 4.0 * half * (double)L->row_len + 5.0 * P * std::log2((double)P) * fft_lines;
+  L->flops = 4.0 * half * (double)entries + 5.0 * P * std::log2((double)P) * fft_lines;
   const double c8 = sizeof(float2);
-  L->bytes = 4.0 * (double)L->n_rep * L->row_len +                              // S^
+  L->bytes = 4.0 * (double)L->n_rep * entries +                              // S^
              4.0 * vol_elems(m) + 4.0 * (double)m->grid.py * m->grid.px * m->grid.nt +  // input, output
              c8 * Q * m->grid.py * (nz + L->NS) * 2 +                            // row-transform buffers
              c8 * half * (nz + L->NS) * 2;                                       // column-transform buffers
@@ -792,10 +729,11 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
 void oam::fft_free(oam_model *m, cudaStream_t st) {
   FftLayout *L = m->fft;
   if (!L) return;
-  for (void *p : {(void *)L->d_tw, (void *)L->d_klo, (void *)L->d_klen, (void *)L->d_koff, (void *)L->d_members, (void *)L->d_krange,
-                  (void *)L->d_noff, (void *)L->d_shat_t, (void *)L->d_shat,
-                  (void *)L->d_w1, (void *)L->d_w2})
+  for (void *p : {(void *)L->d_tw, (void *)L->d_members, (void *)L->d_w1, (void *)L->d_w2})
     if (p) cudaFreeAsync(p, st);
+  for (ApplyRows &A : L->rows)
+    for (void *p : {(void *)A.d_elem, (void *)A.d_window, (void *)A.d_s})
+      if (p) cudaFreeAsync(p, st);
   delete L;
   m->fft = nullptr;
 }
@@ -824,12 +762,12 @@ int xthreads(int P, int KL) { return std::max(64, std::min(kFftThreads, (((P >> 
 template <int KC>
 struct XKernels {
   static oam_status rows_r2c(const FftLayout *L, cudaStream_t st, const float *X, int py, int px, int Ctot, int c0,
-                             int C, float2 *Y) {
+                             int C, int CO, float2 *Y) {
     const size_t sm = sizeof(float2) * xslots<KC / 2>(L->P);
     oam_status rc = set_smem((const void *)k_xfft_rows_r2c<KC>, sm);
     if (rc) return rc;
-    k_xfft_rows_r2c<KC><<<dim3(py, (C + KC - 1) / KC), xthreads(L->P, KC / 2), sm, st>>>(X, py, px, Ctot, c0, C, L->P,
-                                                                                        L->lgP, L->Q, Y);
+    k_xfft_rows_r2c<KC><<<dim3(py, (C + KC - 1) / KC), xthreads(L->P, KC / 2), sm, st>>>(
+        X, py, px, Ctot, c0, C, CO, L->P, L->lgP, L->Q, Y);
     OAM_LAUNCHED();
     return OAM_OK;
   }
@@ -844,12 +782,12 @@ struct XKernels {
     return OAM_OK;
   }
   static oam_status rows_c2r(const FftLayout *L, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0,
-                             int C, float scale, float *X) {
+                             int C, int CO, float scale, float *X) {
     const size_t sm = sizeof(float2) * xslots<KC / 2>(L->P);
     oam_status rc = set_smem((const void *)k_xfft_rows_c2r<KC>, sm);
     if (rc) return rc;
     k_xfft_rows_c2r<KC><<<dim3(py, (Ctot + KC - 1) / KC), xthreads(L->P, KC / 2), sm, st>>>(
-        Z, py, px, Ctot, c0, C, L->P, L->lgP, L->Q, scale, X);
+        Z, py, px, Ctot, c0, C, CO, L->P, L->lgP, L->Q, scale, X);
     OAM_LAUNCHED();
     return OAM_OK;
   }
@@ -858,52 +796,40 @@ struct XKernels {
 // The same in the mixed-radix kernels (P <= 512).
 struct MKernels {
   static oam_status rows_r2c(const FftLayout *L, cudaStream_t st, const float *X, int py, int px, int Ctot, int c0,
-                             int C, float2 *Y) {
-    return mix_rows_r2c(L->P, st, X, py, px, Ctot, c0, C, L->d_tw, Y);
+                             int C, int CO, float2 *Y) {
+    return mix_rows_r2c(L->P, st, X, py, px, Ctot, c0, C, CO, L->d_tw, Y);
   }
   template <bool kInverse>
   static oam_status cols(const FftLayout *L, cudaStream_t st, const float2 *Z, int nin, int nout, int C, float2 *W) {
     return mix_cols(L->P, kInverse, st, Z, nin, nout, C, L->d_tw, W);
   }
   static oam_status rows_c2r(const FftLayout *L, cudaStream_t st, const float2 *Z, int py, int px, int Ctot, int c0,
-                             int C, float scale, float *X) {
-    return mix_rows_c2r(L->P, st, Z, py, px, Ctot, c0, C, L->d_tw, scale, X);
+                             int C, int CO, float scale, float *X) {
+    return mix_rows_c2r(L->P, st, Z, py, px, Ctot, c0, C, CO, L->d_tw, scale, X);
   }
 };
 
 template <class K>
 oam_status run_fft(const oam_model *m, const FftLayout *L, bool fwd, const float *in, float *out, cudaStream_t st) {
-  const int P = L->P, nz = m->grid.nz, py = m->grid.py, px = m->grid.px, NS = L->NS;
-  oam_status rc;
+  const int P = L->P, nz = m->grid.nz, nt = m->grid.nt, py = m->grid.py, px = m->grid.px, NS = L->NS;
   const float scale = 1.0f / ((float)P * (float)P);
-  if (fwd) {
-    if ((rc = K::rows_r2c(L, st, in, py, px, nz, 0, nz, L->d_w2))) return rc;
-    if ((rc = K::template cols<false>(L, st, L->d_w2, py, P, nz, L->d_w1))) return rc;
-    const size_t sa = sizeof(float4) * 2 * nz + sizeof(int) * (2 * nz + 2) + sizeof(long long) * nz;
-    if ((rc = set_smem((const void *)k_fft_apply_fwd, sa))) return rc;
-    const int fchunk = kFwdChunk > 0 ? kFwdChunk : NS;
-    const int fwd_threads = std::min(kApplyMaxThreads, 32 * ((fchunk + 32 / kFwdPhases - 1) / (32 / kFwdPhases)));
-    const unsigned fblocks = (unsigned)(L->n_rep * ((NS + fchunk - 1) / fchunk));
-    k_fft_apply_fwd<<<fblocks, fwd_threads, sa, st>>>(L->d_shat, L->row_stride, L->d_members, L->d_klo, L->d_klen,
-                                                      L->d_koff, L->d_krange, nz, m->n_lo, NS, L->d_w1, L->d_w2);
-    OAM_LAUNCHED();
-    if ((rc = K::template cols<true>(L, st, L->d_w2, P, py, NS, L->d_w1))) return rc;
-    if ((rc = K::rows_c2r(L, st, L->d_w1, py, px, m->grid.nt, m->n_lo, NS, scale, out))) return rc;
-  } else {
-    if ((rc = K::rows_r2c(L, st, in, py, px, m->grid.nt, m->n_lo, NS, L->d_w2))) return rc;
-    if ((rc = K::template cols<false>(L, st, L->d_w2, py, P, NS, L->d_w1))) return rc;
-    const size_t sa = (sizeof(float4) * 2 + sizeof(int2) + sizeof(long long)) * NS;
-    if ((rc = set_smem((const void *)k_fft_apply_adj, sa))) return rc;
-    const int achunk = kAdjChunk > 0 ? kAdjChunk : nz;
-    const int adj_threads = std::min(kApplyMaxThreads, 32 * ((achunk + 15) / 16));
-    const unsigned ablocks = (unsigned)(L->n_rep * ((nz + achunk - 1) / achunk));
-    k_fft_apply_adj<<<ablocks, adj_threads, sa, st>>>(L->d_shat_t, L->row_stride_t, L->d_members, L->d_klo, L->d_klen,
-                                                      L->d_krange, L->d_noff, nz, m->n_lo, NS, L->d_w1, L->d_w2);
-    OAM_LAUNCHED();
-    if ((rc = K::template cols<true>(L, st, L->d_w2, P, py, nz, L->d_w1))) return rc;
-    if ((rc = K::rows_c2r(L, st, L->d_w1, py, px, nz, 0, nz, scale, out))) return rc;
-  }
-  return OAM_OK;
+  const ApplyRows &A = L->rows[fwd ? 0 : 1];
+  // input and output: row lengths, first channels, channels and work-buffer strides
+  const int il = fwd ? nz : nt, i0 = fwd ? 0 : L->n0, ic = fwd ? nz : NS, is = fwd ? L->CZ : L->CS;
+  const int ol = fwd ? nt : nz, o0 = fwd ? L->n0 : 0, oc = fwd ? NS : nz, os = fwd ? L->CS : L->CZ;
+  oam_status rc;
+  if ((rc = K::rows_r2c(L, st, in, py, px, il, i0, ic, is, L->d_w2))) return rc;
+  if ((rc = K::template cols<false>(L, st, L->d_w2, py, P, is, L->d_w1))) return rc;
+  const size_t sa = (2 * sizeof(ulonglong2) + sizeof(int2)) * (A.n_in + kStep);
+  // both directions and every model share the kernel: one limit for all, or calls from several threads would
+  // lower each other's between setting it and the launch
+  if (sa > 48 * 1024 && (rc = set_smem((const void *)k_fft_apply, std::max<size_t>(sa, 227 * 1024)))) return rc;
+  const int rounds = (A.windows + kApplyWarps - 1) / kApplyWarps, warps = (A.windows + rounds - 1) / rounds;
+  k_fft_apply<<<L->n_rep, 32 * warps, sa, st>>>(A.d_s, A.stride, L->d_members, A.d_elem, A.d_window, A.windows,
+                                                A.n_in, is, A.n_out, os, L->d_w1, L->d_w2);
+  OAM_LAUNCHED();
+  if ((rc = K::template cols<true>(L, st, L->d_w2, P, py, os, L->d_w1))) return rc;
+  return K::rows_c2r(L, st, L->d_w1, py, px, ol, o0, oc, os, scale, out);
 }
 
 oam_status run_fft_any(const oam_model *m, bool fwd, const float *in, float *out, cudaStream_t st) {
