@@ -213,7 +213,9 @@ struct LineShape {
   __host__ __device__ int first_row(int seg) const { return segs > 1 ? seg * valid - halo : 0; }  // point 0's row
 };
 oam_status line_r2c(int P, cudaStream_t st, const LineShape &s, const float *in, const float2 *tw, float *packed);
+// Writes the output channels [z0, z1) of line_channels; the others are not touched.
 oam_status line_c2r(int P, cudaStream_t st, const LineShape &s, const float *part, const float2 *tw, float *out);
+void line_channels(const LineShape &s, int *z0, int *z1);
 
 // op_filter.cu: y = F x over the model's py*px A-lines (x and y may alias)
 oam_status fir_apply(const oam_model *m, const float *x, float *y, cudaStream_t st);

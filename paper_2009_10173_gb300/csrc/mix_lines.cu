@@ -5,12 +5,14 @@
 // input, zero-padded to P, as re and im rows of the packed correlation input.
 // Inverse, per (x, channel block): the correlation's re and im rows back to a
 // real y line of the output.  Both move the volume or the signals once and the
-// half spectrum (about 1.2x the lines, twice that for two partial sums) once; 32
+// half spectrum (about 1.2x the lines, the inverse once per partial sum) once; 32
 // channels per block, two neighbours per thread, make every global access a whole
-// 128-byte line per point, and all of a thread's loads are issued before its
-// first use.  At 200x200x300 (cold caches) 41 us forward and 82 to 102 us inverse,
-// against 18 and 36 to 42 us for the bytes at 6.8 TB/s: the loads' latency at two
-// or three blocks per SM (registers) bounds them.
+// 128-byte line per point, and all of a thread's loads are issued before its first
+// use.  At 200x200x300 (cold caches) 40 us forward, issue-bound, and 30, 62, 67 us
+// inverse with 1, 2 and, at three blocks per SM instead of two, 3 partial sums, bound
+// by the loads' latency (18 us of bytes forward, 26 + 9 per sum inverse, at 6.8 TB/s).
+// The output's channels beyond the accumulator are zeroed by a spare warp of the
+// correlation kernel, under its products (here they took 35 us).
 //
 // The correlation has compact support: a position whose window holds only zeros
 // gets exact zeros, and a non-finite input reaches only the positions whose window
@@ -124,13 +126,13 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>())
 
 // kVec: output rows are a whole number of float2 from an 8-byte boundary.
 template <int R1, int R2, bool kVec>
-__global__ void __launch_bounds__(mix_threads<R1, R2, kKH>())
+__global__ void __launch_bounds__(mix_threads<R1, R2, kKH>(), R1 >= 15 && R2 <= 20 ? 3 : 2)
     k_line_c2r(const LineShape s, const float *__restrict__ part, const float2 *__restrict__ tw, float scale,
                float *__restrict__ out) {
   constexpr int P = R1 * R2, Q = P / 2 + 1;
   extern __shared__ float2 sm[];
   __shared__ unsigned words[2][P / 32 + 2];  // grown marks of the rows written: some input, a non-finite one
-  const int x = blockIdx.y, ob = blockIdx.x * kLineCh;
+  const int x = blockIdx.y, ob = s.out_lo / kLineCh * kLineCh + blockIdx.x * kLineCh;
   const int y0 = s.first_row(blockIdx.z), ya = s.out_row(blockIdx.z), yb = min(s.py, ya + s.valid);  // rows written
   float *col = out + (size_t)x * s.out_len + ob;
   const size_t stride = (size_t)s.px * s.out_len;
@@ -143,16 +145,6 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>())
       for (int i = threadIdx.x; i < Q; i += blockDim.x) s.vmax[i] = 0;
       if (threadIdx.x == 0) *s.any_bad = 0;
     }
-  }
-  if (ob >= s.out_lo + s.acc || ob + kLineCh <= s.out_lo) {  // channels outside the accumulator: zeros
-    for (int i = threadIdx.x; i < (yb - ya) * kKH; i += blockDim.x) {
-      const int y = ya + i / kKH, c = 2 * (i % kKH);
-      float *p = col + (size_t)y * stride + c;
-      if (kVec && c < cols) *reinterpret_cast<float2 *>(p) = make_float2(0.0f, 0.0f);
-      if (!kVec && c < cols) p[0] = 0.0f;
-      if (!kVec && c + 1 < cols) p[1] = 0.0f;
-    }
-    return;
   }
   const int w0 = ya >> 5, nw = ((yb - 1) >> 5) - w0 + 1;
   for (int i = threadIdx.x; i < 2 * nw; i += blockDim.x)
@@ -210,7 +202,9 @@ oam_status run(bool inverse, cudaStream_t st, const LineShape &s, const float *i
     if (sm > 40 * 1024)  // static shared memory comes on top
       OAM_CUDA_TRY(
           cudaFuncSetAttribute(k_line_c2r<R1, R2, kVec>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    k_line_c2r<R1, R2, kVec><<<dim3((s.out_len + kLineCh - 1) / kLineCh, s.px, s.segs), threads, sm, st>>>(
+    int z0, z1;
+    line_channels(s, &z0, &z1);
+    k_line_c2r<R1, R2, kVec><<<dim3((z1 - z0 + kLineCh - 1) / kLineCh, s.px, s.segs), threads, sm, st>>>(
         s, in, tw, 1.0f / (float)(R1 * R2), out);
   } else {
     if (sm > 40 * 1024)
@@ -238,6 +232,12 @@ oam_status dispatch(int P, bool inverse, cudaStream_t st, LineShape s, const flo
 }
 
 }  // namespace
+
+// The 32-channel blocks of the output that meet the accumulator, up to the row's end.
+void oam::line_channels(const LineShape &s, int *z0, int *z1) {
+  *z0 = s.out_lo / kLineCh * kLineCh;
+  *z1 = std::min(s.out_len, (s.out_lo + s.acc + kLineCh - 1) / kLineCh * kLineCh);
+}
 
 oam_status oam::line_r2c(int P, cudaStream_t st, const LineShape &s, const float *in, const float2 *tw, float *packed) {
   return dispatch(P, false, st, s, in, tw, packed);

@@ -22,7 +22,8 @@
 // products than the correlation over both axes at a 61x61 window, for a slab
 // (P/2 + 1) / (R + 1) = 4 times the size at 200 lines and two line transforms.
 // Measured on a GB300 against that form (one application): 200x200x300 forward
-// 5.78 -> 0.49 ms, adjoint 5.71 -> 0.47 ms, 96x96x192 forward 0.86 -> 0.10 ms.
+// 5.78 -> 0.45 ms (k_corr_line 0.34), adjoint 5.71 -> 0.45 ms, 96x96x192 forward 0.86 ->
+// 0.10 ms.
 //
 // Mirror folding.  S_v[a] = S_v[-a], so the two mirrored taps share one slab tile
 // and their operand rows are summed before the product:
@@ -46,9 +47,10 @@
 // tensor memory.  The terms are FP16 (22 significant bits together, BF16 terms
 // hold 16) of operands scaled by powers of two: the slab by one for the model,
 // the iterate by one for each frequency, from the magnitudes that the line
-// transform finds.  Few blocks (small scans, or a nearly empty last wave)
-// split the taps over `parts` blocks, whose partial sums the inverse line
-// transform adds in index order.
+// transform finds.  The taps of a tile go to up to four blocks, whose partial sums the
+// inverse line transform adds in index order.  (Adding them in clusters through
+// distributed shared memory was slower: 9000 cycles a block for two blocks' sums, and
+// clusters of four leave SMs idle.)
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -69,6 +71,7 @@ constexpr int kDefaultFoldWarps = 8;
 constexpr int kMaxItems = 8;       // item ring depth (slab tile + folded operand)
 constexpr int kFoldCols = 32;      // tensor-memory columns per folded operand: 2 chunks x (hi, lo) x 8
 constexpr int kSmemLimit = 227 * 1024;
+constexpr int kStageRow = 36;      // floats per row of a fold warp's 32 x 32 epilogue stage
 
 // One ring item: the slab tiles of one (|a|, stage), hi then lo of each of
 // its two 16-deep chunks; 8 bytes, so a block's item tables stay small.  The
@@ -142,6 +145,8 @@ struct CorrParams {
   const unsigned *vmax;  // [frequencies] largest magnitude of the transformed lines, as float bits
   const unsigned *smax;  // the slab's, over its transform (an upper bound)
   float *part;         // partial sums [parts][frequencies][nr][px][acc_cols]
+  float *out;          // the operator's output [positions][out_len]: channels outside z0 .. z1 are zeroed here
+  int positions, out_len, z0, z1;
   int *status;
   long long budget;
 };
@@ -326,9 +331,23 @@ __device__ __forceinline__ void grow_marks(const CorrParams &p, int x, int lane)
   }
 }
 
-// Block (position tile, tap part, frequency).  What bounds it: the fold warps and
-// the MMA issue take about the same time per pair of items (~0.45 us at 320
-// accumulator columns), each waiting on the other through the item ring.
+// Zeros in the output's channels outside z0 .. z1 (whole groups of four) for this
+// block's share of the positions: the store traffic runs under the products.
+__device__ __forceinline__ void zero_outside(const CorrParams &p, int lane) {
+  const int lo4 = p.z0 / 4, n4 = lo4 + (p.out_len - p.z1) / 4;
+  if (n4 <= 0) return;
+  const int blocks = gridDim.x * gridDim.y * gridDim.z, blk = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  const int per = (p.positions + blocks - 1) / blocks;
+  for (int o = blk * per; o < min(p.positions, (blk + 1) * per); ++o) {
+    float4 *row = reinterpret_cast<float4 *>(p.out + (size_t)o * p.out_len);
+    for (int i = lane; i < n4; i += 32) row[i < lo4 ? i : p.z1 / 4 + i - lo4] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
+// Block (position tile, tap part, frequency).  What bounds it: shared memory.  A pair of
+// items reads 64 KB of strip rows (512 cycles at 128 bytes each), the tensor cores read
+// its tiles three times (336) and the copy engine writes them (224 cycles): 1072, and
+// 1100 measured at 320 accumulator columns.
 template <int FW, bool kWide>
 __global__ void __launch_bounds__(96 + 32 * FW, 1)
     k_corr_line(const __grid_constant__ CUtensorMap tmap, const CorrParams p) {
@@ -377,6 +396,11 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
     *abort_flag = 0;
     *never = 0;
     ptx::mbar_fence_init();
+    // the first strips travel while the block sets up
+    for (int st = 0; st < min(2, p.stages); ++st) {
+      ptx::mbar_arrive_expect_tx(&strip_full[st], (uint32_t)(L * 128));
+      tma_load_2d(strips + (size_t)st * p.strip_bytes, &tmap, kStageK * st, qt, &strip_full[st]);
+    }
   }
   for (int i = threadIdx.x; i < p.stages * nj; i += kThreads)
     sitems[i] = p.items[a_of(j0 + i % nj, R) * p.stages + i / nj];
@@ -397,7 +421,7 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
-      int it_slab = 0, loads = 0;  // item pairs and strips requested
+      int it_slab = 0, loads = min(2, p.stages);  // item pairs and strips requested (two before the block's barrier)
       int k = 0;
       uint32_t lap = 0;  // parity of the item ring's current lap
       bool ok = true;
@@ -411,8 +435,6 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
         ++loads;
         return true;
       };
-      for (int st = 0; st < min(2, p.stages) && ok; ++st) ok = load_strip(st);
-      if (!ok) fail(1);
       for (int st = 0; st < p.stages && ok; ++st) {
         const TcItem *row_items = sitems + st * nj;
         for (int j = 0; j < nj; j += 2) {  // pair slot k holds items j (slot 2k) and j + 1 (slot 2k + 1) of the stage
@@ -505,7 +527,8 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
     if (leader) ptx::mma_commit(acc_full);
     __syncwarp();
   } else if (warp == 2 + kFoldWarps) {
-    // ------------------------------------------------------------ marks
+    // ------------------------------------------------------------ marks, zeros
+    zero_outside(p, lane);
     if (blockIdx.y == 0)
       for (int x = freq * gridDim.x + tile; x < p.px; x += gridDim.z * gridDim.x) grow_marks(p, x, lane);
   } else {
@@ -528,7 +551,7 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
     const int row = o / p.sp, x = o % p.sp;
     const int pm = (row - r0) * p.wp + (x - x0);  // its packed offset from the tile's first
     const int q0 = kq * (E / 8);        // first 8-element quarter of the stage
-    const int ef = scale_exp(2.0f * __uint_as_float(p.vmax[freq])), es = scale_exp(__uint_as_float(*p.smax));
+    const int ef = scale_exp(2.0f * __uint_as_float(p.vmax[freq]));
     const uint64_t sc = pack_f32x2(pow2(ef), pow2(ef));
     int k = 0;
     uint32_t lap = 0;
@@ -568,27 +591,42 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
       if (lane == 0) ptx::mbar_arrive(&strip_empty[s]);
     }
 
-    // epilogue: this warp's lane quarter and column share of the accumulator
+    // Epilogue: this warp's lane quarter and column share of the accumulator.  A lane
+    // holds one row; 32-column blocks go through the (now free) strips, rows of 36 floats
+    // so that neither side meets a bank twice, and leave as four whole 128-byte pieces a
+    // store.  6900 cycles a block at 320 columns: the blocks of a wave write together, and
+    // 24 bytes a cycle from each of 152 SMs are the memory's rate.
     bool done = ptx::mbar_wait(acc_full, 0, abort_flag, 4 * p.budget);
     done = __all_sync(0xffffffffu, done && ok);
     ptx::tc_fence_after();
-    const bool valid = done && row < p.nr && x < p.px;
-    const float us = pow2(-es), uf = pow2(-ef);
-    float *dst_row =
-        p.part + ((((size_t)blockIdx.y * gridDim.z + freq) * p.nr + row) * p.px + x) * (size_t)p.acc_cols;
     if (done) {
-      for (int j = blk_begin; j < blk_end; ++j) {
-        const int col = 32 * j;
-        uint32_t r[32];
-        ptx::tmem_ld32(tmem + lane_base + (uint32_t)col, r);
-        ptx::tmem_wait_ld();
-        if (valid) {
-          float4 *dst = reinterpret_cast<float4 *>(dst_row + col);
-          const int nv = std::min(8, (p.acc_cols - col) >> 2);
-          auto val = [&](int i) { return __uint_as_float(r[i]) * us * uf; };  // exact unless it leaves FP32's range
+      const float us = pow2(-scale_exp(__uint_as_float(*p.smax))), uf = pow2(-ef);
+      const int pos = row < p.nr && x < p.px ? row * p.px + x : -1;  // this lane's row in the output
+      float *base = p.part + ((size_t)blockIdx.y * gridDim.z + freq) * p.nr * p.px * p.acc_cols + 4 * (lane & 7);
+      float *dst[8];  // rows 4 i + lane / 8 of the quarter
 #pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (q < nv) dst[q] = make_float4(val(4 * q), val(4 * q + 1), val(4 * q + 2), val(4 * q + 3));
+      for (int i = 0; i < 8; ++i) {
+        const int q = __shfl_sync(0xffffffffu, pos, 4 * i + (lane >> 3));
+        dst[i] = q >= 0 ? base + (size_t)q * p.acc_cols : nullptr;
+      }
+      float *stage = reinterpret_cast<float *>(strips) + fw * 32 * kStageRow;
+      for (int j = blk_begin; j < blk_end; ++j) {
+        uint32_t r[32];
+        ptx::tmem_ld32(tmem + lane_base + (uint32_t)(32 * j), r);
+        ptx::tmem_wait_ld();
+        auto val = [&](int i) { return __uint_as_float(r[i]) * us * uf; };  // exact unless it leaves FP32's range
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          *reinterpret_cast<float4 *>(stage + lane * kStageRow + 4 * q) =
+              make_float4(val(4 * q), val(4 * q + 1), val(4 * q + 2), val(4 * q + 3));
+        __syncwarp();
+        if (32 * j + 4 * (lane & 7) < p.acc_cols) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (dst[i])
+              *reinterpret_cast<float4 *>(dst[i] + 32 * j) =
+                  *reinterpret_cast<const float4 *>(stage + (4 * i + (lane >> 3)) * kStageRow + 4 * (lane & 7));
         }
       }
     }
@@ -818,19 +856,22 @@ oam_status plan_dir(const oam_model *m, const TcLine *T, TcLayout *L, int dir, s
   }
   L->slot_bytes = (max_item + 127) & ~127;
   L->v_stride = (size_t)std::max<long long>(off, 16);
-  // Blocks that share a tile's taps: as many as make the last wave of one block per
-  // SM fullest.  In units of one pair of items (~0.45 us): a block's pairs, about
-  // 12 for its set-up and epilogue, and a part's sums written and read once more.
-  // At least two: the tensor cores truncate when they add to an accumulator, and
-  // the frequencies' sums cancel over depth, so halving the products that one
-  // accumulator takes halves that error (200x200x300 forward 4.4e-6 -> 2.1e-6).
+  // Blocks that share a tile's taps.  At least one per 5 1/3 pairs of taps: the tensor
+  // cores truncate when they add to an accumulator, and the frequencies' sums cancel
+  // over depth, so the fewer products one accumulator takes the less that costs
+  // (200x200x300, 16 pairs, forward with 1, 2, 3, 4 parts: 4.7e-6, 2.3e-6, 1.5e-6,
+  // 1.2e-6 against FP64, and 3.4e-6 for three BF16 products per tap with no transform;
+  // 164x228x154, 11 pairs: 4.4e-6, 2.1e-6, 1.5e-6, 1.2e-6 and 1.9e-6).  Beyond
+  // that, as many as finish first, in units of one pair of items (~0.55 us): a block's
+  // pairs and about 18 for its set-up and epilogue, times the waves of one block per SM,
+  // and a part's sums written and read once more (40 us for 62 MB).
   const int NP = (R + 2) / 2, sms = std::max(1, m->sm_count ? m->sm_count : 152);
   const long long tiles0 = ((long long)T->nr * m->grid.px + kTileM - 1) / kTileM * T->Q;
-  const double part_units = 2.0 * T->Q * T->nr * m->grid.px * L->acc_cols * 4.0 / (6.8e12 * 0.45e-6);
+  const double part_units = (double)T->Q * T->nr * m->grid.px * L->acc_cols * 4.0 / (1.55e12 * 0.55e-6);
   double best = 0;
   L->parts = 0;
-  for (int q = std::min(2, NP); q <= std::min(4, NP); ++q) {
-    const double cost = (double)((tiles0 * q + sms - 1) / sms) * ((double)((NP + q - 1) / q) * L->stages + 12) +
+  for (int q = std::min(4, (3 * NP + 15) / 16); q <= std::min(4, NP); ++q) {
+    const double cost = (double)((tiles0 * q + sms - 1) / sms) * ((double)((NP + q - 1) / q) * L->stages + 18) +
                         (q - 1) * part_units;
     if (!L->parts || cost < best) {
       best = cost;
@@ -926,8 +967,10 @@ oam_status plan_launch(const oam_model *m, const TcLine *T, const TcLayout *L, L
   p.part = T->d_part;
   p.status = m->d_status;
   p.budget = 4000000000LL;  // ~2 s at 2 GHz
-  out->p = p;
+  // the strips and slots, or where they are smaller the fold warps' epilogue stages
   out->smem = (size_t)fixed + (size_t)p.n_items * p.slot_bytes;
+  out->smem = std::max(out->smem, (size_t)2048 + p.items_bytes + sizeof(float) * 32 * kStageRow * L->fold_warps);
+  out->p = p;
   out->tiling = tiling;
   out->n_tiles = (int)(((long long)T->nr * p.sp + kTileM - 1) / kTileM);
   if (out->smem > (size_t)kSmemLimit) return OAM_ERR_UNSUPPORTED;
@@ -973,7 +1016,6 @@ oam_status run_corr(const oam_model *m, const TcLayout *L, const float *in, int 
   s.out_len = out_len;
   s.out_lo = L->out_lo;
   s.acc = L->acc_cols;
-  s.parts = L->parts;
   s.words = T->words;
   s.marks = T->d_marks;
   unsigned *tail = T->d_marks + (size_t)2 * s.px * s.words;
@@ -984,6 +1026,11 @@ oam_status run_corr(const oam_model *m, const TcLayout *L, const float *in, int 
   lp.p.grown = tail + T->Q + 1;
   lp.p.any_bad = s.any_bad;
   lp.p.words = T->words;
+  s.parts = L->parts;
+  lp.p.out = out;
+  lp.p.positions = s.px * s.py;
+  lp.p.out_len = out_len;
+  line_channels(s, &lp.p.z0, &lp.p.z1);
   lp.p.vmax = s.vmax;
   lp.p.smax = T->d_smax;
   ProfScope prof(m, st, L->dir == 0);
