@@ -150,8 +150,8 @@ void free_model(oam_model *m, cudaStream_t st) {
   fft_free(m, st);
   fir_free(m, st);
   for (cudaEvent_t e : m->prof.pool) cudaEventDestroy(e);
-  void *ptrs[] = {m->d_status, m->d_tap_orbit, m->d_patch, m->d_band_lo, m->d_band, m->d_fwd_krange, m->d_fwd_off,
-                  m->d_fwd, m->d_adj_nrange, m->d_adj_off, m->d_adj};
+  void *ptrs[] = {m->d_status, m->d_tap_orbit, m->d_patch, m->d_band_lo, m->d_band, m->rows_fwd.d_taps,
+                  m->rows_fwd.d_rows, m->rows_adj.d_taps, m->rows_adj.d_rows};
   for (void *p : ptrs)
     if (p) cudaFreeAsync(p, st);
   delete m;

@@ -13,8 +13,8 @@
 
 namespace oam {
 
-constexpr int kTimeTile = 64;  // FP32 forward layout: samples per time tile
-constexpr int kDepthTile = 16; // FP32 adjoint layout: depths per depth tile
+constexpr int kOutTile = 32;   // FP32 operators: outputs (samples or depths) per tile
+constexpr int kRowChunk = 16;  // and input elements per stored chunk of slab rows
 constexpr int kRedBlocks = 1024; // max blocks of a reduction kernel (partials buffer size)
 
 // Sensor ring plan (host): rings uniform in polar angle, 8*u_r patches each.
@@ -29,6 +29,17 @@ struct Ring {
 // and area in mm^2.
 struct __align__(32) Patch {
   double x, y, z, w;
+};
+
+// Slab rows of one direction of the FP32 operators: per (orbit, tile of kOutTile
+// outputs), from the kRowChunk-chunk that holds the first input element whose band
+// meets the tile to the one that holds the last, a row of kOutTile values per input
+// element.  taps: per tile, tap (b, a >= 0) and, in the last column, the union over a:
+// x = first element | count << 16, y = first chunk's index in d_rows.
+struct DirectRows {
+  int tiles = 0;
+  uint2 *d_taps = nullptr;   // [tiles][R + 1][R + 2]
+  float *d_rows = nullptr;   // [chunks][kRowChunk][kOutTile]
 };
 
 // Tensor-core operator layout of one direction (forward or adjoint); defined in op_tc.cu.
@@ -67,16 +78,8 @@ struct oam_model {
   int *d_band_lo = nullptr;
   float *d_band = nullptr;        // [n_orb][nz][band_w]
 
-  // FP32 forward layout: per (orbit, time tile) depths [klo, khi), rows of kTimeTile samples
-  int n_ttiles = 0;
-  int *d_fwd_krange = nullptr;    // [n_orb*n_ttiles][2]
-  long long *d_fwd_off = nullptr; // [n_orb*n_ttiles]
-  float *d_fwd = nullptr;
-  // FP32 adjoint layout: per (orbit, depth tile) samples [nlo, nlo+nlen), rows of nlen
-  int n_ktiles = 0;
-  int *d_adj_nrange = nullptr;    // [n_orb*n_ktiles][2] = (nlo, nlen)
-  long long *d_adj_off = nullptr;
-  float *d_adj = nullptr;
+  // FP32 operators' slab rows (OAM_PREC_FP32)
+  oam::DirectRows rows_fwd, rows_adj;
 
   // tensor-core layouts (OAM_PREC_BF16X3) per direction, and the plan and buffers
   // of the line transforms around them
@@ -147,8 +150,6 @@ inline size_t alloc_bytes(size_t count) {
 // slab.cu
 oam_status build_slab(oam_model *m, cudaStream_t st);
 oam_status plan_bands(oam_model *m, const std::vector<double2> &h_range, int widen);
-long long fwd_layout(const oam_model *m, std::vector<int> *kr, std::vector<long long> *off);
-long long adj_layout(const oam_model *m, std::vector<int> *nr, std::vector<long long> *off);
 size_t slab_plan_bytes(const oam_model *m);
 oam_status slab_column(const oam_model *m, int b, int a, int k, float *d_out, cudaStream_t st);
 

@@ -5,229 +5,595 @@
 // offset relative to each scan position; Methods, Efficient reconstruction
 // based on scanning symmetries).  Voxels and samples outside the grids are zero.
 //
-// forward: block = (row y, 64 positions, 64-sample time tile); it walks every
-//   tap (b, a) and the depths whose band meets the time tile, staging 16 depths
-//   of the shifted volume row and the packed slab rows in shared memory.
-// adjoint: block = (row y, 64 positions, 16-depth tile), 64 threads of 4
-//   positions x 4 depths; it walks every tap and the samples of the tile's band
-//   union, 64 samples at a time.
+// One kernel serves both: out[pos][n] += F[pos][k] S[k][n], K = depths and N =
+// samples for the forward operator, the reverse for the adjoint.  The slab is
+// mirror-symmetric (S[b][a] = S[+-b][+-a]; Results, axial symmetry), so the four
+// mirrored taps share their slab rows and their inputs are summed first:
+//   P[pos][k] = X[y + b][x][k] + X[y - b][x][k]          (once per row offset b)
+//   F[pos][k] = P[x + a][k] + P[x - a][k]                (once per tap)
+// which cuts the products 3.9x at 61x61 taps.  A block serves an output tile of kTile
+// and a tile of positions; it walks the row offsets and the 16-deep K chunks whose band
+// meets the output tile, with P in shared memory, and the taps a of each chunk.  A
+// thread keeps 8 positions x 4 outputs in registers as packed pairs of positions.
+//   k_corr_warps  32 positions; the block's eight warps share out the taps, each with
+//                 its own F and slab rows, so nothing but P is exchanged between warps:
+//                 the short chain for small problems.
+//   k_corr_block  128 positions; four warps take each tap together, 32 positions each,
+//                 sharing its slab rows (a quarter of the L2 reads): large problems.
 //
-// Each output sums up to win^2 x band products (about 3e5 at 61 x 61 taps).
-// One FP32 accumulator for all of them loses about sqrt(n) units in the last
-// place, 2e-5 relative at that size, so both kernels sum in three levels: the
-// products of one tap, then the taps of one tap row, then the rows.
+// What bounds both: the FP32 pipe (1.5x the band's products in 32-output tiles, and the
+// moves that make packed operands) at about half its rate, the rest latency between
+// taps.  One application, GB300, from a kernel without folding: 200x200x300 forward,
+// 61x61 taps, 360 -> 53 ms; 32x32x48, 11x11 taps, 283 -> 47 us; 70x37x52 adjoint, 15x15
+// taps, 888 -> 156 us.
+//
+// Each output sums up to win^2 x band products (about 3e5 at 61x61 taps).  One
+// FP32 accumulator for all of them loses about sqrt(n) units in the last place,
+// so the kernels sum in three levels: the products of at most 8 taps of a chunk, then
+// those of a row offset (in registers or shared memory), then the row offsets, in the
+// output.  The order does not depend on the position, so a shifted input gives the
+// shifted output to the bit.
+#include <algorithm>
+
 #include "internal.cuh"
 
 using namespace oam;
 
 namespace {
 
-constexpr int kPos = 64;
+constexpr int kWarps = 8;        // warps per block: warp w takes the taps a = w (mod kWarps)
+constexpr int kThreads = 32 * kWarps;
+constexpr int kPos = 32;         // positions per block
+constexpr int kChunk = kRowChunk;  // K elements per chunk (16)
+constexpr int kTile = kOutTile;  // outputs per block (32)
+constexpr int kFlush = 8;        // a warp's taps per first-level sum
+constexpr int kMaxStrip = 352;   // staged positions a block takes on run-on tiles
+constexpr int kTableR = 31;      // largest half window whose tap table is copied to shared memory
 
-__global__ void __launch_bounds__(256) k_fwd_fp32(const float *__restrict__ H, float *__restrict__ s, int px, int py,
-                                                  int nz, int nt, int R, const int *__restrict__ tap_orbit, int n_tt,
-                                                  const int *__restrict__ krange, const long long *__restrict__ off,
-                                                  const float *__restrict__ P) {
-  const int x0 = blockIdx.x * kPos, y = blockIdx.y, T = blockIdx.z;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int W = 2 * R + 1;
-  __shared__ __align__(16) float Hs[kPos][kDepthTile + 4];  // rows of 16 depths, 16-byte aligned
-  __shared__ float4 Ps[kDepthTile][kTimeTile / 4];
-  float acc[4][4] = {}, row_acc[4][4], tap_acc[4][4];
-  for (int b = -R; b <= R; ++b) {
-    const int yy = y + b;
-    if (yy < 0 || yy >= py) continue;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) row_acc[i][j] = 0.0f;
-    for (int a = -R; a <= R; ++a) {
-      const int xs = x0 + a;
-      if (xs + kPos <= 0 || xs >= px) continue;
-      const int oi = tap_orbit[(b + R) * W + (a + R)] * n_tt + T;
-      const int klo = krange[2 * oi], khi = krange[2 * oi + 1];
-      if (klo >= khi) continue;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) tap_acc[i][j] = 0.0f;
-      const float4 *P4 = reinterpret_cast<const float4 *>(P + off[oi]);
-      // this thread's share of a 16-depth chunk (4 volume values, 4 slab values),
-      // fetched one chunk ahead so the loads run during the previous chunk's FMAs
-      float hv[4];
-      float4 pv;
-      auto fetch = [&](int kc) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int e = tid + 256 * r, p = e >> 4, kk = e & 15;
-          const int x = xs + p, k = kc + kk;
-          hv[r] = (x >= 0 && x < px && k < khi) ? H[((size_t)yy * px + x) * nz + k] : 0.0f;
-        }
-        const int row = tid >> 4, c4 = tid & 15;
-        pv = (kc + row < khi) ? P4[(size_t)(kc - klo + row) * (kTimeTile / 4) + c4] : make_float4(0.f, 0.f, 0.f, 0.f);
-      };
-      fetch(klo);
-      for (int kc = klo; kc < khi; kc += kDepthTile) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int e = tid + 256 * r;
-          Hs[e >> 4][e & 15] = hv[r];
-        }
-        Ps[tid >> 4][tid & 15] = pv;
-        __syncthreads();
-        if (kc + kDepthTile < khi) fetch(kc + kDepthTile);
-        // four depths per step: 4 + 4 16-byte reads for 64 FMAs, each
-        // accumulator still taking its depths in increasing order
-#pragma unroll
-        for (int k4 = 0; k4 < kDepthTile; k4 += 4) {
-          float4 p[4], h[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) p[u] = Ps[k4 + u][tx];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) h[i] = *reinterpret_cast<const float4 *>(&Hs[4 * ty + i][k4]);
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const float hv = u == 0 ? h[i].x : u == 1 ? h[i].y : u == 2 ? h[i].z : h[i].w;
-              tap_acc[i][0] = fmaf(hv, p[u].x, tap_acc[i][0]);
-              tap_acc[i][1] = fmaf(hv, p[u].y, tap_acc[i][1]);
-              tap_acc[i][2] = fmaf(hv, p[u].z, tap_acc[i][2]);
-              tap_acc[i][3] = fmaf(hv, p[u].w, tap_acc[i][3]);
-            }
-        }
-        __syncthreads();
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) row_acc[i][j] += tap_acc[i][j];
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] += row_acc[i][j];
-  }
-  const int n = T * kTimeTile + 4 * tx;
-  if (n >= nt) return;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int x = x0 + 4 * ty + i;
-    if (x < px)
-      *reinterpret_cast<float4 *>(s + ((size_t)y * px + x) * nt + n) =
-          make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+__device__ __forceinline__ uint64_t pack2(float x, float y) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ void copy16_async(void *dst, const void *src, bool real) {  // zeros unless real
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(real ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void copies_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
+}
+
+struct CorrShape {
+  int px, py, R;
+  int len, out_len;  // input and output row lengths
+  int sp;            // positions per tile-grid row: px (tiles run on over rows) or a multiple of the tile
+  int strip;         // staged positions per block: tile + (rows wrapped + 2) R
+  const uint2 *taps;  // [output tile][R + 1][R + 2] (DirectRows)
+  const float *rows;  // slab rows
+};
+
+// K range [lo, hi) of a table entry.
+__device__ __forceinline__ int k_lo(uint2 t) { return (int)(t.x & 0xffffu); }
+__device__ __forceinline__ int k_hi(uint2 t) { return (int)(t.x & 0xffffu) + (int)(t.x >> 16); }
+
+// Float of K quarter kq of staged position r: 64-byte rows, the 16-byte quarters
+// exchanged so that eight neighbouring positions' reads fall in distinct banks.
+__device__ __forceinline__ int p_at(int r, int kq) { return r * kChunk + 4 * (kq ^ ((r >> 1) & 3)); }
+
+// Row and column (-1: padding) of the staged positions of a tile that starts at (y0, x0).
+template <int kN>
+__device__ __forceinline__ void stage_where(const CorrShape &s, int y0, int x0, int2 *where) {
+  const int wp = s.px + s.R;
+  for (int r = threadIdx.x; r < s.strip; r += kN) {
+    const long long q = (long long)y0 * wp + x0 - s.R + r;
+    const int y = q < 0 ? -1 : (int)(q / wp), x = q < 0 ? -1 : (int)(q % wp);
+    where[r] = make_int2(y, x < s.px ? x : -1);
   }
 }
 
-constexpr int kAdjThreads = 64;
+// F of tap a for the position staged at pm, K quarter by quarter: F[k][position m] at d.
+template <int kM>
+__device__ __forceinline__ void fold_tap(const float *P, int pm, int a, float *d, int kq) {
+  float4 f = *reinterpret_cast<const float4 *>(P + p_at(pm + a, kq));
+  if (a > 0) {
+    const float4 h = *reinterpret_cast<const float4 *>(P + p_at(pm - a, kq));
+    f = make_float4(f.x + h.x, f.y + h.y, f.z + h.z, f.w + h.w);
+  }
+  d += 4 * kq * kM;
+  d[0] = f.x;
+  d[kM] = f.y;
+  d[2 * kM] = f.z;
+  d[3 * kM] = f.w;
+}
 
-__global__ void __launch_bounds__(kAdjThreads) k_adj_fp32(const float *__restrict__ s, float *__restrict__ H, int px,
-                                                          int py, int nz, int nt, int R,
-                                                          const int *__restrict__ tap_orbit, int n_kt,
-                                                          const int *__restrict__ nrange,
-                                                          const long long *__restrict__ off,
-                                                          const float *__restrict__ Q) {
-  const int x0 = blockIdx.x * kPos, y = blockIdx.y, K = blockIdx.z;
-  // thread: positions pg + 16 i (i < 4) and depths 4 dg + d (d < 4) of the tile
-  const int tid = threadIdx.x, pg = tid & 15, dg = tid >> 4;
-  const int W = 2 * R + 1;
-  __shared__ float4 Ss[kPos][kTimeTile / 4 + 1];
-  __shared__ float4 Qs[kDepthTile][kTimeTile / 4];
-  float acc[4][4] = {}, row_acc[4][4], tap_acc[4][4];
-  for (int b = -R; b <= R; ++b) {
-    const int yy = y - b;
-    if (yy < 0 || yy >= py) continue;
+// a1[position pair][output] += F[ka .. kb)[8 positions] S[ka .. kb)[4 outputs].
+template <int kM>
+__device__ __forceinline__ void multiply(const float *F, const float *S, int ka, int kb, uint64_t (&a1)[4][4]) {
+  for (int kk = ka; kk < kb; kk += 4) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int d = 0; d < 4; ++d) row_acc[i][d] = 0.0f;
-    for (int a = -R; a <= R; ++a) {
-      const int xs = x0 - a;
-      if (xs + kPos <= 0 || xs >= px) continue;
-      const int oi = tap_orbit[(b + R) * W + (a + R)] * n_kt + K;
-      const int nlo = nrange[2 * oi], nlen = nrange[2 * oi + 1];
-      if (nlen <= 0) continue;
+    for (int u = 0; u < 4; ++u) {
+      const float4 sv = *reinterpret_cast<const float4 *>(S + (kk + u) * kTile);
+      const uint64_t s2[4] = {pack2(sv.x, sv.x), pack2(sv.y, sv.y), pack2(sv.z, sv.z), pack2(sv.w, sv.w)};
+      const ulonglong2 f0 = *reinterpret_cast<const ulonglong2 *>(F + (kk + u) * kM);
+      const ulonglong2 f1 = *reinterpret_cast<const ulonglong2 *>(F + (kk + u) * kM + 4);
+      const uint64_t f2[4] = {f0.x, f0.y, f1.x, f1.y};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int d = 0; d < 4; ++d) tap_acc[i][d] = 0.0f;
-      const float4 *Q4 = reinterpret_cast<const float4 *>(Q + off[oi]);
-      for (int nc = 0; nc < nlen; nc += kTimeTile) {
-#pragma unroll 4
-        for (int r = 0; r < kPos * (kTimeTile / 4) / kAdjThreads; ++r) {
-          const int e = tid + kAdjThreads * r, pp = e >> 4, j4 = e & 15;
-          const int x = xs + pp, j = nc + 4 * j4;
-          Ss[pp][j4] = (x >= 0 && x < px && j < nlen)
-                           ? *reinterpret_cast<const float4 *>(s + ((size_t)yy * px + x) * nt + nlo + j)
-                           : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int j = 0; j < 4; ++j) a1[i][j] = fma2(f2[i], s2[j], a1[i][j]);
+    }
+  }
+}
+
+// ---------------------------------------------------------------- k_corr_warps
+// Shared memory: raw rows of the two row offsets, double-buffered (the first of a pair
+// holds P once added) [2][2][strip][kChunk]; per warp F [kChunk][kPos] and two slots of
+// slab rows [kChunk][kTile]; the tap table (R <= kTableR); per staged position its row
+// and column.
+size_t warps_smem(int strip, int R) {
+  return sizeof(float) * ((size_t)4 * strip * kChunk + kWarps * kChunk * (kPos + 2 * kTile)) +
+         (R <= kTableR ? sizeof(uint2) * (R + 1) * (R + 2) : 0) + sizeof(int2) * strip;
+}
+
+// kVec: input rows are whole float4 from a 16-byte boundary.
+template <bool kVec>
+__global__ void __launch_bounds__(kThreads, 2)
+    k_corr_warps(const CorrShape s, const float *__restrict__ in, float *__restrict__ out) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int R = s.R, NA = R + 1, wp = s.px + R, p_size = s.strip * kChunk;
+  float *Pb = reinterpret_cast<float *>(smem);  // [buffer][side][p_size]
+  float *Fb = Pb + 4 * p_size;                  // [warp][kChunk][kPos]; the warps' sums at the end of a row offset
+  float *Sb = Fb + kWarps * kChunk * kPos;      // [warp][slot][kChunk][kTile]
+  int2 *where = reinterpret_cast<int2 *>(Sb + 2 * kWarps * kChunk * kTile);  // staged position: row y, column x (-1: padding)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int T = blockIdx.y, tile = blockIdx.x;
+  const int y0 = tile * kPos / s.sp, x0 = tile * kPos % s.sp;
+  const int y1 = min((tile * kPos + kPos - 1) / s.sp, s.py - 1);  // rows of the tile
+  const uint2 *tab = s.taps + (size_t)T * NA * (NA + 1);
+  if (R <= kTableR) {
+    uint2 *t = reinterpret_cast<uint2 *>(where + s.strip);
+    for (int i = tid; i < NA * (NA + 1); i += kThreads) t[i] = tab[i];
+    tab = t;
+  }
+  stage_where<kThreads>(s, y0, x0, where);
+  __syncthreads();
+  float *F = Fb + warp * kChunk * kPos, *S = Sb + warp * 2 * kChunk * kTile;
+  // staged index of the position this lane folds
+  const int pm = ((tile * kPos + lane) / s.sp - y0) * wp + ((tile * kPos + lane) % s.sp - x0) + R;
+  const int ng = lane & 7, pg = lane >> 3;  // outputs 4 ng .. +3 of the tile, positions 8 pg .. +7
+
+  // Walk of the (row offset b, chunk c) with work: c0 .. c1 - 1 are b's chunks.
+  int b = -1, c = 0, c1 = 0;
+  auto advance = [&](int &b, int &c, int &c1) {
+    if (++c < c1) return;
+    while (++b <= R) {
+      if (y0 + b >= s.py && y1 - b < 0) continue;  // neither row offset meets the grid
+      const uint2 t = tab[b * (NA + 1) + NA];      // the union of its taps' ranges
+      if (t.x >> 16) {
+        c = k_lo(t) / kChunk;
+        c1 = (k_hi(t) + kChunk - 1) / kChunk;
+        return;
+      }
+    }
+  };
+  // This warp's taps whose range meets chunk c of row offset b, one bit each.
+  auto my_taps = [&](int b, int c, unsigned long long &m0, unsigned long long &m1) {
+    auto word = [&](int i) {
+      const int a = 32 * i + lane;
+      const uint2 t = a < NA ? tab[b * (NA + 1) + a] : make_uint2(0, 0);
+      return __ballot_sync(0xffffffffu, k_lo(t) < (c + 1) * kChunk && k_hi(t) > c * kChunk && (t.x >> 16)) &
+             (0x01010101u << warp);
+    };
+    m0 = m1 = 0;
+    m0 = word(0);
+    if (NA > 32) m0 |= (unsigned long long)word(1) << 32;
+    if (NA > 64) m1 = word(2);
+    if (NA > 96) m1 |= (unsigned long long)word(3) << 32;
+  };
+  auto pop = [&](unsigned long long &m0, unsigned long long &m1) {  // lowest tap, NA when none is left
+    int a = NA;
+    if (m0) {
+      a = __ffsll((long long)m0) - 1;
+      m0 &= m0 - 1;
+    } else if (m1) {
+      a = 63 + __ffsll((long long)m1);
+      m1 &= m1 - 1;
+    }
+    return a;
+  };
+  // Request the raw rows of (b, c) into buffer pb.
+  auto request_rows = [&](int b, int c, int pb) {
+    const int quarters = s.strip * (kChunk / 4);
+    for (int side = 0; side < (b ? 2 : 1); ++side)
+      for (int i = tid; i < quarters; i += kThreads) {
+        const int r = i / (kChunk / 4), kq = i % (kChunk / 4), k = c * kChunk + 4 * kq;
+        const int2 w = where[r];
+        const int y = side ? w.x - b : w.x + b;
+        const bool ok = w.y >= 0 && y >= 0 && y < s.py;
+        const float *src = in + (ok ? ((size_t)y * s.px + w.y) * s.len + k : 0);
+        float *dst = Pb + (2 * pb + side) * p_size + p_at(r, kq);
+        if (kVec) {
+          copy16_async(dst, k < s.len ? src : in, ok && k < s.len);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) dst[q] = ok && k + q < s.len ? src[q] : 0.0f;
         }
+      }
+  };
+  // Request the slab rows of tap a in (b, c) into this warp's slot.
+  auto request_slab = [&](int b, int c, int a, int slot) {
+    if (a >= NA) return;
+    const uint2 t = tab[b * (NA + 1) + a];
+    const float *src = s.rows + ((size_t)t.y + (c - k_lo(t) / kChunk)) * (kChunk * kTile);
+    float *dst = S + slot * kChunk * kTile;
 #pragma unroll
-        for (int r = 0; r < kDepthTile * (kTimeTile / 4) / kAdjThreads; ++r) {
-          const int e = tid + kAdjThreads * r, row = e >> 4, j4 = e & 15, j = nc + 4 * j4;
-          Qs[row][j4] = (j < nlen) ? Q4[((size_t)row * nlen + j) >> 2] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j = 0; j < kChunk * kTile / 128; ++j) copy16_async(dst + 128 * j + 4 * lane, src + 128 * j + 4 * lane, true);
+  };
+
+  uint64_t a1[4][4], a2[4][4];  // [position pair][output]
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a1[i][j] = a2[i][j] = 0;
+  // Add the warps' sums of a row offset to the output: two of a lane's four outputs at
+  // a time through the F buffers, a thread per four position x output pairs.
+  auto flush = [&](bool first) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      __syncthreads();
+      // [warp][position][2 outputs of each group of four]
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 u = unpack2(a2[i][2 * half]), v = unpack2(a2[i][2 * half + 1]);
+        *reinterpret_cast<float2 *>(F + (8 * pg + 2 * i) * 16 + 2 * ng) = make_float2(u.x, v.x);
+        *reinterpret_cast<float2 *>(F + (8 * pg + 2 * i + 1) * 16 + 2 * ng) = make_float2(u.y, v.y);
+        a2[i][2 * half] = a2[i][2 * half + 1] = 0;
+      }
+      __syncthreads();
+      for (int i = tid; i < kPos * 8; i += kThreads) {  // (position, pair of outputs)
+        float2 v = *reinterpret_cast<const float2 *>(Fb + 2 * i);
+#pragma unroll
+        for (int w = 1; w < kWarps; ++w) {
+          const float2 u = *reinterpret_cast<const float2 *>(Fb + w * kChunk * kPos + 2 * i);
+          v.x += u.x;
+          v.y += u.y;
         }
-        __syncthreads();
-        // 4 + 4 16-byte reads for 64 FMAs; each accumulator takes its samples
-        // in increasing order
-#pragma unroll 2
-        for (int j4 = 0; j4 < kTimeTile / 4; ++j4) {
-          float4 v[4], q[4];
+        const int o = tile * kPos + i / 8, y = o / s.sp, x = o % s.sp, n = T * kTile + 4 * (i % 8) + 2 * half;
+        if (y >= s.py || x >= s.px) continue;
+        float *dst = out + ((size_t)y * s.px + x) * s.out_len + n;
+        if (n < s.out_len) dst[0] = first ? v.x : dst[0] + v.x;
+        if (n + 1 < s.out_len) dst[1] = first ? v.y : dst[1] + v.y;
+      }
+    }
+    __syncthreads();
+  };
+
+  int pb = 0, slot = 0;
+  bool first = true;
+  unsigned long long m0 = 0, m1 = 0;
+  int a = NA;  // this warp's tap
+  advance(b, c, c1);
+  if (b <= R) {
+    request_rows(b, c, 0);
+    my_taps(b, c, m0, m1);
+    a = pop(m0, m1);
+    request_slab(b, c, a, 0);
+    copies_commit();
+  }
+  while (b <= R) {
+    const int k0 = c * kChunk;
+    float *P = Pb + 2 * pb * p_size;
+    copies_wait<0>();
+    __syncthreads();
+    if (b > 0) {
+      float4 *p0 = reinterpret_cast<float4 *>(P);
+      const float4 *p1 = reinterpret_cast<const float4 *>(P + p_size);
+      for (int i = tid; i < p_size / 4; i += kThreads) {
+        const float4 u = p0[i], v = p1[i];
+        p0[i] = make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
+      }
+      __syncthreads();
+    }
+    // the next chunk and this warp's taps of it
+    int bn = b, cn = c, c1n = c1, chain = 0;
+    advance(bn, cn, c1n);
+    unsigned long long n0 = 0, n1 = 0;
+    if (bn <= R) my_taps(bn, cn, n0, n1);
+    bool ahead = false;  // the next chunk's rows are requested
+    for (int step = 0; a < NA; ++step) {
+      // request the tap after this one, here or in the next chunk
+      __syncwarp();  // the other slot's tap is done
+      int an = pop(m0, m1);
+      const bool last = an >= NA;
+      if (last) {
+        an = bn <= R ? pop(n0, n1) : NA;
+        request_slab(bn, cn, an, slot ^ 1);
+      } else {
+        request_slab(b, c, an, slot ^ 1);
+      }
+      copies_commit();
+      if (step == 0) {
+        if (bn <= R) request_rows(bn, cn, pb ^ 1);
+        copies_commit();
+        ahead = true;
+      }
+      // F of this tap
 #pragma unroll
-          for (int i = 0; i < 4; ++i) v[i] = Ss[pg + 16 * i][j4];
+      for (int kq = 0; kq < kChunk / 4; ++kq) fold_tap<kPos>(P, pm, a, F + lane, kq);
+      // this tap's slab rows are older than the last two copies (steps 0 and 1: the
+      // next tap's and the next chunk's) or than the last one
+      if (step < 2) copies_wait<2>();
+      else copies_wait<1>();
+      __syncwarp();
+      const uint2 t = tab[b * (NA + 1) + a];
+      const int ka = max(k_lo(t) - k0, 0) & ~3, kb = min(k_hi(t) - k0, kChunk);
+      multiply<kPos>(F + 8 * pg, S + slot * kChunk * kTile + 4 * ng, ka, kb, a1);
+      if (++chain == kFlush || last) {
+        chain = 0;
 #pragma unroll
-          for (int d = 0; d < 4; ++d) q[d] = Qs[4 * dg + d][j4];
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            a2[i][j] = add2(a2[i][j], a1[i][j]);
+            a1[i][j] = 0;
+          }
+      }
+      slot ^= 1;
+      a = an;
+      if (last) break;
+    }
+    if (!ahead) {  // no tap of this warp here: it still stages its share of the next rows
+      if (bn <= R) request_rows(bn, cn, pb ^ 1);
+      a = bn <= R ? pop(n0, n1) : NA;
+      request_slab(bn, cn, a, slot);
+      copies_commit();
+    }
+    if (bn != b) {
+      flush(first);
+      first = false;
+    }
+    b = bn;
+    c = cn;
+    c1 = c1n;
+    m0 = n0;
+    m1 = n1;
+    pb ^= 1;
+  }
+  if (first) flush(true);  // no slab row meets the tile: zeros
+}
+
+// ---------------------------------------------------------------- k_corr_block
+constexpr int kBlockPos = 128;  // positions per block, one thread each for the folding
+constexpr int kBlockStrip = 400;  // staged positions a block takes on run-on tiles
+
+// Shared memory: P [strip][kChunk], F [2][kChunk][kBlockPos], slab rows
+// [2][kChunk][kTile], second-level sums [16][threads] pairs, a row offset's taps, per
+// staged position its row and column.
+size_t block_smem(int strip, int R) {
+  return sizeof(float) * ((size_t)strip * kChunk + 2 * kChunk * (kBlockPos + kTile)) +
+         sizeof(uint64_t) * 16 * kBlockPos + sizeof(uint2) * (R + 2) + sizeof(int2) * strip;
+}
+
+// kVec: as above.
+template <bool kVec>
+__global__ void __launch_bounds__(kBlockPos, 4)
+    k_corr_block(const CorrShape s, const float *__restrict__ in, float *__restrict__ out) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int R = s.R, NA = R + 1, wp = s.px + R;
+  float *P = reinterpret_cast<float *>(smem);
+  float *F = P + (size_t)s.strip * kChunk;
+  float *S = F + 2 * kChunk * kBlockPos;
+  uint64_t *sum2 = reinterpret_cast<uint64_t *>(S + 2 * kChunk * kTile) + threadIdx.x;  // this thread's, kBlockPos apart
+  uint2 *tap = reinterpret_cast<uint2 *>(S + 2 * kChunk * kTile + 32 * kBlockPos);      // [R + 2]
+  int2 *where = reinterpret_cast<int2 *>(tap + NA + 1);
+  const int tid = threadIdx.x, T = blockIdx.y, tile = blockIdx.x;
+  const int y0 = tile * kBlockPos / s.sp, x0 = tile * kBlockPos % s.sp;
+  const int y1 = min((tile * kBlockPos + kBlockPos - 1) / s.sp, s.py - 1);  // rows of the tile
+  stage_where<kBlockPos>(s, y0, x0, where);
+  // staged index of the position this thread folds
+  const int pm = ((tile * kBlockPos + tid) / s.sp - y0) * wp + ((tile * kBlockPos + tid) % s.sp - x0) + R;
+  const int ng = tid & 7, pg = tid >> 3;  // outputs 4 ng .. +3 of the tile, positions 8 pg .. +7
+  const int n = T * kTile + 4 * ng;
+  uint64_t a1[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      a1[i][j] = 0;
+      sum2[(4 * i + j) * kBlockPos] = 0;
+    }
+  // add a row offset's sums to the output
+  auto flush = [&](bool first) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float2 v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        v[j] = unpack2(sum2[(4 * i + j) * kBlockPos]);
+        sum2[(4 * i + j) * kBlockPos] = 0;
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int o = tile * kBlockPos + 8 * pg + 2 * i + h, y = o / s.sp, x = o % s.sp;
+        if (y >= s.py || x >= s.px) continue;
+        float *dst = out + ((size_t)y * s.px + x) * s.out_len + n;
+        float w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = h ? v[j].y : v[j].x;
+        if (s.out_len % 4 == 0) {
+          if (n >= s.out_len) continue;
+          float4 u = first ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4 *>(dst);
+          *reinterpret_cast<float4 *>(dst) =
+              first ? make_float4(w[0], w[1], w[2], w[3]) : make_float4(u.x + w[0], u.y + w[1], u.z + w[2], u.w + w[3]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (n + j < s.out_len) dst[j] = first ? w[j] : dst[j] + w[j];
+        }
+      }
+    }
+  };
+  bool first = true;
+  for (int b = 0; b <= R; ++b) {
+    if (y0 + b >= s.py && y1 - b < 0) continue;  // neither row offset meets the grid
+    __syncthreads();
+    for (int a = tid; a <= NA; a += kBlockPos) tap[a] = s.taps[((size_t)T * NA + b) * (NA + 1) + a];
+    __syncthreads();
+    const uint2 all = tap[NA];
+    if (!(all.x >> 16)) continue;
+    for (int c = k_lo(all) / kChunk; c * kChunk < k_hi(all); ++c) {
+      const int k0 = c * kChunk;
+      // the chunk's taps, one bit each (the same in every warp)
+      unsigned long long m0 = 0, m1 = 0;
+      auto word = [&](int i) {
+        const int a = 32 * i + (tid & 31);
+        const uint2 t = a < NA ? tap[a] : make_uint2(0, 0);
+        return (unsigned long long)__ballot_sync(0xffffffffu,
+                                                 k_lo(t) < k0 + kChunk && k_hi(t) > k0 && (t.x >> 16));
+      };
+      m0 = word(0);
+      if (NA > 32) m0 |= word(1) << 32;
+      if (NA > 64) m1 = word(2);
+      if (NA > 96) m1 |= word(3) << 32;
+      auto request = [&](int buf) {  // the next tap's slab rows; returns it (NA: none is left)
+        int a = NA;
+        if (m0) {
+          a = __ffsll((long long)m0) - 1;
+          m0 &= m0 - 1;
+        } else if (m1) {
+          a = 63 + __ffsll((long long)m1);
+          m1 &= m1 - 1;
+        }
+        if (a < NA) {
+          const float *src = s.rows + ((size_t)tap[a].y + (c - k_lo(tap[a]) / kChunk)) * (kChunk * kTile);
+          static_assert(kChunk * kTile == 4 * kBlockPos, "one 16-byte copy per thread");
+          copy16_async(S + buf * kChunk * kTile + 4 * tid, src + 4 * tid, true);
+        }
+        copies_commit();
+        return a;
+      };
+      __syncthreads();  // the previous chunk's operands are read
+      int buf = 0, chain = 0, a = request(0);
+      for (int i = tid; i < s.strip * (kChunk / 4); i += kBlockPos) {
+        const int r = i / (kChunk / 4), kq = i % (kChunk / 4), k = k0 + 4 * kq;
+        const int2 w = where[r];
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int side = 0; side < (b ? 2 : 1); ++side) {
+          const int y = side ? w.x - b : w.x + b;
+          if (w.y < 0 || y < 0 || y >= s.py) continue;
+          const float *src = in + ((size_t)y * s.px + w.y) * s.len + k;
+          float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (kVec) {
+            if (k < s.len) u = *reinterpret_cast<const float4 *>(src);
+          } else {
+            if (k < s.len) u.x = src[0];
+            if (k + 1 < s.len) u.y = src[1];
+            if (k + 2 < s.len) u.z = src[2];
+            if (k + 3 < s.len) u.w = src[3];
+          }
+          v = make_float4(v.x + u.x, v.y + u.y, v.z + u.z, v.w + u.w);
+        }
+        *reinterpret_cast<float4 *>(P + p_at(r, kq)) = v;
+      }
+      __syncthreads();
+      auto fold = [&](int a, int buf) {
+#pragma unroll
+        for (int kq = 0; kq < kChunk / 4; ++kq) fold_tap<kBlockPos>(P, pm, a, F + buf * kChunk * kBlockPos + tid, kq);
+      };
+      if (a < NA) fold(a, 0);
+      while (a < NA) {
+        copies_wait<0>();
+        __syncthreads();  // this tap's operands are in place, the other buffer is read
+        const int next = request(buf ^ 1);
+        if (next < NA) fold(next, buf ^ 1);
+        multiply<kBlockPos>(F + buf * kChunk * kBlockPos + 8 * pg, S + buf * kChunk * kTile + 4 * ng,
+                            max(k_lo(tap[a]) - k0, 0) & ~3, min(k_hi(tap[a]) - k0, kChunk), a1);
+        if (++chain == kFlush || next >= NA) {
+          chain = 0;
 #pragma unroll
           for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int d = 0; d < 4; ++d) {
-              tap_acc[i][d] = fmaf(v[i].x, q[d].x, tap_acc[i][d]);
-              tap_acc[i][d] = fmaf(v[i].y, q[d].y, tap_acc[i][d]);
-              tap_acc[i][d] = fmaf(v[i].z, q[d].z, tap_acc[i][d]);
-              tap_acc[i][d] = fmaf(v[i].w, q[d].w, tap_acc[i][d]);
+            for (int j = 0; j < 4; ++j) {
+              sum2[(4 * i + j) * kBlockPos] = add2(sum2[(4 * i + j) * kBlockPos], a1[i][j]);
+              a1[i][j] = 0;
             }
         }
-        __syncthreads();
+        a = next;
+        buf ^= 1;
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int d = 0; d < 4; ++d) row_acc[i][d] += tap_acc[i][d];
     }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int d = 0; d < 4; ++d) acc[i][d] += row_acc[i][d];
+    flush(first);
+    first = false;
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int x = x0 + pg + 16 * i;
-    if (x >= px) continue;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-      const int k = K * kDepthTile + 4 * dg + d;
-      if (k < nz) H[((size_t)y * px + x) * nz + k] = acc[i][d];
-    }
-  }
+  if (first) flush(true);  // no slab row meets the tile: zeros
+}
+
+oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaStream_t st) {
+  const oam_grid &g = m->grid;
+  const DirectRows &L = fwd ? m->rows_fwd : m->rows_adj;
+  CorrShape s{};
+  s.px = g.px;
+  s.py = g.py;
+  s.R = m->R;
+  s.len = fwd ? g.nz : g.nt;
+  s.out_len = fwd ? g.nt : g.nz;
+  s.taps = L.d_taps;
+  s.rows = L.d_rows;
+  // The kernel that finishes first, from the blocks with work on the fullest SM, in
+  // units of one 128-position block alone on an SM: alone a block is bound by its chain
+  // of taps (the eight warps' is 0.3 as long), together they share the SM's pipes (0.47
+  // and 0.15 per block: 48x48x64 31x31 taps 1117 against 319 us, 64x64x128 61x61 taps
+  // 6.5 against 3.5 ms, 96x96x128 8.0 against 7.1, 128x128x64 11x11 taps 268 against
+  // 371 us, 200x200x300 53 against 71 ms).
+  const long long busy = fwd ? (m->n_hi - m->n_lo + kTile - 1) / kTile : L.tiles;
+  const int sms = std::max(1, m->sm_count);
+  auto per_sm = [&](int positions) {
+    const long long blocks = ((long long)g.px * g.py + positions - 1) / positions * busy;
+    return (double)((blocks + sms - 1) / sms);
+  };
+  const bool block = std::max(1.0, 0.47 * per_sm(kBlockPos)) <= std::max(0.3, 0.15 * per_sm(kPos));
+  // Tiles run on over scan rows (no idle positions) unless the padding between
+  // many short rows makes the strip too long; then every tile stays in its row.
+  const int tile = block ? kBlockPos : kPos;
+  const int wrap = tile + ((s.px + tile - 2) / s.px + 2) * s.R;
+  const bool run_on = wrap <= (block ? kBlockStrip : kMaxStrip);
+  s.sp = run_on ? s.px : (s.px + tile - 1) / tile * tile;
+  s.strip = run_on ? wrap : tile + 2 * s.R;
+  const long long tiles = ((long long)s.py * s.sp + tile - 1) / tile;
+  const size_t sm = block ? block_smem(s.strip, s.R) : warps_smem(s.strip, s.R);
+  const bool vec = s.len % 4 == 0;
+  auto fn = block ? (vec ? k_corr_block<true> : k_corr_block<false>) : (vec ? k_corr_warps<true> : k_corr_warps<false>);
+  OAM_CUDA_TRY(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  ProfScope prof(m, st, fwd);
+  fn<<<dim3((unsigned)tiles, L.tiles), block ? kBlockPos : kThreads, sm, st>>>(s, in, out);  // tile neighbours share slab rows
+  OAM_LAUNCHED();
+  return OAM_OK;
 }
 
 }  // namespace
 
 oam_status oam::forward_fp32(const oam_model *m, const float *H, float *s, cudaStream_t st) {
-  const oam_grid &g = m->grid;
-  dim3 grid((g.px + kPos - 1) / kPos, g.py, m->n_ttiles);
-  ProfScope prof(m, st, true);
-  k_fwd_fp32<<<grid, 256, 0, st>>>(H, s, g.px, g.py, g.nz, g.nt, m->R, m->d_tap_orbit, m->n_ttiles, m->d_fwd_krange,
-                                   m->d_fwd_off, m->d_fwd);
-  OAM_LAUNCHED();
-  return OAM_OK;
+  return run(m, true, H, s, st);
 }
 
 oam_status oam::adjoint_fp32(const oam_model *m, const float *s, float *H, cudaStream_t st) {
-  const oam_grid &g = m->grid;
-  dim3 grid((g.px + kPos - 1) / kPos, g.py, m->n_ktiles);
-  ProfScope prof(m, st, false);
-  k_adj_fp32<<<grid, kAdjThreads, 0, st>>>(s, H, g.px, g.py, g.nz, g.nt, m->R, m->d_tap_orbit, m->n_ktiles,
-                                           m->d_adj_nrange, m->d_adj_off, m->d_adj);
-  OAM_LAUNCHED();
-  return OAM_OK;
+  return run(m, false, s, H, st);
 }

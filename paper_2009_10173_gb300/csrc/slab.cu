@@ -402,37 +402,24 @@ __global__ void k_slab_values(Geo g, const PatchDW *__restrict__ pdw, int M, con
   }
 }
 
-// FP32 forward layout: rows k in [klo, khi) of kTimeTile samples of tile T.
-__global__ void k_pack_fwd(const float *band, const int *band_lo, const int *band_hi, int band_w, int nz,
-                           int n_ttiles, const int *krange, const long long *off, float *out) {
-  const int ot = blockIdx.x;
-  const int o = ot / n_ttiles, T = ot % n_ttiles;
-  const int klo = krange[2 * ot], khi = krange[2 * ot + 1];
-  const long long base = off[ot];
-  const int total = (khi - klo) * kTimeTile;
-  for (int i = threadIdx.x; i < total; i += blockDim.x) {
-    const int k = klo + i / kTimeTile, n = T * kTimeTile + i % kTimeTile;
-    const int lo = band_lo[o * nz + k], hi = band_hi[o * nz + k];
-    out[base + i] = (n >= lo && n < hi) ? band[((size_t)o * nz + k) * band_w + (n - lo)] : 0.0f;
-  }
-}
-
-// FP32 adjoint layout: kDepthTile rows (depths) of nlen samples from nlo.
-__global__ void k_pack_adj(const float *band, const int *band_lo, const int *band_hi, int band_w, int nz,
-                           int n_ktiles, const int *nrange, const long long *off, float *out) {
-  const int ok = blockIdx.x;
-  const int o = ok / n_ktiles, K = ok % n_ktiles;
-  const int nlo = nrange[2 * ok], nlen = nrange[2 * ok + 1];
-  const long long base = off[ok];
-  const int total = kDepthTile * nlen;
-  for (int i = threadIdx.x; i < total; i += blockDim.x) {
-    const int k = K * kDepthTile + i / nlen, n = nlo + i % nlen;
+// FP32 operators' slab rows (DirectRows) of one direction: row e of (orbit o, tile T)
+// holds, for input element e (forward: depth, adjoint: sample), the tile's outputs.
+__global__ void k_pack_rows(const float *band, const int *band_lo, const int *band_hi, int band_w, int nz, int dir,
+                            int tiles, const uint2 *range, float *out) {
+  const int ot = blockIdx.x, o = ot / tiles, T = ot % tiles;
+  const int lo = (int)(range[ot].x & 0xffffu), hi = lo + (int)(range[ot].x >> 16);
+  if (lo >= hi) return;
+  const int e0 = lo / kRowChunk * kRowChunk, e1 = (hi + kRowChunk - 1) / kRowChunk * kRowChunk;
+  out += (size_t)range[ot].y * kRowChunk * kOutTile;
+  for (int i = threadIdx.x; i < (e1 - e0) * kOutTile; i += blockDim.x) {
+    const int e = e0 + i / kOutTile, q = T * kOutTile + i % kOutTile;
+    const int k = dir == 0 ? e : q, n = dir == 0 ? q : e;
     float v = 0.0f;
     if (k < nz) {
-      const int lo = band_lo[o * nz + k], hi = band_hi[o * nz + k];
-      if (n >= lo && n < hi) v = band[((size_t)o * nz + k) * band_w + (n - lo)];
+      const int bl = band_lo[o * nz + k], bh = band_hi[o * nz + k];
+      if (n >= bl && n < bh) v = band[((size_t)o * nz + k) * band_w + (n - bl)];
     }
-    out[base + i] = v;
+    out[i] = v;
   }
 }
 
@@ -517,74 +504,86 @@ oam_status oam::plan_bands(oam_model *m, const std::vector<double2> &h_range, in
   return OAM_OK;
 }
 
-// FP32 forward layout: per (orbit, 64-sample time tile) the depths [klo, khi)
-// whose band meets the tile, rows of kTimeTile samples.  Returns the floats.
-long long oam::fwd_layout(const oam_model *m, std::vector<int> *kr, std::vector<long long> *off) {
-  const int nz = m->grid.nz, O = m->n_orb, NT = (m->grid.nt + kTimeTile - 1) / kTimeTile;
-  kr->assign((size_t)O * NT * 2, 0);
-  off->assign((size_t)O * NT, 0);
-  long long total = 0;
-  for (int o = 0; o < O; ++o)
-    for (int T = 0; T < NT; ++T) {
-      int klo = nz, khi = 0;
-      for (int k = 0; k < nz; ++k) {
-        int lo = m->h_band_lo[(size_t)o * nz + k], hi = m->h_band_hi[(size_t)o * nz + k];
-        if (hi > lo && lo < (T + 1) * kTimeTile && hi > T * kTimeTile) {
-          klo = std::min(klo, k);
-          khi = std::max(khi, k + 1);
+// FP32 operators' slab rows of one direction (0 forward, 1 adjoint): per (orbit, output
+// tile) the input range and first chunk, as DirectRows packs them.  Returns the chunks.
+static long long plan_rows(const oam_model *m, int dir, int *tiles, std::vector<uint2> *range) {
+  const int nz = m->grid.nz, O = m->n_orb, NT = ((dir == 0 ? m->grid.nt : nz) + kOutTile - 1) / kOutTile;
+  *tiles = NT;
+  range->assign((size_t)O * NT, make_uint2(0, 0));
+  long long chunks = 0;
+  std::vector<int> lo(NT), hi(NT);
+  for (int o = 0; o < O; ++o) {
+    lo.assign(NT, 1 << 30);
+    hi.assign(NT, 0);
+    for (int k = 0; k < nz; ++k) {
+      const int bl = m->h_band_lo[(size_t)o * nz + k], bh = m->h_band_hi[(size_t)o * nz + k];
+      if (bh <= bl) continue;
+      if (dir == 0) {
+        for (int T = bl / kOutTile; T <= (bh - 1) / kOutTile; ++T) {
+          lo[T] = std::min(lo[T], k);
+          hi[T] = std::max(hi[T], k + 1);
         }
+      } else {
+        lo[k / kOutTile] = std::min(lo[k / kOutTile], bl);
+        hi[k / kOutTile] = std::max(hi[k / kOutTile], bh);
       }
-      if (khi <= klo) klo = khi = 0;
-      size_t i = (size_t)o * NT + T;
-      (*kr)[2 * i] = klo;
-      (*kr)[2 * i + 1] = khi;
-      (*off)[i] = total;
-      total += (long long)(khi - klo) * kTimeTile;
     }
-  return total;
+    for (int T = 0; T < NT; ++T) {
+      if (hi[T] <= lo[T]) continue;
+      (*range)[(size_t)o * NT + T] = make_uint2((unsigned)lo[T] | (unsigned)(hi[T] - lo[T]) << 16, (unsigned)chunks);
+      chunks += (hi[T] + kRowChunk - 1) / kRowChunk - lo[T] / kRowChunk;
+    }
+  }
+  return chunks;
 }
 
-// FP32 adjoint layout: per (orbit, 16-depth tile) the union sample range
-// [nlo, nlo + nlen), 4-aligned, rows of nlen samples.  Returns the floats.
-long long oam::adj_layout(const oam_model *m, std::vector<int> *nr, std::vector<long long> *off) {
-  const int nz = m->grid.nz, nt = m->grid.nt, O = m->n_orb, NK = (nz + kDepthTile - 1) / kDepthTile;
-  nr->assign((size_t)O * NK * 2, 0);
-  off->assign((size_t)O * NK, 0);
-  long long total = 0;
-  for (int o = 0; o < O; ++o)
-    for (int K = 0; K < NK; ++K) {
-      int nlo = nt, nhi = 0;
-      for (int k = K * kDepthTile; k < std::min(nz, (K + 1) * kDepthTile); ++k) {
-        int lo = m->h_band_lo[(size_t)o * nz + k], hi = m->h_band_hi[(size_t)o * nz + k];
-        if (hi > lo) {
-          nlo = std::min(nlo, lo);
-          nhi = std::max(nhi, hi);
-        }
+// Build one direction's slab rows.
+static oam_status build_rows(oam_model *m, int dir, DirectRows *L, const int *d_band_hi, cudaStream_t st) {
+  std::vector<uint2> range, taps;
+  const long long chunks = plan_rows(m, dir, &L->tiles, &range);
+  if (chunks > 0xffffffffLL) return OAM_ERR_UNSUPPORTED;
+  const int R = m->R, W = m->W, NA = R + 1;
+  taps.assign((size_t)L->tiles * NA * (NA + 1), make_uint2(0, 0));
+  for (int T = 0; T < L->tiles; ++T)
+    for (int b = 0; b <= R; ++b) {
+      uint2 *row = &taps[((size_t)T * NA + b) * (NA + 1)];
+      unsigned lo = 0xffffffffu, hi = 0;
+      for (int a = 0; a <= R; ++a) {
+        row[a] = range[(size_t)m->h_tap_orbit[(b + R) * W + (a + R)] * L->tiles + T];
+        if (!(row[a].x >> 16)) continue;
+        lo = std::min(lo, row[a].x & 0xffffu);
+        hi = std::max(hi, (row[a].x & 0xffffu) + (row[a].x >> 16));
       }
-      if (nhi <= nlo) {
-        nlo = 0;
-        nhi = 0;
-      }
-      nlo &= ~3;
-      nhi = std::min((nhi + 3) & ~3, nt);
-      size_t i = (size_t)o * NK + K;
-      (*nr)[2 * i] = nlo;
-      (*nr)[2 * i + 1] = nhi - nlo;
-      (*off)[i] = total;
-      total += (long long)kDepthTile * (nhi - nlo);
+      if (hi > lo) row[NA].x = lo | (hi - lo) << 16;
     }
-  return total;
+  oam_status rc;
+  uint2 *d_range = nullptr;
+  if ((rc = dev_alloc(m, &L->d_taps, taps.size())) ||
+      (rc = dev_alloc(m, &L->d_rows, (size_t)chunks * kRowChunk * kOutTile)))
+    return rc;
+  OAM_CUDA_TRY(cudaMallocAsync((void **)&d_range, sizeof(uint2) * range.size(), st));
+  OAM_CUDA_TRY(cudaMemcpyAsync(d_range, range.data(), sizeof(uint2) * range.size(), cudaMemcpyHostToDevice, st));
+  OAM_CUDA_TRY(cudaMemcpyAsync(L->d_taps, taps.data(), sizeof(uint2) * taps.size(), cudaMemcpyHostToDevice, st));
+  k_pack_rows<<<m->n_orb * L->tiles, 256, 0, st>>>(m->d_band, m->d_band_lo, d_band_hi, m->band_w, m->grid.nz, dir,
+                                                   L->tiles, d_range, L->d_rows);
+  OAM_LAUNCHED();
+  OAM_CUDA_TRY(cudaFreeAsync(d_range, st));
+  OAM_CUDA_TRY(cudaStreamSynchronize(st));  // host tables above go out of scope
+  return OAM_OK;
 }
 
 // Device bytes build_slab allocates for a model whose bands are planned.
 size_t oam::slab_plan_bytes(const oam_model *m) {
   const size_t O = m->n_orb, nz = m->grid.nz;
-  std::vector<int> iv;
-  std::vector<long long> lv;
-  const size_t NT = (m->grid.nt + kTimeTile - 1) / kTimeTile, NK = (nz + kDepthTile - 1) / kDepthTile;
   size_t b = alloc_bytes<int>((size_t)m->W * m->W) + alloc_bytes<int>(O * nz) + alloc_bytes<float>(O * nz * m->band_w);
-  b += alloc_bytes<int>(O * NT * 2) + alloc_bytes<long long>(O * NT) + alloc_bytes<float>(fwd_layout(m, &iv, &lv));
-  b += alloc_bytes<int>(O * NK * 2) + alloc_bytes<long long>(O * NK) + alloc_bytes<float>(adj_layout(m, &iv, &lv));
+  if (m->precision != OAM_PREC_FP32) return b;
+  for (int dir = 0; dir < 2; ++dir) {
+    std::vector<uint2> range;
+    int tiles = 0;
+    const long long chunks = plan_rows(m, dir, &tiles, &range);
+    b += alloc_bytes<uint2>((size_t)tiles * (m->R + 1) * (m->R + 2)) +
+         alloc_bytes<float>((size_t)chunks * kRowChunk * kOutTile);
+  }
   return b;
 }
 
@@ -672,40 +671,9 @@ oam_status oam::build_slab(oam_model *m, cudaStream_t st) {
   }
   OAM_LAUNCHED();
 
-  // FP32 forward layout
-  m->n_ttiles = (nt + kTimeTile - 1) / kTimeTile;
-  {
-    const int NT = m->n_ttiles;
-    std::vector<int> kr;
-    std::vector<long long> off;
-    const long long total = fwd_layout(m, &kr, &off);
-    if ((rc = dev_alloc(m, &m->d_fwd_krange, kr.size()))) return rc;
-    if ((rc = dev_alloc(m, &m->d_fwd_off, off.size()))) return rc;
-    if ((rc = dev_alloc(m, &m->d_fwd, (size_t)total))) return rc;
-    OAM_CUDA_TRY(cudaMemcpyAsync(m->d_fwd_krange, kr.data(), sizeof(int) * kr.size(), cudaMemcpyHostToDevice, st));
-    OAM_CUDA_TRY(cudaMemcpyAsync(m->d_fwd_off, off.data(), sizeof(long long) * off.size(), cudaMemcpyHostToDevice, st));
-    k_pack_fwd<<<O * NT, 256, 0, st>>>(m->d_band, m->d_band_lo, d_band_hi, m->band_w, nz, NT, m->d_fwd_krange,
-                                       m->d_fwd_off, m->d_fwd);
-    OAM_LAUNCHED();
-    OAM_CUDA_TRY(cudaStreamSynchronize(st));  // host tables above go out of scope
-  }
-  // FP32 adjoint layout
-  m->n_ktiles = (nz + kDepthTile - 1) / kDepthTile;
-  {
-    const int NK = m->n_ktiles;
-    std::vector<int> nr;
-    std::vector<long long> off;
-    const long long total = adj_layout(m, &nr, &off);
-    if ((rc = dev_alloc(m, &m->d_adj_nrange, nr.size()))) return rc;
-    if ((rc = dev_alloc(m, &m->d_adj_off, off.size()))) return rc;
-    if ((rc = dev_alloc(m, &m->d_adj, (size_t)total))) return rc;
-    OAM_CUDA_TRY(cudaMemcpyAsync(m->d_adj_nrange, nr.data(), sizeof(int) * nr.size(), cudaMemcpyHostToDevice, st));
-    OAM_CUDA_TRY(cudaMemcpyAsync(m->d_adj_off, off.data(), sizeof(long long) * off.size(), cudaMemcpyHostToDevice, st));
-    k_pack_adj<<<O * NK, 256, 0, st>>>(m->d_band, m->d_band_lo, d_band_hi, m->band_w, nz, NK, m->d_adj_nrange,
-                                       m->d_adj_off, m->d_adj);
-    OAM_LAUNCHED();
-    OAM_CUDA_TRY(cudaStreamSynchronize(st));
-  }
+  if (m->precision == OAM_PREC_FP32 && ((rc = build_rows(m, 0, &m->rows_fwd, d_band_hi, st)) ||
+                                        (rc = build_rows(m, 1, &m->rows_adj, d_band_hi, st))))
+    return rc;
   cudaFreeAsync(d_orb_b, st);
   cudaFreeAsync(d_orb_a, st);
   cudaFreeAsync(d_range, st);
