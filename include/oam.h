@@ -223,8 +223,8 @@ oam_status oam_bandpass_taps(double f_lo_hz, double f_hi_hz, double fs_hz, int32
 /* Make the model's forward operator F A and its adjoint A^T F (also inside
  * the solvers, batches and autotuning) for the even FIR taps[0..half_len]
  * (host memory, copied).  taps == NULL or half_len < 0 removes the filter.
- * The transform length is the smallest power of two NF >= nt + min(L, nt-1);
- * NF > 8192 is rejected (OAM_ERR_INVALID_ARG), as are non-finite taps.
+ * info.filter_size is the smallest power of two NF >= nt + min(L, nt-1) (the
+ * device's transform may be shorter, but not than that sum); NF > 8192 is rejected (OAM_ERR_INVALID_ARG), as are non-finite taps.
  * Allocates the filter's spectrum and one signal-sized staging buffer (owned
  * by the model, counted in device_bytes) on `stream` and synchronises it.
  * A batch that uses the model records its graph again on its next run. */

@@ -51,72 +51,82 @@ __device__ __forceinline__ void static_for(F f) {
   }
 }
 
+// The transforms below are written for any complex type with these operations; a type
+// of another file brings its own.
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 cneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 cadd_i(float2 a, float2 b) { return make_float2(a.x - b.y, a.y + b.x); }  // a + i b
+__device__ __forceinline__ float2 csub_i(float2 a, float2 b) { return make_float2(a.x + b.y, a.y - b.x); }  // a - i b
+__device__ __forceinline__ float2 cturn(float2 a) { return make_float2(a.y, -a.x); }                        // -i a
+__device__ __forceinline__ float2 cscale(float s, float2 a) { return make_float2(s * a.x, s * a.y); }
+__device__ __forceinline__ float2 caxpy(float s, float2 a, float2 b) {  // s a + b
+  return make_float2(fmaf(s, a.x, b.x), fmaf(s, a.y, b.y));
+}
+__device__ __forceinline__ float2 caxpy_i(float s, float2 a, float2 b) {  // b - i s a
+  return make_float2(fmaf(s, a.y, b.x), fmaf(-s, a.x, b.y));
+}
+__device__ __forceinline__ float2 croot(float2 a, float c, float s) {  // a (c - i s)
+  return make_float2(a.x * c + a.y * s, a.y * c - a.x * s);
+}
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
 // a W_N^K, W_N = exp(-2 pi i / N)
-template <int N, int K>
-__device__ __forceinline__ float2 mul_root(float2 a) {
+template <int N, int K, class T>
+__device__ __forceinline__ T mul_root(T a) {
   constexpr int k = K % N;
   if constexpr (k == 0) return a;
-  else if constexpr (4 * k == N) return make_float2(a.y, -a.x);
-  else if constexpr (2 * k == N) return make_float2(-a.x, -a.y);
-  else if constexpr (4 * k == 3 * N) return make_float2(-a.y, a.x);
-  else {
-    constexpr float c = (float)turn_cos(k, N), s = (float)turn_sin(k, N);
-    return make_float2(a.x * c + a.y * s, a.y * c - a.x * s);
-  }
+  else if constexpr (4 * k == N) return cturn(a);
+  else if constexpr (2 * k == N) return cneg(a);
+  else if constexpr (4 * k == 3 * N) return cneg(cturn(a));
+  else return croot(a, (float)turn_cos(k, N), (float)turn_sin(k, N));
 }
 
 // In-register forward transform of N points (N a product of 2, 3 and 5).
-template <int N>
-__device__ __forceinline__ void dft(float2 (&v)[N]) {
+template <int N, class T>
+__device__ __forceinline__ void dft(T (&v)[N]) {
   if constexpr (N == 1) {
   } else if constexpr (N == 2) {
-    const float2 a = v[0], b = v[1];
+    const T a = v[0], b = v[1];
     v[0] = cadd(a, b);
     v[1] = csub(a, b);
   } else if constexpr (N == 3) {
     constexpr float s = (float)turn_sin(1, 3);
-    const float2 t = cadd(v[1], v[2]), d = csub(v[1], v[2]);
-    const float2 m = make_float2(fmaf(-0.5f, t.x, v[0].x), fmaf(-0.5f, t.y, v[0].y));
+    const T t = cadd(v[1], v[2]), d = csub(v[1], v[2]), m = caxpy(-0.5f, t, v[0]);
     v[0] = cadd(v[0], t);
-    v[1] = make_float2(fmaf(s, d.y, m.x), fmaf(-s, d.x, m.y));
-    v[2] = make_float2(fmaf(-s, d.y, m.x), fmaf(s, d.x, m.y));
+    v[1] = caxpy_i(s, d, m);
+    v[2] = caxpy_i(-s, d, m);
   } else if constexpr (N == 4) {
-    const float2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]), c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
+    const T a = cadd(v[0], v[2]), b = csub(v[0], v[2]), c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
     v[0] = cadd(a, c);
     v[2] = csub(a, c);
-    v[1] = make_float2(b.x + d.y, b.y - d.x);
-    v[3] = make_float2(b.x - d.y, b.y + d.x);
+    v[1] = csub_i(b, d);
+    v[3] = cadd_i(b, d);
   } else if constexpr (N == 5) {
     constexpr float c1 = (float)turn_cos(1, 5), c2 = (float)turn_cos(2, 5);
     constexpr float s1 = (float)turn_sin(1, 5), s2 = (float)turn_sin(2, 5);
-    const float2 t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]), d1 = csub(v[1], v[4]), d2 = csub(v[2], v[3]);
-    const float2 m1 = make_float2(fmaf(c2, t2.x, fmaf(c1, t1.x, v[0].x)), fmaf(c2, t2.y, fmaf(c1, t1.y, v[0].y)));
-    const float2 m2 = make_float2(fmaf(c1, t2.x, fmaf(c2, t1.x, v[0].x)), fmaf(c1, t2.y, fmaf(c2, t1.y, v[0].y)));
-    const float2 n1 = make_float2(fmaf(s2, d2.x, s1 * d1.x), fmaf(s2, d2.y, s1 * d1.y));
-    const float2 n2 = make_float2(fmaf(-s1, d2.x, s2 * d1.x), fmaf(-s1, d2.y, s2 * d1.y));
+    const T t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]), d1 = csub(v[1], v[4]), d2 = csub(v[2], v[3]);
+    const T m1 = caxpy(c2, t2, caxpy(c1, t1, v[0])), m2 = caxpy(c1, t2, caxpy(c2, t1, v[0]));
+    const T n1 = caxpy(s2, d2, cscale(s1, d1)), n2 = caxpy(-s1, d2, cscale(s2, d1));
     v[0] = cadd(v[0], cadd(t1, t2));
-    v[1] = make_float2(m1.x + n1.y, m1.y - n1.x);
-    v[4] = make_float2(m1.x - n1.y, m1.y + n1.x);
-    v[2] = make_float2(m2.x + n2.y, m2.y - n2.x);
-    v[3] = make_float2(m2.x - n2.y, m2.y + n2.x);
+    v[1] = csub_i(m1, n1);
+    v[4] = cadd_i(m1, n1);
+    v[2] = csub_i(m2, n2);
+    v[3] = cadd_i(m2, n2);
   } else {
     constexpr int A = N % 4 == 0 ? 4 : N % 2 == 0 ? 2 : N % 3 == 0 ? 3 : 5, B = N / A;
     static_assert(A * B == N && (N % 2 == 0 || N % 3 == 0 || N % 5 == 0), "factors 2, 3 and 5 only");
-    float2 w[N];
+    T w[N];
     static_for<0, B>([&](auto j) {
-      float2 t[A];
+      T t[A];
       static_for<0, A>([&](auto i) { t[i()] = v[i() * B + j()]; });
       dft<A>(t);
       static_for<0, A>([&](auto i) { w[i() * B + j()] = mul_root<N, i() * j()>(t[i()]); });
     });
     static_for<0, A>([&](auto i) {
-      float2 t[B];
+      T t[B];
       static_for<0, B>([&](auto j) { t[j()] = w[i() * B + j()]; });
       dft<B>(t);
       static_for<0, B>([&](auto j) { v[i() + A * j()] = t[j()]; });

@@ -13,9 +13,11 @@
 // 0.5 MHz cut-off at 250 MS/s is about as long as the A-line and would widen
 // every band to all of it).
 //
-// On the device F is a circular convolution of length NF, a power of two with
-// NF >= nt + min(L, nt - 1), so no wrap reaches [0, nt).  Each pair of A-lines
-// is one complex line (real and imaginary parts), transformed by a radix-2
+// On the device F is a circular convolution of a length N >= nt + min(L, nt - 1),
+// so no wrap reaches [0, nt).  Each pair of A-lines is one complex line (real and
+// imaginary parts).  From 257 to 4096 points k_fir_mixed transforms it in three
+// mixed-radix passes; shorter and longer ones (k_fir_lines) have a power-of-two
+// length NF and are transformed by a radix-2
 // decimation-in-frequency FFT (natural order in, bit-reversed order out),
 // multiplied by the filter's spectrum (real because the taps are even,
 // pre-scaled by 1/NF, stored in bit-reversed order) and transformed back by a
@@ -34,6 +36,7 @@
 #include <vector>
 
 #include "fft_dev.cuh"
+#include "fft_mixed.cuh"
 #include "internal.cuh"
 
 using namespace oam;
@@ -42,10 +45,12 @@ namespace oam {
 
 struct FirLayout {
   int L = 0;                 // half length as set (taps with |m| >= nt never reach the output)
-  int NF = 0, lgNF = 0, KP = 0;  // transform size, its log2, complex line pairs per block
-  float *d_hb = nullptr;     // [NF] spectrum of the taps over NF, in bit-reversed order
+  int NF = 0, lgNF = 0;      // power-of-two size (info.filter_size), its log2
+  int N = 0;                 // transform size
+  float *d_hb = nullptr;     // [N] spectrum of the taps over N, in the order the forward transform leaves
+  float2 *d_tw = nullptr;    // k_fir_mixed: its passes' twiddles
   float *d_stage = nullptr;  // signal-sized staging buffer: F s ahead of the adjoint
-  size_t bytes = 0;          // device bytes of the two buffers
+  size_t bytes = 0;          // device bytes of the buffers
 };
 
 }  // namespace oam
@@ -377,6 +382,156 @@ __global__ void __launch_bounds__(kFirThreads, 2) k_fir_lines(const float *x, fl
   edge_pass<KP, false>(r0, a, NF, k0, nullptr, y, line0, n_lines, nt);
 }
 
+// The same operations for the transforms of fft_mixed.cuh.
+__device__ __forceinline__ Cx2 cadd(Cx2 a, Cx2 b) { return x_add(a, b); }
+__device__ __forceinline__ Cx2 csub(Cx2 a, Cx2 b) { return x_sub(a, b); }
+__device__ __forceinline__ uint64_t f2_neg(uint64_t a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ Cx2 cneg(Cx2 a) { return Cx2{f2_neg(a.re), f2_neg(a.im)}; }
+__device__ __forceinline__ Cx2 cadd_i(Cx2 a, Cx2 b) { return Cx2{f2_sub(a.re, b.im), f2_add(a.im, b.re)}; }
+__device__ __forceinline__ Cx2 csub_i(Cx2 a, Cx2 b) { return Cx2{f2_add(a.re, b.im), f2_sub(a.im, b.re)}; }
+__device__ __forceinline__ Cx2 cturn(Cx2 a) { return Cx2{a.im, f2_neg(a.re)}; }
+__device__ __forceinline__ Cx2 cscale(float s, Cx2 a) {
+  const uint64_t w = f2_splat(s);
+  return Cx2{f2_mul(w, a.re), f2_mul(w, a.im)};
+}
+__device__ __forceinline__ Cx2 caxpy(float s, Cx2 a, Cx2 b) {
+  const uint64_t w = f2_splat(s);
+  return Cx2{f2_fma(w, a.re, b.re), f2_fma(w, a.im, b.im)};
+}
+__device__ __forceinline__ Cx2 caxpy_i(float s, Cx2 a, Cx2 b) {
+  return Cx2{f2_fma(f2_splat(s), a.im, b.re), f2_fma(f2_splat(-s), a.re, b.im)};
+}
+__device__ __forceinline__ Cx2 croot(Cx2 a, float c, float s) { return x_mul(a, make_float2(c, -s)); }
+
+// Transform sizes of k_fir_mixed, smallest first: N = A B C.
+#define OAM_FIR_SIZES(X)                                                                                \
+  X(384, 6, 8, 8) X(512, 8, 8, 8) X(640, 10, 8, 8) X(768, 12, 8, 8) X(1024, 8, 16, 8) X(1280, 10, 16, 8) \
+  X(1536, 12, 16, 8) X(2048, 16, 16, 8) X(3072, 12, 16, 16) X(4096, 16, 16, 16)
+
+template <int A, int B, int C>
+constexpr int fir_threads() { return B * C > 64 ? 128 : 64; }
+
+// The convolution of the lines 4b .. 4b + 3 (block b), points in the layout of
+// slot<1>.  With i = m BC + q and q = l C + t, forward:
+//   pass 1, per q: DFT over m, times W_N^(q s), in place of m;
+//   pass 2, per (s, t): DFT over l, times W_BC^(t u), in place of l;
+//   middle, per (s, u): DFT over t: frequency s + A (u + B w) at point (s B + u) C + w,
+//           the product with the taps' spectrum hb there, and back;
+// then passes 2 and 1 in reverse.  The inverse transforms run forward ones on values
+// with real and imaginary parts exchanged, after multiplying with the same twiddles.
+// tw: W_N^(q s) [A - 1][BC], then W_BC^(t u) [B - 1][C].
+//
+// What bounds it: latency between the passes' barriers at 16 warps per SM (registers),
+// with shared memory 68% and the issue slots 49% busy; the signals' bytes alone take half
+// the time.  One line pair per block and 64 or 128 threads of at most 128 registers keep
+// four blocks or more per SM in different passes.  Radix 12 and 16 passes with tabulated
+// twiddles, and a size near the least one (1536 for 1024 samples and 511 taps a side, not
+// 2048), take half the operations of the radix-2 stages that served these sizes:
+// 40000 lines of 1024 samples 196 -> 104 us (3.2 TB/s), error 3.2e-7 -> 1.2e-7.
+template <int A, int B, int C>
+__global__ void __launch_bounds__(fir_threads<A, B, C>(), 512 / fir_threads<A, B, C>())
+    k_fir_mixed(const float *x, float *y, long long n_lines, int nt, const float *__restrict__ hb,
+                const float2 *__restrict__ tw) {
+  constexpr int N = A * B * C, M = B * C, T = fir_threads<A, B, C>();
+  static_assert(C % 8 == 0 && N % 8 == 0, "whole 8-point groups");
+  constexpr int dM = M + M / 8, dC = C + C / 8;  // slots between points M and C apart
+  extern __shared__ ulonglong2 a[];              // [N + N / 8]
+  const float2 *tw2 = tw + (A - 1) * M;
+  const long long line0 = 4LL * blockIdx.x, base = line0 * nt;
+  const bool ok1 = line0 + 1 < n_lines, ok2 = line0 + 2 < n_lines, ok3 = line0 + 3 < n_lines;
+  for (int q = threadIdx.x; q < M; q += T) {
+    Cx2 v[A];
+    const float *p = x + base + q;
+#pragma unroll
+    for (int m = 0; m < A; ++m) {
+      const bool in = m * M + q < nt;
+      const float e0 = in ? p[m * M] : 0.0f, e1 = in && ok1 ? p[m * M + nt] : 0.0f;
+      const float e2 = in && ok2 ? p[m * M + 2LL * nt] : 0.0f, e3 = in && ok3 ? p[m * M + 3LL * nt] : 0.0f;
+      v[m] = Cx2{f2_pack(e0, e2), f2_pack(e1, e3)};
+    }
+    mixfft::dft<A>(v);
+    ulonglong2 *o = a + slot<1>(q, 0);
+    o[0] = make_ulonglong2(v[0].re, v[0].im);
+#pragma unroll
+    for (int s = 1; s < A; ++s) {
+      const Cx2 w = x_mul(v[s], __ldg(tw + (s - 1) * M + q));
+      o[s * dM] = make_ulonglong2(w.re, w.im);
+    }
+  }
+  __syncthreads();
+  for (int id = threadIdx.x; id < A * C; id += T) {
+    const int s = id / C, t = id % C;
+    ulonglong2 *o = a + slot<1>(s * M + t, 0);
+    Cx2 v[B];
+#pragma unroll
+    for (int l = 0; l < B; ++l) v[l] = Cx2{o[l * dC].x, o[l * dC].y};
+    mixfft::dft<B>(v);
+    o[0] = make_ulonglong2(v[0].re, v[0].im);
+#pragma unroll
+    for (int u = 1; u < B; ++u) {
+      const Cx2 w = x_mul(v[u], __ldg(tw2 + (u - 1) * C + t));
+      o[u * dC] = make_ulonglong2(w.re, w.im);
+    }
+  }
+  __syncthreads();
+  for (int g = T - 1 - threadIdx.x; g < A * B; g += T) {  // from the other end: pass 2 leaves the last warps idle
+    ulonglong2 *o = a + g * dC;
+    const float4 *h4 = reinterpret_cast<const float4 *>(hb + g * C);
+    Cx2 v[C];
+#pragma unroll
+    for (int w = 0; w < C; ++w) v[w] = Cx2{o[w + w / 8].x, o[w + w / 8].y};
+    mixfft::dft<C>(v);
+#pragma unroll
+    for (int w = 0; w < C; w += 4) {
+      const float4 h = __ldg(h4 + w / 4);
+      const float hs[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint64_t hh = f2_splat(hs[i]);
+        v[w + i] = Cx2{f2_mul(v[w + i].im, hh), f2_mul(v[w + i].re, hh)};  // exchanged from here on
+      }
+    }
+    mixfft::dft<C>(v);
+#pragma unroll
+    for (int w = 0; w < C; ++w) o[w + w / 8] = make_ulonglong2(v[w].re, v[w].im);
+  }
+  __syncthreads();
+  for (int id = threadIdx.x; id < A * C; id += T) {
+    const int s = id / C, t = id % C;
+    ulonglong2 *o = a + slot<1>(s * M + t, 0);
+    Cx2 v[B];
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      v[u] = Cx2{o[u * dC].x, o[u * dC].y};
+      if (u) v[u] = x_mul(v[u], __ldg(tw2 + (u - 1) * C + t));
+    }
+    mixfft::dft<B>(v);
+#pragma unroll
+    for (int l = 0; l < B; ++l) o[l * dC] = make_ulonglong2(v[l].re, v[l].im);
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < M; q += T) {
+    Cx2 v[A];
+    const ulonglong2 *o = a + slot<1>(q, 0);
+#pragma unroll
+    for (int s = 0; s < A; ++s) {
+      v[s] = Cx2{o[s * dM].x, o[s * dM].y};
+      if (s) v[s] = x_mul(v[s], __ldg(tw + (s - 1) * M + q));
+    }
+    mixfft::dft<A>(v);
+    float *p = y + base + q;
+#pragma unroll
+    for (int m = 0; m < A; ++m) {
+      if (m * M + q >= nt) continue;
+      const float2 im = f2_unpack(v[m].re), re = f2_unpack(v[m].im);
+      p[m * M] = re.x;
+      if (ok1) p[m * M + nt] = im.x;
+      if (ok2) p[m * M + 2LL * nt] = re.y;
+      if (ok3) p[m * M + 3LL * nt] = im.y;
+    }
+  }
+}
+
 oam_status set_smem(const void *fn, size_t bytes) {
   if (bytes > 48 * 1024)
     OAM_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
@@ -395,8 +550,31 @@ oam_status launch_fir(const FirLayout *F, const float *x, float *y, long long n_
   return OAM_OK;
 }
 
-// Line pairs per block: about 64 KB of points in shared memory.
-int fir_pairs_per_block(int NF) { return std::max(1, std::min(8, 4096 / NF)); }
+template <int A, int B, int C>
+oam_status launch_mixed(const FirLayout *F, const float *x, float *y, long long n_lines, int nt, cudaStream_t st) {
+  constexpr size_t smem = sizeof(ulonglong2) * (A * B * C + A * B * C / 8);
+  oam_status rc = set_smem((const void *)k_fir_mixed<A, B, C>, smem);
+  if (rc) return rc;
+  const long long blocks = (n_lines + 3) / 4;
+  if (blocks <= 0) return OAM_OK;
+  k_fir_mixed<A, B, C><<<(unsigned)blocks, fir_threads<A, B, C>(), smem, st>>>(x, y, n_lines, nt, F->d_hb, F->d_tw);
+  OAM_LAUNCHED();
+  return OAM_OK;
+}
+
+// k_fir_mixed's passes for `need` points: the smallest size that holds them; none below
+// 257 points, where k_fir_lines puts eight line pairs in a block, and above 4096.
+struct FirPasses {
+  int N = 0, A = 0, B = 0, C = 0;
+};
+FirPasses fir_passes(int need) {
+  if (need <= 256) return {};
+#define OAM_X(n, a, b, c) \
+  if (need <= n) return {n, a, b, c};
+  OAM_FIR_SIZES(OAM_X)
+#undef OAM_X
+  return {};
+}
 
 double sinc(double x) { return x == 0.0 ? 1.0 : std::sin(M_PI * x) / (M_PI * x); }
 
@@ -416,13 +594,14 @@ oam_status oam::fir_apply(const oam_model *m, const float *x, float *y, cudaStre
   const FirLayout *F = m->fir;
   if (!F) return OAM_ERR_INVALID_ARG;
   const long long lines = (long long)m->grid.py * m->grid.px;
-  switch (F->KP) {
-    case 8: return launch_fir<8>(F, x, y, lines, m->grid.nt, st);
-    case 4: return launch_fir<4>(F, x, y, lines, m->grid.nt, st);
-    case 2: return launch_fir<2>(F, x, y, lines, m->grid.nt, st);
-    case 1: return launch_fir<1>(F, x, y, lines, m->grid.nt, st);
+  switch (F->N) {
+#define OAM_X(n, a, b, c) \
+  case n: return launch_mixed<a, b, c>(F, x, y, lines, m->grid.nt, st);
+    OAM_FIR_SIZES(OAM_X)
+#undef OAM_X
+    case kFirMaxSize: return launch_fir<1>(F, x, y, lines, m->grid.nt, st);
+    default: return launch_fir<8>(F, x, y, lines, m->grid.nt, st);
   }
-  return OAM_ERR_DEVICE;
 }
 
 float *oam::fir_stage(const oam_model *m) { return m->fir ? m->fir->d_stage : nullptr; }
@@ -465,26 +644,49 @@ oam_status oam_model_set_filter(oam_model *m, const double *taps, int32_t half_l
     ++lg;
   }
   if (NF > kFirMaxSize) return OAM_ERR_INVALID_ARG;
-  // spectrum of the even taps on NF points (real): h0 + 2 sum_m h_m cos(2 pi f m / NF),
-  // over NF, stored at the bit reversal of f (the order the forward transform leaves)
-  std::vector<double> ct(NF);
-  for (int j = 0; j < NF; ++j) ct[j] = std::cos(2.0 * M_PI * j / NF);
-  std::vector<float> hh(NF);
-  for (int f = 0; f < NF; ++f) {
+  const FirPasses fp = fir_passes(nt + Le);
+  const int N = fp.N ? fp.N : NF;
+  // spectrum of the even taps on N points (real): h0 + 2 sum_m h_m cos(2 pi f m / N), over
+  // N, stored where the forward transform leaves frequency f
+  std::vector<double> ct(N), sn(N);
+  for (int j = 0; j < N; ++j) {
+    ct[j] = std::cos(2.0 * M_PI * j / N);
+    sn[j] = std::sin(2.0 * M_PI * j / N);
+  }
+  std::vector<float> hh(N);
+  for (int f = 0; f < N; ++f) {
     double acc = 0.0;
-    for (int k = Le; k >= 1; --k) acc += taps[k] * ct[(size_t)((long long)f * k % NF)];
+    for (int k = Le; k >= 1; --k) acc += taps[k] * ct[(size_t)((long long)f * k % N)];
     int r = 0;
-    for (int b = 0; b < lg; ++b) r |= ((f >> b) & 1) << (lg - 1 - b);
-    hh[r] = (float)((taps[0] + 2.0 * acc) / NF);
+    if (fp.N) {
+      const int s = f % fp.A, u = f / fp.A % fp.B, w = f / (fp.A * fp.B);
+      r = (s * fp.B + u) * fp.C + w;
+    } else {
+      for (int b = 0; b < lg; ++b) r |= ((f >> b) & 1) << (lg - 1 - b);
+    }
+    hh[r] = (float)((taps[0] + 2.0 * acc) / N);
+  }
+  std::vector<float2> tw;
+  if (fp.N) {
+    const int M = fp.B * fp.C;
+    for (int s = 1; s < fp.A; ++s)
+      for (int q = 0; q < M; ++q) tw.push_back(make_float2((float)ct[(size_t)q * s], (float)-sn[(size_t)q * s]));
+    for (int u = 1; u < fp.B; ++u)
+      for (int t = 0; t < fp.C; ++t) {
+        const size_t j = (size_t)t * u * fp.A;
+        tw.push_back(make_float2((float)ct[j], (float)-sn[j]));
+      }
   }
   FirLayout *F = new (std::nothrow) FirLayout();
   if (!F) return OAM_ERR_OOM;
   F->L = half_len;
   F->NF = NF;
   F->lgNF = lg;
-  F->KP = fir_pairs_per_block(NF);
-  const size_t hbytes = sizeof(float) * hh.size(), sbytes = sizeof(float) * sig_elems(m);
-  if (cudaMallocAsync((void **)&F->d_hb, hbytes, st) != cudaSuccess ||
+  F->N = N;
+  // the spectrum and the twiddles share a buffer
+  const size_t tbytes = sizeof(float2) * tw.size(), hbytes = sizeof(float) * hh.size(),
+               sbytes = sizeof(float) * sig_elems(m);
+  if (cudaMallocAsync((void **)&F->d_hb, hbytes + tbytes, st) != cudaSuccess ||
       cudaMallocAsync((void **)&F->d_stage, sbytes, st) != cudaSuccess) {
     cudaGetLastError();
     if (F->d_hb) cudaFreeAsync(F->d_hb, st);
@@ -493,8 +695,10 @@ oam_status oam_model_set_filter(oam_model *m, const double *taps, int32_t half_l
     delete F;
     return OAM_ERR_OOM;
   }
-  F->bytes = hbytes + sbytes;
+  F->bytes = hbytes + tbytes + sbytes;
+  F->d_tw = reinterpret_cast<float2 *>(F->d_hb + N);
   if (cudaMemcpyAsync(F->d_hb, hh.data(), hbytes, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      (tbytes && cudaMemcpyAsync(F->d_tw, tw.data(), tbytes, cudaMemcpyHostToDevice, st) != cudaSuccess) ||
       cudaStreamSynchronize(st) != cudaSuccess) {
     cudaFreeAsync(F->d_hb, st);
     cudaFreeAsync(F->d_stage, st);
