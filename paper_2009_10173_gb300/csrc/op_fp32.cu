@@ -16,24 +16,28 @@
 // meets the output tile, with P in shared memory, and the taps a of each chunk.  A
 // thread keeps 8 positions x 4 outputs in registers as packed pairs of positions.
 //   k_corr_warps  32 positions; the block's eight warps share out the taps, each with
-//                 its own F and slab rows, so nothing but P is exchanged between warps:
-//                 the short chain for small problems.
+//                 its own F and slab rows, so nothing but P is exchanged between warps,
+//                 and up to eight blocks of a cluster share out the row offsets: the
+//                 short chain for small problems.
 //   k_corr_block  128 positions; four warps take each tap together, 32 positions each,
 //                 sharing its slab rows (a quarter of the L2 reads): large problems.
 //
 // What bounds both: the FP32 pipe (1.5x the band's products in 32-output tiles, and the
 // moves that make packed operands) at about half its rate, the rest latency between
 // taps.  One application, GB300, from a kernel without folding: 200x200x300 forward,
-// 61x61 taps, 360 -> 53 ms; 32x32x48, 11x11 taps, 283 -> 47 us; 70x37x52 adjoint, 15x15
-// taps, 888 -> 156 us.
+// 61x61 taps, 360 -> 50 ms; 32x32x48, 11x11 taps, 283 -> 29 us (42 without clusters);
+// 70x37x52 adjoint, 15x15 taps, 888 -> 94 us (132).
 //
 // Each output sums up to win^2 x band products (about 3e5 at 61x61 taps).  One
 // FP32 accumulator for all of them loses about sqrt(n) units in the last place,
 // so the kernels sum in three levels: the products of at most 8 taps of a chunk, then
-// those of a row offset (in registers or shared memory), then the row offsets, in the
-// output.  The order does not depend on the position, so a shifted input gives the
+// those of a row offset (in registers or shared memory), then the row offsets, in shared
+// memory or the output.  The order does not depend on the position, so a shifted input gives the
 // shifted output to the bit.
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <cmath>
 
 #include "internal.cuh"
 
@@ -147,12 +151,14 @@ __device__ __forceinline__ void multiply(const float *F, const float *S, int ka,
 // Shared memory: raw rows of the two row offsets, double-buffered (the first of a pair
 // holds P once added) [2][2][strip][kChunk]; per warp F [kChunk][kPos] and two slots of
 // slab rows [kChunk][kTile]; the tap table (R <= kTableR); per staged position its row
-// and column.
+// and column; the tile's sums [2][kThreads] pairs.
 size_t warps_smem(int strip, int R) {
-  return sizeof(float) * ((size_t)4 * strip * kChunk + kWarps * kChunk * (kPos + 2 * kTile)) +
+  return sizeof(float) * ((size_t)4 * strip * kChunk + kWarps * kChunk * (kPos + 2 * kTile) + kPos * kTile) +
          (R <= kTableR ? sizeof(uint2) * (R + 1) * (R + 2) : 0) + sizeof(int2) * strip;
 }
 
+// The blocks of a cluster (grid z) share out a tile's row offsets, b = z (mod Z), and
+// add their sums in rank order at the end.
 // kVec: input rows are whole float4 from a 16-byte boundary.
 template <bool kVec>
 __global__ void __launch_bounds__(kThreads, 2)
@@ -162,9 +168,13 @@ __global__ void __launch_bounds__(kThreads, 2)
   float *Pb = reinterpret_cast<float *>(smem);  // [buffer][side][p_size]
   float *Fb = Pb + 4 * p_size;                  // [warp][kChunk][kPos]; the warps' sums at the end of a row offset
   float *Sb = Fb + kWarps * kChunk * kPos;      // [warp][slot][kChunk][kTile]
-  int2 *where = reinterpret_cast<int2 *>(Sb + 2 * kWarps * kChunk * kTile);  // staged position: row y, column x (-1: padding)
+  // the tile's sums: of output pairs [half][position x group of four], over this block's row offsets
+  float2 *sum3 = reinterpret_cast<float2 *>(Sb + 2 * kWarps * kChunk * kTile);
+  int2 *where = reinterpret_cast<int2 *>(sum3 + 2 * kThreads);  // staged position: row y, column x (-1: padding)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int T = blockIdx.y, tile = blockIdx.x;
+  const int T = blockIdx.y, tile = blockIdx.x, Z = gridDim.z;
+  static_assert(kPos * 8 == kThreads, "a thread per position and group of four outputs");
+  sum3[tid] = sum3[kThreads + tid] = make_float2(0.0f, 0.0f);
   const int y0 = tile * kPos / s.sp, x0 = tile * kPos % s.sp;
   const int y1 = min((tile * kPos + kPos - 1) / s.sp, s.py - 1);  // rows of the tile
   const uint2 *tab = s.taps + (size_t)T * NA * (NA + 1);
@@ -181,10 +191,10 @@ __global__ void __launch_bounds__(kThreads, 2)
   const int ng = lane & 7, pg = lane >> 3;  // outputs 4 ng .. +3 of the tile, positions 8 pg .. +7
 
   // Walk of the (row offset b, chunk c) with work: c0 .. c1 - 1 are b's chunks.
-  int b = -1, c = 0, c1 = 0;
+  int b = (int)blockIdx.z - Z, c = 0, c1 = 0;
   auto advance = [&](int &b, int &c, int &c1) {
     if (++c < c1) return;
-    while (++b <= R) {
+    while ((b += Z) <= R) {
       if (y0 + b >= s.py && y1 - b < 0) continue;  // neither row offset meets the grid
       const uint2 t = tab[b * (NA + 1) + NA];      // the union of its taps' ranges
       if (t.x >> 16) {
@@ -253,9 +263,9 @@ __global__ void __launch_bounds__(kThreads, 2)
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) a1[i][j] = a2[i][j] = 0;
-  // Add the warps' sums of a row offset to the output: two of a lane's four outputs at
-  // a time through the F buffers, a thread per four position x output pairs.
-  auto flush = [&](bool first) {
+  // Add the warps' sums of a row offset to the tile's: two of a lane's four outputs at
+  // a time through the F buffers, a thread per pair.
+  auto flush = [&] {
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
       __syncthreads();
@@ -268,26 +278,20 @@ __global__ void __launch_bounds__(kThreads, 2)
         a2[i][2 * half] = a2[i][2 * half + 1] = 0;
       }
       __syncthreads();
-      for (int i = tid; i < kPos * 8; i += kThreads) {  // (position, pair of outputs)
-        float2 v = *reinterpret_cast<const float2 *>(Fb + 2 * i);
+      float2 v = *reinterpret_cast<const float2 *>(Fb + 2 * tid);
 #pragma unroll
-        for (int w = 1; w < kWarps; ++w) {
-          const float2 u = *reinterpret_cast<const float2 *>(Fb + w * kChunk * kPos + 2 * i);
-          v.x += u.x;
-          v.y += u.y;
-        }
-        const int o = tile * kPos + i / 8, y = o / s.sp, x = o % s.sp, n = T * kTile + 4 * (i % 8) + 2 * half;
-        if (y >= s.py || x >= s.px) continue;
-        float *dst = out + ((size_t)y * s.px + x) * s.out_len + n;
-        if (n < s.out_len) dst[0] = first ? v.x : dst[0] + v.x;
-        if (n + 1 < s.out_len) dst[1] = first ? v.y : dst[1] + v.y;
+      for (int w = 1; w < kWarps; ++w) {
+        const float2 u = *reinterpret_cast<const float2 *>(Fb + w * kChunk * kPos + 2 * tid);
+        v.x += u.x;
+        v.y += u.y;
       }
+      float2 &o = sum3[half * kThreads + tid];
+      o = make_float2(o.x + v.x, o.y + v.y);
     }
     __syncthreads();
   };
 
   int pb = 0, slot = 0;
-  bool first = true;
   unsigned long long m0 = 0, m1 = 0;
   int a = NA;  // this warp's tap
   advance(b, c, c1);
@@ -366,10 +370,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       request_slab(bn, cn, a, slot);
       copies_commit();
     }
-    if (bn != b) {
-      flush(first);
-      first = false;
-    }
+    if (bn != b) flush();
     b = bn;
     c = cn;
     c1 = c1n;
@@ -377,7 +378,25 @@ __global__ void __launch_bounds__(kThreads, 2)
     m1 = n1;
     pb ^= 1;
   }
-  if (first) flush(true);  // no slab row meets the tile: zeros
+  // Write the tile: rank z takes the z-th share of the pairs.
+  auto cluster = cooperative_groups::this_cluster();
+  cluster.sync();
+  const int share = 2 * kThreads / Z;
+  for (int j = tid; j < share; j += kThreads) {
+    const int i = blockIdx.z * share + j, half = i / kThreads, e = i % kThreads;
+    float2 v = *cluster.map_shared_rank(sum3 + i, 0);
+    for (int z = 1; z < Z; ++z) {
+      const float2 u = *cluster.map_shared_rank(sum3 + i, z);
+      v.x += u.x;
+      v.y += u.y;
+    }
+    const int o = tile * kPos + e / 8, y = o / s.sp, x = o % s.sp, n = T * kTile + 4 * (e % 8) + 2 * half;
+    if (y >= s.py || x >= s.px) continue;
+    float *dst = out + ((size_t)y * s.px + x) * s.out_len + n;
+    if (n < s.out_len) dst[0] = v.x;
+    if (n + 1 < s.out_len) dst[1] = v.y;
+  }
+  cluster.sync();  // every rank has read this block's sums
 }
 
 // ---------------------------------------------------------------- k_corr_block
@@ -557,19 +576,15 @@ oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaSt
   s.out_len = fwd ? g.nt : g.nz;
   s.taps = L.d_taps;
   s.rows = L.d_rows;
-  // The kernel that finishes first, from the blocks with work on the fullest SM, in
-  // units of one 128-position block alone on an SM: alone a block is bound by its chain
-  // of taps (the eight warps' is 0.3 as long), together they share the SM's pipes (0.47
-  // and 0.15 per block: 48x48x64 31x31 taps 1117 against 319 us, 64x64x128 61x61 taps
-  // 6.5 against 3.5 ms, 96x96x128 8.0 against 7.1, 128x128x64 11x11 taps 268 against
-  // 371 us, 200x200x300 53 against 71 ms).
+  // k_corr_block from three of its blocks with work on the fullest SM on: alone or in twos
+  // they are bound by their chains of taps, which the eight warps cut eightfold.  us,
+  // block against warps, with one: 48x48x64 31x31 taps 950, 259; two: 80x80x64 21x21
+  // taps 516, 362, 64x64x128 61x61 taps 4202, 2976, 96x64x64 11x11 taps 171, 141,
+  // 128x128x64 11x11 taps adjoint 312, 369; three: 128x96x100 15x15 taps adjoint 667,
+  // 705; five: 96x96x128 31x31 taps 1498, 1818, 128x128x64 11x11 taps 218, 358.
   const long long busy = fwd ? (m->n_hi - m->n_lo + kTile - 1) / kTile : L.tiles;
   const int sms = std::max(1, m->sm_count);
-  auto per_sm = [&](int positions) {
-    const long long blocks = ((long long)g.px * g.py + positions - 1) / positions * busy;
-    return (double)((blocks + sms - 1) / sms);
-  };
-  const bool block = std::max(1.0, 0.47 * per_sm(kBlockPos)) <= std::max(0.3, 0.15 * per_sm(kPos));
+  const bool block = ((long long)g.px * g.py + kBlockPos - 1) / kBlockPos * busy > 2LL * sms;
   // Tiles run on over scan rows (no idle positions) unless the padding between
   // many short rows makes the strip too long; then every tile stays in its row.
   const int tile = block ? kBlockPos : kPos;
@@ -579,11 +594,40 @@ oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaSt
   s.strip = run_on ? wrap : tile + 2 * s.R;
   const long long tiles = ((long long)s.py * s.sp + tile - 1) / tile;
   const size_t sm = block ? block_smem(s.strip, s.R) : warps_smem(s.strip, s.R);
+  // Blocks that share out a tile's row offsets: the count that finishes first, in units of
+  // a row offset, 0.6 more for a block's start and end, times the waves at the blocks an
+  // SM holds (the idle part of the last wave counts half).  us with 1, 2, 4, 8: 32x32x48
+  // 11x11 taps forward 43 30 34 44, adjoint 79 44 38 42; 70x37x52 15x15 taps adjoint
+  // 132 116 94 98; 96x64x64 11x11 taps forward 171 191 272 532.
+  int Z = 1;
+  if (!block) {
+    const double slots = (sm <= 112 * 1024 ? 2.0 : 1.0) * sms;
+    double best = 0;
+    for (int z = 1; z <= std::min(8, s.R + 1); z *= 2) {
+      const double waves = (double)(tiles * busy * z) / slots;
+      const double cost = (waves <= 1 ? 1.0 : 0.5 * (waves + std::ceil(waves))) * ((s.R + z) / z + 0.6);
+      if (z == 1 || cost <= best) {
+        best = cost;
+        Z = z;
+      }
+    }
+  }
   const bool vec = s.len % 4 == 0;
   auto fn = block ? (vec ? k_corr_block<true> : k_corr_block<false>) : (vec ? k_corr_warps<true> : k_corr_warps<false>);
   OAM_CUDA_TRY(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   ProfScope prof(m, st, fwd);
-  fn<<<dim3((unsigned)tiles, L.tiles), block ? kBlockPos : kThreads, sm, st>>>(s, in, out);  // tile neighbours share slab rows
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)tiles, L.tiles, Z);  // tile neighbours share slab rows
+  cfg.blockDim = dim3(block ? kBlockPos : kThreads);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = Z;
+  cfg.attrs = &attr;
+  cfg.numAttrs = Z > 1;
+  OAM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, s, in, out));
   OAM_LAUNCHED();
   return OAM_OK;
 }

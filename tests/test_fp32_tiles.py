@@ -3,8 +3,9 @@
 On the CPU: for both position tilings, the staged strip holds the positions
 x +- a of every lane and its padding is outside the grid.  On the GPU, against
 the FP64 oracle at the FP32 operators' tolerance: sizes on both sides of the
-rules that pick the kernel, the tiling and the tap table's place, odd depth counts (scalar loads), partial
-output tiles and taps beyond the grid.
+rules that pick the kernel, the blocks per tile (one to eight, more than there
+are row offsets in a share), the tiling and the tap table's place, odd depth
+counts (scalar loads), partial output tiles and taps beyond the grid.
 """
 import numpy as np
 import pytest
@@ -49,7 +50,7 @@ def test_strips_hold_every_tap(px, py, R, M):
 @pytest.mark.parametrize("over", [
     dict(px=3, py=40, win=61, nz=13, nt=256, dx_m=4e-6, dy_m=4e-6), dict(px=150, py=90, win=7, nz=51, nt=192),
     dict(px=64, py=66, win=9, nz=47, nt=188), dict(px=33, py=5, win=5, nz=3, nt=128),
-    dict(px=131, py=160, win=3, nz=33, nt=160), dict(px=260, py=190, win=5, nz=6, nt=128), dict(px=20, py=12, win=71, nz=17, nt=256, dx_m=4e-6, dy_m=4e-6), dict(px=9, py=3, win=21, nz=16, nt=192, dx_m=8e-6, dy_m=12e-6)],
+    dict(px=32, py=32, win=11, nz=48, nt=192), dict(px=70, py=37, win=15, nz=52, nt=200), dict(px=131, py=160, win=3, nz=33, nt=160), dict(px=260, py=190, win=5, nz=6, nt=128), dict(px=20, py=12, win=71, nz=17, nt=256, dx_m=4e-6, dy_m=4e-6), dict(px=9, py=3, win=21, nz=16, nt=192, dx_m=8e-6, dy_m=12e-6)],
     ids=lambda o: "x".join(str(o[k]) for k in ("px", "py", "win", "nz", "nt")))
 def test_tiles_match_oracle(over):
     import torch
