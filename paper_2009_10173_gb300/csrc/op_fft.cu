@@ -71,6 +71,7 @@ using namespace oam::fftdev;
 
 constexpr int kFftThreads = 256;
 constexpr int kApplyWarps = 5;  // spectral products: warps per block
+constexpr unsigned kAhead = 48 * 1024;  // bytes of a row prefetched to L2
 constexpr int kUnroll = 4;      // 16-byte row loads per lane and step, two steps in flight
 constexpr int kStep = 4 * kUnroll;  // input elements per step
 constexpr int kBuildThreads = 128;
@@ -320,7 +321,12 @@ __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_c2r(const float2 *__r
 // take 7 issue slots per S^ value instead of 20 (a lane per output, scalar loads), and
 // the next step's loads are issued before this step's products.  200x200x300 (0.77 GB),
 // cold caches: 200 us forward, 191 adjoint (3.9 TB/s), against 270 and 217 for the scalar
-// form with its own kernel per direction.
+// form with its own kernel per direction.  What remains is the loads' latency at 20 warps
+// per SM (registers); a block therefore starts by asking L2 for the first 48 KB of its row:
+// a whole application 338 -> 321 us (adjoint 316 -> 309), 256x256x384 573 -> 547 (522 ->
+// 512), 128x128x192 123 -> 119, 64x64x128 41 both.  24 KB give 327 and 559, 64 KB 331 and
+// 566.  Asking for whole rows or for the rows of later blocks evicts the vectors (adjoint
+// 256x256x384 547, 652), loading S^ as evict-first loses what L2 keeps of it (forward 349).
 __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
@@ -346,6 +352,11 @@ __global__ void __launch_bounds__(32 * kApplyWarps, 4)
   ulonglong2 *X = sma;                                            // [n_in + kStep][2]
   int2 *E = reinterpret_cast<int2 *>(X + 2 * (n_in + kStep));     // [n_in + kStep]
   const int r = blockIdx.x;
+  const float4 *row = reinterpret_cast<const float4 *>(S + (size_t)r * stride);
+  if (threadIdx.x == 0)  // the row's start to L2, under the loads of the vectors
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(row),
+                 "r"((unsigned)min(stride * (long long)sizeof(float), (long long)kAhead))
+                 : "memory");
   const int4 mem = members[r];
   {
     float2 *X2 = reinterpret_cast<float2 *>(X);
@@ -364,7 +375,6 @@ __global__ void __launch_bounds__(32 * kApplyWarps, 4)
     }
   }
   __syncthreads();
-  const float4 *row = reinterpret_cast<const float4 *>(S + (size_t)r * stride);
   const int lane = threadIdx.x & 31, ph = lane >> 3;
   for (int w = threadIdx.x >> 5; w < windows; w += blockDim.x >> 5) {
     const int g = 8 * w + (lane & 7);
