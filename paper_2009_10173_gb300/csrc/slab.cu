@@ -402,6 +402,261 @@ __global__ void k_slab_values(Geo g, const PatchDW *__restrict__ pdw, int M, con
   }
 }
 
+// ---------------------------------------------------------------- band values by moments
+// The same sums with a few instructions per patch instead of thirty per (patch, sample)
+// pair: for an integer offset t from the nearest sample the pulse is a polynomial in
+// the fraction, v(t - x/2) = sum_p c_p(t) x^p for x = 2f in [-1, 1], so a sample needs of
+// the patches whose nearest sample is b (a bin) only their moments sum_j w_j x_j^p:
+//   S[n] = sum_b sum_p c_p(n - b) mom[b][p].
+// The truncation |tau| <= cut splits a bin only at t = +-tb, the one integer within half
+// a sample of it; the truncated sums of those two offsets are two more moments.  There x
+// is compared with the edge itself: t - f against the cut, rounded, lets single patches
+// in or out (1.7e-6 of the slab at a cut of three deviations, here 2.5e-8).
+//
+// Per chunk of patches: arrivals; a stable counting sort by bin (warps own index ranges,
+// equal bins within 32 patches are ranked by match_any); threads sum segments of kSeg
+// patches of a bin (Kahan), and the segments are added in order as double words.
+// Everything is a fixed-order sum, and every product that matters is a double-word one,
+// so the result is nearer to the exact sum than adding the patches' FP32 values.
+//
+// What bounds it: issue slots, about evenly in the arrivals, the segments and the last
+// sums (each pair took 30 slots, and half of the lanes' samples are out of a patch's
+// reach).  Model build, 2000 patches, 61x61 taps, and the slab's error against FP64,
+// from k_slab_values: 192 depths 19.9 -> 8.2 ms, 8.2e-8 -> 3.0e-8; 300 depths 31.4 ->
+// 12.9 ms, 9.9e-8 -> 3.5e-8; 384 depths 40.0 -> 16.5 ms, 9.7e-8 -> 3.6e-8; 48 depths,
+// 11x11 taps 0.66 -> 0.42 ms.
+constexpr int kMom = 12;       // monomials
+constexpr int kMomAll = kMom + 2;
+constexpr int kMomFull = 6;    // the first of them in double words in the last sum
+constexpr int kMomChunk = 1024;
+constexpr int kMomThreads = 128;
+constexpr int kSeg = 16;
+
+struct MomShape {
+  int tb;      // edge offset
+  float edge;  // least x with |tb - x / 2| <= cut
+  int B0, nb;  // first bin's sample - lo, and most bins
+};
+size_t mom_smem(const MomShape &s) {
+  const size_t segs = kMomChunk / kSeg + s.nb;
+  return sizeof(float2) * ((size_t)(2 * s.tb + 1) * kMom + kMomChunk + (segs + s.nb) * kMomAll) +
+         sizeof(int) * (size_t)(4 * s.nb + 2 * (s.nb + 1) + segs);
+}
+
+__device__ __forceinline__ void kahan(float &s, float &c, float v) {
+  const float y = __fsub_rn(v, c), u = __fadd_rn(s, y);
+  c = __fsub_rn(__fsub_rn(u, s), y);
+  s = u;
+}
+
+__global__ void __launch_bounds__(kMomThreads, 4)
+    k_slab_moments(Geo g, const PatchDW *__restrict__ pdw, int M, const int *orb_b, const int *orb_a, int nz,
+                   const int *band_lo, const int *band_hi, int band_w, MomShape ms, const float2 *__restrict__ coef_g,
+                   float *__restrict__ band) {
+  extern __shared__ float2 smm[];
+  const int tb = ms.tb, nbm = ms.nb, segm = kMomChunk / kSeg + nbm;
+  float2 *coef = smm;                                // [2 tb + 1][kMom] (high, low)
+  float2 *sorted = coef + (2 * tb + 1) * kMom;       // [kMomChunk] (x, w)
+  float2 *part = sorted + kMomChunk;                 // [segm][kMomAll] (sum, compensation)
+  float2 *mom = part + segm * kMomAll;               // [nbm][kMomAll] (high, low)
+  int *place = reinterpret_cast<int *>(mom + nbm * kMomAll);  // [4][nbm] counts, then places
+  int *start = place + 4 * nbm;                      // [nbm + 1] a bin's first patch in `sorted`
+  int *seg0 = start + nbm + 1;                       // [nbm + 1] and first segment
+  int *seg_bin = seg0 + nbm + 1;                     // [segm]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int o = blockIdx.x, k = blockIdx.y;
+  const int b = orb_b[o], a = orb_a[o];
+  const int lo = band_lo[o * nz + k], hi = band_hi[o * nz + k];
+  const int nb = max(1, min(nbm, hi - lo - 2 * ms.B0 + 1));  // bins in use
+  for (int i = tid; i < (2 * tb + 1) * kMom; i += kMomThreads) coef[i] = coef_g[i];
+  for (int i = tid; i < nbm * kMomAll; i += kMomThreads) mom[i] = make_float2(0.0f, 0.0f);
+  const double rxd = a * g.dx, ryd = b * g.dy, rzd = g.z0 + k * g.dz;
+  const DW rx = to_dw(rxd), ry = to_dw(ryd), rz = to_dw(rzd), r2 = to_dw(rxd * rxd + ryd * ryd + rzd * rzd);
+  const DW Fw = to_dw(g.F), F2w = to_dw(2.0 * g.F), FFw = to_dw(g.F * g.F), ks = to_dw(g.ks), G = to_dw(g.G);
+  for (int j0 = 0; j0 < M; j0 += kMomChunk) {
+    const int cnt = min(kMomChunk, M - j0);
+    __syncthreads();
+    for (int i = tid; i < 4 * nbm; i += kMomThreads) place[i] = 0;
+    __syncthreads();
+    // arrivals, and each patch's place among its warp's patches of its bin
+    constexpr int kIter = kMomChunk / kMomThreads;
+    int at[kIter];     // bin | place << 16, -1: none
+    float2 xw[kIter];
+#pragma unroll
+    for (int i = 0; i < kIter; ++i) {
+      const int j = (warp * kIter + i) * 32 + lane;
+      int bin = -1;
+      xw[i] = make_float2(0.0f, 0.0f);
+      if (j < cnt) {
+        const PatchDW p = pdw[j0 + j];
+        const DW rn = dw_add(dw_add(dw_mul(rx, DW{p.xh, p.xl}), dw_mul(ry, DW{p.yh, p.yl})), dw_mul(rz, DW{p.zh, p.zl}));
+        const DW num = dw_add(dw_mul(F2w, rn), r2);
+        const DW d = dw_sqrt(dw_add(FFw, num));
+        const DW dd = dw_div(num, dw_add(d, Fw));  // d - F, metres
+        const DW D = dw_add(dw_mul(ks, dd), G);    // arrival, samples
+        const float nr = rintf(D.h);
+        const float f = __fadd_rn(__fsub_rn(D.h, nr), D.l);  // D.h - nr is exact
+        bin = __float2int_rn(nr) - lo - ms.B0;
+        if (bin < 0 || bin >= nb) bin = -1;  // meets no sample of the band
+        xw[i] = make_float2(2.0f * f, __fdiv_rn(p.w, dw_add(Fw, dd).h));  // (mm^2 / 1e3) / metres = mm^2 / mm
+      }
+      const unsigned same = __match_any_sync(0xffffffffu, bin);
+      const int rank = __popc(same & ((1u << lane) - 1u));
+      at[i] = bin < 0 ? -1 : bin | (place[warp * nbm + bin] + rank) << 16;
+      __syncwarp();
+      if (bin >= 0 && rank == 0) place[warp * nbm + bin] += __popc(same);
+      __syncwarp();
+    }
+    __syncthreads();
+    if (warp == 0) {  // first places and segments of the bins
+      int c0 = 0, s0 = 0;
+      for (int i0 = 0; i0 < nb; i0 += 32) {
+        const int i = i0 + lane;
+        int n[4] = {0, 0, 0, 0}, total = 0;
+        if (i < nb) {
+#pragma unroll
+          for (int w = 0; w < 4; ++w) total += n[w] = place[w * nbm + i];
+        }
+        const int segs = (total + kSeg - 1) / kSeg;
+        int c = total, s = segs;  // inclusive sums
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const int c2 = __shfl_up_sync(0xffffffffu, c, off), s2 = __shfl_up_sync(0xffffffffu, s, off);
+          if (lane >= off) {
+            c += c2;
+            s += s2;
+          }
+        }
+        if (i < nb) {
+          int at0 = c0 + c - total;
+          start[i] = at0;
+          seg0[i] = s0 + s - segs;
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
+            place[w * nbm + i] = at0;
+            at0 += n[w];
+          }
+          for (int q = 0; q < segs; ++q) seg_bin[s0 + s - segs + q] = i;
+        }
+        c0 += __shfl_sync(0xffffffffu, c, 31);
+        s0 += __shfl_sync(0xffffffffu, s, 31);
+      }
+      if (lane == 0) {
+        start[nb] = c0;
+        seg0[nb] = s0;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kIter; ++i)
+      if (at[i] >= 0) sorted[place[warp * nbm + (at[i] & 0xffff)] + (at[i] >> 16)] = xw[i];
+    __syncthreads();
+    for (int s = tid; s < seg0[nb]; s += kMomThreads) {
+      const int bin = seg_bin[s], i0 = start[bin] + (s - seg0[bin]) * kSeg, i1 = min(i0 + kSeg, start[bin + 1]);
+      float sum[kMomAll], comp[kMomAll];
+#pragma unroll
+      for (int p = 0; p < kMomAll; ++p) sum[p] = comp[p] = 0.0f;
+      for (int i = i0; i < i1; ++i) {
+        const float2 q = sorted[i];
+        float pw = q.y, ep = 0.0f, em = 0.0f;
+#pragma unroll
+        for (int p = 0; p < kMom; ++p) {
+          kahan(sum[p], comp[p], pw);
+          ep = fmaf(coef[2 * tb * kMom + p].x, pw, ep);
+          em = fmaf(coef[p].x, pw, em);
+          pw *= q.x;
+        }
+        if (q.x >= ms.edge) kahan(sum[kMom], comp[kMom], ep);
+        if (q.x <= -ms.edge) kahan(sum[kMom + 1], comp[kMom + 1], em);
+      }
+#pragma unroll
+      for (int p = 0; p < kMomAll; ++p) part[s * kMomAll + p] = make_float2(sum[p], -comp[p]);
+    }
+    __syncthreads();
+    for (int i = tid; i < nb * kMomAll; i += kMomThreads) {
+      const int bin = i / kMomAll, p = i % kMomAll;
+      DW v{mom[i].x, mom[i].y};
+      for (int s = seg0[bin]; s < seg0[bin + 1]; ++s) {
+        const float2 u = part[s * kMomAll + p];
+        v = dw_add(v, fast_two_sum(u.x, u.y));
+      }
+      mom[i] = make_float2(v.h, v.l);
+    }
+  }
+  __syncthreads();
+  float *row = band + ((size_t)o * nz + k) * band_w;
+  for (int i = tid; i < band_w; i += kMomThreads) {
+    if (lo + i >= hi) {
+      row[i] = 0.0f;
+      continue;
+    }
+    const int c = i - ms.B0;  // this sample's bin
+    float acc = 0.0f, err = 0.0f;
+    auto add = [&](float h, float l) {
+      const DW s = two_sum(acc, h);
+      acc = s.h;
+      err += s.l + l;
+    };
+    for (int bin = max(0, c - tb + 1); bin <= min(nb - 1, c + tb - 1); ++bin) {
+      const float2 *m = mom + bin * kMomAll, *w = coef + (c - bin + tb) * kMom;
+      float rest = 0.0f;
+#pragma unroll
+      for (int p = kMom - 1; p >= kMomFull; --p) rest = fmaf(w[p].x, m[p].x, rest);
+#pragma unroll
+      for (int p = kMomFull - 1; p >= 0; --p) {
+        const DW pr = two_prod(w[p].x, m[p].x);
+        rest += fmaf(w[p].y, m[p].x, fmaf(w[p].x, m[p].y, pr.l));
+        add(pr.h, 0.0f);
+      }
+      err += rest;
+    }
+    if (c - tb >= 0 && c - tb < nb) add(mom[(c - tb) * kMomAll + kMom].x, mom[(c - tb) * kMomAll + kMom].y);
+    if (c + tb >= 0 && c + tb < nb) add(mom[(c + tb) * kMomAll + kMom + 1].x, mom[(c + tb) * kMomAll + kMom + 1].y);
+    row[i] = acc + err;
+  }
+}
+
+// The pulse's polynomials c_p(t), t = -tb .. tb, as (high, low) pairs: interpolation at
+// Chebyshev points in FP64.  False when they miss the pulse by more than 1e-9 of its
+// largest value (a carrier or an envelope that varies too fast within a sample).
+bool pulse_polynomials(double sigma, double omega, int tb, std::vector<float2> *out) {
+  auto pulse = [&](double tau) {
+    return -std::exp(-tau * tau / (2.0 * sigma * sigma)) *
+           (tau / (sigma * sigma) * std::cos(omega * tau) + omega * std::sin(omega * tau));
+  };
+  double T[kMom][kMom] = {};  // monomial coefficients of the Chebyshev polynomials
+  T[0][0] = T[1][1] = 1.0;
+  for (int j = 2; j < kMom; ++j)
+    for (int p = 0; p < kMom; ++p) T[j][p] = (p ? 2.0 * T[j - 1][p - 1] : 0.0) - T[j - 2][p];
+  double node[4 * kMom];  // cos(pi i / (2 kMom)): the points are at odd i
+  for (int i = 0; i < 4 * kMom; ++i) node[i] = std::cos(M_PI * i / (2 * kMom));
+  out->resize((size_t)(2 * tb + 1) * kMom);
+  double top = 0.0, miss = 0.0;
+  for (int t = 0; t <= tb; ++t) {  // v is odd: c_p(-t) = (-1)^(p + 1) c_p(t)
+    double c[kMom] = {}, v[kMom];
+    for (int i = 0; i < kMom; ++i) v[i] = pulse(t - 0.5 * node[2 * i + 1]);
+    for (int j = 0; j < kMom; ++j) {
+      double aj = 0.0;
+      for (int i = 0; i < kMom; ++i) aj += v[i] * node[j * (2 * i + 1) % (4 * kMom)];
+      aj *= (j ? 2.0 : 1.0) / kMom;
+      for (int p = 0; p < kMom; ++p) c[p] += aj * T[j][p];
+    }
+    for (int i = 0; i <= kMom; i += 2) {  // between the points, where the error peaks
+      const double x = node[2 * i], want = pulse(t - 0.5 * x);
+      double got = 0.0;
+      for (int p = kMom - 1; p >= 0; --p) got = got * x + c[p];
+      top = std::max(top, std::fabs(want));
+      miss = std::max(miss, std::fabs(got - want));
+    }
+    for (int p = 0; p < kMom; ++p) {
+      const float h = (float)c[p], l = (float)(c[p] - (double)h);
+      (*out)[(size_t)(tb - t) * kMom + p] = p % 2 ? make_float2(h, l) : make_float2(-h, -l);
+      (*out)[(size_t)(tb + t) * kMom + p] = make_float2(h, l);
+    }
+  }
+  return miss <= 1e-9 * top;
+}
+
 // FP32 operators' slab rows (DirectRows) of one direction: row e of (orbit o, tile T)
 // holds, for input element e (forward: depth, adjoint: sample), the tile's outputs.
 __global__ void k_pack_rows(const float *band, const int *band_lo, const int *band_hi, int band_w, int nz, int dir,
@@ -664,10 +919,32 @@ oam_status oam::build_slab(oam_model *m, cudaStream_t st) {
     k_slab33_values<<<dim3(O, nz), threads, sm, st>>>(g3, m->d_patch, m->M, d_orb_b, d_orb_a, nz, nt, m->d_band_lo,
                                                       d_band_hi, m->band_w, m->d_band);
   } else {
-    const int threads = m->band_w <= 128 ? 128 : 256;
-    const int T0 = (int)std::floor(m->cut + 0.5) + 1;  // rotation table half-length
-    k_slab_values<<<dim3(O, nz), threads, sizeof(float2) * (2 * T0 + 1), st>>>(
-        g, d_pdw, m->M, d_orb_b, d_orb_a, nz, m->d_band_lo, d_band_hi, m->band_w, T0, m->d_band);
+    // k_slab_values where the pulse varies too fast within a sample for the polynomials, is
+    // shorter than two samples a side, or its bins exceed the shared memory of two blocks
+    // per SM
+    MomShape ms{};
+    ms.tb = (int)std::floor(m->cut - 0.5) + 1;
+    const double edge = 2.0 * (ms.tb - m->cut);
+    ms.edge = (float)edge;
+    if ((double)ms.edge < edge) ms.edge = std::nextafter(ms.edge, INFINITY);
+    ms.B0 = std::max(0, (int)std::floor(m->cut) - 1);
+    ms.nb = std::max(1, m->band_w - 2 * ms.B0 + 1);
+    std::vector<float2> coef;
+    if (m->cut >= 2.0 && m->cut <= 64.0 && mom_smem(ms) <= 100 * 1024 &&
+        pulse_polynomials(m->sigma_s, m->omega, ms.tb, &coef)) {
+      float2 *d_coef = nullptr;
+      OAM_CUDA_TRY(cudaMallocAsync((void **)&d_coef, sizeof(float2) * coef.size(), st));
+      OAM_CUDA_TRY(cudaMemcpyAsync(d_coef, coef.data(), sizeof(float2) * coef.size(), cudaMemcpyHostToDevice, st));
+      OAM_CUDA_TRY(cudaFuncSetAttribute(k_slab_moments, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+      k_slab_moments<<<dim3(O, nz), kMomThreads, mom_smem(ms), st>>>(
+          g, d_pdw, m->M, d_orb_b, d_orb_a, nz, m->d_band_lo, d_band_hi, m->band_w, ms, d_coef, m->d_band);
+      cudaFreeAsync(d_coef, st);
+    } else {
+      const int threads = m->band_w <= 128 ? 128 : 256;
+      const int T0 = (int)std::floor(m->cut + 0.5) + 1;  // rotation table half-length
+      k_slab_values<<<dim3(O, nz), threads, sizeof(float2) * (2 * T0 + 1), st>>>(
+          g, d_pdw, m->M, d_orb_b, d_orb_a, nz, m->d_band_lo, d_band_hi, m->band_w, T0, m->d_band);
+    }
   }
   OAM_LAUNCHED();
 
