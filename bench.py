@@ -30,21 +30,15 @@ LSQR_ITERS, FISTA_ITERS, POWER_ITERS, LAMBDA_REL = 50, 100, 20, 1e-3
 # operator applications per step: LSQR 1 + 2*50; FISTA 2*20 power + 1 lambda + 2*100
 OPS_PER_STEP = (1 + 2 * LSQR_ITERS) + (2 * POWER_ITERS + 1 + 2 * FISTA_ITERS)
 FP32_LANES_PER_SM = 128
-# DRAM bytes per launch of the tensor-core operator kernel (k_corr_fold) per
-# direction on this workload: dram__bytes_read.sum + dram__bytes_write.sum of an
-# ncu capture of the same kernel on a 96x96-position case of this workload (576
-# blocks), scaled by blocks processed (2504 / 576; profiles/k_corr_fold_fwd_ and
-# k_corr_fold_adj_96x96x300_win61.md).  Set to None when the kernel changes.
-TC_TRAFFIC_BYTES = {"forward": (106.70e6 + 61.04e6) * 2504 / 576, "adjoint": (100.98e6 + 56.94e6) * 2504 / 576}
-# DRAM bytes per application of the lateral-FFT form on this workload:
-# dram__bytes_read.sum + dram__bytes_write.sum over the five launches of one
-# forward, from an ncu capture of the full 200x200x300 workload (1.191 GB read,
-# 0.250 GB written).  Set to None when those kernels change.
-FFT_TRAFFIC_BYTES = 1.4414e9
+# DRAM bytes per application of the operators on this workload, from a capture of
+# all their launches (dram__bytes_read.sum + dram__bytes_write.sum); None until the
+# current kernels are captured.
+TC_TRAFFIC_BYTES = None
+FFT_TRAFFIC_BYTES = None
 # Band-pass filter along time: half length of the 0.5-80 MHz FIR, and the DRAM
-# bytes of one application (ncu, profiles/k_fir_lines_200x200x1024_L511.md).
+# bytes of one application (None as above).
 FIR_HALF = 511
-FIR_TRAFFIC_BYTES = 163.96e6 + 120.01e6
+FIR_TRAFFIC_BYTES = None
 
 
 def parse():
@@ -644,7 +638,7 @@ def run_ours(args, rank, world, acc=None):
         fir_size = mm.info.filter_size
         mm.close()
         return {"bandpass_filter": {"band_hz": [0.5e6, 80e6], "taps": 2 * FIR_HALF + 1, "transform": fir_size,
-                                    "ms": fir_ms, "roofline": {"bound": "hbm", "kernel": "k_fir_lines",
+                                    "ms": fir_ms, "roofline": {"bound": "hbm", "kernel": "k_fir_mixed",
                                                                "achieved": gbs, "peak": hbm, "unit": "GB/s",
                                                                "frac": gbs / hbm, "bytes_per_launch": fir_bytes,
                                                                "traffic": FIR_TRAFFIC_BYTES}},
@@ -729,16 +723,20 @@ def run_ours(args, rank, world, acc=None):
     elif prec == B.OAM_PREC_FP32:
         mhz = peaks.get("sm_max_mhz", 2070.0)
         peak = sms * FP32_LANES_PER_SM * 2 * mhz * 1e6 / 1e12
-        roof = {"bound": "alu", "kernel": f"{dom} (FP32 FFMA)", "achieved": achieved, "peak": peak,
-                "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
+        # the four mirrored taps share one product: the folded operator's flops
+        half = (cfg["win"] - 1) // 2
+        folded = achieved * ((half + 1) / cfg["win"]) ** 2
+        roof = {"bound": "alu", "kernel": f"{dom} (FP32, mirror-folded)", "achieved": folded, "peak": peak,
+                "unit": "TFLOP/s", "frac": folded / peak, "traffic": None, "algorithmic_tflops": achieved,
                 "peak_source": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 flop x {mhz:g} MHz"}
     else:
         peak = peaks.get("bf16_tflops_sustained", 1700.0)
-        roof = {"bound": "tensor", "kernel": f"{dom} (tcgen05 split-BF16, mirror-folded)", "achieved": achieved,
-                "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": TC_TRAFFIC_BYTES[dom] if TC_TRAFFIC_BYTES else None,
-                "executed_tflops": (info.exec_flops_adjoint if dom == "adjoint" else info.exec_flops_forward) /
-                                   (dom_ms * 1e-3) / 1e12,
+        # the flops that the tensor cores are given: transformed and mirror-folded, the
+        # form needs a fraction of the direct sums' flops
+        done = (info.exec_flops_adjoint if dom == "adjoint" else info.exec_flops_forward) / (dom_ms * 1e-3) / 1e12
+        roof = {"bound": "tensor", "kernel": f"{dom} (3 launches, tcgen05 split products per lateral frequency)",
+                "achieved": done, "peak": peak, "unit": "TFLOP/s", "frac": done / peak,
+                "traffic": TC_TRAFFIC_BYTES[dom] if TC_TRAFFIC_BYTES else None, "algorithmic_tflops": achieved,
                 "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (of measured)"}
     line = {"metric": METRIC, "value": value, "unit": "volumes/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": per_step, "higher_is_better": True, "scaling": "weak",

@@ -4,9 +4,9 @@
 // over the scan grid (Methods, Efficient reconstruction based on scanning
 // symmetries: the model is the same for every scanning position).  With the
 // volume and the signals zero-padded to P x P, P >= max(py, px) + R one of the
-// mixed-radix transform sizes up to 512 or a power of two, no circular wrap reaches the output window, and the
-// correlation theorem restates both operators exactly per lateral frequency
-// (v, u):
+// mixed-radix transform sizes up to 512 or a power of two, no circular wrap
+// reaches the output window, and the correlation theorem restates both operators
+// exactly per lateral frequency (v, u):
 //   A:    s^(v,u,n) = sum_k S^(v,u,k,n) H^(v,u,k)
 //   A^T:  H^(v,u,k) = sum_n S^(v,u,k,n) s^(v,u,n)
 // The slab is mirror-symmetric in both lateral offsets (the patch set is;

@@ -3,9 +3,9 @@
 //
 // Distances use the cancellation-free form d - F = (2F r.n + |r|^2) / (d + F)
 // in FP64, so the arrival sample fs*(d/c - t0) = (fs/c)(d - F) + fs(F/c - t0)
-// keeps full precision; the EIR derivative is evaluated in FP32 at
-// tau = n - D_j (|tau| <= trunc_sigma * sigma_s), tau being the FP32 rounding
-// of the exact offset, and summed over patches with a compensated FP32 sum.
+// keeps full precision; the EIR derivative, a polynomial in the fraction of a sample
+// between an arrival and its nearest sample, is summed over patches as moments
+// (k_slab_moments), or evaluated in FP32 per patch (k_slab_values).
 #include <algorithm>
 #include <climits>
 #include <cmath>

@@ -6,7 +6,7 @@ A small command-line driver for profiling and timing through the C-ABI:
         --px 96 --py 96 --nz 300 --nt 1024 --win 61 --reps 3
 
 prints one JSON line with the mean CUDA-event time per call.  ``--op filter``
-times the band-pass filter on the signals (one k_fir_lines launch per call,
+times the band-pass filter on the signals (one kernel launch per call,
 ``--band`` and ``--filter-half`` set the FIR); ``--op sweep`` times an LSQR
 sweep over ``--damps`` Tikhonov weights.
 """
