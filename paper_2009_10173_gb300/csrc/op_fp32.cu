@@ -22,11 +22,14 @@
 //   k_corr_block  128 positions; four warps take each tap together, 32 positions each,
 //                 sharing its slab rows (a quarter of the L2 reads): large problems.
 //
-// What bounds both: the FP32 pipe (1.5x the band's products in 32-output tiles, and the
-// moves that make packed operands) at about half its rate, the rest latency between
-// taps.  One application, GB300, from a kernel without folding: 200x200x300 forward,
-// 61x61 taps, 360 -> 50 ms; 32x32x48, 11x11 taps, 283 -> 29 us (42 without clusters);
-// 70x37x52 adjoint, 15x15 taps, 888 -> 94 us (132).
+// What bounds them: k_corr_block the shared memory (84 % of its rate, with the FP32 pipe
+// at 64 %: three 16-byte reads per 16 packed products, and the folding's two reads and a
+// write per input), for 1.5x the band's products in 32-output tiles; other maps of lanes
+// to positions and outputs read more (55 and 51 ms against 50 below).  k_corr_warps the
+// chain of staging, folding and products per chunk.  One application, GB300, from a
+// kernel without folding: 200x200x300 forward, 61x61 taps, 360 -> 50 ms; 32x32x48, 11x11
+// taps, 283 -> 29 us (42 without clusters); 70x37x52 adjoint, 15x15 taps, 888 -> 94 us
+// (132).
 //
 // Each output sums up to win^2 x band products (about 3e5 at 61x61 taps).  One
 // FP32 accumulator for all of them loses about sqrt(n) units in the last place,
