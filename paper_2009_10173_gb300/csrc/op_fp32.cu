@@ -617,7 +617,9 @@ oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaSt
   }
   const bool vec = s.len % 4 == 0;
   auto fn = block ? (vec ? k_corr_block<true> : k_corr_block<false>) : (vec ? k_corr_warps<true> : k_corr_warps<false>);
-  OAM_CUDA_TRY(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  // one limit for all launches: calls from several threads would lower each other's
+  // between setting it and the launch
+  OAM_CUDA_TRY(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   ProfScope prof(m, st, fwd);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)tiles, L.tiles, Z);  // tile neighbours share slab rows

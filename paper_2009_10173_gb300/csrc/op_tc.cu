@@ -980,7 +980,7 @@ oam_status plan_launch(const oam_model *m, const TcLine *T, const TcLayout *L, L
 template <int FW, bool kWide>
 oam_status launch_corr(const Launch &lp, const TcLayout *L, dim3 grid, cudaStream_t st) {
   OAM_CUDA_TRY(
-      cudaFuncSetAttribute(k_corr_line<FW, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lp.smem));
+      cudaFuncSetAttribute(k_corr_line<FW, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
   k_corr_line<FW, kWide><<<grid, 96 + 32 * FW, lp.smem, st>>>(lp.tiling == 2 ? L->tmap_scan : L->tmap, lp.p);
   OAM_LAUNCHED();
   return OAM_OK;
