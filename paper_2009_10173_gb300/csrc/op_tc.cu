@@ -795,6 +795,40 @@ void tile_cols(int lo, int hi, int *col, int *n) {
   *n = ((hi - *col) + 15) & ~15;
 }
 
+// Blocks that share a tile's taps.  At least one per 5 1/3 pairs of taps: the tensor
+// cores truncate when they add to an accumulator, and the frequencies' sums cancel
+// over depth, so the fewer products one accumulator takes the less that costs
+// (200x200x300, 16 pairs, forward with 1, 2, 3, 4 parts: 4.7e-6, 2.3e-6, 1.5e-6,
+// 1.2e-6 against FP64, and 3.4e-6 for three BF16 products per tap with no transform;
+// 164x228x154, 11 pairs: 4.4e-6, 2.1e-6, 1.5e-6, 1.2e-6 and 1.9e-6).  Beyond
+// that, as many as finish first, in units of one pair of items (~0.55 us): a block's
+// pairs and about 18 for its set-up and epilogue, times the waves of one block per SM,
+// and a part's sums written and read once more (40 us for 62 MB).
+int choose_parts(const TcLine *T, int px, int R, int stages, int acc_cols) {
+  constexpr int kSms = 152;  // of every device: the footprint query has none to ask
+  const int NP = (R + 2) / 2;
+  const long long tiles0 = ((long long)T->nr * px + kTileM - 1) / kTileM * T->Q;
+  const double part_units = (double)T->Q * T->nr * px * acc_cols * 4.0 / (1.55e12 * 0.55e-6);
+  double best = 0;
+  int parts = 0;
+  for (int q = std::min(4, (3 * NP + 15) / 16); q <= std::min(4, NP); ++q) {
+    const double cost = (double)((tiles0 * q + kSms - 1) / kSms) * ((double)((NP + q - 1) / q) * stages + 18) +
+                        (q - 1) * part_units;
+    if (!parts || cost < best) {
+      best = cost;
+      parts = q;
+    }
+  }
+  return parts;
+}
+
+// K stages and accumulator columns of one direction for the support [n_lo, n_hi).
+void dir_sizes(int dir, int nz, int n_lo, int n_hi, int *stages, int *acc_cols) {
+  const int support = n_hi - (n_lo & ~15);
+  *stages = ((dir == 0 ? nz : support) + kStageK - 1) / kStageK;
+  *acc_cols = ((dir == 0 ? support : nz) + 15) & ~15;
+}
+
 // One direction's item and tile tables from the band form (host only): per (|a|,
 // stage) the union of the row offsets' bands.
 oam_status plan_dir(const oam_model *m, const TcLine *T, TcLayout *L, int dir, std::vector<TcItem> &items,
@@ -802,17 +836,9 @@ oam_status plan_dir(const oam_model *m, const TcLine *T, TcLayout *L, int dir, s
   const int nz = m->grid.nz, R = m->R, W = m->W;
   const int t_lo = m->n_lo & ~15;
   L->dir = dir;
-  if (dir == 0) {
-    L->stages = (nz + kStageK - 1) / kStageK;
-    L->acc_cols = ((m->n_hi - t_lo) + 15) & ~15;
-    L->out_lo = t_lo;
-    L->in_lo = 0;
-  } else {
-    L->stages = ((m->n_hi - t_lo) + kStageK - 1) / kStageK;
-    L->acc_cols = (nz + 15) & ~15;
-    L->out_lo = 0;
-    L->in_lo = t_lo;
-  }
+  dir_sizes(dir, nz, m->n_lo, m->n_hi, &L->stages, &L->acc_cols);
+  L->out_lo = dir == 0 ? t_lo : 0;
+  L->in_lo = dir == 0 ? 0 : t_lo;
   L->in_elems = kStageK * L->stages;
   if (pow2_cols(L->acc_cols) > 512) return OAM_ERR_UNSUPPORTED;
 
@@ -856,28 +882,7 @@ oam_status plan_dir(const oam_model *m, const TcLine *T, TcLayout *L, int dir, s
   }
   L->slot_bytes = (max_item + 127) & ~127;
   L->v_stride = (size_t)std::max<long long>(off, 16);
-  // Blocks that share a tile's taps.  At least one per 5 1/3 pairs of taps: the tensor
-  // cores truncate when they add to an accumulator, and the frequencies' sums cancel
-  // over depth, so the fewer products one accumulator takes the less that costs
-  // (200x200x300, 16 pairs, forward with 1, 2, 3, 4 parts: 4.7e-6, 2.3e-6, 1.5e-6,
-  // 1.2e-6 against FP64, and 3.4e-6 for three BF16 products per tap with no transform;
-  // 164x228x154, 11 pairs: 4.4e-6, 2.1e-6, 1.5e-6, 1.2e-6 and 1.9e-6).  Beyond
-  // that, as many as finish first, in units of one pair of items (~0.55 us): a block's
-  // pairs and about 18 for its set-up and epilogue, times the waves of one block per SM,
-  // and a part's sums written and read once more (40 us for 62 MB).
-  const int NP = (R + 2) / 2, sms = std::max(1, m->sm_count ? m->sm_count : 152);
-  const long long tiles0 = ((long long)T->nr * m->grid.px + kTileM - 1) / kTileM * T->Q;
-  const double part_units = (double)T->Q * T->nr * m->grid.px * L->acc_cols * 4.0 / (1.55e12 * 0.55e-6);
-  double best = 0;
-  L->parts = 0;
-  for (int q = std::min(4, (3 * NP + 15) / 16); q <= std::min(4, NP); ++q) {
-    const double cost = (double)((tiles0 * q + sms - 1) / sms) * ((double)((NP + q - 1) / q) * L->stages + 18) +
-                        (q - 1) * part_units;
-    if (!L->parts || cost < best) {
-      best = cost;
-      L->parts = q;
-    }
-  }
+  L->parts = choose_parts(T, m->grid.px, R, L->stages, L->acc_cols);
   return OAM_OK;
 }
 
@@ -1040,8 +1045,11 @@ oam_status run_corr(const oam_model *m, const TcLayout *L, const float *in, int 
   return line_c2r(T->P, st, s, T->d_part, T->d_tw, out);
 }
 
+size_t part_floats(const oam_model *m, const TcLine *T, int parts, int acc_cols) {
+  return (size_t)parts * T->Q * T->nr * m->grid.px * acc_cols;
+}
 size_t part_floats(const oam_model *m, const TcLine *T, const TcLayout *L) {
-  return (size_t)L->parts * T->Q * T->nr * m->grid.px * L->acc_cols;
+  return part_floats(m, T, L->parts, L->acc_cols);
 }
 size_t mark_words(const oam_model *m, const TcLine *T) { return (size_t)4 * m->grid.px * T->words + T->Q + 1; }
 
@@ -1065,7 +1073,15 @@ oam_status oam::tc_plan_bytes(const oam_model *m, size_t *bytes) {
     if ((rc = plan_launch(m, &T, L, &lp))) return rc;
     b += alloc_bytes<TcItem>(items.size()) + alloc_bytes<uint8_t>(L->v_stride * T.Q) +
          alloc_bytes<float>((size_t)T.rows * T.Q * L->in_elems);
-    part = std::max(part, part_floats(m, &T, L));
+    // The bands planned here are up to kSlack samples wider at either end than those of
+    // the build, and a narrower support can take more parts: the most that any of them takes.
+    constexpr int kSlack = 4;
+    for (int lo = m->n_lo; lo <= m->n_lo + kSlack; ++lo)
+      for (int hi = std::max(lo, m->n_hi - kSlack); hi <= m->n_hi; ++hi) {
+        int stages, acc;
+        dir_sizes(dir, m->grid.nz, lo, hi, &stages, &acc);
+        part = std::max(part, part_floats(m, &T, choose_parts(&T, m->grid.px, m->R, stages, acc), acc));
+      }
   }
   *bytes = b + alloc_bytes<float>(part) + alloc_bytes<float2>(T.P) + alloc_bytes<unsigned>(mark_words(m, &T)) + alloc_bytes<unsigned>(1);
   return OAM_OK;
