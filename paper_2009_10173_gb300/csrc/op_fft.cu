@@ -435,19 +435,23 @@ __global__ void __launch_bounds__(32 * kApplyWarps, 4)
 // ---------------------------------------------------------------- S^ build
 // Pass 1: T[b'][u][e] = sum_{a'=0..R} w_a' cos(2 pi u a' / P) S[b'][a'][k_e][n_e]
 // for every row entry e = (k_e, n_e); w_0 = 1, w_{>0} = 2 (the +-a' pair).
-// Block (entry block, b').
+// Block (entry block, b').  tw: the roots rounded from FP64 (none above 512 points):
+// cospif of a rounded 2 m / P, exact for powers of two alone, is off by up to 2e-7.
+__device__ __forceinline__ void load_cosines(float *cosT, const float2 *tw, int P) {
+  for (int m = threadIdx.x; m < P; m += blockDim.x) cosT[m] = tw ? tw[m].x : cospif(2.0f * (float)m / (float)P);
+  __syncthreads();
+}
 __global__ void __launch_bounds__(kBuildThreads) k_shat_pass1(const float *__restrict__ band,
                                                               const int *__restrict__ band_lo,
                                                               const int *__restrict__ band_hi, int band_w,
                                                               const int *__restrict__ tap_orbit, int R, int W,
                                                               int nz, const int2 *__restrict__ entry_kn,
                                                               long long row_len, int P, int Q,
-                                                              float *__restrict__ T) {
+                                                              const float2 *__restrict__ tw, float *__restrict__ T) {
   extern __shared__ float smb[];
   float *cosT = smb;           // [P]
   float *sv = smb + P;         // [R+1][blockDim]: weighted slab values of this thread's entry
-  for (int m = threadIdx.x; m < P; m += blockDim.x) cosT[m] = cospif(2.0f * (float)m / (float)P);
-  __syncthreads();
+  load_cosines(cosT, tw, P);
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int bp = blockIdx.y;
   if (e >= row_len) return;
@@ -474,7 +478,8 @@ __global__ void __launch_bounds__(kBuildThreads) k_shat_pass1(const float *__res
 // Pass 2: S^[r][e] = sum_{b'=0..R} w_b' cos(2 pi v0 b' / P) T[b'][u0][e] for
 // every orbit r = (v0, u0) with this u0.  Block (entry block, u0).
 __global__ void __launch_bounds__(kBuildThreads) k_shat_pass2(const float *__restrict__ T, long long row_len, int R,
-                                                              int P, int Q, const int *__restrict__ rep_of,
+                                                              int P, int Q, const float2 *__restrict__ tw,
+                                                              const int *__restrict__ rep_of,
                                                               const int2 *__restrict__ entry_kn, int n0,
                                                               const int2 *__restrict__ by_depth,
                                                               const int2 *__restrict__ by_sample,
@@ -483,8 +488,7 @@ __global__ void __launch_bounds__(kBuildThreads) k_shat_pass2(const float *__res
   extern __shared__ float smb[];
   float *cosT = smb;    // [P]
   float *tv = smb + P;  // [R+1][blockDim]
-  for (int m = threadIdx.x; m < P; m += blockDim.x) cosT[m] = cospif(2.0f * (float)m / (float)P);
-  __syncthreads();
+  load_cosines(cosT, tw, P);
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int u0 = blockIdx.y;
   if (e >= row_len) return;
@@ -711,9 +715,9 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
     OAM_CUDA_TRY(cudaFuncSetAttribute(k_shat_pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb));
   }
   k_shat_pass1<<<dim3(eblocks, R + 1), kBuildThreads, sb, st>>>(
-      m->d_band, m->d_band_lo, d_band_hi, m->band_w, m->d_tap_orbit, R, W, nz, d_entry, entries, P, Q, d_T);
+      m->d_band, m->d_band_lo, d_band_hi, m->band_w, m->d_tap_orbit, R, W, nz, d_entry, entries, P, Q, L->d_tw, d_T);
   OAM_LAUNCHED();
-  k_shat_pass2<<<dim3(eblocks, Q), kBuildThreads, sb, st>>>(d_T, entries, R, P, Q, d_rep_of, d_entry, L->n0,
+  k_shat_pass2<<<dim3(eblocks, Q), kBuildThreads, sb, st>>>(d_T, entries, R, P, Q, L->d_tw, d_rep_of, d_entry, L->n0,
                                                             L->rows[0].d_elem, L->rows[1].d_elem, L->rows[0].stride,
                                                             L->rows[1].stride, L->rows[0].d_s, L->rows[1].d_s);
   OAM_LAUNCHED();
