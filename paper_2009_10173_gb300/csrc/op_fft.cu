@@ -343,6 +343,28 @@ __device__ __forceinline__ uint64_t splat2(float v) {
   return r;
 }
 
+// Sums over the quarters of a warp's [output][member] sums; quarter ph keeps member ph.
+__device__ __forceinline__ void sum_quarters(const uint64_t (&acc)[4][4], int ph, uint64_t (&c)[4]) {
+  const bool hi = ph & 2, odd = ph & 1;
+  uint64_t b[4][2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      b[i][j] = add2(hi ? acc[i][2 + j] : acc[i][j],
+                     __shfl_xor_sync(0xffffffffu, hi ? acc[i][j] : acc[i][2 + j], 16));
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    c[i] = add2(odd ? b[i][1] : b[i][0], __shfl_xor_sync(0xffffffffu, odd ? b[i][0] : b[i][1], 8));
+}
+// Eight FP32 values' exponents below the largest.
+__device__ __forceinline__ bool all_finite(const uint64_t (&c)[4]) {
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) ok = ok && (~c[i] & 0x7f800000u) && (~c[i] >> 32 & 0x7f800000u);
+  return ok;
+}
+
 __global__ void __launch_bounds__(32 * kApplyWarps, 4)
     k_fft_apply(const float *__restrict__ S, long long stride, const int4 *__restrict__ members,
                 const int2 *__restrict__ elem, const int2 *__restrict__ window, int windows, int n_in, int in_stride,
@@ -412,17 +434,21 @@ __global__ void __launch_bounds__(32 * kApplyWarps, 4)
       for (int q = 0; q < kUnroll; ++q) v[q] = next[q];
     }
     // sum the quarters, each keeping the member of its number
-    uint64_t b[4][2], c[4];
-    const bool hi = ph & 2, odd = ph & 1;
+    uint64_t c[4];
+    sum_quarters(acc, ph, c);
+    // A lane added zeros for the elements that do not meet its group; where the sums are
+    // not finite they are taken again without those elements, so that a non-finite one
+    // reaches no sample beyond its band's groups.
+    if (__any_sync(0xffffffffu, !all_finite(c))) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 2; ++j)
-        b[i][j] = add2(hi ? acc[i][2 + j] : acc[i][j],
-                       __shfl_xor_sync(0xffffffffu, hi ? acc[i][j] : acc[i][2 + j], 16));
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      c[i] = add2(odd ? b[i][1] : b[i][0], __shfl_xor_sync(0xffffffffu, odd ? b[i][0] : b[i][1], 8));
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0;
+      for (int e = win.x + ph; e < win.y; e += 4)
+        if (g >= (E[e].y & 0xffff) && g < (int)((unsigned)E[e].y >> 16)) add(e, load(e));
+      __syncwarp();
+      sum_quarters(acc, ph, c);
+    }
     const int f = ph == 0 ? mem.x : ph == 1 ? mem.y : ph == 2 ? mem.z : mem.w;
     if (f >= 0 && 4 * g < n_out) {  // whole groups: out_stride is a multiple of 4
       ulonglong2 *o = reinterpret_cast<ulonglong2 *>(out + (size_t)f * out_stride + 4 * g);
