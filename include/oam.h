@@ -62,12 +62,19 @@ typedef enum {
   OAM_PREC_FP32 = 0,  /* plain FP32 slab and FP32 CUDA-core operators */
   OAM_PREC_BF16X3 = 1, /* two-term 16-bit splits (hi+lo) of the slab and the iterate on
                           tcgen05 tensor cores, FP32 accumulation in tensor memory:
-                          hi*hi + hi*lo + lo*hi, at least as accurate as BF16 terms
-                          (the terms are FP16 of operands scaled by powers of two).
+                          hi*hi + hi*lo + lo*hi (the terms are FP16 of operands scaled by
+                          powers of two, 22 bits together).
                           The scan's y axis is taken to the lateral frequency domain
                           by FP32 line transforms, so each frequency is a correlation
                           along x; positions whose window holds only zeros get exact
-                          zeros, those whose window holds a non-finite value NaN */
+                          zeros, those whose window holds a non-finite value NaN.
+                          Error: at most 1e-5 of a position's own output (about 2e-6;
+                          three products of BF16 terms give 1.3e-5) and 5e-7 (about
+                          2e-7) of the strongest output on the lines along y through
+                          its window: a position whose window holds nothing above
+                          1/60 of what stands elsewhere on those lines is less exact
+                          relative to its own output than a direct sum of BF16 terms,
+                          as in the lateral-FFT form; OAM_PREC_FP32 sums directly */
   OAM_PREC_FFT = 2     /* FP32 lateral-FFT form of the same operators: both are 2-D
                           correlations over the scan grid (Methods, Efficient
                           reconstruction based on scanning symmetries), restated

@@ -207,7 +207,7 @@ struct LineShape {
   int out_len, out_lo, acc, parts;  // output row length, output channel of accumulator column 0, columns, partial sums
   int words;               // 32-row mark words per column
   unsigned *marks;         // [2][px][words]: positions with a non-zero, with a non-finite input
-  unsigned *vmax;          // [frequencies] largest magnitude of the transformed lines, as float bits
+  unsigned *vmax;          // [frequencies][px] largest magnitude of the transformed lines, as float bits
   int *any_bad;            // some position has a non-finite input
   const unsigned *grown;   // [2][px][words]: positions whose window holds one
   __host__ __device__ int out_row(int seg) const { return seg * valid; }  // first output row of a segment

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>())
       }
       top = fmaxf(fmaxf(fabsf(re.x), fabsf(re.y)), fmaxf(fabsf(im.x), fabsf(im.y)));
     }
-    // the frequency's largest magnitude (non-negative floats compare as integers)
+    // the frequency's largest magnitude on this line (non-negative floats compare as integers)
     unsigned t = __float_as_uint(top);
 #pragma unroll
     for (int off = kKH / 2; off; off >>= 1) t = max(t, __shfl_xor_sync(0xffffffffu, t, off));
@@ -120,8 +120,10 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>())
     }
   }
   __syncthreads();
-  for (int u = threadIdx.x; u < Q; u += blockDim.x)
-    if (umax[u] > __ldcg(s.vmax + u)) atomicMax(s.vmax + u, umax[u]);
+  for (int u = threadIdx.x; u < Q; u += blockDim.x) {
+    unsigned *top = s.vmax + (size_t)u * s.px + x;
+    if (umax[u] > __ldcg(top)) atomicMax(top, umax[u]);
+  }
 }
 
 // kVec: output rows are a whole number of float2 from an 8-byte boundary.
@@ -141,10 +143,8 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>(), R1 >= 15 && R2 <= 
   if (blockIdx.x == 0 && blockIdx.z == 0) {
     for (int i = threadIdx.x; i < 2 * s.words; i += blockDim.x)
       s.marks[(size_t)(i < s.words ? x : s.px + x) * s.words + i % s.words] = 0;
-    if (x == 0) {
-      for (int i = threadIdx.x; i < Q; i += blockDim.x) s.vmax[i] = 0;
-      if (threadIdx.x == 0) *s.any_bad = 0;
-    }
+    for (int i = threadIdx.x; i < Q; i += blockDim.x) s.vmax[(size_t)i * s.px + x] = 0;
+    if (x == 0 && threadIdx.x == 0) *s.any_bad = 0;
   }
   const int w0 = ya >> 5, nw = ((yb - 1) >> 5) - w0 + 1;
   for (int i = threadIdx.x; i < 2 * nw; i += blockDim.x)

@@ -46,8 +46,8 @@
 // folded iterate: D += F_hi S_hi + F_hi S_lo + F_lo S_hi, accumulated in FP32 in
 // tensor memory.  The terms are FP16 (22 significant bits together, BF16 terms
 // hold 16) of operands scaled by powers of two: the slab by one for the model,
-// the iterate by one for each frequency, from the magnitudes that the line
-// transform finds.  The taps of a tile go to up to four blocks, whose partial sums the
+// the iterate by one for each frequency and row, from the magnitudes that the line
+// transform finds on the lines of the row's window.  The taps of a tile go to up to four blocks, whose partial sums the
 // inverse line transform adds in index order.  (Adding them in clusters through
 // distributed shared memory was slower: 9000 cycles a block for two blocks' sums, and
 // clusters of four leave SMs idle.)
@@ -120,7 +120,7 @@ struct TcLine {
   int nr = 0, rows = 0;       // packed rows and positions per frequency
   int words = 0;              // mark words per column
   float2 *d_tw = nullptr;     // [P] roots
-  unsigned *d_marks = nullptr;  // [2][px][words], [Q] magnitudes, the non-finite flag, [2][px][words] grown
+  unsigned *d_marks = nullptr;  // [2][px][words], [Q][px] magnitudes, the non-finite flag, [2][px][words] grown
   unsigned *d_smax = nullptr;   // bound of the transformed slab's magnitude, as float bits
   float *d_part = nullptr;    // partial sums [parts][Q][nr][px][acc_cols]
 };
@@ -142,7 +142,7 @@ struct CorrParams {
   unsigned *grown;        // [2][px][words]: positions whose window holds one
   const int *any_bad;     // some position has a non-finite input
   int words;
-  const unsigned *vmax;  // [frequencies] largest magnitude of the transformed lines, as float bits
+  const unsigned *vmax;  // [frequencies][px] largest magnitude of the transformed lines, as float bits
   const unsigned *smax;  // the slab's, over its transform (an upper bound)
   float *part;         // partial sums [parts][frequencies][nr][px][acc_cols]
   float *out;          // the operator's output [positions][out_len]: channels outside z0 .. z1 are zeroed here
@@ -368,6 +368,7 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + 512);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + 516);
   volatile int *never = reinterpret_cast<volatile int *>(smem + 520);  // stays 0: waits that ignore abort
+  uint8_t *line_exp = smem + 640;  // [strip_rows <= 256] biased exponents of the strip's lines (0: padding)
   TcItem *sitems = reinterpret_cast<TcItem *>(smem + 1024);           // [stages][nj]: this part's items
   uint8_t *strips = smem + 1024 + p.items_bytes;                       // [3][strip_bytes]: stage st in buffer st % 3
   uint8_t *slots = strips + 3 * p.strip_bytes;                         // [K][slot_bytes]
@@ -404,6 +405,10 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
   }
   for (int i = threadIdx.x; i < p.stages * nj; i += kThreads)
     sitems[i] = p.items[a_of(j0 + i % nj, R) * p.stages + i / nj];
+  for (int i = threadIdx.x; i < L; i += kThreads) {
+    const int q = r0 * p.wp + x0 - R + i, x = q < 0 ? p.px : q % p.wp;
+    line_exp[i] = x < p.px ? (uint8_t)(__ldg(p.vmax + (size_t)freq * p.px + x) >> 23) : 0;
+  }
   if (warp == 1) {
     ptx::tmem_alloc(tmem_slot, p.tmem_cols);
     ptx::tmem_relinquish();
@@ -551,7 +556,12 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
     const int row = o / p.sp, x = o % p.sp;
     const int pm = (row - r0) * p.wp + (x - x0);  // its packed offset from the tile's first
     const int q0 = kq * (E / 8);        // first 8-element quarter of the stage
-    const int ef = scale_exp(2.0f * __uint_as_float(p.vmax[freq]));
+    // The row's own scale, from the largest magnitude of the lines in its window: one of the
+    // whole scan would leave FP16's range to columns 1e-6 below its strongest.
+    int top = 0;
+#pragma unroll 8
+    for (int i = pm; i <= pm + 2 * R; ++i) top = max(top, (int)line_exp[i]);
+    const int ef = min(126, 140 - top);  // the fold doubles: into [2^14, 2^15), below FP16's largest 65504
     const uint64_t sc = pack_f32x2(pow2(ef), pow2(ef));
     int k = 0;
     uint32_t lap = 0;
@@ -1025,10 +1035,10 @@ oam_status run_corr(const oam_model *m, const TcLayout *L, const float *in, int 
   s.marks = T->d_marks;
   unsigned *tail = T->d_marks + (size_t)2 * s.px * s.words;
   s.vmax = tail;
-  s.any_bad = reinterpret_cast<int *>(tail + T->Q);
-  s.grown = tail + T->Q + 1;
+  s.any_bad = reinterpret_cast<int *>(tail + (size_t)s.px * T->Q);
+  s.grown = tail + (size_t)s.px * T->Q + 1;
   lp.p.marks = s.marks;
-  lp.p.grown = tail + T->Q + 1;
+  lp.p.grown = tail + (size_t)s.px * T->Q + 1;
   lp.p.any_bad = s.any_bad;
   lp.p.words = T->words;
   s.parts = L->parts;
@@ -1051,7 +1061,7 @@ size_t part_floats(const oam_model *m, const TcLine *T, int parts, int acc_cols)
 size_t part_floats(const oam_model *m, const TcLine *T, const TcLayout *L) {
   return part_floats(m, T, L->parts, L->acc_cols);
 }
-size_t mark_words(const oam_model *m, const TcLine *T) { return (size_t)4 * m->grid.px * T->words + T->Q + 1; }
+size_t mark_words(const oam_model *m, const TcLine *T) { return (size_t)m->grid.px * (4 * T->words + T->Q) + 1; }
 
 }  // namespace
 
