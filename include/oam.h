@@ -67,7 +67,8 @@ typedef enum {
                           The scan's y axis is taken to the lateral frequency domain
                           by FP32 line transforms, so each frequency is a correlation
                           along x; positions whose window holds only zeros get exact
-                          zeros, those whose window holds a non-finite value NaN.
+                          zeros, those whose window holds a non-finite value NaN in
+                          the samples (depths) that its 32-channel block reaches.
                           Error: at most 1e-5 of a position's own output (about 2e-6;
                           three products of BF16 terms give 1.3e-5) and 5e-7 (about
                           2e-7) of the strongest output on the lines along y through

@@ -206,10 +206,15 @@ struct LineShape {
   int nr;                  // packed rows per frequency: 2 segs (re and im)
   int out_len, out_lo, acc, parts;  // output row length, output channel of accumulator column 0, columns, partial sums
   int words;               // 32-row mark words per column
-  unsigned *marks;         // [2][px][words]: positions with a non-zero, with a non-finite input
+  // Marks, a bit per position of a column: plane 0 those with a non-zero input, plane 1 + b
+  // those with a non-finite one among the packed channels 32 b .. 32 b + 31.
+  int planes;
+  unsigned *marks;         // [planes][px][words]
   unsigned *vmax;          // [frequencies][px] largest magnitude of the transformed lines, as float bits
   int *any_bad;            // some position has a non-finite input
-  const unsigned *grown;   // [2][px][words]: positions whose window holds one
+  const unsigned *grown;   // [planes][px][words]: positions whose window holds one
+  const int *spoiled;      // any_bad while the marks were grown
+  const int2 *reach;       // [planes - 1] accumulator columns [x, y) that a plane's channels reach
   __host__ __device__ int out_row(int seg) const { return seg * valid; }  // first output row of a segment
   __host__ __device__ int first_row(int seg) const { return segs > 1 ? seg * valid - halo : 0; }  // point 0's row
 };

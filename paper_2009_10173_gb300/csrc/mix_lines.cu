@@ -16,12 +16,13 @@
 //
 // The correlation has compact support: a position whose window holds only zeros
 // gets exact zeros, and a non-finite input reaches only the positions whose window
-// holds it.  A transform along y would spread both over the line.  So the forward
-// transform marks the positions that hold a non-zero and those that hold a
-// non-finite value (taken as zero by the transform), one bit each; a spare warp of
-// the correlation kernel grows the marks by the window while the products run
-// (op_tc.cu); the inverse writes zeros where the window of an output position holds
-// no input, NaN where it holds a non-finite one, and clears the marks.
+// holds it, and of those the samples (depths) that the slab couples with its channel.
+// A transform along y would spread both over the line.  So the forward transform marks
+// the positions that hold a non-zero and, per 32 channels, those that hold a non-finite
+// value (taken as zero by the transform), one bit each; a spare warp of the correlation
+// kernel grows the marks by the window while the products run (op_tc.cu); the inverse
+// writes zeros where the window of an output position holds no input, NaN in the 32
+// channels that a non-finite one reaches, and clears the marks.
 #include <algorithm>
 #include <cfloat>
 
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>())
     if ((threadIdx.x & 31) == 0) {
       mark_rows(s.marks + (size_t)x * s.words, y0 + 32 * w, b);
       if (n) {
-        mark_rows(s.marks + (size_t)(s.px + x) * s.words, y0 + 32 * w, n);
+        mark_rows(s.marks + ((size_t)(1 + blockIdx.x) * s.px + x) * s.words, y0 + 32 * w, n);
         *s.any_bad = 1;
       }
     }
@@ -141,16 +142,24 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>(), R1 >= 15 && R2 <= 
   const int cols = min(kLineCh, s.out_len - ob);
   // this application's marks are grown: clear them for the next
   if (blockIdx.x == 0 && blockIdx.z == 0) {
-    for (int i = threadIdx.x; i < 2 * s.words; i += blockDim.x)
-      s.marks[(size_t)(i < s.words ? x : s.px + x) * s.words + i % s.words] = 0;
+    const int planes = *s.spoiled ? s.planes : 1;
+    for (int i = threadIdx.x; i < planes * s.words; i += blockDim.x)
+      s.marks[((size_t)(i / s.words) * s.px + x) * s.words + i % s.words] = 0;
     for (int i = threadIdx.x; i < Q; i += blockDim.x) s.vmax[(size_t)i * s.px + x] = 0;
     if (x == 0 && threadIdx.x == 0) *s.any_bad = 0;
   }
   const int w0 = ya >> 5, nw = ((yb - 1) >> 5) - w0 + 1;
-  for (int i = threadIdx.x; i < 2 * nw; i += blockDim.x)
-    words[i / nw][i % nw] = __ldg(s.grown + (size_t)(i < nw ? x : s.px + x) * s.words + w0 + i % nw);
-  const size_t f_off = (size_t)s.nr * s.px * s.acc, im_off = (size_t)s.px * s.acc, p_off = Q * f_off;
   const int z0 = ob - s.out_lo;  // accumulator column of the block's first channel (even: out_lo is 16-aligned)
+  for (int i = threadIdx.x; i < nw; i += blockDim.x) {
+    const size_t at = (size_t)x * s.words + w0 + i, plane = (size_t)s.px * s.words;
+    words[0][i] = __ldg(s.grown + at);
+    unsigned bad = 0;
+    if (*s.spoiled)
+      for (int b = 0; b < s.planes - 1; ++b)
+        if (s.reach[b].x < z0 + kLineCh && s.reach[b].y > z0) bad |= __ldg(s.grown + (1 + b) * plane + at);
+    words[1][i] = bad;
+  }
+  const size_t f_off = (size_t)s.nr * s.px * s.acc, im_off = (size_t)s.px * s.acc, p_off = Q * f_off;
   const float *zc = part + ((size_t)(2 * blockIdx.z) * s.px + x) * s.acc + z0;
   auto load = [&](int i2, int l, float2 (&v)[R1]) {
     const bool ok = z0 + 2 * l >= 0 && z0 + 2 * l < s.acc;

@@ -108,6 +108,8 @@ struct TcLayout {
   uint8_t *d_data = nullptr;  // [P/2 + 1][v_stride]
   size_t v_stride = 0;        // bytes of one frequency's tiles
   float *d_pack = nullptr;    // packed input [(P/2 + 1) rows][in_elems]
+  std::vector<int2> reach;    // [stages] accumulator columns [x, y) that a stage's elements reach
+  int2 *d_reach = nullptr;
   CUtensorMap tmap;       // FP32 packed input [qtot][in_elems], box 32 x (128 + 2R), 128-byte swizzle
   CUtensorMap tmap_scan;  // the same with the scan-grid strip positions (when they fit one box)
 };
@@ -118,9 +120,9 @@ struct TcLine {
   int halo = 0;               // rows coupled along y: min(R, py - 1)
   int segs = 1, valid = 0;    // segments of a line, output rows of each
   int nr = 0, rows = 0;       // packed rows and positions per frequency
-  int words = 0;              // mark words per column
+  int words = 0, planes = 0;  // mark words per column, planes (LineShape) of the direction with more
   float2 *d_tw = nullptr;     // [P] roots
-  unsigned *d_marks = nullptr;  // [2][px][words], [Q][px] magnitudes, the non-finite flag, [2][px][words] grown
+  unsigned *d_marks = nullptr;  // [planes][px][words], [Q][px] magnitudes, two flags, [planes][px][words] grown
   unsigned *d_smax = nullptr;   // bound of the transformed slab's magnitude, as float bits
   float *d_part = nullptr;    // partial sums [parts][Q][nr][px][acc_cols]
 };
@@ -138,10 +140,11 @@ struct CorrParams {
   size_t v_stride;
   int slot_bytes, n_items, strip_rows, strip_bytes, items_bytes;
   int acc_cols, tmem_cols, fold_col0;
-  const unsigned *marks;  // [2][px][words]: positions with a non-zero, with a non-finite input
-  unsigned *grown;        // [2][px][words]: positions whose window holds one
+  const unsigned *marks;  // [planes][px][words] (LineShape): positions with a non-zero, with a non-finite input
+  unsigned *grown;        // [planes][px][words]: positions whose window holds one
   const int *any_bad;     // some position has a non-finite input
-  int words;
+  int *spoiled;           // the same, for the inverse transform
+  int words, planes;
   const unsigned *vmax;  // [frequencies][px] largest magnitude of the transformed lines, as float bits
   const unsigned *smax;  // the slab's, over its transform (an upper bound)
   float *part;         // partial sums [parts][frequencies][nr][px][acc_cols]
@@ -306,14 +309,14 @@ __device__ __forceinline__ void mma_cols(uint32_t d, uint32_t a, uint64_t b, uin
 // R rows: one warp, lanes over columns, then over the rows of a word.
 __device__ __forceinline__ void grow_marks(const CorrParams &p, int x, int lane) {
   const int xa = max(0, x - p.R), xb = min(p.px - 1, x + p.R);
-  const bool bad = *p.any_bad != 0;
-  for (int which = 0; which < 2; ++which) {
+  const int planes = *p.any_bad ? p.planes : 1;
+  for (int which = 0; which < planes; ++which) {
     const unsigned *src = p.marks + (size_t)(which * p.px) * p.words;
     unsigned *dst = p.grown + (size_t)(which * p.px + x) * p.words;
     unsigned win[5] = {0, 0, 0, 0, 0};  // words w - 2 .. w + 2 (R <= 64)
     for (int j = -2; j < p.words; ++j) {  // word j + 2 joins; word j is complete
       unsigned m = 0;
-      if (j + 2 < p.words && (which == 0 || bad))
+      if (j + 2 < p.words)
         for (int xx = xa + lane; xx <= xb; xx += 32) m |= __ldcg(src + (size_t)xx * p.words + j + 2);
 #pragma unroll
       for (int i = 0; i < 4; ++i) win[i] = win[i + 1];
@@ -534,6 +537,7 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
   } else if (warp == 2 + kFoldWarps) {
     // ------------------------------------------------------------ marks, zeros
     zero_outside(p, lane);
+    if (lane == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) *p.spoiled = *p.any_bad;
     if (blockIdx.y == 0)
       for (int x = freq * gridDim.x + tile; x < p.px; x += gridDim.z * gridDim.x) grow_marks(p, x, lane);
   } else {
@@ -853,6 +857,7 @@ oam_status plan_dir(const oam_model *m, const TcLine *T, TcLayout *L, int dir, s
   if (pow2_cols(L->acc_cols) > 512) return OAM_ERR_UNSUPPORTED;
 
   items.assign((size_t)(R + 1) * L->stages, TcItem{});
+  L->reach.assign(L->stages, make_int2(L->acc_cols, 0));
   tiles.clear();
   long long off = 0;
   int max_item = 16;
@@ -879,6 +884,7 @@ oam_status plan_dir(const oam_model *m, const TcLine *T, TcLayout *L, int dir, s
         if (hi <= lo) continue;
         int col, n;
         tile_cols(lo, hi, &col, &n);
+        L->reach[s] = make_int2(std::min(L->reach[s].x, col), std::max(L->reach[s].y, col + n));
         it.c16[c] = (uint8_t)(col / 16);
         it.n16[c] = (uint8_t)(n / 16);
         L->wide = L->wide || n > 256;
@@ -908,6 +914,8 @@ oam_status build_dir(oam_model *m, TcLayout *L, int dir, cudaStream_t st, int *d
   if ((rc = dev_alloc(m, &L->d_items, items.size()))) return rc;
   if ((rc = dev_alloc(m, &L->d_data, L->v_stride * T->Q))) return rc;
   if ((rc = dev_alloc(m, &L->d_pack, qtot * L->in_elems))) return rc;
+  if ((rc = dev_alloc(m, &L->d_reach, L->reach.size()))) return rc;
+  OAM_CUDA_TRY(cudaMemcpyAsync(L->d_reach, L->reach.data(), sizeof(int2) * L->reach.size(), cudaMemcpyHostToDevice, st));
   OAM_CUDA_TRY(cudaMemcpyAsync(L->d_items, items.data(), sizeof(TcItem) * items.size(), cudaMemcpyHostToDevice, st));
   // padding positions and channels stay zero: the line transform writes the others
   OAM_CUDA_TRY(cudaMemsetAsync(L->d_pack, 0, sizeof(float) * qtot * L->in_elems, st));
@@ -1033,14 +1041,20 @@ oam_status run_corr(const oam_model *m, const TcLayout *L, const float *in, int 
   s.acc = L->acc_cols;
   s.words = T->words;
   s.marks = T->d_marks;
-  unsigned *tail = T->d_marks + (size_t)2 * s.px * s.words;
+  s.planes = 1 + L->stages;
+  unsigned *tail = T->d_marks + (size_t)T->planes * s.px * s.words;
   s.vmax = tail;
-  s.any_bad = reinterpret_cast<int *>(tail + (size_t)s.px * T->Q);
-  s.grown = tail + (size_t)s.px * T->Q + 1;
+  tail += (size_t)s.px * T->Q;
+  s.any_bad = reinterpret_cast<int *>(tail);
+  lp.p.spoiled = s.any_bad + 1;
+  s.spoiled = lp.p.spoiled;
+  s.grown = tail + 2;
+  s.reach = L->d_reach;
   lp.p.marks = s.marks;
-  lp.p.grown = tail + (size_t)s.px * T->Q + 1;
+  lp.p.grown = tail + 2;
   lp.p.any_bad = s.any_bad;
-  lp.p.words = T->words;
+  lp.p.words = s.words;
+  lp.p.planes = s.planes;
   s.parts = L->parts;
   lp.p.out = out;
   lp.p.positions = s.px * s.py;
@@ -1061,7 +1075,9 @@ size_t part_floats(const oam_model *m, const TcLine *T, int parts, int acc_cols)
 size_t part_floats(const oam_model *m, const TcLine *T, const TcLayout *L) {
   return part_floats(m, T, L->parts, L->acc_cols);
 }
-size_t mark_words(const oam_model *m, const TcLine *T) { return (size_t)m->grid.px * (4 * T->words + T->Q) + 1; }
+size_t mark_words(const oam_model *m, const TcLine *T) {
+  return (size_t)m->grid.px * ((size_t)2 * T->planes * T->words + T->Q) + 2;
+}
 
 }  // namespace
 
@@ -1081,7 +1097,8 @@ oam_status oam::tc_plan_bytes(const oam_model *m, size_t *bytes) {
     if ((rc = plan_dir(m, &T, L, dir, items, tiles))) return rc;
     Launch lp;
     if ((rc = plan_launch(m, &T, L, &lp))) return rc;
-    b += alloc_bytes<TcItem>(items.size()) + alloc_bytes<uint8_t>(L->v_stride * T.Q) +
+    T.planes = std::max(T.planes, 1 + L->stages);
+    b += alloc_bytes<TcItem>(items.size()) + alloc_bytes<int2>(L->stages) + alloc_bytes<uint8_t>(L->v_stride * T.Q) +
          alloc_bytes<float>((size_t)T.rows * T.Q * L->in_elems);
     // The bands planned here are up to kSlack samples wider at either end than those of
     // the build, and a narrower support can take more parts: the most that any of them takes.
@@ -1103,11 +1120,8 @@ oam_status oam::tc_build(oam_model *m, cudaStream_t st) {
   oam_status rc = plan_line(m, T);
   if (rc) return rc;
   const std::vector<float2> roots = mix_roots(T->P);
-  if ((rc = dev_alloc(m, &T->d_tw, roots.size())) || (rc = dev_alloc(m, &T->d_marks, mark_words(m, T))) ||
-      (rc = dev_alloc(m, &T->d_smax, 1)))
-    return rc;
+  if ((rc = dev_alloc(m, &T->d_tw, roots.size())) || (rc = dev_alloc(m, &T->d_smax, 1))) return rc;
   OAM_CUDA_TRY(cudaMemcpyAsync(T->d_tw, roots.data(), sizeof(float2) * roots.size(), cudaMemcpyHostToDevice, st));
-  OAM_CUDA_TRY(cudaMemsetAsync(T->d_marks, 0, sizeof(unsigned) * mark_words(m, T), st));
   OAM_CUDA_TRY(cudaMemsetAsync(T->d_smax, 0, sizeof(unsigned), st));
   const size_t nb = (size_t)m->n_orb * m->grid.nz;
   k_slab_max<<<4 * std::max(1, m->sm_count), 256, 0, st>>>(m->d_band, nb * m->band_w, (float)m->W, T->d_smax);
@@ -1124,14 +1138,17 @@ oam_status oam::tc_build(oam_model *m, cudaStream_t st) {
   for (TcLayout *L : {m->tc_fwd, m->tc_adj}) {
     Launch lp;
     if ((rc = plan_launch(m, T, L, &lp))) return rc;
+    T->planes = std::max(T->planes, 1 + L->stages);
   }
+  if ((rc = dev_alloc(m, &T->d_marks, mark_words(m, T)))) return rc;
+  OAM_CUDA_TRY(cudaMemsetAsync(T->d_marks, 0, sizeof(unsigned) * mark_words(m, T), st));
   return dev_alloc(m, &T->d_part, std::max(part_floats(m, T, m->tc_fwd), part_floats(m, T, m->tc_adj)));
 }
 
 void oam::tc_free(oam_model *m, cudaStream_t st) {
   for (TcLayout *L : {m->tc_fwd, m->tc_adj}) {
     if (!L) continue;
-    for (void *p : {(void *)L->d_items, (void *)L->d_data, (void *)L->d_pack})
+    for (void *p : {(void *)L->d_items, (void *)L->d_data, (void *)L->d_pack, (void *)L->d_reach})
       if (p) cudaFreeAsync(p, st);
     delete L;
   }

@@ -41,3 +41,41 @@ def test_fft_form_keeps_other_bands_finite(direction, value):
         assert bad[meets[e]].all()
         assert not (bad & ~reach).any() and not reach.all()
     m.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("direction", ["forward", "adjoint"])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_split_form_keeps_other_bands(direction, value):
+    """Positions outside the window are untouched; inside it, the outputs that the 32 channels
+    around the value do not reach are those of the same input with a zero in its place."""
+    import torch
+
+    from paper_2009_10173_gb300 import binding as B
+    cfg, meets, m = setup(B.OAM_PREC_BF16X3, px=20, py=30, nz=192, dz_m=8e-6, z0_rel_m=-192 * 4e-6, nt=768)
+    op = getattr(m, direction)
+    if direction == "adjoint":
+        meets = meets.T
+    n, partial = np.flatnonzero(meets.any(1)), False
+    for e in (int(n[0]), int(n[len(n) // 2]), int(n[-1])):
+        x = torch.randn(m.vol_shape if direction == "forward" else m.sig_shape, device="cuda")
+        x[15, 8, e] = 0
+        want = op(x).clone()
+        x[15, 8, e] = value
+        got = op(x)
+        bad = ~torch.isfinite(got)
+        window = torch.zeros_like(bad)
+        window[13:18, 6:11] = True
+        assert not (bad & ~window).any()
+        here = bad[13:18, 6:11].any(0).any(0).cpu().numpy()
+        o = np.flatnonzero(meets[max(0, e - 47):e + 48].any(0))
+        reach = np.zeros_like(here)
+        reach[max(0, o[0] - 48):o[-1] + 49] = True
+        assert here[meets[e]].all() and not (here & ~reach).any()
+        partial = partial or not reach.all()
+        keep = ~bad
+        assert torch.equal(got[keep], want[keep])
+        x[15, 8, e] = 0  # nothing of the marks is left
+        assert torch.equal(op(x), want)
+    assert partial
+    m.close()
