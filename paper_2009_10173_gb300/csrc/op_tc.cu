@@ -1016,6 +1016,10 @@ oam_status launch_corr_fw(const Launch &lp, const TcLayout *L, dim3 grid, cudaSt
   return launch_corr<8, kWide>(lp, L, grid, st);
 }
 
+size_t mark_words(const oam_model *m, const TcLine *T) {
+  return (size_t)m->grid.px * ((size_t)2 * T->planes * T->words + T->Q) + 2;
+}
+
 oam_status run_corr(const oam_model *m, const TcLayout *L, const float *in, int in_len, float *out, int out_len,
                     cudaStream_t st) {
   const TcLine *T = m->tc_line;
@@ -1063,10 +1067,13 @@ oam_status run_corr(const oam_model *m, const TcLayout *L, const float *in, int 
   lp.p.vmax = s.vmax;
   lp.p.smax = T->d_smax;
   ProfScope prof(m, st, L->dir == 0);
-  if ((rc = line_r2c(T->P, st, s, in, T->d_tw, L->d_pack))) return rc;
   const dim3 grid(lp.n_tiles, L->parts, T->Q);
-  if ((rc = L->wide ? launch_corr_fw<true>(lp, L, grid, st) : launch_corr_fw<false>(lp, L, grid, st))) return rc;
-  return line_c2r(T->P, st, s, T->d_part, T->d_tw, out);
+  rc = line_r2c(T->P, st, s, in, T->d_tw, L->d_pack);
+  if (!rc) rc = L->wide ? launch_corr_fw<true>(lp, L, grid, st) : launch_corr_fw<false>(lp, L, grid, st);
+  if (!rc) rc = line_c2r(T->P, st, s, T->d_part, T->d_tw, out);
+  // the inverse clears the marks and magnitudes; without it they would reach the next application
+  if (rc) cudaMemsetAsync(T->d_marks, 0, sizeof(unsigned) * mark_words(m, T), st);
+  return rc;
 }
 
 size_t part_floats(const oam_model *m, const TcLine *T, int parts, int acc_cols) {
@@ -1074,9 +1081,6 @@ size_t part_floats(const oam_model *m, const TcLine *T, int parts, int acc_cols)
 }
 size_t part_floats(const oam_model *m, const TcLine *T, const TcLayout *L) {
   return part_floats(m, T, L->parts, L->acc_cols);
-}
-size_t mark_words(const oam_model *m, const TcLine *T) {
-  return (size_t)m->grid.px * ((size_t)2 * T->planes * T->words + T->Q) + 2;
 }
 
 }  // namespace
