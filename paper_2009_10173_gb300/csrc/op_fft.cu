@@ -736,9 +736,10 @@ oam_status oam::fft_build(oam_model *m, cudaStream_t st) {
   cudaMemcpyAsync(d_rep_of, rep_of.data(), sizeof(int) * rep_of.size(), cudaMemcpyHostToDevice, st);
   const unsigned eblocks = (unsigned)((entries + kBuildThreads - 1) / kBuildThreads);
   const size_t sb = sizeof(float) * ((size_t)P + (size_t)(R + 1) * kBuildThreads);
-  if (sb > 48 * 1024) {
-    OAM_CUDA_TRY(cudaFuncSetAttribute(k_shat_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb));
-    OAM_CUDA_TRY(cudaFuncSetAttribute(k_shat_pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb));
+  if (sb > 48 * 1024) {  // one limit for every model: builds from several threads would lower each other's
+    const int limit = std::max<int>((int)sb, 227 * 1024);
+    OAM_CUDA_TRY(cudaFuncSetAttribute(k_shat_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+    OAM_CUDA_TRY(cudaFuncSetAttribute(k_shat_pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
   }
   k_shat_pass1<<<dim3(eblocks, R + 1), kBuildThreads, sb, st>>>(
       m->d_band, m->d_band_lo, d_band_hi, m->band_w, m->d_tap_orbit, R, W, nz, d_entry, entries, P, Q, L->d_tw, d_T);

@@ -915,7 +915,9 @@ oam_status oam::build_slab(oam_model *m, cudaStream_t st) {
     const size_t sm = sizeof(double) * (2 * g3.T + 1 + (size_t)k33Chunk * g3.len) + sizeof(int) * (k33Chunk + 2) +
                       sizeof(double) * k33Chunk;
     if (threads > 1024 || sm > 200 * 1024) return OAM_ERR_UNSUPPORTED;
-    if (sm > 48 * 1024) OAM_CUDA_TRY(cudaFuncSetAttribute(k_slab33_values, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > 48 * 1024)  // one limit for every model: builds from several threads would lower each other's
+      OAM_CUDA_TRY(
+          cudaFuncSetAttribute(k_slab33_values, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     k_slab33_values<<<dim3(O, nz), threads, sm, st>>>(g3, m->d_patch, m->M, d_orb_b, d_orb_a, nz, nt, m->d_band_lo,
                                                       d_band_hi, m->band_w, m->d_band);
   } else {
