@@ -18,8 +18,16 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// A coefficient as a pair of FP32 terms: rounded to one, and with th / beta rounded before
+// the difference in k_lsqr_v, 30 steps at 128x128x192 ended 2.79e-6 from FP64, so 2.76e-6.
+struct F2 {
+  float h, l;
+};
+__device__ __forceinline__ F2 split2(double v) { return F2{(float)v, (float)(v - (double)(float)v)}; }
+
 struct Scalars {
   // LSQR
+  F2 u_old, v_new, v_old;  // coefficients of the last u (alpha / beta) and of A^T u and the last v (1 / beta, beta)
   double alpha, beta, rhobar, phibar, damp;
   double inv_alpha, inv_beta, cx, cw;
   double anorm2, arnorm;
@@ -189,6 +197,7 @@ __global__ void k_lsqr_alpha0(const float *th, size_t n, Scalars *S, DampState *
   if (finish_blocks<false>(S, acc, 0.0, &ta, &tb) && threadIdx.x == 0) {
     S->alpha = sqrt(ta);
     S->inv_alpha = S->alpha > 0 ? 1.0 / S->alpha : 0.0;
+    S->u_old = split2(S->alpha);  // the first u is normalised
     if (!(S->alpha > 0)) S->stop_at = -1;
     S->rhobar = S->alpha;
     S->phibar = S->beta;
@@ -220,12 +229,6 @@ __global__ void k_lsqr_vw0(const float *th, float *v, float *w, float *x, size_t
   }
 }
 
-// A coefficient as a pair of FP32 terms: rounded to one, and with th / beta rounded before
-// the difference, 30 steps at 128x128x192 ended 2.79e-6 from FP64, so 2.76e-6.
-struct F2 {
-  float h, l;
-  __device__ __forceinline__ explicit F2(double v) : h((float)v), l((float)(v - (double)h)) {}
-};
 // y - a x and a x - b y, rounded once but for terms of the second order.
 __device__ __forceinline__ float nmul_add(F2 a, float x, float y) { return fmaf(-a.l, x, fmaf(-a.h, x, y)); }
 __device__ __forceinline__ float mul_sub(F2 a, float x, F2 b, float y) {
@@ -246,7 +249,7 @@ __device__ __forceinline__ float4 mul_sub4(F2 a, float4 x, F2 b, float4 y) {
 // A pass saved is 100 MB at 128x128x768 (13 us of a 330 us step) and a launch of six.
 __global__ void k_lsqr_u(const float *ts, float *u, size_t n, Scalars *S, int it, DampState *D, int nd) {
   if (it > S->stop_at) return;
-  const F2 al(it ? mul_rn(S->alpha, S->inv_beta) : S->alpha);
+  const F2 al = S->u_old;
   double acc = 0;
   const size_t hop = (size_t)gridDim.x * blockDim.x, n4 = n / 4;
   size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
@@ -272,6 +275,8 @@ __global__ void k_lsqr_u(const float *ts, float *u, size_t n, Scalars *S, int it
   if (finish_blocks<false>(S, acc, 0.0, &ta, &tb) && threadIdx.x == 0) {
     S->beta = sqrt(ta);
     S->inv_beta = S->beta > 0 ? 1.0 / S->beta : 0.0;
+    S->v_new = split2(S->inv_beta);
+    S->v_old = split2(S->beta);
     S->anorm2 = __dadd_rn(S->anorm2, sumsq_rn(S->beta, S->damp));
     for (int i = 0; i < nd; ++i) D[i].anorm2 = __dadd_rn(D[i].anorm2, sumsq_rn(S->beta, D[i].damp));
     if (!(S->beta > 0)) S->stop_at = it;
@@ -303,7 +308,7 @@ __device__ __forceinline__ void lsqr_rotate(double alpha, double beta, double da
 // solve's own damp and for each of the nd damps of a sweep in D.
 __global__ void k_lsqr_v(const float *th, float *v, size_t n, Scalars *S, int it, DampState *D, int nd) {
   if (it > S->stop_at) return;
-  const F2 be(S->beta), ib(S->inv_beta);
+  const F2 be = S->v_old, ib = S->v_new;
   double acc = 0;
   const size_t hop = (size_t)gridDim.x * blockDim.x, n4 = n / 4;
   size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
@@ -330,6 +335,7 @@ __global__ void k_lsqr_v(const float *th, float *v, size_t n, Scalars *S, int it
     const double alpha = sqrt(ta);
     S->alpha = alpha;
     S->inv_alpha = alpha > 0 ? 1.0 / alpha : 0.0;
+    S->u_old = split2(mul_rn(alpha, S->inv_beta));
     S->anorm2 = __dadd_rn(S->anorm2, mul_rn(alpha, alpha));
     if (!(alpha > 0) && S->stop_at > it) S->stop_at = it;
     double rhobar = S->rhobar, phibar = S->phibar, cx, cw, arnorm;
