@@ -15,6 +15,7 @@
 // and a tile of positions; it walks the row offsets and the 16-deep K chunks whose band
 // meets the output tile, with P in shared memory, and the taps a of each chunk.  A
 // thread keeps 8 positions x 4 outputs in registers as packed pairs of positions.
+//   k_corr_one    one tap: a banded product per position, nothing folded.
 //   k_corr_warps  32 positions; the block's eight warps share out the taps, each with
 //                 its own F and slab rows, so nothing but P is exchanged between warps,
 //                 and up to eight blocks of a cluster share out the row offsets: the
@@ -48,7 +49,7 @@ using namespace oam;
 
 namespace {
 
-constexpr int kWarps = 8;        // warps per block: warp w takes the taps a = w (mod kWarps)
+constexpr int kWarps = 8;        // warps per block
 constexpr int kThreads = 32 * kWarps;
 constexpr int kPos = 32;         // positions per block
 constexpr int kChunk = kRowChunk;  // K elements per chunk (16)
@@ -93,6 +94,7 @@ struct CorrShape {
   int len, out_len;  // input and output row lengths
   int sp;            // positions per tile-grid row: px (tiles run on over rows) or a multiple of the tile
   int strip;         // staged positions per block: tile + (rows wrapped + 2) R
+  int group;         // chunks staged together (1, 2, 4 or 8)
   const uint2 *taps;  // [output tile][R + 1][R + 2] (DirectRows)
   const float *rows;  // slab rows
 };
@@ -150,24 +152,142 @@ __device__ __forceinline__ void multiply(const float *F, const float *S, int ka,
   }
 }
 
+// ---------------------------------------------------------------- k_corr_one
+constexpr int kOneThreads = 128;
+constexpr int kOneK = 128;          // K elements staged at once
+constexpr int kOneRow = kOneK + 4;  // floats per staged position: eight of them meet distinct banks
+
+// A window of one tap is a banded product per position: the block's 32 positions and the
+// tile's slab rows are staged 128 K elements at a time, the four warps take every fourth
+// four of them and add their sums in shared memory at the end.
+// What bounds it: the staging's latency, under four blocks an SM; the kernels below pay a
+// chain of chunks with barriers for folding that one tap does not have.  us a call, from
+// those: 48x48x101 forward 16.5 -> 8.0, 64x64x128 27 -> 8.0 (adjoint 21 -> 7.9),
+// 128x128x64 16.5 -> 14.4 (37 -> 10.2), 200x200x300 125 -> 85 (97 -> 68).
+template <bool kVec>
+__global__ void __launch_bounds__(kOneThreads, 4)
+    k_corr_one(const CorrShape s, const float *__restrict__ in, float *__restrict__ out) {
+  __shared__ __align__(16) float X[kPos * kOneRow];
+  __shared__ __align__(16) float S[kOneK * kTile];
+  static_assert(kPos * kOneRow >= 3 * kPos * kTile, "three warps' sums in the inputs' place");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockIdx.y;
+  const long long o0 = (long long)blockIdx.x * kPos, positions = (long long)s.py * s.px;
+  const uint2 t = s.taps[(size_t)T * 2];  // one tap a row
+  const int lo = (int)(t.x >> 16) ? k_lo(t) / kChunk * kChunk : 0, hi = (int)(t.x >> 16) ? k_hi(t) : 0;
+  if (hi == 0 && s.out_len % 4 == 0) {  // no slab row meets the tile: zeros
+    for (int i = tid; i < kPos * (kTile / 4); i += kOneThreads) {
+      const int r = i / (kTile / 4), n = T * kTile + 4 * (i % (kTile / 4));
+      if (o0 + r < positions && n < s.out_len)
+        *reinterpret_cast<float4 *>(out + (o0 + r) * s.out_len + n) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    return;
+  }
+  const float *rows = s.rows + (size_t)t.y * kChunk * kTile;
+  const int ng = lane & 7, pg = lane >> 3;  // outputs 4 ng .. +3 of the tile, positions pg, pg + 4, .. pg + 28
+  uint64_t sum[8][2], acc[8][2];            // [position][output pair]
+#pragma unroll
+  for (int i = 0; i < 8; ++i) sum[i][0] = sum[i][1] = 0;
+  for (int k0 = lo; k0 < hi; k0 += kOneK) {
+    const int n = min(kOneK, hi - k0), n4 = (n + 3) / 4;
+    __syncthreads();
+    for (int i = tid; i < kPos * (kOneK / 4); i += kOneThreads) {
+      const int r = i / (kOneK / 4), k = 4 * (i % (kOneK / 4));
+      if (k >= n) continue;
+      const bool ok = o0 + r < positions;
+      const float *src = in + (ok ? (o0 + r) * s.len + k0 + k : 0);
+      float *dst = X + r * kOneRow + k;
+      if (kVec) {
+        copy16_async(dst, src, ok);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dst[q] = ok && k0 + k + q < s.len ? src[q] : 0.0f;
+      }
+    }
+    for (int i = tid; i < 4 * n4 * (kTile / 4); i += kOneThreads)  // whole chunks are stored
+      copy16_async(S + 4 * i, rows + (size_t)(k0 - lo) * kTile + 4 * i, true);
+    copies_commit();
+    copies_wait<0>();
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = 0;
+    for (int q = warp; q < n4; q += kOneThreads / 32) {
+      ulonglong2 w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) w[u] = *reinterpret_cast<const ulonglong2 *>(S + (4 * q + u) * kTile + 4 * ng);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 f = *reinterpret_cast<const float4 *>(X + (pg + 4 * i) * kOneRow + 4 * q);
+        const uint64_t f2[4] = {pack2(f.x, f.x), pack2(f.y, f.y), pack2(f.z, f.z), pack2(f.w, f.w)};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          acc[i][0] = fma2(f2[u], w[u].x, acc[i][0]);
+          acc[i][1] = fma2(f2[u], w[u].y, acc[i][1]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      sum[i][0] = add2(sum[i][0], acc[i][0]);
+      sum[i][1] = add2(sum[i][1], acc[i][1]);
+    }
+  }
+  __syncthreads();
+  if (warp) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      *reinterpret_cast<ulonglong2 *>(X + ((warp - 1) * kPos + pg + 4 * i) * kTile + 4 * ng) =
+          make_ulonglong2(sum[i][0], sum[i][1]);
+  }
+  __syncthreads();
+  if (warp) return;
+  const int n = T * kTile + 4 * ng;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(X + (w * kPos + pg + 4 * i) * kTile + 4 * ng);
+      sum[i][0] = add2(sum[i][0], v.x);
+      sum[i][1] = add2(sum[i][1], v.y);
+    }
+    if (o0 + pg + 4 * i >= positions) continue;
+    float *dst = out + (o0 + pg + 4 * i) * s.out_len + n;
+    const float2 a = unpack2(sum[i][0]), b = unpack2(sum[i][1]);
+    if (s.out_len % 4 == 0) {
+      if (n < s.out_len) *reinterpret_cast<float4 *>(dst) = make_float4(a.x, a.y, b.x, b.y);
+    } else {
+      if (n < s.out_len) dst[0] = a.x;
+      if (n + 1 < s.out_len) dst[1] = a.y;
+      if (n + 2 < s.out_len) dst[2] = b.x;
+      if (n + 3 < s.out_len) dst[3] = b.y;
+    }
+  }
+}
+
 // ---------------------------------------------------------------- k_corr_warps
+// A window of few taps leaves warps without one, so the block stages a group of G chunks
+// and warp w takes chunk w / (kWarps / G) of it and the taps a = w (mod kWarps / G): the
+// fewer taps, the more chunks at once.  us from one chunk at a time: 3x3 taps, 48x48x101
+// 27 -> 23 (adjoint 24 -> 17), 64x64x128 47 -> 37 (41 -> 27); 7x7 taps 84 -> 76 (86 -> 76).
+int chunk_group(int R) { return R == 1 ? 4 : R <= 3 ? 2 : 1; }
+
 // Shared memory: raw rows of the two row offsets, double-buffered (the first of a pair
-// holds P once added) [2][2][strip][kChunk]; per warp F [kChunk][kPos] and two slots of
+// holds P once added) [2][2][group][strip][kChunk]; per warp F [kChunk][kPos] and two slots of
 // slab rows [kChunk][kTile]; the tap table (R <= kTableR); per staged position its row
 // and column; the tile's sums [2][kThreads] pairs.
-size_t warps_smem(int strip, int R) {
-  return sizeof(float) * ((size_t)4 * strip * kChunk + kWarps * kChunk * (kPos + 2 * kTile) + kPos * kTile) +
+size_t warps_smem(int strip, int R, int group) {
+  return sizeof(float) * ((size_t)4 * group * strip * kChunk + kWarps * kChunk * (kPos + 2 * kTile) + kPos * kTile) +
          (R <= kTableR ? sizeof(uint2) * (R + 1) * (R + 2) : 0) + sizeof(int2) * strip;
 }
 
 // The blocks of a cluster (grid z) share out a tile's row offsets, b = z (mod Z), and
 // add their sums in rank order at the end.
-// kVec: input rows are whole float4 from a 16-byte boundary.
-template <bool kVec>
+// kVec: input rows are whole float4 from a 16-byte boundary.  kGroups: groups of chunks.
+template <bool kVec, bool kGroups>
 __global__ void __launch_bounds__(kThreads, 2)
     k_corr_warps(const CorrShape s, const float *__restrict__ in, float *__restrict__ out) {
   extern __shared__ __align__(16) uint8_t smem[];
-  const int R = s.R, NA = R + 1, wp = s.px + R, p_size = s.strip * kChunk;
+  const int G = kGroups ? s.group : 1;
+  const int R = s.R, NA = R + 1, wp = s.px + R, p_size = G * s.strip * kChunk;
   float *Pb = reinterpret_cast<float *>(smem);  // [buffer][side][p_size]
   float *Fb = Pb + 4 * p_size;                  // [warp][kChunk][kPos]; the warps' sums at the end of a row offset
   float *Sb = Fb + kWarps * kChunk * kPos;      // [warp][slot][kChunk][kTile]
@@ -193,10 +313,18 @@ __global__ void __launch_bounds__(kThreads, 2)
   const int pm = ((tile * kPos + lane) / s.sp - y0) * wp + ((tile * kPos + lane) % s.sp - x0) + R;
   const int ng = lane & 7, pg = lane >> 3;  // outputs 4 ng .. +3 of the tile, positions 8 pg .. +7
 
-  // Walk of the (row offset b, chunk c) with work: c0 .. c1 - 1 are b's chunks.
+  // this warp's chunk of a group, and its taps
+  const int share = kWarps / G, own = kGroups ? warp / share : 0;
+  unsigned own_taps = 0x01010101u << warp;
+  if (kGroups) {
+    own_taps = 0;
+    for (int a = warp % share; a < 32; a += share) own_taps |= 1u << a;
+  }
+
+  // Walk of the (row offset b, group of chunks from c) with work: c0 .. c1 - 1 are b's chunks.
   int b = (int)blockIdx.z - Z, c = 0, c1 = 0;
   auto advance = [&](int &b, int &c, int &c1) {
-    if (++c < c1) return;
+    if ((c += G) < c1) return;
     while ((b += Z) <= R) {
       if (y0 + b >= s.py && y1 - b < 0) continue;  // neither row offset meets the grid
       const uint2 t = tab[b * (NA + 1) + NA];      // the union of its taps' ranges
@@ -207,13 +335,14 @@ __global__ void __launch_bounds__(kThreads, 2)
       }
     }
   };
-  // This warp's taps whose range meets chunk c of row offset b, one bit each.
+  // This warp's taps whose range meets its chunk of the group from c of row offset b, one bit each.
   auto my_taps = [&](int b, int c, unsigned long long &m0, unsigned long long &m1) {
+    c += own;
     auto word = [&](int i) {
       const int a = 32 * i + lane;
       const uint2 t = a < NA ? tab[b * (NA + 1) + a] : make_uint2(0, 0);
       return __ballot_sync(0xffffffffu, k_lo(t) < (c + 1) * kChunk && k_hi(t) > c * kChunk && (t.x >> 16)) &
-             (0x01010101u << warp);
+             own_taps;
     };
     m0 = m1 = 0;
     m0 = word(0);
@@ -234,15 +363,17 @@ __global__ void __launch_bounds__(kThreads, 2)
   };
   // Request the raw rows of (b, c) into buffer pb.
   auto request_rows = [&](int b, int c, int pb) {
-    const int quarters = s.strip * (kChunk / 4);
+    const int quarters = G * s.strip * (kChunk / 4), lg = kGroups ? 31 - __clz(G) : 0;
     for (int side = 0; side < (b ? 2 : 1); ++side)
       for (int i = tid; i < quarters; i += kThreads) {
-        const int r = i / (kChunk / 4), kq = i % (kChunk / 4), k = c * kChunk + 4 * kq;
+        // a position's chunks follow one another, as they do in its input row
+        const int r = i / (kChunk / 4) >> lg, h = kGroups ? i / (kChunk / 4) & (G - 1) : 0, kq = i % (kChunk / 4);
+        const int k = (c + h) * kChunk + 4 * kq;
         const int2 w = where[r];
         const int y = side ? w.x - b : w.x + b;
         const bool ok = w.y >= 0 && y >= 0 && y < s.py;
         const float *src = in + (ok ? ((size_t)y * s.px + w.y) * s.len + k : 0);
-        float *dst = Pb + (2 * pb + side) * p_size + p_at(r, kq);
+        float *dst = Pb + (2 * pb + side) * p_size + h * s.strip * kChunk + p_at(r, kq);
         if (kVec) {
           copy16_async(dst, k < s.len ? src : in, ok && k < s.len);
         } else {
@@ -251,9 +382,10 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
       }
   };
-  // Request the slab rows of tap a in (b, c) into this warp's slot.
+  // Request the slab rows of tap a in this warp's chunk of the group into its slot.
   auto request_slab = [&](int b, int c, int a, int slot) {
     if (a >= NA) return;
+    c += own;
     const uint2 t = tab[b * (NA + 1) + a];
     const float *src = s.rows + ((size_t)t.y + (c - k_lo(t) / kChunk)) * (kChunk * kTile);
     float *dst = S + slot * kChunk * kTile;
@@ -306,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     copies_commit();
   }
   while (b <= R) {
-    const int k0 = c * kChunk;
+    const int k0 = (c + own) * kChunk;
     float *P = Pb + 2 * pb * p_size;
     copies_wait<0>();
     __syncthreads();
@@ -344,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       }
       // F of this tap
 #pragma unroll
-      for (int kq = 0; kq < kChunk / 4; ++kq) fold_tap<kPos>(P, pm, a, F + lane, kq);
+      for (int kq = 0; kq < kChunk / 4; ++kq) fold_tap<kPos>(P + own * s.strip * kChunk, pm, a, F + lane, kq);
       // this tap's slab rows are older than the last two copies (steps 0 and 1: the
       // next tap's and the next chunk's) or than the last one
       if (step < 2) copies_wait<2>();
@@ -384,9 +516,9 @@ __global__ void __launch_bounds__(kThreads, 2)
   // Write the tile: rank z takes the z-th share of the pairs.
   auto cluster = cooperative_groups::this_cluster();
   cluster.sync();
-  const int share = 2 * kThreads / Z;
-  for (int j = tid; j < share; j += kThreads) {
-    const int i = blockIdx.z * share + j, half = i / kThreads, e = i % kThreads;
+  const int part = 2 * kThreads / Z;
+  for (int j = tid; j < part; j += kThreads) {
+    const int i = blockIdx.z * part + j, half = i / kThreads, e = i % kThreads;
     float2 v = *cluster.map_shared_rank(sum3 + i, 0);
     for (int z = 1; z < Z; ++z) {
       const float2 u = *cluster.map_shared_rank(sum3 + i, z);
@@ -579,6 +711,15 @@ oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaSt
   s.out_len = fwd ? g.nt : g.nz;
   s.taps = L.d_taps;
   s.rows = L.d_rows;
+  const bool vec = s.len % 4 == 0;
+  if (m->R == 0) {
+    ProfScope prof(m, st, fwd);
+    const dim3 grid((unsigned)(((long long)g.px * g.py + kPos - 1) / kPos), L.tiles);
+    if (vec) k_corr_one<true><<<grid, kOneThreads, 0, st>>>(s, in, out);
+    else k_corr_one<false><<<grid, kOneThreads, 0, st>>>(s, in, out);
+    OAM_LAUNCHED();
+    return OAM_OK;
+  }
   // k_corr_block from three of its blocks with work on the fullest SM on: alone or in twos
   // they are bound by their chains of taps, which the eight warps cut eightfold.  us,
   // block against warps, with one: 48x48x64 31x31 taps 950, 259; two: 80x80x64 21x21
@@ -587,7 +728,10 @@ oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaSt
   // 705; five: 96x96x128 31x31 taps 1498, 1818, 128x128x64 11x11 taps 218, 358.
   const long long busy = fwd ? (m->n_hi - m->n_lo + kTile - 1) / kTile : L.tiles;
   const int sms = std::max(1, m->sm_count);
-  const bool block = ((long long)g.px * g.py + kBlockPos - 1) / kBlockPos * busy > 2LL * sms;
+  // Inputs of one or two chunks leave the warps nothing to share but their set-up (from one
+  // block per SM on: 128x128x4 forward, 3x3 taps 15, 49; 9x9 taps 42, 70).
+  const long long blocks = ((long long)g.px * g.py + kBlockPos - 1) / kBlockPos * busy;
+  const bool block = blocks > (s.len <= 2 * kChunk ? 1LL : 2LL) * sms;
   // Tiles run on over scan rows (no idle positions) unless the padding between
   // many short rows makes the strip too long; then every tile stays in its row.
   const int tile = block ? kBlockPos : kPos;
@@ -596,7 +740,8 @@ oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaSt
   s.sp = run_on ? s.px : (s.px + tile - 1) / tile * tile;
   s.strip = run_on ? wrap : tile + 2 * s.R;
   const long long tiles = ((long long)s.py * s.sp + tile - 1) / tile;
-  const size_t sm = block ? block_smem(s.strip, s.R) : warps_smem(s.strip, s.R);
+  s.group = chunk_group(s.R);
+  const size_t sm = block ? block_smem(s.strip, s.R) : warps_smem(s.strip, s.R, s.group);
   // Blocks that share out a tile's row offsets: the count that finishes first, in units of
   // a row offset, 0.6 more for a block's start and end, times the waves at the blocks an
   // SM holds (the idle part of the last wave counts half).  us with 1, 2, 4, 8: 32x32x48
@@ -615,8 +760,10 @@ oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaSt
       }
     }
   }
-  const bool vec = s.len % 4 == 0;
-  auto fn = block ? (vec ? k_corr_block<true> : k_corr_block<false>) : (vec ? k_corr_warps<true> : k_corr_warps<false>);
+  void (*const kernels[2][2][2])(const CorrShape, const float *, float *) = {
+      {{k_corr_warps<false, false>, k_corr_warps<false, true>}, {k_corr_warps<true, false>, k_corr_warps<true, true>}},
+      {{k_corr_block<false>, k_corr_block<false>}, {k_corr_block<true>, k_corr_block<true>}}};
+  auto fn = kernels[block][vec][s.group > 1];
   // one limit for all launches: calls from several threads would lower each other's
   // between setting it and the launch
   OAM_CUDA_TRY(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
