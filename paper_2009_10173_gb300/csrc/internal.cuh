@@ -205,6 +205,7 @@ struct LineShape {
   int wp, rows;            // positions per packed row (px + R), packed positions per frequency
   int nr;                  // packed rows per frequency: 2 segs (re and im)
   int out_len, out_lo, acc, parts;  // output row length, output channel of accumulator column 0, columns, partial sums
+  bool zeros;              // the inverse writes the zeros outside the accumulator too
   int words;               // 32-row mark words per column
   // Marks, a bit per position of a column: plane 0 those with a non-zero input, plane 1 + b
   // those with a non-finite one among the packed channels 32 b .. 32 b + 31.
@@ -219,7 +220,7 @@ struct LineShape {
   __host__ __device__ int first_row(int seg) const { return segs > 1 ? seg * valid - halo : 0; }  // point 0's row
 };
 oam_status line_r2c(int P, cudaStream_t st, const LineShape &s, const float *in, const float2 *tw, float *packed);
-// Writes the output channels [z0, z1) of line_channels; the others are not touched.
+// Writes the output channels [z0, z1) of line_channels; the others are zeroed or (s.zeros unset) not touched.
 oam_status line_c2r(int P, cudaStream_t st, const LineShape &s, const float *part, const float2 *tw, float *out);
 void line_channels(const LineShape &s, int *z0, int *z1);
 

@@ -12,7 +12,8 @@
 // inverse with 1, 2 and, at three blocks per SM instead of two, 3 partial sums, bound
 // by the loads' latency (18 us of bytes forward, 26 + 9 per sum inverse, at 6.8 TB/s).
 // The output's channels beyond the accumulator are zeroed by a spare warp of the
-// correlation kernel, under its products (here they took 35 us).
+// correlation kernel where its products hide that (35 us here), else by blocks of the
+// inverse (op_tc.cu, zeros_in_inverse).
 //
 // The correlation has compact support: a position whose window holds only zeros
 // gets exact zeros, and a non-finite input reaches only the positions whose window
@@ -135,7 +136,7 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>(), R1 >= 15 && R2 <= 
   constexpr int P = R1 * R2, Q = P / 2 + 1;
   extern __shared__ float2 sm[];
   __shared__ unsigned words[2][P / 32 + 2];  // grown marks of the rows written: some input, a non-finite one
-  const int x = blockIdx.y, ob = s.out_lo / kLineCh * kLineCh + blockIdx.x * kLineCh;
+  const int x = blockIdx.y, ob = (s.zeros ? 0 : s.out_lo / kLineCh * kLineCh) + blockIdx.x * kLineCh;
   const int y0 = s.first_row(blockIdx.z), ya = s.out_row(blockIdx.z), yb = min(s.py, ya + s.valid);  // rows written
   float *col = out + (size_t)x * s.out_len + ob;
   const size_t stride = (size_t)s.px * s.out_len;
@@ -147,6 +148,13 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>(), R1 >= 15 && R2 <= 
       s.marks[((size_t)(i / s.words) * s.px + x) * s.words + i % s.words] = 0;
     for (int i = threadIdx.x; i < Q; i += blockDim.x) s.vmax[(size_t)i * s.px + x] = 0;
     if (x == 0 && threadIdx.x == 0) *s.any_bad = 0;
+  }
+  if (ob + kLineCh <= s.out_lo || ob >= s.out_lo + s.acc) {  // outside the accumulator (whole float4 there)
+    for (int i = threadIdx.x; i < (yb - ya) * (kLineCh / 4); i += blockDim.x) {
+      const int y = ya + i / (kLineCh / 4), c = 4 * (i % (kLineCh / 4));
+      if (c < cols) *reinterpret_cast<float4 *>(col + (size_t)y * stride + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    return;
   }
   const int w0 = ya >> 5, nw = ((yb - 1) >> 5) - w0 + 1;
   const int z0 = ob - s.out_lo;  // accumulator column of the block's first channel (even: out_lo is 16-aligned)
@@ -213,6 +221,7 @@ oam_status run(bool inverse, cudaStream_t st, const LineShape &s, const float *i
           cudaFuncSetAttribute(k_line_c2r<R1, R2, kVec>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     int z0, z1;
     line_channels(s, &z0, &z1);
+    if (s.zeros) z0 = 0, z1 = s.out_len;
     k_line_c2r<R1, R2, kVec><<<dim3((z1 - z0 + kLineCh - 1) / kLineCh, s.px, s.segs), threads, sm, st>>>(
         s, in, tw, 1.0f / (float)(R1 * R2), out);
   } else {

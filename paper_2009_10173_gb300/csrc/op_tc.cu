@@ -1016,6 +1016,22 @@ oam_status launch_corr_fw(const Launch &lp, const TcLayout *L, dim3 grid, cudaSt
   return launch_corr<8, kWide>(lp, L, grid, st);
 }
 
+// Which kernel zeroes the output's channels outside the accumulator, by the time that it
+// adds (us).  A spare warp of each correlation block takes 0.08 a position and 0.035 a
+// store, of which the block's products hide most: 200x200x300, 61 taps 76 under 340.  The
+// inverse's own blocks write 3.2 TB/s but hide nothing: 35 there.  With few blocks or few
+// taps the spare warps are last: 64x64x128, 3 taps, 33 blocks, 20.7 against 9.5 for the
+// kernel without them; 32x32x48, 1 tap 13.0 against 7.1; 200x200x300, 1 tap 75 against 42.
+bool zeros_in_inverse(const oam_model *m, const TcLine *T, const TcLayout *L, const Launch &lp, int out_len) {
+  const int outside4 = (lp.p.z0 + out_len - lp.p.z1) / 4, sms = std::max(1, m->sm_count);
+  if (outside4 <= 0) return false;
+  const long long blocks = (long long)lp.n_tiles * L->parts * T->Q, positions = (long long)m->grid.px * m->grid.py;
+  const int pairs = ((m->R + 2) / 2 + L->parts - 1) / L->parts;
+  const double products = 0.55 * (pairs * L->stages + 8) * (double)((blocks + sms - 1) / sms);
+  const double spare = (double)positions / (double)std::min<long long>(blocks, sms) * (0.08 + 0.035 * ((outside4 + 31) / 32));
+  return spare - 0.8 * products > (double)positions * outside4 * 16 / 3.2e6;
+}
+
 size_t mark_words(const oam_model *m, const TcLine *T) {
   return (size_t)m->grid.px * ((size_t)2 * T->planes * T->words + T->Q) + 2;
 }
@@ -1064,6 +1080,8 @@ oam_status run_corr(const oam_model *m, const TcLayout *L, const float *in, int 
   lp.p.positions = s.px * s.py;
   lp.p.out_len = out_len;
   line_channels(s, &lp.p.z0, &lp.p.z1);
+  s.zeros = zeros_in_inverse(m, T, L, lp, out_len);
+  if (s.zeros) lp.p.z0 = 0, lp.p.z1 = out_len;  // none are left to the correlation
   lp.p.vmax = s.vmax;
   lp.p.smax = T->d_smax;
   ProfScope prof(m, st, L->dir == 0);
