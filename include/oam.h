@@ -75,7 +75,10 @@ typedef enum {
                           its window: a position whose window holds nothing above
                           1/60 of what stands elsewhere on those lines is less exact
                           relative to its own output than a direct sum of BF16 terms,
-                          as in the lateral-FFT form; OAM_PREC_FP32 sums directly */
+                          as in the lateral-FFT form; OAM_PREC_FP32 sums directly.
+                          Windows of one tap, and small problems of up to nine folded
+                          taps (at most three offsets a side, more on single rows), are
+                          summed by the FP32 kernels, which are faster there */
   OAM_PREC_FFT = 2     /* FP32 lateral-FFT form of the same operators: both are 2-D
                           correlations over the scan grid (Methods, Efficient
                           reconstruction based on scanning symmetries), restated
@@ -142,9 +145,10 @@ typedef struct {
   double flops_per_op; /* algorithmic flops of one forward (= one adjoint): 2*px*py*nnz_in_grid */
   size_t device_bytes; /* device memory owned by the model */
   double exec_flops_forward, exec_flops_adjoint; /* flops issued per application: tensor-core
-                                                    flops (3 BF16 products, band and tile padding)
+                                                    flops (3 products of 16-bit terms, band and tile padding)
                                                     for OAM_PREC_BF16X3, banded spectral products
-                                                    and FFTs for OAM_PREC_FFT; 0 for OAM_PREC_FP32 */
+                                                    and FFTs for OAM_PREC_FFT; 0 for OAM_PREC_FP32
+                                                    and where OAM_PREC_BF16X3 takes its kernels */
   double op_bytes;     /* OAM_PREC_FFT: device bytes read + written per application (the
                           spectral slab dominates); 0 otherwise */
   int32_t filter_half_len; /* L of the band-pass filter set by oam_model_set_filter, -1: none */
@@ -340,7 +344,8 @@ oam_status oam_solver_work_bytes(const oam_model *model, int32_t solver, size_t 
  * fits), and the position tiling (oam_model_set_tiling).  The choice is kept
  * in the model (read it with oam_model_get_tiles and oam_model_get_tiling).
  * Allocates and frees a scratch volume and signal buffer; synchronises
- * `stream`.  No-op for the other precisions.  The paper has no counterpart
+ * `stream`.  No-op for the other precisions, and without effect on a direction
+ * that OAM_PREC_BF16X3 sums by the FP32 kernels.  The paper has no counterpart
  * (tuning of this implementation). */
 oam_status oam_model_autotune(oam_model *model, int32_t reps, void *stream, int32_t *ring_forward,
                               int32_t *ring_adjoint);

@@ -411,9 +411,9 @@ oam_status oam_adjoint(const oam_model *m, const float *d_s, float *d_H, void *s
 // A filtered model (oam_model_set_filter) applies F A and A^T F.
 oam_status oam::apply_forward(const oam_model *m, const float *H, float *s, cudaStream_t st) {
   oam_status rc;
-  if (m->precision == OAM_PREC_BF16X3) rc = forward_tc(m, H, s, st);
-  else if (m->precision == OAM_PREC_FFT) rc = forward_fft(m, H, s, st);
-  else rc = forward_fp32(m, H, s, st);
+  if (m->precision == OAM_PREC_FFT) rc = forward_fft(m, H, s, st);
+  else if (uses_direct(m, true)) rc = forward_fp32(m, H, s, st);
+  else rc = forward_tc(m, H, s, st);
   if (rc || !m->fir) return rc;
   return fir_apply(m, s, s, st);
 }
@@ -425,7 +425,7 @@ oam_status oam::apply_adjoint(const oam_model *m, const float *s, float *H, cuda
     if (rc) return rc;
     s = fs;
   }
-  if (m->precision == OAM_PREC_BF16X3) return adjoint_tc(m, s, H, st);
   if (m->precision == OAM_PREC_FFT) return adjoint_fft(m, s, H, st);
-  return adjoint_fp32(m, s, H, st);
+  if (uses_direct(m, false)) return adjoint_fp32(m, s, H, st);
+  return adjoint_tc(m, s, H, st);
 }

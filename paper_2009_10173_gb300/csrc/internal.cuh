@@ -38,6 +38,7 @@ struct __align__(32) Patch {
 // x = first element | count << 16, y = first chunk's index in d_rows.
 struct DirectRows {
   int tiles = 0;
+  long long items = 0;       // (tile, tap, chunk) triples with work
   uint2 *d_taps = nullptr;   // [tiles][R + 1][R + 2]
   float *d_rows = nullptr;   // [chunks][kRowChunk][kOutTile]
 };
@@ -78,7 +79,7 @@ struct oam_model {
   int *d_band_lo = nullptr;
   float *d_band = nullptr;        // [n_orb][nz][band_w]
 
-  // FP32 operators' slab rows (OAM_PREC_FP32)
+  // FP32 operators' slab rows (OAM_PREC_FP32, and OAM_PREC_BF16X3 with few taps)
   oam::DirectRows rows_fwd, rows_adj;
 
   // tensor-core layouts (OAM_PREC_BF16X3) per direction, and the plan and buffers
@@ -154,6 +155,9 @@ size_t slab_plan_bytes(const oam_model *m);
 oam_status slab_column(const oam_model *m, int b, int a, int k, float *d_out, cudaStream_t st);
 
 // op_fp32.cu
+// Does the model apply its operator by the FP32 kernels: the plain form, and the split
+// form where its transforms would take longer than the sums.
+bool uses_direct(const oam_model *m, bool fwd);
 oam_status forward_fp32(const oam_model *m, const float *H, float *s, cudaStream_t st);
 oam_status adjoint_fp32(const oam_model *m, const float *s, float *H, cudaStream_t st);
 

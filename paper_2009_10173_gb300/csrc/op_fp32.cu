@@ -786,6 +786,21 @@ oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaSt
 
 }  // namespace
 
+// The split form takes three launches and two transforms, so small sums are faster here.  us
+// of that form and of these kernels, with the triples of all position tiles: one tap 64x64x128
+// 25, 8; 200x200x300 141, 85.  3x3 taps 600x1x128 37, 12 (0.7e3), 32x32x48 21, 12 (1e3),
+// 48x48x101 23, 23 (4.6e3), 128x128x4 32, 15 (4.1e3), adjoint 28, 23 (6.1e3); 64x64x128
+// 27, 37 (9.7e3), adjoint 25, 27.  5x5 taps 32x32x48 23, 16 (2.3e3), 48x48x101 23, 37 (1.0e4).
+// One row of 17 taps 600x1x128 36, 23 (3.4e3), of 31 taps 45, 70.  Above nine folded taps it
+// gains little (32x32x48, 7x7 taps 23, 19; 9x9 taps 21, 27), so those keep no rows.
+bool oam::uses_direct(const oam_model *m, bool fwd) {
+  if (m->precision != OAM_PREC_BF16X3) return m->precision == OAM_PREC_FP32;
+  const DirectRows &L = fwd ? m->rows_fwd : m->rows_adj;
+  if (!L.d_rows) return false;
+  const long long tiles = ((long long)m->grid.px * m->grid.py + kPos - 1) / kPos;
+  return m->R == 0 || tiles * L.items <= 6500;
+}
+
 oam_status oam::forward_fp32(const oam_model *m, const float *H, float *s, cudaStream_t st) {
   return run(m, true, H, s, st);
 }

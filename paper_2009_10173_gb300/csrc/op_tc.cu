@@ -1188,7 +1188,7 @@ void oam::tc_free(oam_model *m, cudaStream_t st) {
 double oam::tc_exec_flops(const oam_model *m, int dir) {
   const TcLayout *L = dir == 0 ? m->tc_fwd : m->tc_adj;
   Launch lp;
-  if (!L || plan_launch(m, m->tc_line, L, &lp)) return 0.0;
+  if (!L || uses_direct(m, dir == 0) || plan_launch(m, m->tc_line, L, &lp)) return 0.0;
   return 3.0 * 2.0 * kTileM * (double)lp.n_tiles * m->tc_line->Q * L->cols;
 }
 

@@ -759,6 +759,15 @@ oam_status oam::plan_bands(oam_model *m, const std::vector<double2> &h_range, in
   return OAM_OK;
 }
 
+// Row and column offsets that couple two positions of the scan.
+static int row_offsets(const oam_model *m) { return std::min(m->R, m->grid.py - 1) + 1; }
+static int col_offsets(const oam_model *m) { return std::min(m->R, m->grid.px - 1) + 1; }
+// The split form keeps FP32 rows for windows of up to nine folded taps (uses_direct).
+static bool needs_rows(const oam_model *m) {
+  return m->precision == OAM_PREC_FP32 ||
+         (m->precision == OAM_PREC_BF16X3 && row_offsets(m) * col_offsets(m) <= 9);
+}
+
 // FP32 operators' slab rows of one direction (0 forward, 1 adjoint): per (orbit, output
 // tile) the input range and first chunk, as DirectRows packs them.  Returns the chunks.
 static long long plan_rows(const oam_model *m, int dir, int *tiles, std::vector<uint2> *range) {
@@ -767,7 +776,11 @@ static long long plan_rows(const oam_model *m, int dir, int *tiles, std::vector<
   range->assign((size_t)O * NT, make_uint2(0, 0));
   long long chunks = 0;
   std::vector<int> lo(NT), hi(NT);
+  std::vector<char> used(O, 0);
+  for (int b = 0; b < row_offsets(m); ++b)
+    for (int a = 0; a < col_offsets(m); ++a) used[m->h_tap_orbit[(b + m->R) * m->W + (a + m->R)]] = 1;
   for (int o = 0; o < O; ++o) {
+    if (!used[o]) continue;
     lo.assign(NT, 1 << 30);
     hi.assign(NT, 0);
     for (int k = 0; k < nz; ++k) {
@@ -800,12 +813,14 @@ static oam_status build_rows(oam_model *m, int dir, DirectRows *L, const int *d_
   const int R = m->R, W = m->W, NA = R + 1;
   taps.assign((size_t)L->tiles * NA * (NA + 1), make_uint2(0, 0));
   for (int T = 0; T < L->tiles; ++T)
-    for (int b = 0; b <= R; ++b) {
+    for (int b = 0; b < row_offsets(m); ++b) {
       uint2 *row = &taps[((size_t)T * NA + b) * (NA + 1)];
       unsigned lo = 0xffffffffu, hi = 0;
-      for (int a = 0; a <= R; ++a) {
+      for (int a = 0; a < col_offsets(m); ++a) {
         row[a] = range[(size_t)m->h_tap_orbit[(b + R) * W + (a + R)] * L->tiles + T];
         if (!(row[a].x >> 16)) continue;
+        L->items += ((row[a].x & 0xffffu) + (row[a].x >> 16) + kRowChunk - 1) / kRowChunk -
+                    (row[a].x & 0xffffu) / kRowChunk;
         lo = std::min(lo, row[a].x & 0xffffu);
         hi = std::max(hi, (row[a].x & 0xffffu) + (row[a].x >> 16));
       }
@@ -831,7 +846,7 @@ static oam_status build_rows(oam_model *m, int dir, DirectRows *L, const int *d_
 size_t oam::slab_plan_bytes(const oam_model *m) {
   const size_t O = m->n_orb, nz = m->grid.nz;
   size_t b = alloc_bytes<int>((size_t)m->W * m->W) + alloc_bytes<int>(O * nz) + alloc_bytes<float>(O * nz * m->band_w);
-  if (m->precision != OAM_PREC_FP32) return b;
+  if (!needs_rows(m)) return b;
   for (int dir = 0; dir < 2; ++dir) {
     std::vector<uint2> range;
     int tiles = 0;
@@ -950,7 +965,7 @@ oam_status oam::build_slab(oam_model *m, cudaStream_t st) {
   }
   OAM_LAUNCHED();
 
-  if (m->precision == OAM_PREC_FP32 && ((rc = build_rows(m, 0, &m->rows_fwd, d_band_hi, st)) ||
+  if (needs_rows(m) && ((rc = build_rows(m, 0, &m->rows_fwd, d_band_hi, st)) ||
                                         (rc = build_rows(m, 1, &m->rows_adj, d_band_hi, st))))
     return rc;
   cudaFreeAsync(d_orb_b, st);

@@ -52,7 +52,7 @@ def test_split_form_keeps_other_bands(direction, value):
     import torch
 
     from paper_2009_10173_gb300 import binding as B
-    cfg, meets, m = setup(B.OAM_PREC_BF16X3, px=20, py=30, nz=192, dz_m=8e-6, z0_rel_m=-192 * 4e-6, nt=768)
+    cfg, meets, m = setup(B.OAM_PREC_BF16X3, px=20, py=30, win=9, nz=192, dz_m=8e-6, z0_rel_m=-192 * 4e-6, nt=768)
     op = getattr(m, direction)
     if direction == "adjoint":
         meets = meets.T
@@ -65,9 +65,9 @@ def test_split_form_keeps_other_bands(direction, value):
         got = op(x)
         bad = ~torch.isfinite(got)
         window = torch.zeros_like(bad)
-        window[13:18, 6:11] = True
+        window[11:20, 4:13] = True
         assert not (bad & ~window).any()
-        here = bad[13:18, 6:11].any(0).any(0).cpu().numpy()
+        here = bad[11:20, 4:13].any(0).any(0).cpu().numpy()
         o = np.flatnonzero(meets[max(0, e - 47):e + 48].any(0))
         reach = np.zeros_like(here)
         reach[max(0, o[0] - 48):o[-1] + 49] = True
