@@ -938,7 +938,10 @@ oam_status oam::build_slab(oam_model *m, cudaStream_t st) {
   } else {
     // k_slab_values where the pulse varies too fast within a sample for the polynomials, is
     // shorter than two samples a side, or its bins exceed the shared memory of two blocks
-    // per SM
+    // per SM; and for few patches, which do not repay the moments' last sums (build of 192
+    // depths, 61x61 taps, ms, moments against values: 64 patches 4.5, 3.5; 256 5.6, 4.9; 512
+    // 5.9, 6.9; 48 depths, 11x11 taps, 256 patches 0.32, 0.30, 512 0.31, 0.35)
+    constexpr int kMomPatches = 352;
     MomShape ms{};
     ms.tb = (int)std::floor(m->cut - 0.5) + 1;
     const double edge = 2.0 * (ms.tb - m->cut);
@@ -947,7 +950,7 @@ oam_status oam::build_slab(oam_model *m, cudaStream_t st) {
     ms.B0 = std::max(0, (int)std::floor(m->cut) - 1);
     ms.nb = std::max(1, m->band_w - 2 * ms.B0 + 1);
     std::vector<float2> coef;
-    if (m->cut >= 2.0 && m->cut <= 64.0 && mom_smem(ms) <= 100 * 1024 &&
+    if (m->M >= kMomPatches && m->cut >= 2.0 && m->cut <= 64.0 && mom_smem(ms) <= 100 * 1024 &&
         pulse_polynomials(m->sigma_s, m->omega, ms.tb, &coef)) {
       float2 *d_coef = nullptr;
       OAM_CUDA_TRY(cudaMallocAsync((void **)&d_coef, sizeof(float2) * coef.size(), st));
