@@ -673,7 +673,7 @@ __global__ void k_slab_max(const float *__restrict__ band, size_t n, float terms
 
 __global__ void __launch_bounds__(kPackThreads) k_pack_tiles(const float *__restrict__ band, const int *band_lo,
                                                              const int *band_hi, int band_w, int nz, int dir, int t_lo,
-                                                             const int *tap_orbit, int R, int halo, int P, int Q,
+                                                             const int *tap_orbit, int R, int halo, int P,
                                                              const float2 *__restrict__ tw, const unsigned *smax,
                                                              const TcTile *tiles, size_t v_stride, uint8_t *data) {
   extern __shared__ float smp[];
@@ -699,18 +699,40 @@ __global__ void __launch_bounds__(kPackThreads) k_pack_tiles(const float *__rest
   }
   const float sc = pow2(scale_exp(__uint_as_float(*smax)));
   __half *dst = reinterpret_cast<__half *>(data + t.off) + i;
-  for (int f = 0; f < Q; ++f) {
-    float v = 0.0f;
-    for (int b = 0, j = 0; b <= halo; ++b) {  // j = f b mod P
-      v = fmaf(cosT[j], sv[b * kPackThreads + tid], v);
-      j += f;
-      if (j >= P) j -= P;
-    }
+  auto put = [&](int f, float v) {
     v *= sc;
     const __half h = __float2half_rn(v);
     __half *d = dst + (size_t)f * (v_stride / sizeof(__half));
     d[0] = h;
     d[16 * t.n] = __float2half_rn(v - __half2float(h));
+  };
+  // Frequencies f and P / 2 - f (P is a multiple of 4) differ in the sign of the odd row
+  // offsets' terms; four pairs at a time share a slab value.
+  for (int f0 = 0; f0 <= P / 4; f0 += 4) {
+    float even[4] = {}, odd[4] = {};
+    int j[4] = {}, step[4];  // j = f b mod P
+#pragma unroll
+    for (int q = 0; q < 4; ++q) step[q] = f0 + q;
+    auto term = [&](int b, float (&sum)[4]) {
+      const float v = sv[b * kPackThreads + tid];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        sum[q] = fmaf(cosT[j[q]], v, sum[q]);
+        j[q] += step[q];
+        if (j[q] >= P) j[q] -= P;
+      }
+    };
+    for (int b = 0; b <= halo; b += 2) {
+      term(b, even);
+      if (b < halo) term(b + 1, odd);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int f = f0 + q;
+      if (f > P / 4) break;
+      put(f, even[q] + odd[q]);
+      if (f < P / 4) put(P / 2 - f, even[q] - odd[q]);
+    }
   }
 }
 
@@ -776,31 +798,23 @@ oam_status plan_line(const oam_model *m, TcLine *T) {
   return OAM_OK;
 }
 
-// Sample (forward) or depth (adjoint) range [lo, hi) of the slab of orbit o in one
-// 16-deep K chunk, from accumulator column 0.
-void chunk_range(const oam_model *m, int o, int dir, int chunk, int t_lo, int *plo, int *phi) {
+// Sample (forward) or depth (adjoint) range [x, y) of the slab of every orbit in each
+// 16-deep K chunk, from accumulator column 0: [orbit][chunks] (x >= y: none), in one pass
+// over the bands.
+std::vector<int2> chunk_ranges(const oam_model *m, int dir, int chunks, int t_lo) {
   const int nz = m->grid.nz;
-  int lo = 1 << 30, hi = -1;
-  if (dir == 0) {
-    for (int k = 16 * chunk; k < std::min(nz, 16 * chunk + 16); ++k) {
-      const int bl = m->h_band_lo[(size_t)o * nz + k], bh = m->h_band_hi[(size_t)o * nz + k];
-      if (bh > bl) {
-        lo = std::min(lo, bl - t_lo);
-        hi = std::max(hi, bh - t_lo);
-      }
-    }
-  } else {
-    const int n0 = t_lo + 16 * chunk, n1 = n0 + 16;
+  std::vector<int2> r((size_t)m->n_orb * chunks, make_int2(1 << 30, -1));
+  for (int o = 0; o < m->n_orb; ++o) {
+    int2 *row = r.data() + (size_t)o * chunks;
     for (int k = 0; k < nz; ++k) {
-      const int bl = m->h_band_lo[(size_t)o * nz + k], bh = m->h_band_hi[(size_t)o * nz + k];
-      if (bh > bl && bl < n1 && bh > n0) {
-        lo = std::min(lo, k);
-        hi = std::max(hi, k + 1);
-      }
+      const int bl = m->h_band_lo[(size_t)o * nz + k] - t_lo, bh = m->h_band_hi[(size_t)o * nz + k] - t_lo;
+      if (bh <= bl) continue;
+      const int lo = dir == 0 ? bl : k, hi = dir == 0 ? bh : k + 1;
+      const int c0 = dir == 0 ? k / 16 : bl / 16, c1 = dir == 0 ? k / 16 : (bh - 1) / 16;
+      for (int c = c0; c <= c1; ++c) row[c] = make_int2(std::min(row[c].x, lo), std::max(row[c].y, hi));
     }
   }
-  *plo = lo;
-  *phi = hi;
+  return r;
 }
 
 // Columns [col, col + n) of a tile over a range, whole 16-column groups.
@@ -858,6 +872,8 @@ oam_status plan_dir(const oam_model *m, const TcLine *T, TcLayout *L, int dir, s
 
   items.assign((size_t)(R + 1) * L->stages, TcItem{});
   L->reach.assign(L->stages, make_int2(L->acc_cols, 0));
+  const int chunks = 2 * L->stages;
+  const std::vector<int2> ranges = chunk_ranges(m, dir, chunks, t_lo);
   tiles.clear();
   long long off = 0;
   int max_item = 16;
@@ -871,8 +887,9 @@ oam_status plan_dir(const oam_model *m, const TcLine *T, TcLayout *L, int dir, s
         const int chunk = 2 * s + c;
         int lo = 1 << 30, hi = -1;
         for (int b = 0; b <= R; ++b) {
-          int bl, bh, col, n;
-          chunk_range(m, m->h_tap_orbit[(b + R) * W + (a + R)], dir, chunk, t_lo, &bl, &bh);
+          const int2 r = ranges[(size_t)m->h_tap_orbit[(b + R) * W + (a + R)] * chunks + chunk];
+          const int bl = r.x, bh = r.y;
+          int col, n;
           if (bh <= bl) continue;
           // a single offset's band wider than 256 columns is not taken
           tile_cols(bl, bh, &col, &n);
@@ -928,7 +945,7 @@ oam_status build_dir(oam_model *m, TcLayout *L, int dir, cudaStream_t st, int *d
     const dim3 grid((unsigned)tiles.size(), (unsigned)((16 * n_max + kPackThreads - 1) / kPackThreads));
     const size_t sm = sizeof(float) * ((size_t)T->P + (size_t)(T->halo + 1) * kPackThreads);  // at most 35 KB
     k_pack_tiles<<<grid, kPackThreads, sm, st>>>(m->d_band, m->d_band_lo, d_band_hi, m->band_w, nz, dir, t_lo,
-                                                 m->d_tap_orbit, m->R, T->halo, T->P, T->Q, T->d_tw, T->d_smax,
+                                                 m->d_tap_orbit, m->R, T->halo, T->P, T->d_tw, T->d_smax,
                                                  d_tiles, L->v_stride, L->d_data);
     OAM_LAUNCHED();
     OAM_CUDA_TRY(cudaFreeAsync(d_tiles, st));
