@@ -28,6 +28,7 @@
 #include <set>
 #include <vector>
 
+#include "f32x2.cuh"
 #include "fft_dev.cuh"
 #include "internal.cuh"
 
@@ -159,63 +160,32 @@ __device__ __forceinline__ void xpass(int P, int k, Src src, Dst dst) {
   }
 }
 
-// A whole transform of KL lines of P = 2^lgP points (lgP >= 4) through the
-// shared slots `a`: `first` reads the input (forward: natural point i;
-// inverse: the point at position i, i.e. frequency bitrev(i)), `last` takes
-// position i's result (forward: frequency bitrev(i); inverse: point i).  With
-// kLastToSmem the last pass writes the slots too (followed by a barrier) and
-// `last` is not called.
+// A whole transform of KL lines of P = 2^lgP points (lgP 10 or 11: one pass of two or
+// three stages and two of four) through the shared slots `a`: `first` reads the input
+// (forward: natural point i; inverse: the point at position i, i.e. frequency bitrev(i)),
+// `last` takes position i's result (forward: frequency bitrev(i); inverse: point i).  With
+// kLastToSmem the last pass writes the slots too (followed by a barrier) and `last` is not
+// called.
 template <int KL, bool kForward, bool kLastToSmem, class First, class Last>
 __device__ __forceinline__ void xtransform(float2 *a, int P, int lgP, First first, Last last) {
-  const int np = (lgP + 3) / 4, r0 = lgP - 4 * (np - 1);
   auto from_smem = [&](int i, int l) { return a[xslot<KL>(i, l)]; };
   auto to_smem = [&](int i, int l, float2 v) { a[xslot<KL>(i, l)] = v; };
-  // pass p covers stages [kf, kf + rr): forward passes run p = 0 .. np-1 with
-  // kf = 4 (np-1-p) (the first has r0 stages), inverse passes the reverse
-  for (int pi = 0; pi < np; ++pi) {
-    const int pp = kForward ? pi : np - 1 - pi;  // which stage block
-    const int kf = 4 * (np - 1 - pp), rr = pp == 0 ? r0 : 4;
-    const bool is_first = pi == 0, is_last = pi == np - 1;
-    if (is_first && is_last) {
-      if (kLastToSmem) {
-        switch (rr) {
-          case 1: xpass<KL, 1, kForward>(P, kf, first, to_smem); break;
-          case 2: xpass<KL, 2, kForward>(P, kf, first, to_smem); break;
-          case 3: xpass<KL, 3, kForward>(P, kf, first, to_smem); break;
-          default: xpass<KL, 4, kForward>(P, kf, first, to_smem); break;
-        }
-      } else {
-        switch (rr) {
-          case 1: xpass<KL, 1, kForward>(P, kf, first, last); break;
-          case 2: xpass<KL, 2, kForward>(P, kf, first, last); break;
-          case 3: xpass<KL, 3, kForward>(P, kf, first, last); break;
-          default: xpass<KL, 4, kForward>(P, kf, first, last); break;
-        }
-      }
-    } else if (is_first) {
-      switch (rr) {
-        case 1: xpass<KL, 1, kForward>(P, kf, first, to_smem); break;
-        case 2: xpass<KL, 2, kForward>(P, kf, first, to_smem); break;
-        case 3: xpass<KL, 3, kForward>(P, kf, first, to_smem); break;
-        default: xpass<KL, 4, kForward>(P, kf, first, to_smem); break;
-      }
-    } else if (is_last && !kLastToSmem) {
-      switch (rr) {
-        case 1: xpass<KL, 1, kForward>(P, kf, from_smem, last); break;
-        case 2: xpass<KL, 2, kForward>(P, kf, from_smem, last); break;
-        case 3: xpass<KL, 3, kForward>(P, kf, from_smem, last); break;
-        default: xpass<KL, 4, kForward>(P, kf, from_smem, last); break;
-      }
-    } else {
-      switch (rr) {
-        case 1: xpass<KL, 1, kForward>(P, kf, from_smem, to_smem); break;
-        case 2: xpass<KL, 2, kForward>(P, kf, from_smem, to_smem); break;
-        case 3: xpass<KL, 3, kForward>(P, kf, from_smem, to_smem); break;
-        default: xpass<KL, 4, kForward>(P, kf, from_smem, to_smem); break;
-      }
-    }
-    if (!is_last || kLastToSmem) __syncthreads();
+  auto short_pass = [&](auto src, auto dst) {  // stages 8 and up
+    if (lgP == 10) xpass<KL, 2, kForward>(P, 8, src, dst);
+    else xpass<KL, 3, kForward>(P, 8, src, dst);
+  };
+  if (kForward) short_pass(first, to_smem);
+  else xpass<KL, 4, kForward>(P, 0, first, to_smem);
+  __syncthreads();
+  xpass<KL, 4, kForward>(P, 4, from_smem, to_smem);
+  __syncthreads();
+  if constexpr (kForward) {
+    if constexpr (kLastToSmem) xpass<KL, 4, kForward>(P, 0, from_smem, to_smem);
+    else xpass<KL, 4, kForward>(P, 0, from_smem, last);
+  } else {
+    short_pass(from_smem, last);
   }
+  if (kLastToSmem) __syncthreads();
 }
 
 // Real rows -> half spectrum along x (arguments and results as k_mix_rows_r2c).
@@ -327,21 +297,6 @@ __global__ void __launch_bounds__(kFftThreads) k_xfft_rows_c2r(const float2 *__r
 // 512), 128x128x192 123 -> 119, 64x64x128 41 both.  24 KB give 327 and 559, 64 KB 331 and
 // 566.  Asking for whole rows or for the rows of later blocks evicts the vectors (adjoint
 // 256x256x384 547, 652), loading S^ as evict-first loses what L2 keeps of it (forward 349).
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t splat2(float v) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
-  return r;
-}
 
 // Sums over the quarters of a warp's [output][member] sums; quarter ph keeps member ph.
 __device__ __forceinline__ void sum_quarters(const uint64_t (&acc)[4][4], int ph, uint64_t (&c)[4]) {
@@ -351,11 +306,11 @@ __device__ __forceinline__ void sum_quarters(const uint64_t (&acc)[4][4], int ph
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j)
-      b[i][j] = add2(hi ? acc[i][2 + j] : acc[i][j],
+      b[i][j] = f2_add(hi ? acc[i][2 + j] : acc[i][j],
                      __shfl_xor_sync(0xffffffffu, hi ? acc[i][j] : acc[i][2 + j], 16));
 #pragma unroll
   for (int i = 0; i < 4; ++i)
-    c[i] = add2(odd ? b[i][1] : b[i][0], __shfl_xor_sync(0xffffffffu, odd ? b[i][0] : b[i][1], 8));
+    c[i] = f2_add(odd ? b[i][1] : b[i][0], __shfl_xor_sync(0xffffffffu, odd ? b[i][0] : b[i][1], 8));
 }
 // Eight FP32 values' exponents below the largest.
 __device__ __forceinline__ bool all_finite(const uint64_t (&c)[4]) {
@@ -413,11 +368,11 @@ __global__ void __launch_bounds__(32 * kApplyWarps, 4)
     };
     auto add = [&](int e, float4 v) {
       const ulonglong2 h0 = X[2 * e], h1 = X[2 * e + 1];
-      const uint64_t h[4] = {h0.x, h0.y, h1.x, h1.y}, s[4] = {splat2(v.x), splat2(v.y), splat2(v.z), splat2(v.w)};
+      const uint64_t h[4] = {h0.x, h0.y, h1.x, h1.y}, s[4] = {f2_splat(v.x), f2_splat(v.y), f2_splat(v.z), f2_splat(v.w)};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma2(s[i], h[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) acc[i][j] = f2_fma(s[i], h[j], acc[i][j]);
     };
     // the next step's loads are issued before this step's products
     float4 v[kUnroll], next[kUnroll];

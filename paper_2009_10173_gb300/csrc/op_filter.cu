@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "fft_dev.cuh"
+#include "f32x2.cuh"
 #include "fft_mixed.cuh"
 #include "internal.cuh"
 
@@ -63,39 +64,6 @@ constexpr int kFirThreads = 256;
 constexpr int kFirMaxSize = 8192;  // largest transform: 144 KiB of shared memory for one line pair
 
 size_t fir_smem(int NF, int KP) { return sizeof(ulonglong2) * ((size_t)KP * NF + NF / 8); }
-
-// Packed FP32 pairs (two lanes of one 64-bit register) and their arithmetic.
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {  // a b + c
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_splat(float v) { return f2_pack(v, v); }
-__device__ __forceinline__ float2 f2_unpack(uint64_t v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
 
 // The same point of two complex lines c and c + 1: re = (re_c, re_c+1),
 // im = (im_c, im_c+1).  Every operation below acts on both lines at once.
@@ -385,7 +353,6 @@ __global__ void __launch_bounds__(kFirThreads, 2) k_fir_lines(const float *x, fl
 // The same operations for the transforms of fft_mixed.cuh.
 __device__ __forceinline__ Cx2 cadd(Cx2 a, Cx2 b) { return x_add(a, b); }
 __device__ __forceinline__ Cx2 csub(Cx2 a, Cx2 b) { return x_sub(a, b); }
-__device__ __forceinline__ uint64_t f2_neg(uint64_t a) { return a ^ 0x8000000080000000ull; }
 __device__ __forceinline__ Cx2 cneg(Cx2 a) { return Cx2{f2_neg(a.re), f2_neg(a.im)}; }
 __device__ __forceinline__ Cx2 cadd_i(Cx2 a, Cx2 b) { return Cx2{f2_sub(a.re, b.im), f2_add(a.im, b.re)}; }
 __device__ __forceinline__ Cx2 csub_i(Cx2 a, Cx2 b) { return Cx2{f2_add(a.re, b.im), f2_sub(a.im, b.re)}; }

@@ -43,6 +43,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "f32x2.cuh"
 #include "internal.cuh"
 
 using namespace oam;
@@ -58,26 +59,6 @@ constexpr int kFlush = 8;        // a warp's taps per first-level sum
 constexpr int kMaxStrip = 352;   // staged positions a block takes on run-on tiles
 constexpr int kTableR = 31;      // largest half window whose tap table is copied to shared memory
 
-__device__ __forceinline__ uint64_t pack2(float x, float y) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(uint64_t v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
 __device__ __forceinline__ void copy16_async(void *dst, const void *src, bool real) {  // zeros unless real
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
                "r"(real ? 16 : 0)
@@ -140,14 +121,14 @@ __device__ __forceinline__ void multiply(const float *F, const float *S, int ka,
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const float4 sv = *reinterpret_cast<const float4 *>(S + (kk + u) * kTile);
-      const uint64_t s2[4] = {pack2(sv.x, sv.x), pack2(sv.y, sv.y), pack2(sv.z, sv.z), pack2(sv.w, sv.w)};
+      const uint64_t s2[4] = {f2_pack(sv.x, sv.x), f2_pack(sv.y, sv.y), f2_pack(sv.z, sv.z), f2_pack(sv.w, sv.w)};
       const ulonglong2 f0 = *reinterpret_cast<const ulonglong2 *>(F + (kk + u) * kM);
       const ulonglong2 f1 = *reinterpret_cast<const ulonglong2 *>(F + (kk + u) * kM + 4);
       const uint64_t f2[4] = {f0.x, f0.y, f1.x, f1.y};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) a1[i][j] = fma2(f2[i], s2[j], a1[i][j]);
+        for (int j = 0; j < 4; ++j) a1[i][j] = f2_fma(f2[i], s2[j], a1[i][j]);
     }
   }
 }
@@ -217,18 +198,18 @@ __global__ void __launch_bounds__(kOneThreads, 4)
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const float4 f = *reinterpret_cast<const float4 *>(X + (pg + 4 * i) * kOneRow + 4 * q);
-        const uint64_t f2[4] = {pack2(f.x, f.x), pack2(f.y, f.y), pack2(f.z, f.z), pack2(f.w, f.w)};
+        const uint64_t f2[4] = {f2_pack(f.x, f.x), f2_pack(f.y, f.y), f2_pack(f.z, f.z), f2_pack(f.w, f.w)};
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          acc[i][0] = fma2(f2[u], w[u].x, acc[i][0]);
-          acc[i][1] = fma2(f2[u], w[u].y, acc[i][1]);
+          acc[i][0] = f2_fma(f2[u], w[u].x, acc[i][0]);
+          acc[i][1] = f2_fma(f2[u], w[u].y, acc[i][1]);
         }
       }
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      sum[i][0] = add2(sum[i][0], acc[i][0]);
-      sum[i][1] = add2(sum[i][1], acc[i][1]);
+      sum[i][0] = f2_add(sum[i][0], acc[i][0]);
+      sum[i][1] = f2_add(sum[i][1], acc[i][1]);
     }
   }
   __syncthreads();
@@ -246,12 +227,12 @@ __global__ void __launch_bounds__(kOneThreads, 4)
 #pragma unroll
     for (int w = 0; w < 3; ++w) {
       const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(X + (w * kPos + pg + 4 * i) * kTile + 4 * ng);
-      sum[i][0] = add2(sum[i][0], v.x);
-      sum[i][1] = add2(sum[i][1], v.y);
+      sum[i][0] = f2_add(sum[i][0], v.x);
+      sum[i][1] = f2_add(sum[i][1], v.y);
     }
     if (o0 + pg + 4 * i >= positions) continue;
     float *dst = out + (o0 + pg + 4 * i) * s.out_len + n;
-    const float2 a = unpack2(sum[i][0]), b = unpack2(sum[i][1]);
+    const float2 a = f2_unpack(sum[i][0]), b = f2_unpack(sum[i][1]);
     if (s.out_len % 4 == 0) {
       if (n < s.out_len) *reinterpret_cast<float4 *>(dst) = make_float4(a.x, a.y, b.x, b.y);
     } else {
@@ -407,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       // [warp][position][2 outputs of each group of four]
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float2 u = unpack2(a2[i][2 * half]), v = unpack2(a2[i][2 * half + 1]);
+        const float2 u = f2_unpack(a2[i][2 * half]), v = f2_unpack(a2[i][2 * half + 1]);
         *reinterpret_cast<float2 *>(F + (8 * pg + 2 * i) * 16 + 2 * ng) = make_float2(u.x, v.x);
         *reinterpret_cast<float2 *>(F + (8 * pg + 2 * i + 1) * 16 + 2 * ng) = make_float2(u.y, v.y);
         a2[i][2 * half] = a2[i][2 * half + 1] = 0;
@@ -491,7 +472,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         for (int i = 0; i < 4; ++i)
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            a2[i][j] = add2(a2[i][j], a1[i][j]);
+            a2[i][j] = f2_add(a2[i][j], a1[i][j]);
             a1[i][j] = 0;
           }
       }
@@ -581,7 +562,7 @@ __global__ void __launch_bounds__(kBlockPos, 4)
       float2 v[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        v[j] = unpack2(sum2[(4 * i + j) * kBlockPos]);
+        v[j] = f2_unpack(sum2[(4 * i + j) * kBlockPos]);
         sum2[(4 * i + j) * kBlockPos] = 0;
       }
 #pragma unroll
@@ -686,7 +667,7 @@ __global__ void __launch_bounds__(kBlockPos, 4)
           for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              sum2[(4 * i + j) * kBlockPos] = add2(sum2[(4 * i + j) * kBlockPos], a1[i][j]);
+              sum2[(4 * i + j) * kBlockPos] = f2_add(sum2[(4 * i + j) * kBlockPos], a1[i][j]);
               a1[i][j] = 0;
             }
         }

@@ -57,6 +57,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "f32x2.cuh"
 #include "internal.cuh"
 #include "tc_ptx.cuh"
 
@@ -168,25 +169,6 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
 // the same MMA time while its fold work is the same for every pair.
 __device__ __forceinline__ int a_of(int j, int R) { return (j & 1) ? R - (j >> 1) : (j >> 1); }
 
-// Packed FP32 pairs (two lanes of one 64-bit register) and their arithmetic.
-__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t sub_f32x2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t pack_f32x2(float x, float y) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ void unpack_f32x2(uint64_t v, float &x, float &y) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-}
 
 // Staged FP32 rows are 128 bytes with the TMA's 128-byte swizzle: 16-byte
 // chunk c of row r sits at chunk c ^ (r & 7).  Read the 8 elements of
@@ -207,16 +189,11 @@ __device__ __forceinline__ void add_row(const float *strip, int row, int q, uint
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const ulonglong2 u = r2[(2 * q + i) ^ (row & 7)];
-    v[2 * i] = add_f32x2(v[2 * i], u.x);
-    v[2 * i + 1] = add_f32x2(v[2 * i + 1], u.y);
+    v[2 * i] = f2_add(v[2 * i], u.x);
+    v[2 * i + 1] = f2_add(v[2 * i + 1], u.y);
   }
 }
 
-__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
 
 // 2^e, -126 <= e <= 127.
 __device__ __forceinline__ float pow2(int e) { return __int_as_float((e + 127) << 23); }
@@ -233,14 +210,12 @@ __device__ __forceinline__ int scale_exp(float top) {
 __device__ __forceinline__ void split_f16(const uint64_t (&v)[4], uint32_t (&hv)[4], uint32_t (&lv)[4]) {
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    float x, y;
-    unpack_f32x2(v[e], x, y);
-    x = __uint_as_float(__float_as_uint(x) & 0xffffe000u);
-    y = __uint_as_float(__float_as_uint(y) & 0xffffe000u);
+    const float2 u = f2_unpack(v[e]);
+    const float x = __uint_as_float(__float_as_uint(u.x) & 0xffffe000u);
+    const float y = __uint_as_float(__float_as_uint(u.y) & 0xffffe000u);
     const __half2 h2 = __floats2half2_rn(x, y);
-    float lx, ly;
-    unpack_f32x2(sub_f32x2(v[e], pack_f32x2(x, y)), lx, ly);
-    const __half2 l2 = __floats2half2_rn(lx, ly);
+    const float2 rest = f2_unpack(f2_sub(v[e], f2_pack(x, y)));
+    const __half2 l2 = __floats2half2_rn(rest.x, rest.y);
     hv[e] = *reinterpret_cast<const uint32_t *>(&h2);
     lv[e] = *reinterpret_cast<const uint32_t *>(&l2);
   }
@@ -264,7 +239,7 @@ __device__ __forceinline__ void fold_item(const float *X1, int m, int R, int a, 
 #pragma unroll
   for (int i = 0; i < NQ; ++i) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) f[i][e] = mul_f32x2(f[i][e], sc);
+    for (int e = 0; e < 4; ++e) f[i][e] = f2_mul(f[i][e], sc);
     uint32_t hv[4], lv[4];
     split_f16(f[i], hv, lv);
     const int hb = E == 8 ? 0 : 16 * (i >> 1) + 4 * (i & 1);  // word of the quarter's first hi pair
@@ -566,7 +541,7 @@ __global__ void __launch_bounds__(96 + 32 * FW, 1)
 #pragma unroll 8
     for (int i = pm; i <= pm + 2 * R; ++i) top = max(top, (int)line_exp[i]);
     const int ef = min(126, 140 - top);  // the fold doubles: into [2^14, 2^15), below FP16's largest 65504
-    const uint64_t sc = pack_f32x2(pow2(ef), pow2(ef));
+    const uint64_t sc = f2_pack(pow2(ef), pow2(ef));
     int k = 0;
     uint32_t lap = 0;
     for (int st = 0; st < p.stages && ok; ++st) {
