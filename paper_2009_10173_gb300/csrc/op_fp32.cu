@@ -709,10 +709,10 @@ oam_status run(const oam_model *m, bool fwd, const float *in, float *out, cudaSt
   // 705; five: 96x96x128 31x31 taps 1498, 1818, 128x128x64 11x11 taps 218, 358.
   const long long busy = fwd ? (m->n_hi - m->n_lo + kTile - 1) / kTile : L.tiles;
   const int sms = std::max(1, m->sm_count);
-  // Inputs of one or two chunks leave the warps nothing to share but their set-up (from one
+  // Inputs of one chunk leave the warps nothing to share but their set-up (from one
   // block per SM on: 128x128x4 forward, 3x3 taps 15, 49; 9x9 taps 42, 70).
   const long long blocks = ((long long)g.px * g.py + kBlockPos - 1) / kBlockPos * busy;
-  const bool block = blocks > (s.len <= 2 * kChunk ? 1LL : 2LL) * sms;
+  const bool block = blocks > (s.len <= kChunk ? 1LL : 2LL) * sms;
   // Tiles run on over scan rows (no idle positions) unless the padding between
   // many short rows makes the strip too long; then every tile stays in its row.
   const int tile = block ? kBlockPos : kPos;
