@@ -122,10 +122,8 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>())
     }
   }
   __syncthreads();
-  for (int u = threadIdx.x; u < Q; u += blockDim.x) {
-    unsigned *top = s.vmax + (size_t)u * s.px + x;
-    if (umax[u] > __ldcg(top)) atomicMax(top, umax[u]);
-  }
+  for (int u = threadIdx.x; u < Q; u += blockDim.x)
+    if (umax[u]) atomicMax(s.vmax + (size_t)u * s.px + x, umax[u]);
 }
 
 // kVec: output rows are a whole number of float2 from an 8-byte boundary.
@@ -141,9 +139,10 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>(), R1 >= 15 && R2 <= 
   float *col = out + (size_t)x * s.out_len + ob;
   const size_t stride = (size_t)s.px * s.out_len;
   const int cols = min(kLineCh, s.out_len - ob);
+  const bool spoiled = __ldg(s.spoiled) != 0;
   // this application's marks are grown: clear them for the next
   if (blockIdx.x == 0 && blockIdx.z == 0) {
-    const int planes = *s.spoiled ? s.planes : 1;
+    const int planes = spoiled ? s.planes : 1;
     for (int i = threadIdx.x; i < planes * s.words; i += blockDim.x)
       s.marks[((size_t)(i / s.words) * s.px + x) * s.words + i % s.words] = 0;
     for (int i = threadIdx.x; i < Q; i += blockDim.x) s.vmax[(size_t)i * s.px + x] = 0;
@@ -162,7 +161,7 @@ __global__ void __launch_bounds__(mix_threads<R1, R2, kKH>(), R1 >= 15 && R2 <= 
     const size_t at = (size_t)x * s.words + w0 + i, plane = (size_t)s.px * s.words;
     words[0][i] = __ldg(s.grown + at);
     unsigned bad = 0;
-    if (*s.spoiled)
+    if (spoiled)
       for (int b = 0; b < s.planes - 1; ++b)
         if (s.reach[b].x < z0 + kLineCh && s.reach[b].y > z0) bad |= __ldg(s.grown + (1 + b) * plane + at);
     words[1][i] = bad;
