@@ -432,7 +432,7 @@ def run_serve(args):
     shutil.rmtree(workdir, ignore_errors=True)
     line = {"metric": "served reconstructions: volumes/s and p50/p99 latency", "unit": "volumes/s",
             "value": max(r["volumes_per_s"] for r in results), "n_gpus": 1, "higher_is_better": True,
-            "dtype": "bf16" if prec == B.OAM_PREC_BF16X3 else "f32", "data": "synthetic",
+            "dtype": "fp16" if prec == B.OAM_PREC_BF16X3 else "f32", "data": "synthetic",
             "config": {"workload": "served: Poisson arrivals, sizes as the batched workload (scan 64-256^2, "
                                    "128-384 depths, 512-1024 samples, seeded sensors) plus 5 % 200x200x300 "
                                    "volumes; 30 LSQR + 50 FISTA (+20 power) each",
@@ -527,9 +527,10 @@ def run_ours(args, rank, world, acc=None):
                 raise
             prec = B.OAM_PREC_FP32
     prec_name = {B.OAM_PREC_FP32: "fp32 CUDA-core operators",
-                 B.OAM_PREC_BF16X3: "split-BF16 (hi*hi+hi*lo+lo*hi) tcgen05 operators, FP32 accumulate",
+                 B.OAM_PREC_BF16X3: "two-term 16-bit splits (FP16, hi*hi+hi*lo+lo*hi) on tcgen05, FP32 line "
+                                     "transforms and accumulation",
                  B.OAM_PREC_FFT: "FP32 lateral-FFT form of the same operators (correlation theorem on a "
-                                 "256x256 zero-padded grid, real slab spectrum per frequency orbit)"}[prec]
+                                 "240x240 zero-padded grid, real slab spectrum per frequency orbit)"}[prec]
 
     # synthetic input for this rank: vessel tree + microspheres, clean signals by A, 20 dB noise
     from paper_2009_10173_gb300 import replicas
@@ -637,7 +638,7 @@ def run_ours(args, rank, world, acc=None):
         sweep_ms, single_ms = e[0].elapsed_time(e[1]), e[1].elapsed_time(e[2])
         fir_size = mm.info.filter_size
         mm.close()
-        return {"bandpass_filter": {"band_hz": [0.5e6, 80e6], "taps": 2 * FIR_HALF + 1, "transform": fir_size,
+        return {"bandpass_filter": {"band_hz": [0.5e6, 80e6], "taps": 2 * FIR_HALF + 1, "filter_size": fir_size,
                                     "ms": fir_ms, "roofline": {"bound": "hbm", "kernel": "k_fir_mixed",
                                                                "achieved": gbs, "peak": hbm, "unit": "GB/s",
                                                                "frac": gbs / hbm, "bytes_per_launch": fir_bytes,
@@ -740,7 +741,7 @@ def run_ours(args, rank, world, acc=None):
                 "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (of measured)"}
     line = {"metric": METRIC, "value": value, "unit": "volumes/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": per_step, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "bf16" if prec == B.OAM_PREC_BF16X3 else "f32", "data": "synthetic",
+            "vs_baseline": None, "dtype": "fp16" if prec == B.OAM_PREC_BF16X3 else "f32", "data": "synthetic",
             "config": config_dict(prec_name),
             "p50_ms": statistics.median(step_ms), "p99_ms": float(np.percentile(step_ms, 99)),
             "op_tflops_algorithmic": OPS_PER_STEP * info.flops_per_op / (per_step * 1e-3) / 1e12,

@@ -84,8 +84,10 @@ typedef enum {
                           reconstruction based on scanning symmetries), restated
                           exactly by the correlation theorem on a zero-padded
                           P x P grid (P >= max(py, px) + R, an even size with factors
-                          2, 3 and 5 up to 512, else 1024 or 2048), with the slab's real lateral spectrum stored once
-                          per frequency orbit */
+                          2, 3 and 5 up to 512, else 1024 or 2048), with the slab's real
+                          lateral spectrum stored once per frequency orbit; non-finite
+                          inputs spread over every position, in the samples (depths) that
+                          their bands and those of the neighbour channel hold */
 } oam_precision;
 
 /* How Eq. 1 is discretised into the model slab.
@@ -152,7 +154,8 @@ typedef struct {
   double op_bytes;     /* OAM_PREC_FFT: device bytes read + written per application (the
                           spectral slab dominates); 0 otherwise */
   int32_t filter_half_len; /* L of the band-pass filter set by oam_model_set_filter, -1: none */
-  int32_t filter_size;     /* its transform length NF (0: none) */
+  int32_t filter_size;     /* smallest power of two NF that holds its convolution (0: none); the
+                              device's transform may be shorter */
 } oam_model_info;
 
 /* Build the model slab on the device (Methods: Forward modeling, Eqs. 1-4;
@@ -236,7 +239,8 @@ oam_status oam_bandpass_taps(double f_lo_hz, double f_hi_hz, double fs_hz, int32
  * the solvers, batches and autotuning) for the even FIR taps[0..half_len]
  * (host memory, copied).  taps == NULL or half_len < 0 removes the filter.
  * info.filter_size is the smallest power of two NF >= nt + min(L, nt-1) (the
- * device's transform may be shorter, but not than that sum); NF > 8192 is rejected (OAM_ERR_INVALID_ARG), as are non-finite taps.
+ * device's transform may be shorter, but not than that sum); NF > 8192 is
+ * rejected (OAM_ERR_INVALID_ARG), as are non-finite taps.
  * Allocates the filter's spectrum and one signal-sized staging buffer (owned
  * by the model, counted in device_bytes) on `stream` and synchronises it.
  * A batch that uses the model records its graph again on its next run. */
