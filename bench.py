@@ -30,11 +30,11 @@ LSQR_ITERS, FISTA_ITERS, POWER_ITERS, LAMBDA_REL = 50, 100, 20, 1e-3
 # operator applications per step: LSQR 1 + 2*50; FISTA 2*20 power + 1 lambda + 2*100
 OPS_PER_STEP = (1 + 2 * LSQR_ITERS) + (2 * POWER_ITERS + 1 + 2 * FISTA_ITERS)
 FP32_LANES_PER_SM = 128
-# DRAM bytes per application of the operators on this workload, from a capture of
-# all their launches (dram__bytes_read.sum + dram__bytes_write.sum); None until the
-# current kernels are captured.
-TC_TRAFFIC_BYTES = None
-FFT_TRAFFIC_BYTES = None
+# DRAM bytes per application of the operators on this workload (dram__bytes_read.sum +
+# dram__bytes_write.sum over their launches; profiles/split_form_kernels.md and
+# profiles/lateral_fft_kernels.md).  Set to None when the kernels change.
+TC_TRAFFIC_BYTES = {"forward": 1070.3e6, "adjoint": 946.1e6}
+FFT_TRAFFIC_BYTES = 1289.1e6
 # Band-pass filter along time: half length of the 0.5-80 MHz FIR, and the DRAM
 # bytes of one application (None as above).
 FIR_HALF = 511
