@@ -36,9 +36,9 @@ FP32_LANES_PER_SM = 128
 TC_TRAFFIC_BYTES = {"forward": 1070.3e6, "adjoint": 946.1e6}
 FFT_TRAFFIC_BYTES = 1289.1e6
 # Band-pass filter along time: half length of the 0.5-80 MHz FIR, and the DRAM
-# bytes of one application (None as above).
+# bytes of one application (profiles/operator_and_filter_kernels.md).
 FIR_HALF = 511
-FIR_TRAFFIC_BYTES = None
+FIR_TRAFFIC_BYTES = 163.9e6 + 117.2e6
 
 
 def parse():
