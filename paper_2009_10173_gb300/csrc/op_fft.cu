@@ -393,7 +393,8 @@ __global__ void __launch_bounds__(32 * kApplyWarps, 4)
     sum_quarters(acc, ph, c);
     // A lane added zeros for the elements that do not meet its group; where the sums are
     // not finite they are taken again without those elements, so that a non-finite one
-    // reaches no sample beyond its band's groups.
+    // reaches no sample beyond its band's groups.  (1 to 3 us of an application; predicated
+    // products cost 10 %, a look at the vectors while they are loaded 2 to 4 %.)
     if (__any_sync(0xffffffffu, !all_finite(c))) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)

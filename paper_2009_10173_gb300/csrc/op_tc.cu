@@ -22,7 +22,7 @@
 // products than the correlation over both axes at a 61x61 window, for a slab
 // (P/2 + 1) / (R + 1) = 4 times the size at 200 lines and two line transforms.
 // Measured on a GB300 against that form (one application): 200x200x300 forward
-// 5.78 -> 0.45 ms (k_corr_line 0.34), adjoint 5.71 -> 0.45 ms, 96x96x192 forward 0.86 ->
+// 5.78 -> 0.46 ms (k_corr_line 0.34), adjoint 5.71 -> 0.46 ms, 96x96x192 forward 0.86 ->
 // 0.10 ms.
 //
 // Mirror folding.  S_v[a] = S_v[-a], so the two mirrored taps share one slab tile
